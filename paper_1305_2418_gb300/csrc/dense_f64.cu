@@ -7,6 +7,8 @@
 // pipe, not HBM, bounds these kernels.
 #include <algorithm>
 
+#include "colour_split.cuh"
+#include "dfloat.cuh"
 #include "mgfr_internal.cuh"
 
 namespace {
@@ -246,25 +248,8 @@ __global__ void __launch_bounds__(64) k_coarse(double* __restrict__ ug, double* 
   Eg[t] = E[t];
 }
 
-template <int MODE>  // 0: residual of (u,E,f); 1: plain vector x (in u)
-__global__ void __launch_bounds__(BS) k_norm(const double* __restrict__ u,
-                                             const double* __restrict__ E,
-                                             const double* __restrict__ f, int lg, long long n,
-                                             Model m, double ih2, double* __restrict__ partials) {
-  double ss = 0.0, mx = 0.0;
-  const long long stride = (long long)gridDim.x * blockDim.x;
-  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n; t += stride) {
-    double r;
-    if (MODE == 0) {
-      const int N = 1 << lg;
-      const int k = (int)(t & (N - 1)), j = (int)((t >> lg) & (N - 1)), i = (int)(t >> (2 * lg));
-      r = f[t] - Lpoint(u, E, i, j, k, lg, m, ih2);
-    } else {
-      r = u[t];
-    }
-    ss = fma(r, r, ss);
-    mx = fmax(mx, fabs(r));
-  }
+// block sums of (sum, max) into partials[2 block], [2 block + 1]
+__device__ __forceinline__ void block_norms(double ss, double mx, double* __restrict__ partials) {
   __shared__ double s1[BS / 32], s2[BS / 32];
   for (int o = 16; o > 0; o >>= 1) {
     ss += __shfl_xor_sync(0xffffffffu, ss, o);
@@ -284,6 +269,69 @@ __global__ void __launch_bounds__(BS) k_norm(const double* __restrict__ u,
     partials[2 * blockIdx.x] = a;
     partials[2 * blockIdx.x + 1] = b;
   }
+}
+
+template <int MODE>  // 0: residual of (u,E,f); 1: plain vector x (in u)
+__global__ void __launch_bounds__(BS) k_norm(const double* __restrict__ u,
+                                             const double* __restrict__ E,
+                                             const double* __restrict__ f, int lg, long long n,
+                                             Model m, double ih2, double* __restrict__ partials) {
+  double ss = 0.0, mx = 0.0;
+  const long long stride = (long long)gridDim.x * blockDim.x;
+  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n; t += stride) {
+    double r;
+    if (MODE == 0) {
+      const int N = 1 << lg;
+      const int k = (int)(t & (N - 1)), j = (int)((t >> lg) & (N - 1)), i = (int)(t >> (2 * lg));
+      r = f[t] - Lpoint(u, E, i, j, k, lg, m, ih2);
+    } else {
+      r = u[t];
+    }
+    ss = fma(r, r, ss);
+    mx = fmax(mx, fabs(r));
+  }
+  block_norms(ss, mx, partials);
+}
+
+// The residual of the FP64 iterate as the right-hand side of the FP32
+// deviation cycle (colour-split r32, u32 = u), and its norms as k_norm<0>
+// forms them.  One pass per V-cycle: FP64 pipe bound, about 32 FP64
+// instructions per cell against about 400 of an FP64 V-cycle.
+__global__ void __launch_bounds__(BS) k_resid_dev(const double* __restrict__ u,
+                                                  const double* __restrict__ E,
+                                                  const double* __restrict__ f, int lg, Model m,
+                                                  double ih2, float* __restrict__ r32,
+                                                  float* __restrict__ u32,
+                                                  double* __restrict__ partials) {
+  double ss = 0.0;
+  long long mx = 0;  // bits of max |r| (ordered like the values)
+  const unsigned n = 1u << (3 * lg);
+  const int M = (1 << lg) - 1;
+  for (unsigned t = blockIdx.x * blockDim.x + threadIdx.x; t < n; t += gridDim.x * blockDim.x) {
+    const int k = (int)(t & M), j = (int)((t >> lg) & M), i = (int)(t >> (2 * lg));
+    const double r = f[t] - Lpoint(u, E, i, j, k, lg, m, ih2);
+    const unsigned p = pdx(i, j, k, lg);
+    r32[p] = f_from_double_bits(r);
+    u32[p] = f_from_double_bits(u[t]);
+    ss = fma(r, r, ss);
+    const long long b = __double_as_longlong(r) & 0x7fffffffffffffffLL;
+    mx = b > mx ? b : mx;
+  }
+  block_norms(ss, __longlong_as_double(mx), partials);
+}
+
+// u += sign e (FP32 correction; a value that is not finite is left out, the
+// residual then shows that the cycle gained nothing), E = e^u
+__global__ void __launch_bounds__(BS) k_apply_dev(double* __restrict__ u, double* __restrict__ E,
+                                                  const float* __restrict__ e32, int lg,
+                                                  float sign) {
+  const unsigned t = blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= (1u << (3 * lg))) return;
+  const int M = (1 << lg) - 1;
+  const float e = e32[pdx((int)(t >> (2 * lg)), (int)((t >> lg) & M), (int)(t & M), lg)];
+  const double v = u[t] + (isfinite(e) ? d_from_float_bits(sign * e) : 0.0);
+  u[t] = v;
+  E[t] = exp(v);
 }
 
 __global__ void k_finish(const double* __restrict__ partials, int nparts, double* __restrict__ out) {
@@ -370,6 +418,17 @@ void resid_norm(DenseLevel& L, const Model& m, double* partials, int nparts, dou
   int nb = (int)std::min<long long>(nparts, nblocks(L.n, BS));
   k_norm<0><<<nb, BS, 0, s>>>(L.u, L.E, L.f, L.lg, L.n, m, L.ih2, partials);
   k_finish<<<1, 256, 0, s>>>(partials, nb, out);
+}
+
+void resid_dev(DenseLevel& L, const Model& m, double* partials, int nparts, double* out,
+               cudaStream_t s) {
+  const int nb = (int)std::min<long long>(nparts, nblocks(L.n, BS));
+  k_resid_dev<<<nb, BS, 0, s>>>(L.u, L.E, L.f, L.lg, m, L.ih2, L.r32, L.u32, partials);
+  k_finish<<<1, 256, 0, s>>>(partials, nb, out);
+}
+
+void apply_dev(DenseLevel& L, float sign, cudaStream_t s) {
+  k_apply_dev<<<nblocks(L.n, BS), BS, 0, s>>>(L.u, L.E, L.e32, L.lg, sign);
 }
 
 void norm(const double* x, long long n, double* partials, int nparts, double* out, cudaStream_t s) {

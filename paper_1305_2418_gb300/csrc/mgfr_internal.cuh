@@ -42,8 +42,9 @@ struct DenseLevel {
   double *u = nullptr, *E = nullptr, *f = nullptr, *uold = nullptr;
   // FP32 nonlinear FAS (mixed precision, phase A)
   float *u32 = nullptr, *f32 = nullptr, *uold32 = nullptr;
-  // FP32 linear multigrid on the Jacobian system (mixed precision, phase B)
-  float *e32 = nullptr, *r32 = nullptr, *w32 = nullptr;
+  // FP32 correction and right-hand side: the linear multigrid on the Jacobian
+  // system (mixed form, phase B) and the deviation cycles of the FP64 form
+  float *e32 = nullptr, *r32 = nullptr;
   // multigrid mask of partial-level solves (Sec. 3.3): only cells with
   // mask > mthr are relaxed; nullptr = all cells.
   const float* mask = nullptr;
@@ -79,6 +80,12 @@ void resid_norm(DenseLevel& L, const Model& m, double* partials, int nparts, dou
 // sum x^2 and max|x| into out[0], out[1] (device).
 void norm(const double* x, long long n, double* partials, int nparts, double* out, cudaStream_t s);
 void force(const DenseLevel& L, const Model& m, double* fr, double* acc, cudaStream_t s);
+// r = f - L(u): norms as resid_norm, and the deviation problem of the FP32
+// cycle (mg32.cuh, MG_DEV): r32 = r, u32 = u
+void resid_dev(DenseLevel& L, const Model& m, double* partials, int nparts, double* out,
+               cudaStream_t s);
+// u += sign e32 (where finite), E = e^u
+void apply_dev(DenseLevel& L, float sign, cudaStream_t s);
 }  // namespace f64
 
 // ---- FP32 dense kernels, mixed precision (dense_f32.cu) -------------------
@@ -88,15 +95,6 @@ void force(const DenseLevel& L, const Model& m, double* fr, double* acc, cudaStr
 namespace f32 {
 // C-order FP64 x -> colour-split FP32 y on level L's grid
 void from64(const double* x, float* y, const DenseLevel& L, cudaStream_t s);
-void sweep(DenseLevel& L, const Model& m, int colour, float step_cap, cudaStream_t s);
-void restrict_resid(DenseLevel& F, DenseLevel& C, const Model& m, double* partials, int nparts,
-                    cudaStream_t s);
-void fas_rhs(DenseLevel& C, const Model& m, cudaStream_t s);
-void prolong_corr(DenseLevel& F, DenseLevel& C, int linear, cudaStream_t s);
-void coarse_solve(DenseLevel& C, const Model& m, float step_cap, int max_sweeps, cudaStream_t s);
-// FP32 residual norms of the FP32 iterate (sum r^2, max|r|) into out.
-void norm32(DenseLevel& L, const Model& m, double* partials, int nparts, double* out,
-            cudaStream_t s);
 // Phase B.  From to_df until state_to_fp64, L.u and L.E hold the iterate and
 // e^u as double-float pairs (hi + lo floats in each 8-byte slot).
 // FP64-accurate residual in double-float (fdf: f as pairs, see f_to_df);
@@ -104,12 +102,6 @@ void norm32(DenseLevel& L, const Model& m, double* partials, int nparts, double*
 // max|r|) into out.
 void resid_df(DenseLevel& L, const double* fdf, const Model& m, double* partials, int nparts,
               double* out, cudaStream_t s);
-// Linear Gauss-Seidel on J(u32) e = r (J: Jacobian of L at u32).
-void lin_sweep(DenseLevel& L, const Model& m, int colour, cudaStream_t s);
-void lin_restrict(DenseLevel& F, DenseLevel& C, const Model& m, cudaStream_t s);
-void lin_prolong(DenseLevel& F, DenseLevel& C, int linear, cudaStream_t s);
-void lin_coarse(DenseLevel& C, const Model& m, int sweeps, cudaStream_t s);
-void zero(float* x, long long n, cudaStream_t s);
 // u += clamp(e, cap); E = e^u (double-float)
 void apply_corr(DenseLevel& L, double cap, cudaStream_t s);
 // u = u32, E = e^u as double-float pairs
@@ -136,10 +128,11 @@ struct mgfr_ctx {
   std::string err;
   DenseHier dh;
   double* host_scal = nullptr;  // pinned: norms read back by the host
-  // captured V-cycle graphs (FP64 / FP32 nonlinear / linear phase)
-  cudaGraphExec_t g_v64 = nullptr, g_v32 = nullptr, g_lin = nullptr;
-  char graph_key[256] = {0}, key32[256] = {0}, keylin[256] = {0};
-  long long updates_v64 = 0, updates_v32 = 0, updates_lin = 0;
+  // captured V-cycle graphs (FP64 all through / FP64 with FP32 corrections /
+  // FP32 nonlinear / linear phase)
+  cudaGraphExec_t g_v64 = nullptr, g_dev = nullptr, g_v32 = nullptr, g_lin = nullptr;
+  char graph_key[256] = {0}, keydev[256] = {0}, key32[256] = {0}, keylin[256] = {0};
+  long long updates_v64 = 0, updates_dev = 0, updates_v32 = 0, updates_lin = 0;
   void* amr = nullptr;    // refined hierarchy workspace (amr.cu)
   void* batch = nullptr;  // batched-solve workspace (batch.cu)
   void* unet = nullptr;   // learned initial guess network (unet.cu)
@@ -150,10 +143,10 @@ struct mgfr_ctx {
     cudaEvent_t a, b;
     long long cells;
   };
-  std::vector<ProfRec> prof[4];  // per graph: 0 v64, 1 v32, 2 lin, 3 refined
+  std::vector<ProfRec> prof[5];  // per graph: 0 v64, 1 v32, 2 lin, 3 refined, 4 dev
   std::vector<cudaEvent_t> evpool;
   int capturing = -1;            // graph being captured (-1: none)
-  long long graph_kernels[4] = {0, 0, 0, 0};  // kernel nodes per captured graph
+  long long graph_kernels[5] = {0, 0, 0, 0, 0};  // kernel nodes per captured graph
   long long launches = 0;        // kernels launched by the current call
   int u_prev_N = 0;              // grid of the solution held in dh.L[0].u (0: none)
   double* u_learn = nullptr;     // learned initial guess of a solve (MGFR_START_LEARNED)

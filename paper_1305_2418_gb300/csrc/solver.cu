@@ -13,6 +13,7 @@
 
 #include "mgfr_internal.cuh"
 #include "amr.cuh"
+#include "mg32.cuh"
 
 #define CLIGHT_OVER_H0 2997.92458
 
@@ -195,7 +196,7 @@ mgfr_status start_guess(mgfr_ctx* c, int N, const double* x, double dscale, cons
 static void free_dense(DenseHier& H) {
   for (int l = 0; l < MGFR_MAX_DENSE; ++l) {
     DenseLevel& L = H.L[l];
-    void* ps[] = {L.u, L.E, L.f, L.uold, L.u32, L.f32, L.uold32, L.e32, L.r32, L.w32};
+    void* ps[] = {L.u, L.E, L.f, L.uold, L.u32, L.f32, L.uold32, L.e32, L.r32};
     for (void* p : ps)
       if (p) cudaFree(p);
     L = DenseLevel();
@@ -207,12 +208,11 @@ static void free_dense(DenseHier& H) {
 }
 
 static void drop_graphs(mgfr_ctx* c) {
-  if (c->g_v64) cudaGraphExecDestroy(c->g_v64);
-  if (c->g_v32) cudaGraphExecDestroy(c->g_v32);
-  if (c->g_lin) cudaGraphExecDestroy(c->g_lin);
-  c->g_v64 = c->g_v32 = c->g_lin = nullptr;
-  c->graph_key[0] = c->key32[0] = c->keylin[0] = 0;
-  for (int g = 0; g < 3; ++g) prof_clear(c, g);
+  for (cudaGraphExec_t g : {c->g_v64, c->g_dev, c->g_v32, c->g_lin})
+    if (g) cudaGraphExecDestroy(g);
+  c->g_v64 = c->g_dev = c->g_v32 = c->g_lin = nullptr;
+  c->graph_key[0] = c->keydev[0] = c->key32[0] = c->keylin[0] = 0;
+  for (int g = 0; g < 5; ++g) prof_clear(c, g);
 }
 
 // Allocate the dense hierarchy N, N/2, ..., 4 (FP64 arrays always; FP32 ones
@@ -220,6 +220,8 @@ static void drop_graphs(mgfr_ctx* c) {
 static mgfr_status ensure_dense(mgfr_ctx* c, int N, bool mixed) {
   DenseHier& H = c->dh;
   if (H.N == N && (H.mixed || !mixed)) return MGFR_OK;
+  mgfr_status ps = mg32_prepare(c);
+  if (ps != MGFR_OK) return ps;
   drop_graphs(c);
   free_dense(H);
   c->u_prev_N = 0;
@@ -238,11 +240,11 @@ static mgfr_status ensure_dense(mgfr_ctx* c, int N, bool mixed) {
     MG_CK(c, cudaMalloc(&L.E, b8));
     MG_CK(c, cudaMalloc(&L.f, b8));
     if (l > 0) MG_CK(c, cudaMalloc(&L.uold, b8));
+    MG_CK(c, cudaMalloc(&L.u32, b4));
+    MG_CK(c, cudaMalloc(&L.e32, b4));
+    MG_CK(c, cudaMalloc(&L.r32, b4));
     if (mixed) {
-      MG_CK(c, cudaMalloc(&L.u32, b4));
       MG_CK(c, cudaMalloc(&L.f32, b4));
-      MG_CK(c, cudaMalloc(&L.e32, b4));
-      MG_CK(c, cudaMalloc(&L.r32, b4));
       if (l > 0) MG_CK(c, cudaMalloc(&L.uold32, b4));
     }
   }
@@ -344,6 +346,64 @@ static mgfr_status sync_read(mgfr_ctx* c) {
   return MGFR_OK;
 }
 
+static Mg32Par mg32_par(const Model& m, const mgfr_config& g, Mg32Op op) {
+  Mg32Par p;
+  p.aRt = (float)m.aRt;
+  p.aRt_np1 = (float)m.aRt_np1;
+  p.inv_np1 = (float)m.inv_np1;
+  p.cap = (float)g.step_cap;
+  p.n_pre = g.n_pre;
+  p.n_post = g.n_post;
+  p.linear = g.prolong_linear;
+  // the FP64 form solves its 4^3 grid to kCoarseRel64, the mixed form by a
+  // fixed number of sweeps
+  p.coarse_sweeps = op == MG_DEV ? 200 : 40;
+  p.coarse_rel = op == MG_DEV ? (float)kCoarseRel64 : 0.f;
+  return p;
+}
+
+// The FP32 V-cycles (mg32.cuh): phase A of the mixed form (MG_NL, u32, f32,
+// uold32), phase B (MG_LIN, e32, r32 at u32) and the corrections of the FP64
+// form (MG_DEV, e32, r32 at u32); the half-sweeps of the base level are timed
+// as family `fam`.
+struct CycleProf {
+  mgfr_ctx* c;
+  int fam;
+  long long cells;
+};
+
+static long long cycle32(mgfr_ctx* c, Mg32Op op, const Model& m, int fam, int n_cycles = 1) {
+  DenseHier& H = c->dh;
+  const mgfr_config& g = c->cfg;
+  Mg32Level L[MGFR_MAX_DENSE];
+  for (int l = 0; l < H.nlev; ++l) {
+    const DenseLevel& D = H.L[l];
+    L[l].lg = D.lg;
+    L[l].ih2 = (float)D.ih2;
+    L[l].h2 = (float)(D.h * D.h);
+    L[l].x = op == MG_NL ? D.u32 : D.e32;
+    L[l].r = op == MG_NL ? D.f32 : D.r32;
+    L[l].w = op == MG_NL ? D.uold32 : D.u32;
+  }
+  const Mg32Par p = mg32_par(m, g, op);
+  CycleProf pr{c, fam, H.L[0].n};
+  Mg32Hook hook;
+  hook.arg = &pr;
+  hook.begin = [](void* a) { prof_begin(((CycleProf*)a)->c, ((CycleProf*)a)->fam, ((CycleProf*)a)->cells); };
+  hook.end = [](void* a) { prof_end(((CycleProf*)a)->c); };
+  long long upd = 0;
+  for (int q = 0; q < n_cycles; ++q)
+    upd += mg32_cycle(op, L, H.nlev, p, c->s, g.profile ? &hook : nullptr);
+  return upd;
+}
+
+static void norm32(mgfr_ctx* c, const Model& m) {
+  DenseHier& H = c->dh;
+  const DenseLevel& D = H.L[0];
+  const Mg32Level L{D.lg, (float)D.ih2, (float)(D.h * D.h), D.u32, D.f32, nullptr};
+  mg32_norm(L, mg32_par(m, c->cfg, MG_NL), H.partials, H.nparts, H.scal, c->s);
+}
+
 // FP64 base-level solve on the already-filled hierarchy (f on level 0, u/E
 // initialised).  Fills stats (vcycles, updates, norms).
 mgfr_status dense_solve64(mgfr_ctx* c, const Model& m, double box, mgfr_stats* st) {
@@ -352,7 +412,7 @@ mgfr_status dense_solve64(mgfr_ctx* c, const Model& m, double box, mgfr_stats* s
   const mgfr_config& g = c->cfg;
   double* hs = c->host_scal;
   f64::norm(L0.f, L0.n, H.partials, H.nparts, H.scal + 2, c->s);
-  f64::resid_norm(L0, m, H.partials, H.nparts, H.scal, c->s);
+  f64::resid_dev(L0, m, H.partials, H.nparts, H.scal, c->s);
   c->launches += 4;
   MG_CK(c, cudaMemcpyAsync(hs, H.scal, 4 * sizeof(double), cudaMemcpyDeviceToHost, c->s));
   mgfr_status rs = sync_read(c);
@@ -363,35 +423,80 @@ mgfr_status dense_solve64(mgfr_ctx* c, const Model& m, double box, mgfr_stats* s
   const double target = g.tol_rel * (fn > 0.0 ? fn : r0);
   long long updates_per = 0;
   char key[256];
-  make_key(key, sizeof(key), "v64", H.N, box, m, g);
+  // the V-cycle with its correction in FP32: the same nonlinear V-cycle in the
+  // deviation from the iterate, which FP32 resolves to its own relative
+  // accuracy (the iterate, e^u, the residual and the test stay in FP64)
+  make_key(key, sizeof(key), "dev", H.N, box, m, g);
+  auto bodydev = [&]() {
+    cudaMemsetAsync(L0.e32, 0, sizeof(float) * (size_t)L0.n, c->s);
+    updates_per = cycle32(c, MG_DEV, m, 0);
+    f64::apply_dev(L0, 1.f, c->s);
+    f64::resid_dev(L0, m, H.partials, H.nparts, H.scal, c->s);
+    cudaMemcpyAsync(hs, H.scal, 2 * sizeof(double), cudaMemcpyDeviceToHost, c->s);
+  };
+  if (!c->g_dev || std::strcmp(key, c->keydev) != 0) {
+    if (c->g_dev) cudaGraphExecDestroy(c->g_dev);
+    c->g_dev = nullptr;
+    mgfr_status cs = capture(c, 4, &c->g_dev, bodydev);
+    if (cs != MGFR_OK) return cs;
+    std::strcpy(c->keydev, key);
+    c->updates_dev = updates_per;
+  }
+  // the V-cycle in FP64 throughout, for a start far from the solution, whose
+  // residual (kDevMax ||f|| and more; ||f|| at the zero start) FP32 cannot
+  // resolve against f, and from the first FP32 cycle that gains nothing (its
+  // correction is taken back)
+  constexpr double kDevMax = 2.0;
   auto body64 = [&]() {
     updates_per = 0;
     vcycle64(c, m, 0, updates_per);
     f64::resid_norm(L0, m, H.partials, H.nparts, H.scal, c->s);
     cudaMemcpyAsync(hs, H.scal, 2 * sizeof(double), cudaMemcpyDeviceToHost, c->s);
   };
-  if (!c->g_v64 || std::strcmp(key, c->graph_key) != 0) {
-    if (c->g_v64) cudaGraphExecDestroy(c->g_v64);
-    c->g_v64 = nullptr;
-    mgfr_status cs = capture(c, 0, &c->g_v64, body64);
-    if (cs != MGFR_OK) return cs;
-    std::strcpy(c->graph_key, key);
-    c->updates_v64 = updates_per;
-  }
+  const double ref = fn > 0.0 ? fn : r0;
+  bool dev_ok = true;
   double r = r0;
   int it = 0;
+  long long updates = 0;
   while (r > target && it < g.max_vcycles) {
-    if ((rs = issue(c, 0, c->g_v64, body64)) != MGFR_OK) return rs;
+    const bool dev = dev_ok && r <= kDevMax * ref;
+    if (!dev) {
+      make_key(key, sizeof(key), "v64", H.N, box, m, g);
+      if (!c->g_v64 || std::strcmp(key, c->graph_key) != 0) {
+        if (c->g_v64) cudaGraphExecDestroy(c->g_v64);
+        c->g_v64 = nullptr;
+        if ((rs = capture(c, 0, &c->g_v64, body64)) != MGFR_OK) return rs;
+        std::strcpy(c->graph_key, key);
+        c->updates_v64 = updates_per;
+      }
+      rs = issue(c, 0, c->g_v64, body64);
+    } else {
+      rs = issue(c, 4, c->g_dev, bodydev);
+    }
+    if (rs != MGFR_OK) return rs;
     rs = sync_read(c);
     if (rs != MGFR_OK) return rs;
-    prof_collect(c, 0, st);
-    r = std::sqrt(hs[0]);
+    prof_collect(c, dev ? 4 : 0, st);
+    const double rn = std::sqrt(hs[0]);
+    updates += dev ? c->updates_dev : c->updates_v64;
+    if (dev && !(rn < r)) {
+      f64::apply_dev(L0, -1.f, c->s);
+      c->launches += 1;
+      dev_ok = false;
+      continue;
+    }
     ++it;
+    r = rn;
     if (!std::isfinite(r)) break;
+    // the deviation cycle starts from u32 and r32 of this iterate
+    if (!dev && dev_ok && r <= kDevMax * ref) {
+      f64::resid_dev(L0, m, H.partials, H.nparts, H.scal, c->s);
+      c->launches += 2;
+    }
   }
   if (st) {
     st->vcycles = it;
-    st->cell_updates += (long long)it * c->updates_v64;
+    st->cell_updates += updates;
     st->res_l2_init = r0;
     st->res_l2_final = r;
     st->res_max_final = hs[1];
@@ -404,68 +509,6 @@ mgfr_status dense_solve64(mgfr_ctx* c, const Model& m, double box, mgfr_stats* s
 
 
 // ---- mixed precision ---------------------------------------------------------
-// Phase A: FP32 nonlinear FAS V-cycle (same steps as vcycle64).
-static void vcycle32(mgfr_ctx* c, const Model& m, int l, long long& updates) {
-  DenseHier& H = c->dh;
-  DenseLevel& F = H.L[l];
-  DenseLevel& C = H.L[l + 1];
-  const mgfr_config& g = c->cfg;
-  const float cap = (float)g.step_cap;
-  for (int s = 0; s < g.n_pre; ++s) {
-    for (int col = 0; col < 2; ++col) {
-      if (l == 0) prof_begin(c, 0, F.n);
-      f32::sweep(F, m, col, cap, c->s);
-      if (l == 0) prof_end(c);
-    }
-    updates += F.n;
-  }
-  f32::restrict_resid(F, C, m, H.partials, H.nparts, c->s);
-  f32::fas_rhs(C, m, c->s);
-  if (C.N > 4)
-    vcycle32(c, m, l + 1, updates);
-  else
-    f32::coarse_solve(C, m, cap, 40, c->s);
-  f32::prolong_corr(F, C, g.prolong_linear, c->s);
-  for (int s = 0; s < g.n_post; ++s) {
-    for (int col = 0; col < 2; ++col) {
-      if (l == 0) prof_begin(c, 0, F.n);
-      f32::sweep(F, m, col, cap, c->s);
-      if (l == 0) prof_end(c);
-    }
-    updates += F.n;
-  }
-}
-
-// Phase B: FP32 linear V-cycle on J(u) e = r (correction scheme).
-static void vcycle_lin(mgfr_ctx* c, const Model& m, int l, long long& updates) {
-  DenseHier& H = c->dh;
-  DenseLevel& F = H.L[l];
-  DenseLevel& C = H.L[l + 1];
-  const mgfr_config& g = c->cfg;
-  for (int s = 0; s < g.n_pre; ++s) {
-    for (int col = 0; col < 2; ++col) {
-      if (l == 0) prof_begin(c, 1, F.n);
-      f32::lin_sweep(F, m, col, c->s);
-      if (l == 0) prof_end(c);
-    }
-    updates += F.n;
-  }
-  f32::lin_restrict(F, C, m, c->s);
-  if (C.N > 4)
-    vcycle_lin(c, m, l + 1, updates);
-  else
-    f32::lin_coarse(C, m, 40, c->s);
-  f32::lin_prolong(F, C, g.prolong_linear, c->s);
-  for (int s = 0; s < g.n_post; ++s) {
-    for (int col = 0; col < 2; ++col) {
-      if (l == 0) prof_begin(c, 1, F.n);
-      f32::lin_sweep(F, m, col, c->s);
-      if (l == 0) prof_end(c);
-    }
-    updates += F.n;
-  }
-}
-
 // Mixed form: FP32 nonlinear V-cycles until ||r|| <= mixed_switch ||f|| (or
 // they stall), then FP64 defect correction: r = f - L(u) in FP64, FP32 linear
 // V-cycles on J e = r, u += e in FP64, until the FP64 stopping test holds.
@@ -482,7 +525,7 @@ mgfr_status dense_solve_mixed(mgfr_ctx* c, const Model& m, double box, mgfr_stat
   f64::norm(L0.f, L0.n, H.partials, H.nparts, H.scal + 2, c->s);
   f32::from64(L0.f, L0.f32, L0, c->s);
   f32::from64(L0.u, L0.u32, L0, c->s);
-  f32::norm32(L0, m, H.partials, H.nparts, H.scal, c->s);
+  norm32(c, m);
   c->launches += 6;
   MG_CK(c, cudaMemcpyAsync(hs, H.scal, 4 * sizeof(double), cudaMemcpyDeviceToHost, c->s));
   mgfr_status rs = sync_read(c);
@@ -500,9 +543,8 @@ mgfr_status dense_solve_mixed(mgfr_ctx* c, const Model& m, double box, mgfr_stat
   make_key(key, sizeof(key), "v32", H.N, box, m, g);
   long long upd = 0;
   auto body32 = [&]() {
-    upd = 0;
-    vcycle32(c, m, 0, upd);
-    f32::norm32(L0, m, H.partials, H.nparts, H.scal, c->s);
+    upd = cycle32(c, MG_NL, m, 0);
+    norm32(c, m);
     cudaMemcpyAsync(hs, H.scal, 2 * sizeof(double), cudaMemcpyDeviceToHost, c->s);
   };
   if (!c->g_v32 || std::strcmp(key, c->key32) != 0) {
@@ -515,8 +557,7 @@ mgfr_status dense_solve_mixed(mgfr_ctx* c, const Model& m, double box, mgfr_stat
   }
   make_key(key, sizeof(key), "lin", H.N, box, m, g);
   auto bodylin = [&]() {
-    upd = 0;
-    for (int q = 0; q < g.mixed_inner; ++q) vcycle_lin(c, m, 0, upd);
+    upd = cycle32(c, MG_LIN, m, 1, g.mixed_inner);
     f32::apply_corr(L0, g.step_cap, c->s);
     prof_begin(c, 2, L0.n);
     f32::resid_df(L0, H.fdf, m, H.partials, H.nparts, H.scal, c->s);
