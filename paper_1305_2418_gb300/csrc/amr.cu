@@ -25,7 +25,7 @@
 #include <vector>
 
 #include "amr.cuh"
-#include "dfloat.cuh"
+#include "lean_fp64.cuh"
 
 namespace {
 
@@ -686,16 +686,22 @@ __global__ void k_source_lvl(const double* __restrict__ mass, long long n, doubl
 // masses, scale = N_l^3 / Np).
 struct EffPar {
   double scale, c3, inv_np1;
+  int n;
 };
 
-__device__ __forceinline__ double eff_density(double mass, double u, const EffPar& q) {
-  return (mass * q.scale - 1.0) / 3.0 + q.c3 * (1.0 - exp(-u * q.inv_np1));
+// u and (for n = 1, where e^{-u/2} = 1/sqrt(E)) E = e^u of the cell
+__device__ __forceinline__ double eff_density(double d, double u, double E, const EffPar& q) {
+  const double s = q.n == 1 ? lean_rsqrt(E) : lean_exp(-u * q.inv_np1);
+  return fma(d, 1.0 / 3.0, fma(-q.c3, s, q.c3));
 }
 
 __global__ void k_eff_level(const double* __restrict__ mass, const double* __restrict__ u,
-                            long long n, EffPar q, double* __restrict__ out) {
+                            const double* __restrict__ E, long long n, EffPar q,
+                            double* __restrict__ out) {
   const long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (c < n) out[c] = eff_density(mass[c], u[c], q);
+  if (c < n)
+    out[c] = eff_density(fma(mass[c], q.scale, -1.0), q.n == 1 ? 0.0 : u[c], q.n == 1 ? E[c] : 1.0,
+                         q);
 }
 
 // Each leaf cell of level l hands its mass to the cells of the nested
@@ -704,29 +710,47 @@ __global__ void k_eff_level(const double* __restrict__ mass, const double* __res
 // contrast as a density (plain stores: leaves do not overlap); a leaf at
 // l > lpm lies in one PM cell and adds its contrast 8^-(l-lpm) (atomics).
 // The contrast is delta_eff (what 0), delta (what 1) or delta + delta_eff
-// (what 2, the right-hand side of Eq. (30)).
+// (what 2, the right-hand side of Eq. (30)).  FP64 pipe bound; the eight
+// daughters of an oct beyond lpm fall into one PM cell, so their lanes add up
+// first and the oct costs one atomic instead of eight (78 M cells of a 256^3
+// base with two levels took 4.1 ms with an FP64 exponential and an atomic per
+// leaf).
 __global__ void k_eff_pm(int l, int lpm, TreeView T, const double* __restrict__ mass,
-                         const double* __restrict__ u, long long n, EffPar q, int what,
-                         double* __restrict__ out) {
+                         const double* __restrict__ u, const double* __restrict__ E, long long n,
+                         EffPar q, int what, double* __restrict__ out) {
   const long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (c >= n || T.son[l][c] >= 0) return;  // not a leaf
-  const double d = mass[c] * q.scale - 1.0;
-  const double eff = what == 1 ? d : (what == 0 ? eff_density(mass[c], u[c], q)
-                                                : d + eff_density(mass[c], u[c], q));
-  long long I, J, K;
-  cell_coords(T, l, c, &I, &J, &K);
-  const long long Npm = 1LL << (T.lg0 + lpm);
+  const bool leaf = c < n && T.son[l][c] < 0;
+  double eff = 0.0;
+  if (leaf) {
+    const double d = fma(mass[c], q.scale, -1.0);
+    eff = what == 1 ? d : eff_density(d, q.n == 1 ? 0.0 : u[c], q.n == 1 ? E[c] : 1.0, q);
+    if (what == 2) eff += d;
+  }
   if (l <= lpm) {
+    if (!leaf) return;
+    long long I, J, K;
+    cell_coords(T, l, c, &I, &J, &K);
+    const long long Npm = 1LL << (T.lg0 + lpm);
     const long long s = 1LL << (lpm - l);
     for (long long a = 0; a < s; ++a)
       for (long long b = 0; b < s; ++b)
         for (long long e = 0; e < s; ++e)
           out[((I * s + a) * Npm + (J * s + b)) * Npm + (K * s + e)] = eff;
-  } else {
-    const int sh = l - lpm;
-    atomicAdd(out + ((I >> sh) * Npm + (J >> sh)) * Npm + (K >> sh),
-              eff / (double)(1LL << (3 * sh)));
+    return;
   }
+  // whole warps reach here (l >= 1: cells come in octs of 8 lanes)
+  unsigned any = __ballot_sync(0xffffffffu, leaf);
+  any = (any >> (threadIdx.x & 24)) & 0xffu;
+  if (any == 0u) return;
+  const unsigned oct = 0xffu << (threadIdx.x & 24);
+  for (int o = 4; o > 0; o >>= 1) eff += __shfl_xor_sync(oct, eff, o);
+  if (threadIdx.x & 7) return;
+  const int4 p = T.opos[l][c >> 3];  // the parent at level l - 1 >= lpm
+  const int sh = l - lpm;
+  const long long Npm = 1LL << (T.lg0 + lpm);
+  atomicAdd(out + ((long long)(p.x >> (sh - 1)) * Npm + (p.y >> (sh - 1))) * Npm +
+                (p.z >> (sh - 1)),
+            eff / (double)(1LL << (3 * sh)));
 }
 
 __global__ void k_nan_check(const double* __restrict__ x, long long n,
@@ -1422,7 +1446,7 @@ static EffPar eff_par(const AmrWork* A, int l) {
   const double Nl = (double)(1LL << (A->lg0 + l));
   const double a3 = A->a * A->a * A->a, rho = A->omega_m / a3;
   const double Rt = rho + 4.0 * (1.0 - A->omega_m);
-  return EffPar{Nl * Nl * Nl / (double)A->Np, Rt / (3.0 * rho), 1.0 / (A->nexp + 1)};
+  return EffPar{Nl * Nl * Nl / (double)A->Np, Rt / (3.0 * rho), 1.0 / (A->nexp + 1), A->nexp};
 }
 
 mgfr_status mgfr_get_effective_density(mgfr_ctx* c, int level, double* out_dev) {
@@ -1436,7 +1460,8 @@ mgfr_status mgfr_get_effective_density(mgfr_ctx* c, int level, double* out_dev) 
   MG_CK(c, cudaStreamWaitEvent(c->s, c->ev_in, 0));
   AmrLevel& L = A->L[level];
   const double* u = level == 0 ? c->dh.L[0].u : L.u;
-  k_eff_level<<<nblocks(L.ncell, BS), BS, 0, c->s>>>(L.mass, u, L.ncell, eff_par(A, level),
+  const double* E = level == 0 ? c->dh.L[0].E : L.E;
+  k_eff_level<<<nblocks(L.ncell, BS), BS, 0, c->s>>>(L.mass, u, E, L.ncell, eff_par(A, level),
                                                      out_dev);
   MG_CK(c, cudaEventRecord(c->ev_out, c->s));
   MG_CK(c, cudaStreamWaitEvent(c->user, c->ev_out, 0));
@@ -1462,7 +1487,8 @@ mgfr_status amr_density_pm(mgfr_ctx* c, int lpm, int what, double* out_dev, int*
   for (int l = 0; l < A->nlev; ++l) {
     AmrLevel& L = A->L[l];
     const double* u = l == 0 ? c->dh.L[0].u : L.u;
-    k_eff_pm<<<nblocks(L.ncell, BS), BS, 0, c->s>>>(l, lpm, T, L.mass, u, L.ncell,
+    const double* E = l == 0 ? c->dh.L[0].E : L.E;
+    k_eff_pm<<<nblocks(L.ncell, BS), BS, 0, c->s>>>(l, lpm, T, L.mass, u, E, L.ncell,
                                                     eff_par(A, l), what, out_dev);
     c->launches += 1;
   }

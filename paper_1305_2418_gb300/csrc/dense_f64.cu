@@ -8,7 +8,7 @@
 #include <algorithm>
 
 #include "colour_split.cuh"
-#include "dfloat.cuh"
+#include "lean_fp64.cuh"
 #include "mgfr_internal.cuh"
 
 namespace {
@@ -293,10 +293,28 @@ __global__ void __launch_bounds__(BS) k_norm(const double* __restrict__ u,
   block_norms(ss, mx, partials);
 }
 
+// f - L(u) at a cell as Lpoint forms it, the factor 1/2 of the face
+// coefficients taken out of the sum (exact) and 1/sqrt(E) by lean_rsqrt: 28
+// FP64 instructions against 43
+__device__ __forceinline__ double resid_lean(const double* __restrict__ u,
+                                             const double* __restrict__ E, double f, int i, int j,
+                                             int k, int lg, const Model& m, double ih2h) {
+  const int M = (1 << lg) - 1;
+  const unsigned c = cidx(i, j, k, lg);
+  const unsigned nb[6] = {cidx((i - 1) & M, j, k, lg), cidx((i + 1) & M, j, k, lg),
+                          cidx(i, (j - 1) & M, k, lg), cidx(i, (j + 1) & M, k, lg),
+                          cidx(i, j, (k - 1) & M, lg), cidx(i, j, (k + 1) & M, lg)};
+  const double uc = u[c], Ec = E[c];
+  double s = 0.0;
+#pragma unroll
+  for (int q = 0; q < 6; ++q) s = fma(E[nb[q]] + Ec, u[nb[q]] - uc, s);
+  const double n = m.n == 1 ? lean_rsqrt(Ec) : lean_exp(-uc * m.inv_np1);
+  return f - fma(s, ih2h, m.aRt * (1.0 - n));
+}
+
 // The residual of the FP64 iterate as the right-hand side of the FP32
 // deviation cycle (colour-split r32, u32 = u), and its norms as k_norm<0>
-// forms them.  One pass per V-cycle: FP64 pipe bound, about 32 FP64
-// instructions per cell against about 400 of an FP64 V-cycle.
+// forms them (ih2: 1/(2 h^2)).  One pass per V-cycle, bound by the FP64 pipe.
 __global__ void __launch_bounds__(BS) k_resid_dev(const double* __restrict__ u,
                                                   const double* __restrict__ E,
                                                   const double* __restrict__ f, int lg, Model m,
@@ -309,7 +327,7 @@ __global__ void __launch_bounds__(BS) k_resid_dev(const double* __restrict__ u,
   const int M = (1 << lg) - 1;
   for (unsigned t = blockIdx.x * blockDim.x + threadIdx.x; t < n; t += gridDim.x * blockDim.x) {
     const int k = (int)(t & M), j = (int)((t >> lg) & M), i = (int)(t >> (2 * lg));
-    const double r = f[t] - Lpoint(u, E, i, j, k, lg, m, ih2);
+    const double r = resid_lean(u, E, f[t], i, j, k, lg, m, ih2);
     const unsigned p = pdx(i, j, k, lg);
     r32[p] = f_from_double_bits(r);
     u32[p] = f_from_double_bits(u[t]);
@@ -331,7 +349,7 @@ __global__ void __launch_bounds__(BS) k_apply_dev(double* __restrict__ u, double
   const float e = e32[pdx((int)(t >> (2 * lg)), (int)((t >> lg) & M), (int)(t & M), lg)];
   const double v = u[t] + (isfinite(e) ? d_from_float_bits(sign * e) : 0.0);
   u[t] = v;
-  E[t] = exp(v);
+  E[t] = lean_exp(v);
 }
 
 __global__ void k_finish(const double* __restrict__ partials, int nparts, double* __restrict__ out) {
@@ -423,7 +441,7 @@ void resid_norm(DenseLevel& L, const Model& m, double* partials, int nparts, dou
 void resid_dev(DenseLevel& L, const Model& m, double* partials, int nparts, double* out,
                cudaStream_t s) {
   const int nb = (int)std::min<long long>(nparts, nblocks(L.n, BS));
-  k_resid_dev<<<nb, BS, 0, s>>>(L.u, L.E, L.f, L.lg, m, L.ih2, L.r32, L.u32, partials);
+  k_resid_dev<<<nb, BS, 0, s>>>(L.u, L.E, L.f, L.lg, m, 0.5 * L.ih2, L.r32, L.u32, partials);
   k_finish<<<1, 256, 0, s>>>(partials, nb, out);
 }
 

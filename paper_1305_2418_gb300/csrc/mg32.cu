@@ -55,7 +55,8 @@ struct PF {
 
 // ---- point operations: xc, xn[6] the unknown at the cell and its neighbours
 // (-x, +x, -y, +y, -z, +z), wc, wn[6] the linearisation point -------------------
-template <int OP>
+// (EXACT: with the correctly rounded division, on the 4^3 grid)
+template <int OP, bool EXACT = false>
 __device__ __forceinline__ float point_update(float xc, const float* xn, float wc, const float* wn,
                                               float r, const PF& m, float ih2, float h2) {
   if constexpr (OP == MG_NL) {
@@ -72,7 +73,7 @@ __device__ __forceinline__ float point_update(float xc, const float* xn, float w
     const float s = __expf(-xc * m.inv_np1);
     const float L = sbd * ih2 + m.aRt * (1.f - s);
     const float dL = (0.5f * Ec * sd - sb) * ih2 + m.aRt_np1 * s;
-    const float step = __fdividef(L - r, dL);
+    const float step = EXACT ? (L - r) / dL : __fdividef(L - r, dL);
     return xc - fminf(fmaxf(step, -m.cap), m.cap);
   } else if constexpr (OP == MG_LIN) {
     const float Ec = __expf(wc), q2 = 0.5f * ih2;
@@ -85,7 +86,7 @@ __device__ __forceinline__ float point_update(float xc, const float* xn, float w
       s = fmaf(-off, xn[q], s);
     }
     const float diag = d * q2 + m.aRt_np1 * __expf(-wc * m.inv_np1);
-    return __fdividef(s, diag);
+    return EXACT ? s / diag : __fdividef(s, diag);
   } else if constexpr (OP == MG_DEV) {
     // D = L(w + x) - L(w): per neighbour, twice the new face coefficient
     // b = E_j + E_i with E = e^{w + x} = e^w e^x, and its change t
@@ -640,8 +641,8 @@ struct Bot {
     }
   }
   // the 4^3 grid by the first warp (one colour's 32 cells per half-sweep):
-  // until no cell changes by more than its rounding, or the residual has
-  // dropped by `rel` (checked every four sweeps), or `sweeps`
+  // until no cell changes any more (DEV and POI: by more than its rounding), or
+  // the residual has dropped by `rel` (checked every four sweeps), or `sweeps`
   __device__ void coarse(const BotGrid& g, const PF& m, float ih2, float h2, int sweeps,
                          float rel) {
     if (threadIdx.x >= 32) return;
@@ -685,8 +686,9 @@ struct Bot {
 #pragma unroll
         for (int e = 0; e < 6; ++e) xn[e] = x[nb[q][e]];
         const float old = x[c[q]];
-        const float v = point_update<OP>(old, xn, wc[q], wn[q], r[c[q]], m, ih2, h2);
-        changed = changed || fabsf(v - old) > 1.2e-7f * fabsf(v);
+        constexpr bool exact = OP == MG_NL || OP == MG_LIN;
+        const float v = point_update<OP, exact>(old, xn, wc[q], wn[q], r[c[q]], m, ih2, h2);
+        changed = changed || (exact ? v != old : fabsf(v - old) > 1.2e-7f * fabsf(v));
         __syncwarp();
         x[c[q]] = v;
         __syncwarp();
