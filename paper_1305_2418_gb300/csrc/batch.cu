@@ -2,9 +2,10 @@
 //
 // Each solve is the mixed-precision form of the base-level solve (Puchwein,
 // Baldi & Springel 2013, Sec. 3.3): FP32 nonlinear FAS V-cycles (mode A)
-// until the FP32 residual reaches mixed_switch or stalls, then FP64 defect
-// correction (mode B): r = f - L(u) in FP64, one FP32 linear V-cycle on
-// J(u) e = r, u += e.  All solves advance together through one V-cycle
+// until the FP32 residual reaches mixed_switch or stalls, then defect correction
+// (mode B): r = f - L(u) in double-float or FP64, one FP32 linear V-cycle on
+// J(u) e = r, u += e.  The FP32 arrays are stored by red-black colour and worked
+// on four cells per thread (mg32_dev.cuh).  All solves advance together through one V-cycle
 // schedule aligned on grid size: at size 2^k every solve with N >= 2^k works
 // on its level of that size, so one phase covers all solves; solves are
 // sorted by N (descending) so the participants of size 2^k are a prefix and
@@ -22,16 +23,19 @@
 #include <string>
 #include <vector>
 
-#include "mgfr_internal.cuh"
+#include "lean_fp64.cuh"
+#include "mg32_dev.cuh"
 
 #define BMAXL 9  // levels per solve: N <= 1024 -> 1024..4
+constexpr int kMaxBatch = 4096;  // solves of one call
 
 struct BSolve {
   int N, lg, nlev;
   float ih2[BMAXL];
   double ih2_0, h0;
   float aRt, aRt_np1, inv_np1;  // FP32 model
-  double aRt64, aRt_np1_64, inv_np1_64, src, fbar, gscale;
+  double aRt64, inv_np1_64, src, fbar, gscale;
+  dfl aRt_df, inv_np1_df, ih2h_df;  // alpha Rt, 1/(n+1), 1/(2 h^2)
   int n;
   float* u32[BMAXL];
   float* f32[BMAXL];
@@ -64,7 +68,7 @@ struct BArgs {
   int P[16];  // participants per log2 size
   int n_pre, n_post, linear, max_cycles;
   float cap32;
-  double cap64, tol, sw;
+  double tol, sw;
   unsigned* bar_count;
   unsigned* bar_gen;
   int* err;
@@ -106,147 +110,68 @@ __device__ bool gsync(const BArgs& A) {
   return *(volatile int*)A.err == 0;
 }
 
-struct NB6 {
-  float v[6];
-};
+__device__ __forceinline__ PF batch_pf(const BArgs& A, const BSolve& S) {
+  return PF{S.aRt, S.aRt_np1, S.inv_np1, A.cap32};
+}
 
-__device__ __forceinline__ NB6 nbr6(const float* __restrict__ x, int i, int j, int k, int lg) {
+// ---- per-item operations on four cells (mg32_dev.cuh) -----------------------
+__device__ __forceinline__ void op_sweep(const BArgs& A, const BSolve& S, int mode, int l,
+                                         int colour, unsigned t) {
+  const int lg = S.lg - l;
+  const size_t half = (size_t)1 << (3 * lg - 1);
+  const size_t s = colour * half, o = half - s;
+  if (mode == BM_A)
+    vec_sweep<MG_NL>(t, S.u32[l] + s, S.u32[l] + o, S.f32[l] + s, nullptr, nullptr, lg, colour,
+                     batch_pf(A, S), S.ih2[l], 0.f);
+  else
+    vec_sweep<MG_LIN>(t, S.e32[l] + s, S.e32[l] + o, S.r32[l] + s, S.u32[l] + s, S.u32[l] + o, lg,
+                      colour, batch_pf(A, S), S.ih2[l], 0.f);
+}
+
+// restriction from level l to l+1 at four coarse cells
+__device__ __forceinline__ void op_restrict(const BArgs& A, const BSolve& S, int mode, int l,
+                                            unsigned t) {
+  if (mode == BM_A)
+    vec_restrict<MG_NL>(t, S.u32[l], S.f32[l], nullptr, S.lg - l, S.u32[l + 1], S.f32[l + 1],
+                        S.uold32[l + 1], batch_pf(A, S), S.ih2[l]);
+  else
+    vec_restrict<MG_LIN>(t, S.e32[l], S.r32[l], S.u32[l], S.lg - l, S.e32[l + 1], S.r32[l + 1],
+                         S.u32[l + 1], batch_pf(A, S), S.ih2[l]);
+}
+
+// one cell of a colour-split level: the index, the unknown and its neighbours
+__device__ __forceinline__ unsigned cell_nbrs(const float* __restrict__ x, unsigned c, int lg,
+                                              float* o) {
   const int M = (1 << lg) - 1;
-  NB6 r;
-  r.v[0] = x[cidx((i - 1) & M, j, k, lg)];
-  r.v[1] = x[cidx((i + 1) & M, j, k, lg)];
-  r.v[2] = x[cidx(i, (j - 1) & M, k, lg)];
-  r.v[3] = x[cidx(i, (j + 1) & M, k, lg)];
-  r.v[4] = x[cidx(i, j, (k - 1) & M, lg)];
-  r.v[5] = x[cidx(i, j, (k + 1) & M, lg)];
-  return r;
+  const int i = (int)(c >> (2 * lg)), j = (int)((c >> lg) & M), k = (int)(c & M);
+  unsigned q[6];
+  pnb6(i, j, k, lg, q);
+#pragma unroll
+  for (int e = 0; e < 6; ++e) o[e] = x[q[e]];
+  return pdx(i, j, k, lg);
 }
 
-// FP32 L at a cell (e^u by the SFU)
-__device__ __forceinline__ float L32(const BSolve& S, const float* u, int i, int j, int k, int lg,
-                                     float ih2) {
-  const float uc = u[cidx(i, j, k, lg)], Ec = __expf(uc);
-  const NB6 nb = nbr6(u, i, j, k, lg);
-  float sbd = 0.f;
-#pragma unroll
-  for (int q = 0; q < 6; ++q) sbd = fmaf(0.5f * (__expf(nb.v[q]) + Ec), nb.v[q] - uc, sbd);
-  return sbd * ih2 + S.aRt * (1.f - __expf(-uc * S.inv_np1));
-}
-
-// Jacobian row of L at u (FP32): off-diagonal and diagonal
-__device__ __forceinline__ void jrow(const BSolve& S, float uc, const NB6& un, float ih2,
-                                     float* off, float* diag) {
-  const float Ec = __expf(uc), h2 = 0.5f * ih2;
-  float d = 0.f;
-#pragma unroll
-  for (int q = 0; q < 6; ++q) {
-    const float En = __expf(un.v[q]), du = un.v[q] - uc;
-    off[q] = h2 * fmaf(En, du, Ec + En);
-    d += fmaf(Ec, du, -Ec - En);
+// FAS right-hand side of level l (the 4^3 level has no vectors: cell by cell)
+__device__ __forceinline__ void op_fas(const BArgs& A, const BSolve& S, int l, unsigned t) {
+  const int lg = S.lg - l;
+  if (lg > 2) {
+    vec_fas(t, S.u32[l], S.f32[l], lg, batch_pf(A, S), S.ih2[l]);
+    return;
   }
-  *diag = d * h2 + S.aRt_np1 * __expf(-uc * S.inv_np1);
-}
-
-// ---- per-item operations ---------------------------------------------------
-__device__ void op_sweep(const BArgs& A, const BSolve& S, int mode, int l, int colour,
-                         long long t) {
-  const int lg = S.lg - l, N = 1 << lg, M = N - 1;
-  const int k2 = (int)(t & ((N >> 1) - 1));
-  const long long r = t >> (lg - 1);
-  const int j = (int)(r & M), i = (int)(r >> lg);
-  const int k = 2 * k2 + ((i + j + colour) & 1);
-  const long long c = cidx(i, j, k, lg);
-  const float ih2 = S.ih2[l];
-  if (mode == BM_A) {
-    float* u = S.u32[l];
-    const float uc = u[c], Ec = __expf(uc);
-    const NB6 nb = nbr6(u, i, j, k, lg);
-    float sbd = 0.f, sd = 0.f, sb = 0.f;
-#pragma unroll
-    for (int q = 0; q < 6; ++q) {
-      const float b = 0.5f * (__expf(nb.v[q]) + Ec), du = nb.v[q] - uc;
-      sbd = fmaf(b, du, sbd);
-      sd += du;
-      sb += b;
-    }
-    const float s = __expf(-uc * S.inv_np1);
-    const float L = sbd * ih2 + S.aRt * (1.f - s);
-    const float dL = (0.5f * Ec * sd - sb) * ih2 + S.aRt_np1 * s;
-    float step = __fdividef(L - S.f32[l][c], dL);
-    step = fminf(fmaxf(step, -A.cap32), A.cap32);
-    u[c] = uc - step;
-  } else {
-    const float* u = S.u32[l];
-    float* e = S.e32[l];
-    const NB6 un = nbr6(u, i, j, k, lg), en = nbr6(e, i, j, k, lg);
-    float off[6], diag;
-    jrow(S, u[c], un, ih2, off, &diag);
-    float s = S.r32[l][c];
-#pragma unroll
-    for (int q = 0; q < 6; ++q) s = fmaf(-off[q], en.v[q], s);
-    e[c] = __fdividef(s, diag);
+  for (unsigned c = 4 * t; c < 4 * t + 4; ++c) {
+    float n[6];
+    const unsigned q = cell_nbrs(S.u32[l], c, lg, n);
+    S.f32[l][q] += point_apply<MG_NL>(S.u32[l][q], n, 0.f, n, batch_pf(A, S), S.ih2[l]);
   }
 }
 
-// restriction from level l to l+1 at coarse cell t
-__device__ void op_restrict(const BSolve& S, int mode, int l, long long t) {
-  const int lgf = S.lg - l, lgc = lgf - 1, Nc = 1 << lgc;
-  const int K = (int)(t & (Nc - 1)), J = (int)((t >> lgc) & (Nc - 1)), I = (int)(t >> (2 * lgc));
-  const float ih2 = S.ih2[l];
-  float su = 0.f, sr = 0.f;
-  for (int q = 0; q < 8; ++q) {
-    const int i = 2 * I + (q >> 2), j = 2 * J + ((q >> 1) & 1), k = 2 * K + (q & 1);
-    const long long c = cidx(i, j, k, lgf);
-    const float* u = S.u32[l];
-    su += u[c];
-    if (mode == BM_A) {
-      sr += S.f32[l][c] - L32(S, u, i, j, k, lgf, ih2);
-    } else {
-      const NB6 un = nbr6(u, i, j, k, lgf), en = nbr6(S.e32[l], i, j, k, lgf);
-      float off[6], diag;
-      jrow(S, u[c], un, ih2, off, &diag);
-      float Je = diag * S.e32[l][c];
-#pragma unroll
-      for (int p = 0; p < 6; ++p) Je = fmaf(off[p], en.v[p], Je);
-      sr += S.r32[l][c] - Je;
-    }
-  }
-  if (mode == BM_A) {
-    S.u32[l + 1][t] = 0.125f * su;
-    S.uold32[l + 1][t] = 0.125f * su;
-    S.f32[l + 1][t] = 0.125f * sr;
-  } else {
-    S.u32[l + 1][t] = 0.125f * su;
-    S.r32[l + 1][t] = 0.125f * sr;
-    S.e32[l + 1][t] = 0.f;
-  }
-}
-
-__device__ void op_fas(const BSolve& S, int l, long long t) {
-  const int lg = S.lg - l, N = 1 << lg;
-  const int k = (int)(t & (N - 1)), j = (int)((t >> lg) & (N - 1)), i = (int)(t >> (2 * lg));
-  S.f32[l][t] += L32(S, S.u32[l], i, j, k, lg, S.ih2[l]);
-}
-
-// prolongation from level l+1 to fine cell t of level l
-__device__ void op_prolong(const BArgs& A, const BSolve& S, int mode, int l, long long t) {
-  const int lgf = S.lg - l, N = 1 << lgf, lgc = lgf - 1, Mc = (N >> 1) - 1;
-  const int k = (int)(t & (N - 1)), j = (int)((t >> lgf) & (N - 1)), i = (int)(t >> (2 * lgf));
-  const int I = i >> 1, J = j >> 1, K = k >> 1;
-  const float* uc = mode == BM_A ? S.u32[l + 1] : S.e32[l + 1];
-  const float* uo = mode == BM_A ? S.uold32[l + 1] : nullptr;
-  auto corr = [&](int a, int b, int c) {
-    const long long q = cidx(a & Mc, b & Mc, c & Mc, lgc);
-    return uo ? uc[q] - uo[q] : uc[q];
-  };
-  float v = corr(I, J, K);
-  if (A.linear) {
-    v += ((i & 1) ? 0.125f : -0.125f) * (corr(I + 1, J, K) - corr(I - 1, J, K));
-    v += ((j & 1) ? 0.125f : -0.125f) * (corr(I, J + 1, K) - corr(I, J - 1, K));
-    v += ((k & 1) ? 0.125f : -0.125f) * (corr(I, J, K + 1) - corr(I, J, K - 1));
-  }
-  float* dst = mode == BM_A ? S.u32[l] : S.e32[l];
-  dst[t] += v;
+// prolongation from level l+1 to the daughters of four of its cells
+__device__ __forceinline__ void op_prolong(const BArgs& A, const BSolve& S, int mode, int l,
+                                           unsigned t) {
+  if (mode == BM_A)
+    vec_prolong<MG_NL>(t, S.u32[l], S.u32[l + 1], S.uold32[l + 1], S.lg - l, A.linear);
+  else
+    vec_prolong<MG_LIN>(t, S.e32[l], S.e32[l + 1], nullptr, S.lg - l, A.linear);
 }
 
 // 4^3 coarse level of one solve by one block (64 threads used)
@@ -259,164 +184,218 @@ __device__ void op_coarse(const BArgs& A, const BSolve& S, int mode) {
   const int q[6] = {(((i + 3) & 3) << 4) | (j << 2) | k, (((i + 1) & 3) << 4) | (j << 2) | k,
                     (i << 4) | (((j + 3) & 3) << 2) | k, (i << 4) | (((j + 1) & 3) << 2) | k,
                     (i << 4) | (j << 2) | ((k + 3) & 3), (i << 4) | (j << 2) | ((k + 1) & 3)};
+  const unsigned g = pdx(i, j, k, 2);
+  const PF m = batch_pf(A, S);
   const float ih2 = S.ih2[l];
+  float rhs = 0.f, wc = 0.f, wn[6] = {0, 0, 0, 0, 0, 0};
   if (on) {
-    sh[t] = mode == BM_A ? S.u32[l][t] : S.e32[l][t];
-    sh2[t] = S.u32[l][t];
+    sh[t] = mode == BM_A ? S.u32[l][g] : S.e32[l][g];
+    sh2[t] = S.u32[l][g];
+    rhs = mode == BM_A ? S.f32[l][g] : S.r32[l][g];
   }
   __syncthreads();
-  float off[6] = {0, 0, 0, 0, 0, 0}, diag = 1.f, rhs = 0.f;
   if (on && mode != BM_A) {
-    NB6 un;
-    for (int d = 0; d < 6; ++d) un.v[d] = sh2[q[d]];
-    jrow(S, sh2[t], un, ih2, off, &diag);
-    rhs = S.r32[l][t];
+    wc = sh2[t];
+    for (int d = 0; d < 6; ++d) wn[d] = sh2[q[d]];
   }
-  const float f = on && mode == BM_A ? S.f32[l][t] : 0.f;
   for (int s = 0; s < 40; ++s)
     for (int col = 0; col < 2; ++col) {
       if (on && colour == col) {
-        if (mode == BM_A) {
-          const float uc = sh[t], Ec = __expf(uc);
-          float sbd = 0.f, sd = 0.f, sb = 0.f;
-          for (int d = 0; d < 6; ++d) {
-            const float un = sh[q[d]], b = 0.5f * (__expf(un) + Ec), du = un - uc;
-            sbd = fmaf(b, du, sbd);
-            sd += du;
-            sb += b;
-          }
-          const float sN = __expf(-uc * S.inv_np1);
-          const float L = sbd * ih2 + S.aRt * (1.f - sN);
-          const float dL = (0.5f * Ec * sd - sb) * ih2 + S.aRt_np1 * sN;
-          float step = (L - f) / dL;
-          step = fminf(fmaxf(step, -A.cap32), A.cap32);
-          sh[t] = uc - step;
-        } else {
-          float acc = rhs;
-          for (int d = 0; d < 6; ++d) acc = fmaf(-off[d], sh[q[d]], acc);
-          sh[t] = acc / diag;
-        }
+        float xn[6];
+        for (int d = 0; d < 6; ++d) xn[d] = sh[q[d]];
+        sh[t] = mode == BM_A ? point_update<MG_NL, true>(sh[t], xn, 0.f, wn, rhs, m, ih2, 0.f)
+                             : point_update<MG_LIN, true>(sh[t], xn, wc, wn, rhs, m, ih2, 0.f);
       }
       __syncthreads();
     }
   if (on) {
     if (mode == BM_A)
-      S.u32[l][t] = sh[t];
+      S.u32[l][g] = sh[t];
     else
-      S.e32[l][t] = sh[t];
+      S.e32[l][g] = sh[t];
   }
   __syncthreads();
 }
 
-__device__ __forceinline__ double nls64(const BSolve& S, double u, double E) {
-  return S.n == 1 ? rsqrt(E) : exp(-u * S.inv_np1_64);
+// ---- the iterate of the defect correction: u, e^u and f of the finest level,
+// in double-float pairs (DF) or FP64, C order -------------------------------
+__device__ __forceinline__ dfl* dfp(double* p) { return reinterpret_cast<dfl*>(p); }
+
+// u = v (FP32 or FP64), E = e^u
+template <bool DF>
+__device__ __forceinline__ void set_u(const BSolve& S, unsigned t, double v) {
+  if (DF) {
+    const dfl x = df_from_double_bits(v);
+    dfp(S.u64)[t] = x;
+    dfp(S.E64)[t] = df_exp(x);
+  } else {
+    S.u64[t] = v;
+    S.E64[t] = lean_exp(v);
+  }
 }
 
-// FP64 residual at finest cell t: writes r32, u32 (= u), e32 = 0; returns r
-__device__ double op_resid64(const BSolve& S, long long t) {
+// u += clamp(e), E = e^u
+template <bool DF>
+__device__ __forceinline__ void add_e(const BArgs& A, const BSolve& S, unsigned t) {
+  const int lg = S.lg, M = (1 << lg) - 1;
+  const float e = S.e32[0][pdx((int)(t >> (2 * lg)), (int)((t >> lg) & M), (int)(t & M), lg)];
+  const float d = fminf(fmaxf(e, -A.cap32), A.cap32);
+  if (DF) {
+    const dfl x = df_add_f(dfp(S.u64)[t], d);
+    dfp(S.u64)[t] = x;
+    dfp(S.E64)[t] = df_exp(x);
+  } else {
+    const double x = S.u64[t] + d_from_float_bits(d);
+    S.u64[t] = x;
+    S.E64[t] = lean_exp(x);
+  }
+}
+
+// residual at finest cell t: writes r32, u32 (= u), e32 = 0; returns r rounded
+template <bool DF>
+__device__ __forceinline__ float op_resid(const BSolve& S, unsigned t) {
   const int lg = S.lg, M = (1 << lg) - 1;
   const int k = (int)(t & M), j = (int)((t >> lg) & M), i = (int)(t >> (2 * lg));
-  const long long nb[6] = {cidx((i - 1) & M, j, k, lg), cidx((i + 1) & M, j, k, lg),
-                           cidx(i, (j - 1) & M, k, lg), cidx(i, (j + 1) & M, k, lg),
-                           cidx(i, j, (k - 1) & M, lg), cidx(i, j, (k + 1) & M, lg)};
-  const double uc = S.u64[t], Ec = S.E64[t];
-  double sbd = 0.0;
+  const unsigned nb[6] = {cidx((i - 1) & M, j, k, lg), cidx((i + 1) & M, j, k, lg),
+                          cidx(i, (j - 1) & M, k, lg), cidx(i, (j + 1) & M, k, lg),
+                          cidx(i, j, (k - 1) & M, lg), cidx(i, j, (k + 1) & M, lg)};
+  float rf, uf;
+  if (DF) {
+    const dfl *u = dfp(S.u64), *E = dfp(S.E64);
+    const dfl uc = u[t], Ec = E[t];
+    dfl acc = {0.f, 0.f};
 #pragma unroll
-  for (int q = 0; q < 6; ++q) sbd = fma(0.5 * (S.E64[nb[q]] + Ec), S.u64[nb[q]] - uc, sbd);
-  const double r = S.f64[t] - (sbd * S.ih2_0 + S.aRt64 * (1.0 - nls64(S, uc, Ec)));
-  S.r32[0][t] = (float)r;
-  S.u32[0][t] = (float)uc;
-  S.e32[0][t] = 0.f;
-  return r;
+    for (int q = 0; q < 6; ++q)
+      acc = df_add_abs(acc, df_mul(df_add_abs(E[nb[q]], Ec), df_add_abs(u[nb[q]], df_neg(uc))));
+    const dfl sN = S.n == 1 ? df_rsqrt(Ec) : df_exp(df_neg(df_mul(uc, S.inv_np1_df)));
+    const dfl L = df_add(df_mul(acc, S.ih2h_df), df_mul(S.aRt_df, df_add_f(df_neg(sN), 1.f)));
+    rf = df_sub(dfp(S.f64)[t], L).hi;
+    uf = uc.hi;
+  } else {
+    const double uc = S.u64[t], Ec = S.E64[t];
+    double s = 0.0;
+#pragma unroll
+    for (int q = 0; q < 6; ++q) s = fma(S.E64[nb[q]] + Ec, S.u64[nb[q]] - uc, s);
+    const double sN = S.n == 1 ? lean_rsqrt(Ec) : lean_exp(-uc * S.inv_np1_64);
+    rf = f_from_double_bits(S.f64[t] - fma(s, 0.5 * S.ih2_0, S.aRt64 * (1.0 - sN)));
+    uf = f_from_double_bits(uc);
+  }
+  const unsigned p = pdx(i, j, k, lg);
+  S.r32[0][p] = rf;
+  S.u32[0][p] = uf;
+  S.e32[0][p] = 0.f;
+  return rf;
 }
 
-// warp-level accumulation of (r^2, |r|, f^2) into the solve's state; all
-// lanes of a warp belong to the same solve (per-solve item counts are
-// multiples of 32)
-__device__ __forceinline__ void accum(BState* st, double r, double f, bool live) {
-  double ss = live ? r * r : 0.0, mx = live ? fabs(r) : 0.0, ff = live ? f * f : 0.0;
+// a thread's sums over its cells of one solve (FP32 squares summed in FP64
+// every few cells) into the solve's state; whole warps, one solve
+struct Acc {
+  double ss = 0.0, ff = 0.0;
+  float s4 = 0.f, mx = 0.f;
+  int n = 0;
+  __device__ __forceinline__ void add(float r) {
+    s4 = fmaf(r, r, s4);
+    mx = fmaxf(mx, fabsf(r));
+    if ((++n & 3) == 0) flush();
+  }
+  __device__ __forceinline__ void flush() {
+    ss += (double)s4;
+    s4 = 0.f;
+  }
+};
+__device__ __forceinline__ void accum(BState* st, Acc& a) {
+  a.flush();
+  double ss = a.ss, ff = a.ff;
+  float mx = a.mx;
   for (int o = 16; o > 0; o >>= 1) {
     ss += __shfl_xor_sync(0xffffffffu, ss, o);
     ff += __shfl_xor_sync(0xffffffffu, ff, o);
-    mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
   }
-  if ((threadIdx.x & 31) == 0 && live) {
-    atomicAdd(&st->acc_ss, ss);
-    atomicAdd(&st->acc_ff, ff);
-    atomicMax(&st->acc_max, (unsigned long long)__double_as_longlong(mx));
+  if ((threadIdx.x & 31) == 0) {
+    if (ss != 0.0) atomicAdd(&st->acc_ss, ss);
+    if (ff != 0.0) atomicAdd(&st->acc_ff, ff);
+    atomicMax(&st->acc_max, (unsigned long long)__double_as_longlong((double)mx));
   }
 }
 
-// items of size 2^k over the participant prefix: `shift` = log2(items per solve)
+// items of size 2^k over the participant prefix: `shift` = log2(items per
+// solve); the solves' modes are read from shared memory (they change only
+// where load_modes follows)
 #define FOR_ITEMS(A, k, shift, ...)                                                         \
   do {                                                                                     \
     const long long tot_ = (long long)(A).P[k] << (shift);                                 \
     for (long long g_ = blockIdx.x * (long long)blockDim.x + threadIdx.x; g_ < tot_;       \
          g_ += (long long)gridDim.x * blockDim.x) {                                        \
       const int s = (int)(g_ >> (shift));                                                  \
-      const long long t = g_ & ((1LL << (shift)) - 1);                                     \
+      const unsigned t = (unsigned)(g_ & ((1LL << (shift)) - 1));                          \
       const BSolve& S = (A).S[s];                                                          \
-      const int mode = *(volatile const int*)&(A).st[s].mode;                              \
+      const int mode = smode[s];                                                           \
       __VA_ARGS__                                                                          \
     }                                                                                      \
   } while (0)
 
-// finest-level items of every solve (sizes differ): walk solves in turn
-#define FOR_FINEST(A, ...)                                                                \
-  do {                                                                                     \
-    long long base_ = 0;                                                                   \
-    for (int s = 0; s < (A).ns; ++s) {                                                     \
-      const BSolve& S = (A).S[s];                                                          \
-      const long long n_ = 1LL << (3 * S.lg);                                              \
-      const int mode = *(volatile const int*)&(A).st[s].mode;                              \
-      const long long gs_ = (long long)gridDim.x * blockDim.x;                             \
-      const long long g0_ = blockIdx.x * (long long)blockDim.x + threadIdx.x;              \
-      long long first_ = (g0_ - base_ % gs_ + gs_) % gs_;                                  \
-      for (long long t = first_; t < n_; t += gs_) {                                       \
-        __VA_ARGS__                                                                        \
-      }                                                                                    \
-      base_ += n_;                                                                         \
-    }                                                                                      \
-  } while (0)
+// body(S, mode, t, acc) at the finest-level cells t of the solves whose mode
+// `want` accepts (sizes differ: the solves in turn); with `sum`, acc of every
+// thread goes to the solve's state.  Cell counts and the grid stride are
+// multiples of 32, so whole warps reach accum.
+template <class Want, class Body>
+__device__ __forceinline__ void for_finest(const BArgs& A, const unsigned char* smode, bool sum,
+                                           Want want, Body body) {
+  unsigned base = 0;
+  const unsigned gs = gridDim.x * blockDim.x, g0 = blockIdx.x * blockDim.x + threadIdx.x;
+  for (int s = 0; s < A.ns; ++s) {
+    const BSolve& S = A.S[s];
+    const int mode = smode[s];
+    const unsigned n = 1u << (3 * S.lg);
+    unsigned t = g0 >= base ? g0 - base : g0 + gs - base;
+    base = (base + n % gs) % gs;
+    if (!want(mode)) continue;
+    Acc acc;
+    for (; t < n; t += gs) body(S, mode, t, acc);
+    if (sum) accum(&A.st[s], acc);
+  }
+}
 
-__global__ void __launch_bounds__(512) k_batch(BArgs A) {
+// modes of all solves into shared memory (after a barrier that follows a change)
+__device__ __forceinline__ void load_modes(const BArgs& A, unsigned char* smode) {
+  for (int s = threadIdx.x; s < A.ns; s += blockDim.x)
+    smode[s] = (unsigned char)*(volatile const int*)&A.st[s].mode;
+  __syncthreads();
+}
+
+// DF: the iterate of the defect correction in double-float pairs on the FP32
+// pipes (its residual took 43 FP64 instructions per cell); FP64 for tolerances
+// that come near the pairs' 48 bits.  Bound by issue slots (55% busy at 32
+// warps per SM; 64 registers, a few spilled, against one block of 128: 45 and
+// 50 ms).  96 solves of 32^3..128^3: 157 ms with one cell per thread in C order
+// (half of every line unused per half-sweep), FP64 residuals and a warp
+// reduction per 32 cells; 45 ms now.
+template <bool DF>
+__global__ void __launch_bounds__(512, 2) k_batch(BArgs A) {
+  __shared__ unsigned char smode[kMaxBatch];
+  load_modes(A, smode);
   // ---- set-up: f = src delta, u from the initial guess -----------------------
-  FOR_FINEST(A, {
-    (void)mode;
+  auto all = [](int) { return true; };
+  for_finest(A, smode, true, all, [&](const BSolve& S, int, unsigned t, Acc& acc) {
     const double f = S.src * S.delta[t];
     const double u0 = S.uinit ? S.uinit[t] : 0.0;
-    S.f64[t] = f;
-    S.f32[0][t] = (float)f;
-    S.u64[t] = u0;
-    S.E64[t] = exp(u0);
-    S.u32[0][t] = (float)u0;
+    const int lg = S.lg, M = (1 << lg) - 1;
+    const unsigned p = pdx((int)(t >> (2 * lg)), (int)((t >> lg) & M), (int)(t & M), lg);
+    if (DF)
+      dfp(S.f64)[t] = df_from_double_bits(f);
+    else
+      S.f64[t] = f;
+    S.f32[0][p] = f_from_double_bits(f);
+    S.u32[0][p] = f_from_double_bits(u0);
+    set_u<DF>(S, t, u0);
+    acc.ff = fma(f, f, acc.ff);
   });
   if (!gsync(A)) return;
-  // initial FP64 residual and ||f||.  Lanes of a warp walk consecutive cells
-  // of one solve (cell counts and the grid stride are multiples of 32), so
-  // the warp reductions in accum() see whole warps.
-  {
-    const long long gs = (long long)gridDim.x * blockDim.x;
-    const long long g0 = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    long long base = 0;
-    for (int s = 0; s < A.ns; ++s) {
-      const BSolve& S = A.S[s];
-      const long long n = 1LL << (3 * S.lg);
-      const long long first = (g0 - base % gs + gs) % gs;
-      // all lanes of a warp iterate together: pad the loop to whole warps
-      const long long lane_first = first;
-      for (long long t = lane_first; t - (threadIdx.x & 31) < n; t += gs) {
-        const bool live = t < n;
-        double r = 0.0, f = 0.0;
-        if (live) {
-          r = op_resid64(S, t);
-          f = S.f64[t];
-        }
-        accum(&A.st[s], r, f, live);
-      }
-      base += n;
-    }
-  }
+  // initial residual
+  for_finest(A, smode, true, all, [&](const BSolve& S, int, unsigned t, Acc& acc) {
+    acc.add(op_resid<DF>(S, t));
+  });
   if (!gsync(A)) return;
   if (blockIdx.x == 0) {
     for (int s = threadIdx.x; s < A.ns; s += blockDim.x) {
@@ -434,84 +413,62 @@ __global__ void __launch_bounds__(512) k_batch(BArgs A) {
     }
   }
   if (!gsync(A)) return;
+  load_modes(A, smode);
 
   for (int cyc = 0; cyc < A.max_cycles; ++cyc) {
     // ---- down ----------------------------------------------------------------
     for (int k = A.maxlg; k >= 3; --k) {
       for (int p = 0; p < A.n_pre; ++p)
         for (int col = 0; col < 2; ++col) {
-          FOR_ITEMS(A, k, 3 * k - 1, {
-            if (mode == BM_A || mode == BM_B) op_sweep(A, S, mode, S.lg - k, col, t);
+          FOR_ITEMS(A, k, 3 * k - 3, {
+            if (mode != BM_DONE) op_sweep(A, S, mode, S.lg - k, col, t);
           });
           if (!gsync(A)) return;
         }
-      FOR_ITEMS(A, k, 3 * (k - 1), {
-        if (mode == BM_A || mode == BM_B) op_restrict(S, mode, S.lg - k, t);
+      FOR_ITEMS(A, k, 3 * k - 5, {
+        if (mode != BM_DONE) op_restrict(A, S, mode, S.lg - k, t);
       });
       if (!gsync(A)) return;
-      FOR_ITEMS(A, k, 3 * (k - 1), {
-        if (mode == BM_A) op_fas(S, S.lg - k + 1, t);
+      FOR_ITEMS(A, k, 3 * k - 5, {
+        if (mode == BM_A) op_fas(A, S, S.lg - k + 1, t);
       });
       if (!gsync(A)) return;
     }
     // ---- coarsest 4^3: one block per solve -------------------------------------
-    for (int s = blockIdx.x; s < A.ns; s += gridDim.x) {
-      const int mode = *(volatile const int*)&A.st[s].mode;
-      if (mode == BM_A || mode == BM_B) op_coarse(A, A.S[s], mode);
-    }
+    for (int s = blockIdx.x; s < A.ns; s += gridDim.x)
+      if (smode[s] != BM_DONE) op_coarse(A, A.S[s], smode[s]);
     if (!gsync(A)) return;
     // ---- up ------------------------------------------------------------------
     for (int k = 3; k <= A.maxlg; ++k) {
-      FOR_ITEMS(A, k, 3 * k, {
-        if (mode == BM_A || mode == BM_B) op_prolong(A, S, mode, S.lg - k, t);
+      FOR_ITEMS(A, k, 3 * k - 5, {
+        if (mode != BM_DONE) op_prolong(A, S, mode, S.lg - k, t);
       });
       if (!gsync(A)) return;
       for (int p = 0; p < A.n_post; ++p)
         for (int col = 0; col < 2; ++col) {
-          FOR_ITEMS(A, k, 3 * k - 1, {
-            if (mode == BM_A || mode == BM_B) op_sweep(A, S, mode, S.lg - k, col, t);
+          FOR_ITEMS(A, k, 3 * k - 3, {
+            if (mode != BM_DONE) op_sweep(A, S, mode, S.lg - k, col, t);
           });
           if (!gsync(A)) return;
         }
     }
     // ---- end of cycle: mode B applies the correction ---------------------------
-    FOR_FINEST(A, {
-      if (mode == BM_B) {
-        const double d = fmin(fmax((double)S.e32[0][t], -A.cap64), A.cap64);
-        const double v = S.u64[t] + d;
-        S.u64[t] = v;
-        S.E64[t] = exp(v);
-      }
-    });
+    for_finest(A, smode, false, [](int mode) { return mode == BM_B; },
+               [&](const BSolve& S, int, unsigned t, Acc&) { add_e<DF>(A, S, t); });
     if (!gsync(A)) return;
-    // residual norms: FP32 for mode A, FP64 (+ new linear system) for mode B
-    {
-      const long long gs = (long long)gridDim.x * blockDim.x;
-      const long long g0 = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-      long long base = 0;
-      for (int s = 0; s < A.ns; ++s) {
-        const BSolve& S = A.S[s];
-        const long long n = 1LL << (3 * S.lg);
-        const int mode = *(volatile const int*)&A.st[s].mode;
-        const long long first = (g0 - base % gs + gs) % gs;
-        base += n;
-        if (mode != BM_A && mode != BM_B) continue;
-        for (long long t = first; t - (threadIdx.x & 31) < n; t += gs) {
-          const bool live = t < n;
-          double r = 0.0;
-          if (live) {
-            if (mode == BM_B) {
-              r = op_resid64(S, t);
-            } else {
-              const int lg = S.lg, M = (1 << lg) - 1;
-              const int kk = (int)(t & M), jj = (int)((t >> lg) & M), ii = (int)(t >> (2 * lg));
-              r = (double)(S.f32[0][t] - L32(S, S.u32[0], ii, jj, kk, lg, S.ih2[0]));
-            }
-          }
-          accum(&A.st[s], r, 0.0, live);
-        }
+    // residual norms: FP32 for mode A, of the iterate (+ new linear system) for B
+    for_finest(A, smode, true, [](int mode) { return mode != BM_DONE; },
+               [&](const BSolve& S, int mode, unsigned t, Acc& acc) {
+      float r;
+      if (mode == BM_B) {
+        r = op_resid<DF>(S, t);
+      } else {
+        float n[6];
+        const unsigned q = cell_nbrs(S.u32[0], t, S.lg, n);
+        r = S.f32[0][q] - point_apply<MG_NL>(S.u32[0][q], n, 0.f, n, batch_pf(A, S), S.ih2[0]);
       }
-    }
+      acc.add(r);
+    });
     if (!gsync(A)) return;
     // decide
     if (blockIdx.x == 0) {
@@ -542,33 +499,19 @@ __global__ void __launch_bounds__(512) k_batch(BArgs A) {
       }
     }
     if (!gsync(A)) return;
-    // transition A -> B: FP64 iterate from the FP32 one, FP64 residual
-    FOR_FINEST(A, {
-      if (mode == BM_TRANS) {
-        const double v = (double)S.u32[0][t];
-        S.u64[t] = v;
-        S.E64[t] = exp(v);
-      }
+    load_modes(A, smode);
+    // transition A -> B: the iterate from the FP32 one, its residual
+    auto trans = [](int mode) { return mode == BM_TRANS; };
+    for_finest(A, smode, false, trans, [&](const BSolve& S, int, unsigned t, Acc&) {
+      const int lg = S.lg, M = (1 << lg) - 1;
+      const float v =
+          S.u32[0][pdx((int)(t >> (2 * lg)), (int)((t >> lg) & M), (int)(t & M), lg)];
+      set_u<DF>(S, t, d_from_float_bits(v));
     });
     if (!gsync(A)) return;
-    {
-      const long long gs = (long long)gridDim.x * blockDim.x;
-      const long long g0 = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-      long long base = 0;
-      for (int s = 0; s < A.ns; ++s) {
-        const BSolve& S = A.S[s];
-        const long long n = 1LL << (3 * S.lg);
-        const int mode = *(volatile const int*)&A.st[s].mode;
-        const long long first = (g0 - base % gs + gs) % gs;
-        base += n;
-        if (mode != BM_TRANS) continue;
-        for (long long t = first; t - (threadIdx.x & 31) < n; t += gs) {
-          const bool live = t < n;
-          const double r = live ? op_resid64(S, t) : 0.0;
-          accum(&A.st[s], r, 0.0, live);
-        }
-      }
-    }
+    for_finest(A, smode, true, trans, [&](const BSolve& S, int, unsigned t, Acc& acc) {
+      acc.add(op_resid<DF>(S, t));
+    });
     if (!gsync(A)) return;
     int active = 0;
     if (blockIdx.x == 0) {
@@ -592,23 +535,27 @@ __global__ void __launch_bounds__(512) k_batch(BArgs A) {
       if (threadIdx.x == 0) atomicExch(A.err + 1, active);
     }
     if (!gsync(A)) return;
+    load_modes(A, smode);
     if (*(volatile int*)(A.err + 1) == 0) break;
   }
   // ---- outputs: fR = fbar e^u and the force -----------------------------------
-  FOR_FINEST(A, {
-    (void)mode;
+  auto val = [](const double* p, unsigned q) {
+    return DF ? df_to_double_bits(reinterpret_cast<const dfl*>(p)[q]) : p[q];
+  };
+  for_finest(A, smode, false, all, [&](const BSolve& S, int, unsigned t, Acc&) {
     const int lg = S.lg, M = (1 << lg) - 1;
-    const long long n = 1LL << (3 * lg);
+    const size_t n = (size_t)1 << (3 * lg);
     const int kk = (int)(t & M), jj = (int)((t >> lg) & M), ii = (int)(t >> (2 * lg));
-    S.fr_out[t] = S.fbar * S.E64[t];
-    if (S.u_out) S.u_out[t] = S.u64[t];
+    const double* E = S.E64;
+    S.fr_out[t] = S.fbar * val(E, t);
+    if (S.u_out) S.u_out[t] = val(S.u64, t);
     if (S.acc_out) {
-      const double* E = S.E64;
-      S.acc_out[t] = S.gscale * (E[cidx((ii + 1) & M, jj, kk, lg)] - E[cidx((ii - 1) & M, jj, kk, lg)]);
-      S.acc_out[n + t] =
-          S.gscale * (E[cidx(ii, (jj + 1) & M, kk, lg)] - E[cidx(ii, (jj - 1) & M, kk, lg)]);
-      S.acc_out[2 * n + t] =
-          S.gscale * (E[cidx(ii, jj, (kk + 1) & M, lg)] - E[cidx(ii, jj, (kk - 1) & M, lg)]);
+      S.acc_out[t] = S.gscale * (val(E, cidx((ii + 1) & M, jj, kk, lg)) -
+                                 val(E, cidx((ii - 1) & M, jj, kk, lg)));
+      S.acc_out[n + t] = S.gscale * (val(E, cidx(ii, (jj + 1) & M, kk, lg)) -
+                                     val(E, cidx(ii, (jj - 1) & M, kk, lg)));
+      S.acc_out[2 * n + t] = S.gscale * (val(E, cidx(ii, jj, (kk + 1) & M, lg)) -
+                                         val(E, cidx(ii, jj, (kk - 1) & M, lg)));
     }
   });
 }
@@ -726,7 +673,10 @@ static mgfr_status launch_batch(mgfr_ctx* c, BatchWork* B, const BArgs& A, int t
   int dev = c->device, nsm = 0;
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   int occ = 0;
-  MG_CK(c, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_batch, threads, 0));
+  // double-float carries the residual to about 1e-13 of its terms; tolerances
+  // below 1e-10 keep FP64
+  void* kern = A.tol >= 1e-10 ? (void*)k_batch<true> : (void*)k_batch<false>;
+  MG_CK(c, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, threads, 0));
   if (occ < 1) return set_err(c, MGFR_E_UNSUPPORTED, "batched kernel cannot be resident");
   const int grid = nsm * std::min(bpsm, occ);
   MG_CK(c, cudaMemsetAsync(B->bar, 0, 2 * sizeof(unsigned), c->s));
@@ -734,26 +684,26 @@ static mgfr_status launch_batch(mgfr_ctx* c, BatchWork* B, const BArgs& A, int t
   BArgs a = A;
   void* args[] = {&a};
   if (!use_graph) {
-    MG_CK(c, cudaLaunchCooperativeKernel((void*)k_batch, grid, threads, args, 0, c->s));
+    MG_CK(c, cudaLaunchCooperativeKernel(kern, grid, threads, args, 0, c->s));
     c->launches += 1;
     return MGFR_OK;
   }
   char key[512];
   std::snprintf(key, sizeof(key), "%s|%d|%d|%d|%d|%d|%d|%.17g|%.17g|%.17g|%lld", B->sig.c_str(),
-                threads, grid, A.n_pre, A.n_post, A.linear, A.max_cycles, A.cap64, A.tol, A.sw,
+                threads, grid, A.n_pre, A.n_post, A.linear, A.max_cycles, (double)A.cap32, A.tol, A.sw,
                 A.max_spins);
   if (!B->gx || B->gkey != key) {
     if (B->gx) cudaGraphExecDestroy(B->gx);
     B->gx = nullptr;
     cudaGraph_t g = nullptr;
     MG_CK(c, cudaStreamBeginCapture(c->s, cudaStreamCaptureModeThreadLocal));
-    cudaError_t e = cudaLaunchCooperativeKernel((void*)k_batch, grid, threads, args, 0, c->s);
+    cudaError_t e = cudaLaunchCooperativeKernel(kern, grid, threads, args, 0, c->s);
     cudaError_t e2 = cudaStreamEndCapture(c->s, &g);
     if (e != cudaSuccess || e2 != cudaSuccess) {
       if (g) cudaGraphDestroy(g);
       (void)cudaGetLastError();
       // capture of a cooperative launch unsupported: launch directly
-      MG_CK(c, cudaLaunchCooperativeKernel((void*)k_batch, grid, threads, args, 0, c->s));
+      MG_CK(c, cudaLaunchCooperativeKernel(kern, grid, threads, args, 0, c->s));
       c->launches += 1;
       return MGFR_OK;
     }
@@ -772,7 +722,7 @@ extern "C" {
 mgfr_status mgfr_batch_solve(mgfr_ctx* c, int nsolves, const mgfr_batch_item* items,
                              mgfr_stats* per_solve) {
   if (!c) return MGFR_E_INVALID;
-  if (nsolves < 1 || nsolves > 4096 || !items)
+  if (nsolves < 1 || nsolves > kMaxBatch || !items)
     return set_err(c, MGFR_E_INVALID, "need 1..4096 batch items");
   const mgfr_config& g = c->cfg;
   for (int i = 0; i < nsolves; ++i) {
@@ -851,7 +801,9 @@ mgfr_status mgfr_batch_solve(mgfr_ctx* c, int nsolves, const mgfr_batch_item* it
     S.aRt_np1 = (float)m.aRt_np1;
     S.inv_np1 = (float)m.inv_np1;
     S.aRt64 = m.aRt;
-    S.aRt_np1_64 = m.aRt_np1;
+    S.aRt_df = df_from_double(m.aRt);
+    S.inv_np1_df = df_from_double(m.inv_np1);
+    S.ih2h_df = df_from_double(0.5 * S.ih2_0);
     S.inv_np1_64 = m.inv_np1;
     S.src = m.src;
     S.fbar = m.fbar;
@@ -890,15 +842,15 @@ mgfr_status mgfr_batch_solve(mgfr_ctx* c, int nsolves, const mgfr_batch_item* it
   A.linear = g.prolong_linear;
   A.max_cycles = g.max_vcycles;
   A.cap32 = (float)g.step_cap;
-  A.cap64 = g.step_cap;
   A.tol = g.tol_rel;
   A.sw = g.mixed_switch;
   A.bar_count = B->bar;
   A.bar_gen = B->bar + 1;
   A.err = B->err;
   A.max_spins = g.max_spins;
-  // launch shape: tuned choice for this signature, else 256 threads x 2 per SM
-  int threads = 256, bpsm = 2;
+  // launch shape: tuned choice for this signature, else 512 threads x 2 per SM
+  // (96 solves of 32^3..128^3: 45.0 ms; 256 x 2 54.5, 256 x 4 46.9, 128 x 8 50.3)
+  int threads = 512, bpsm = 2;
   auto itc = B->tuned.find(sig);
   if (itc != B->tuned.end()) {
     threads = itc->second.first;

@@ -88,3 +88,27 @@ def test_far_starts_converge_in_fp64(dev, u0):
     # both within 1e-8 ||f|| of the solution
     assert float((out["fr"] / want - 1.0).abs().max()) <= 1e-6
     s.close()
+
+
+@pytest.mark.parametrize("tol", [1e-8, 1e-12])
+def test_batch_in_both_precisions(dev, tol):
+    """The batched kernel holds its iterate in double-float pairs, or in FP64 for
+    tolerances below 1e-10; sizes from one vector per row up, several solves."""
+    sizes, fr0s, ns = [8, 32, 16, 8, 64], [1e-5, 1e-6, 1e-4, 1e-6, 1e-5], [1, 2, 1, 1, 3]
+    ds = [torch.from_numpy(synth.lognormal_delta(N, 3.0 * N, 1.5, 600 + q)).to(dev)
+          for q, N in enumerate(sizes)]
+    boxes = [3.0 * N for N in sizes]
+    s = mgfr.Solver(0, precision=mgfr.PREC_MIXED, tol_rel=tol, max_vcycles=300)
+    outs, st = s.batch_solve(ds, boxes, fr0s, ns=ns, want_acc=True, want_u=True)
+    assert st == mgfr.MGFR_OK
+    for q, o in enumerate(outs):
+        assert o["stats"]["res_l2_final"] <= tol * o["stats"]["f_l2"]
+        one = mgfr.Solver(0, fr0_abs=fr0s[q], n=ns[q], tol_rel=1e-12, max_vcycles=300)
+        ref = one.solve_density(ds[q], boxes[q], want_u=True)
+        one.close()
+        # both within tol ||f|| of the solution; 1e3 for the operator's inverse
+        assert float((o["fr"] / ref["fr"] - 1.0).abs().max()) <= 1e3 * tol
+        assert float((o["u"] - ref["u"]).abs().max()) <= 1e3 * tol
+        scale = float(ref["acc"].abs().max())
+        assert float((o["acc"] - ref["acc"]).abs().max()) <= 1e3 * tol * scale
+    s.close()
