@@ -180,6 +180,8 @@ mgfr_status set_err(mgfr_ctx* c, mgfr_status st, const std::string& msg);
 bool validate_cfg(const mgfr_config* c, std::string& why);
 void batch_free(mgfr_ctx* c);
 void unet_free(mgfr_ctx* c);
+// give back the convolution primitive's scratch on this device (unet.cu)
+void conv_scratch_trim(int dev);
 void pm_free(mgfr_ctx* c);
 #define MG_CK(ctx, call)                                                                  \
   do {                                                                                    \

@@ -197,46 +197,48 @@ __global__ void k_wgrad_reduce(const float* __restrict__ partials, int S, long l
   dW[i] = s;
 }
 
-// db[c] = sum over voxels of g[m][c].  The additions follow one fixed order:
-// for each slot t < 256 the voxels m = t, t + 256, t + 512, ... in turn, then
-// a pairwise tree over the 256 slot sums (stride 128, 64, ..., 1).  Stage 1
-// gives every (slot, channel) pair its own thread (consecutive threads take
-// consecutive channels of one voxel, so a warp's loads are contiguous) and
-// keeps 32 loads of the chain in flight; stage 2 runs the tree, one block
-// per channel.
-constexpr int BG_SLOTS = 256;
+// db[c] = sum over voxels of g[m][c].  Each thread sums 8 channels (16-byte
+// loads) of its voxels, the block's threads of a channel group are added in
+// order, and the blocks' sums in order by one warp per channel: fixed orders,
+// short chains (one thread per (slot, channel) with 4096-element chains took
+// 78 us per full-resolution layer; this is bound by reading g).
+constexpr int BG_BLOCKS = 152;
+constexpr int BG_BS = 256;
 
-__global__ void __launch_bounds__(128) k_bias_slots(const __nv_bfloat16* __restrict__ g, int ldg,
-                                                    int offg, long long Mtot, int Cout,
-                                                    float* __restrict__ part) {
-  const long long T = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (T >= (long long)BG_SLOTS * Cout) return;
-  const int c = (int)(T % Cout), t = (int)(T / Cout);
-  constexpr int U = 32;
-  float s = 0.f;
-  long long m = t;
-  for (; m + (U - 1) * (long long)BG_SLOTS < Mtot; m += U * (long long)BG_SLOTS) {
-    float v[U];
+__global__ void __launch_bounds__(BG_BS) k_bias_part(const __nv_bfloat16* __restrict__ g, int ldg,
+                                                     int offg, long long Mtot, int Cout,
+                                                     float* __restrict__ part) {
+  __shared__ float red[BG_BS][8];
+  const int ng = Cout / 8, vpb = BG_BS / ng;  // channel groups, voxels per pass
+  const int c8 = threadIdx.x % ng, vo = threadIdx.x / ng;
+  float s[8] = {};
+  if (vo < vpb)
+    for (long long m = (long long)blockIdx.x * vpb + vo; m < Mtot; m += (long long)gridDim.x * vpb) {
+      const uint4 q = *reinterpret_cast<const uint4*>(g + m * ldg + offg + 8 * c8);
+      const unsigned w[4] = {q.x, q.y, q.z, q.w};
 #pragma unroll
-    for (int q = 0; q < U; ++q) v[q] = __bfloat162float(g[(m + q * BG_SLOTS) * ldg + offg + c]);
+      for (int i = 0; i < 4; ++i) {
+        s[2 * i] += __uint_as_float(w[i] << 16);
+        s[2 * i + 1] += __uint_as_float(w[i] & 0xffff0000u);
+      }
+    }
 #pragma unroll
-    for (int q = 0; q < U; ++q) s += v[q];
+  for (int i = 0; i < 8; ++i) red[threadIdx.x][i] = s[i];
+  __syncthreads();
+  for (int c = threadIdx.x; c < Cout; c += BG_BS) {
+    float a = 0.f;
+    for (int v = 0; v < vpb; ++v) a += red[v * ng + c / 8][c & 7];
+    part[(long long)blockIdx.x * Cout + c] = a;
   }
-  for (; m < Mtot; m += BG_SLOTS) s += __bfloat162float(g[m * ldg + offg + c]);
-  part[(long long)t * Cout + c] = s;
 }
 
-__global__ void __launch_bounds__(BG_SLOTS) k_bias_tree(const float* __restrict__ part, int Cout,
-                                                        float* __restrict__ db) {
-  __shared__ float red[BG_SLOTS];
-  const int c = blockIdx.x, t = threadIdx.x;
-  red[t] = part[(long long)t * Cout + c];
-  __syncthreads();
-  for (int w = BG_SLOTS / 2; w > 0; w >>= 1) {
-    if (t < w) red[t] += red[t + w];
-    __syncthreads();
-  }
-  if (t == 0) db[c] = red[0];
+__global__ void __launch_bounds__(32) k_bias_sum(const float* __restrict__ part, int nb, int Cout,
+                                                 float* __restrict__ db) {
+  const int c = blockIdx.x, lane = threadIdx.x;
+  float s = 0.f;
+  for (int q = lane; q < nb; q += 32) s += part[(long long)q * Cout + c];
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if (lane == 0) db[c] = s;
 }
 
 constexpr int WG_S_TARGET = 608;  // about 4 blocks per SM of partial tiles
@@ -278,9 +280,8 @@ void nn_wgrad_finish(float* partials, int S, int Cin, int Cout, float* dW, TView
   if (!db) return;
   // the bias stages reuse the partials (read by k_wgrad_reduce before them on
   // this stream); they hold S * 27 * Cin * Cout >= 432 * Cout floats (Cin >= 16)
-  const long long nt = (long long)BG_SLOTS * Cout;
-  k_bias_slots<<<(unsigned)((nt + 127) / 128), 128, 0, s>>>(g.p, g.ld, g.off, Mtot, Cout, partials);
-  k_bias_tree<<<Cout, BG_SLOTS, 0, s>>>(partials, Cout, db);
+  k_bias_part<<<BG_BLOCKS, BG_BS, 0, s>>>(g.p, g.ld, g.off, Mtot, Cout, partials);
+  k_bias_sum<<<Cout, 32, 0, s>>>(partials, BG_BLOCKS, Cout, db);
 }
 
 long long nn_wgrad_scratch(int Cin, int Cout) {

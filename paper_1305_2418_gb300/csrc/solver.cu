@@ -699,6 +699,7 @@ void mgfr_destroy(mgfr_ctx* c) {
   amr_free(c);
   batch_free(c);
   unet_free(c);
+  conv_scratch_trim(c->device);
   pm_free(c);
   if (c->u_learn) cudaFree(c->u_learn);
   for (auto e : c->evpool) cudaEventDestroy(e);

@@ -20,9 +20,11 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <mutex>
 #include <random>
 #include <vector>
 
+#include "lean_fp64.cuh"
 #include "nn_kernels.cuh"
 
 namespace {
@@ -50,105 +52,227 @@ const ConvSpec kConvs[14] = {
 // output's own variable: asinh(u_scr / 0.01) / 5 (of order one).
 constexpr double U_SCALE_F = 0.01;  // the output variable's scale (U_SCALE below)
 
-__global__ void k_features(const double* __restrict__ delta, const double* __restrict__ fr0s,
-                           long long per, long long M, __nv_bfloat16* __restrict__ x,
-                           double scr, double np1, double dscale) {
+// the features in FP64 throughout (bf16 of the FP32-rounded value)
+__device__ __noinline__ void features64(double d, double scr, double np1, __nv_bfloat16* ln,
+                                        __nv_bfloat16* scv) {
+  *ln = __float2bfloat16((float)log(fmax(1.0 + d, 1e-3)));
+  const double ul = fmin(fmax(-np1 * log(fmax(1.0 + scr * d, 1e-6)), -20.0), 5.0);
+  *scv = __float2bfloat16((float)(asinh(ul / U_SCALE_F) / 5.0));
+}
+
+// whether an FP32 value accurate to 8 ulp decides its rounding to bf16: it is
+// further than 12 ulp from the midpoint of two bf16 values
+__device__ __forceinline__ bool bf16_decided(float v) {
+  const int low = (int)(__float_as_uint(v) & 0xffffu) - 0x8000;
+  return low > 12 || low < -12;
+}
+
+// ln(max(1 + y, lo)) of the FP64 sum 1 + y to a few FP32 ulp: log1pf of what the
+// sum kept of y where 1 + y is near 1
+__device__ __forceinline__ float ln1p(double y, float lo) {
+  const double x = 1.0 + y;
+  const float yf = f_from_double_bits(x - 1.0);
+  return fabsf(yf) < 0.5f ? log1pf(yf) : logf(fmaxf(f_from_double_bits(x), lo));
+}
+
+__global__ void k_fr0_feature(const double* __restrict__ fr0s, int B,
+                              __nv_bfloat16* __restrict__ out) {
+  const int b = blockIdx.x * blockDim.x + threadIdx.x;
+  if (b < B) out[b] = __float2bfloat16((float)(log10(fr0s[b]) + 5.0));
+}
+
+// The features are bf16: FP32 functions (log1pf, logf and asinhf, each within a
+// few ulp, 8 at most together) decide them except within 12 FP32 ulp of a rounding midpoint (one
+// value in 2700), where the FP64 form decides, so the result is that of FP64
+// everywhere.  Memory bound (40 bytes per voxel); the FP64 functions took 5.2 ms
+// for 256^3.
+__global__ void __launch_bounds__(BS) k_features(const double* __restrict__ delta,
+                                                 const __nv_bfloat16* __restrict__ ffr0, int lg3,
+                                                 long long M, __nv_bfloat16* __restrict__ x,
+                                                 double scr, double np1, double dscale) {
   const long long m = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (m >= M) return;
   const double d = dscale * delta[m];
-  const double fr0 = fr0s[m / per];
-  __nv_bfloat16* o = x + m * 16;
-  o[0] = __float2bfloat16((float)log(fmax(1.0 + d, 1e-3)));
-  o[1] = __float2bfloat16((float)(log10(fr0) + 5.0));
-  o[2] = __float2bfloat16(1.f);
-  const double ul = fmin(fmax(-np1 * log(fmax(1.0 + scr * d, 1e-6)), -20.0), 5.0);
-  o[3] = __float2bfloat16((float)(asinh(ul / U_SCALE_F) / 5.0));
-  for (int c = 4; c < 16; ++c) o[c] = __float2bfloat16(0.f);
+  const float l = ln1p(d, 1e-3f);
+  const float ul =
+      fminf(fmaxf(-(float)np1 * ln1p(scr * d, 1e-6f), -20.f), 5.f);
+  const float a = asinhf(ul * (float)(1.0 / U_SCALE_F)) * 0.2f;
+  __nv_bfloat16 ln = __float2bfloat16(l), sc = __float2bfloat16(a);
+  if (!(bf16_decided(l) && bf16_decided(a))) features64(d, scr, np1, &ln, &sc);
+  auto bits = [](__nv_bfloat16 v) { return (unsigned)__bfloat16_as_ushort(v); };
+  uint4* o = reinterpret_cast<uint4*>(x + m * 16);
+  o[0] = make_uint4(bits(ln) | (bits(ffr0[m >> lg3]) << 16),
+                    bits(__float2bfloat16(1.f)) | (bits(sc) << 16), 0u, 0u);
+  o[1] = make_uint4(0u, 0u, 0u, 0u);
+}
+
+// ---- elementwise kernels on 8-channel (16-byte BF16, 32-byte FP32) chunks; a
+// thread's chunk index is e = voxel (C/8) + chunk, C/8 a power of two ----------
+struct B8 {
+  float v[8];
+};
+__device__ __forceinline__ B8 ldb8(const __nv_bfloat16* p) {
+  const uint4 q = *reinterpret_cast<const uint4*>(p);
+  const unsigned w[4] = {q.x, q.y, q.z, q.w};
+  B8 r;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    r.v[2 * i] = __uint_as_float(w[i] << 16);
+    r.v[2 * i + 1] = __uint_as_float(w[i] & 0xffff0000u);
+  }
+  return r;
+}
+__device__ __forceinline__ uint4 packb8(const float* v) {
+  unsigned w[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+    w[i] = (unsigned)__bfloat16_as_ushort(__float2bfloat16(v[2 * i])) |
+           ((unsigned)__bfloat16_as_ushort(__float2bfloat16(v[2 * i + 1])) << 16);
+  return make_uint4(w[0], w[1], w[2], w[3]);
+}
+__device__ __forceinline__ B8 ldf8(const float* p) {
+  const float4 a = reinterpret_cast<const float4*>(p)[0], b = reinterpret_cast<const float4*>(p)[1];
+  return B8{{a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w}};
+}
+__device__ __forceinline__ void stf8(float* p, const B8& x) {
+  reinterpret_cast<float4*>(p)[0] = make_float4(x.v[0], x.v[1], x.v[2], x.v[3]);
+  reinterpret_cast<float4*>(p)[1] = make_float4(x.v[4], x.v[5], x.v[6], x.v[7]);
+}
+// daughter q of coarse voxel mc (grid 2^lgc), parent of fine voxel mf (2^lgf)
+__device__ __forceinline__ unsigned daughter(unsigned mc, int lgc, int q) {
+  const unsigned Mc = (1u << lgc) - 1;
+  const unsigned K = mc & Mc, J = (mc >> lgc) & Mc, bI = mc >> (2 * lgc);  // sample and I
+  return (((2 * bI + (q >> 2)) << (lgc + 1)) + 2 * J + ((q >> 1) & 1) << (lgc + 1)) + 2 * K +
+         (q & 1);
+}
+__device__ __forceinline__ unsigned parent(unsigned mf, int lgf) {
+  const unsigned Mf = (1u << lgf) - 1;
+  const unsigned k = mf & Mf, j = (mf >> lgf) & Mf, bi = mf >> (2 * lgf);
+  return (((bi >> 1) << (lgf - 1)) + (j >> 1) << (lgf - 1)) + (k >> 1);
 }
 
 // 2^3 average pooling: y[M'][c] from x (full res, view)
-__global__ void k_pool(TView x, TView y, int C, int lgDc, long long Mc) {
-  const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (t >= Mc * C) return;
-  const long long mc = t / C;
-  const int c = (int)(t % C);
-  const long long per = 1LL << (3 * lgDc);
-  const long long b = mc / per, r = mc % per;
-  const int Dc = 1 << lgDc, lgDf = lgDc + 1;
-  const int I = (int)(r >> (2 * lgDc)), J = (int)((r >> lgDc) & (Dc - 1)), K = (int)(r & (Dc - 1));
-  float s = 0.f;
+__global__ void __launch_bounds__(BS) k_pool(TView x, TView y, int lc8, int lgDc, long long n) {
+  const long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  if (e >= n) return;
+  const unsigned mc = (unsigned)(e >> lc8);
+  const int c = 8 * (int)(e & ((1 << lc8) - 1));
+  float s[8] = {};
+#pragma unroll
   for (int q = 0; q < 8; ++q) {
-    const long long mf = (b << (3 * lgDf)) +
-                         ((((long long)(2 * I + (q >> 2)) << lgDf) + (2 * J + ((q >> 1) & 1))) << lgDf) +
-                         (2 * K + (q & 1));
-    s += __bfloat162float(x.p[mf * x.ld + x.off + c]);
+    const B8 v = ldb8(x.p + (size_t)daughter(mc, lgDc, q) * x.ld + x.off + c);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) s[i] += v.v[i];
   }
-  y.p[mc * y.ld + y.off + c] = __float2bfloat16(0.125f * s);
+#pragma unroll
+  for (int i = 0; i < 8; ++i) s[i] *= 0.125f;
+  *reinterpret_cast<uint4*>(y.p + (size_t)mc * y.ld + y.off + c) = packb8(s);
 }
 
 // g_fine[child][c] += g_coarse[parent][c] / 8
-__global__ void k_pool_bwd(FView gc, FView gf, int C, int lgDf, long long Mf) {
-  const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (t >= Mf * C) return;
-  const long long mf = t / C;
-  const int c = (int)(t % C);
-  const long long per = 1LL << (3 * lgDf);
-  const long long b = mf / per, r = mf % per;
-  const int Df = 1 << lgDf, lgDc = lgDf - 1;
-  const int i = (int)(r >> (2 * lgDf)), j = (int)((r >> lgDf) & (Df - 1)), k = (int)(r & (Df - 1));
-  const long long mc = (b << (3 * lgDc)) + ((((long long)(i >> 1) << lgDc) + (j >> 1)) << lgDc) + (k >> 1);
-  gf.p[mf * gf.ld + gf.off + c] += 0.125f * gc.p[mc * gc.ld + gc.off + c];
+__global__ void __launch_bounds__(BS) k_pool_bwd(FView gc, FView gf, int lc8, int lgDf,
+                                                 long long n) {
+  const long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  if (e >= n) return;
+  const unsigned mf = (unsigned)(e >> lc8);
+  const int c = 8 * (int)(e & ((1 << lc8) - 1));
+  const B8 g = ldf8(gc.p + (size_t)parent(mf, lgDf) * gc.ld + gc.off + c);
+  float* q = gf.p + (size_t)mf * gf.ld + gf.off + c;
+  B8 v = ldf8(q);
+#pragma unroll
+  for (int i = 0; i < 8; ++i) v.v[i] += 0.125f * g.v[i];
+  stf8(q, v);
 }
 
-// nearest upsampling: y[fine][c] = x[parent][c]
-__global__ void k_up(TView x, TView y, int C, int lgDf, long long Mf) {
-  const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (t >= Mf * C) return;
-  const long long mf = t / C;
-  const int c = (int)(t % C);
-  const long long per = 1LL << (3 * lgDf);
-  const long long b = mf / per, r = mf % per;
-  const int Df = 1 << lgDf, lgDc = lgDf - 1;
-  const int i = (int)(r >> (2 * lgDf)), j = (int)((r >> lgDf) & (Df - 1)), k = (int)(r & (Df - 1));
-  const long long mc = (b << (3 * lgDc)) + ((((long long)(i >> 1) << lgDc) + (j >> 1)) << lgDc) + (k >> 1);
-  y.p[mf * y.ld + y.off + c] = x.p[mc * x.ld + x.off + c];
+// nearest upsampling: y[fine][c] = x[parent][c] (one channel per thread took
+// 2.7 ms for the three levels of a 256^3 box)
+__global__ void __launch_bounds__(BS) k_up(TView x, TView y, int lc8, int lgDf, long long n) {
+  const long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  if (e >= n) return;
+  const unsigned mf = (unsigned)(e >> lc8);
+  const int c = 8 * (int)(e & ((1 << lc8) - 1));
+  *reinterpret_cast<uint4*>(y.p + (size_t)mf * y.ld + y.off + c) =
+      *reinterpret_cast<const uint4*>(x.p + (size_t)parent(mf, lgDf) * x.ld + x.off + c);
 }
 
 // g_coarse[parent][c] = sum of the 8 children's gradients
-__global__ void k_up_bwd(FView gf, FView gc, int C, int lgDc, long long Mc) {
-  const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (t >= Mc * C) return;
-  const long long mc = t / C;
-  const int c = (int)(t % C);
-  const long long per = 1LL << (3 * lgDc);
-  const long long b = mc / per, r = mc % per;
-  const int Dc = 1 << lgDc, lgDf = lgDc + 1;
-  const int I = (int)(r >> (2 * lgDc)), J = (int)((r >> lgDc) & (Dc - 1)), K = (int)(r & (Dc - 1));
-  float s = 0.f;
+__global__ void __launch_bounds__(BS) k_up_bwd(FView gf, FView gc, int lc8, int lgDc,
+                                               long long n) {
+  const long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  if (e >= n) return;
+  const unsigned mc = (unsigned)(e >> lc8);
+  const int c = 8 * (int)(e & ((1 << lc8) - 1));
+  B8 s{};
+#pragma unroll
   for (int q = 0; q < 8; ++q) {
-    const long long mf = (b << (3 * lgDf)) +
-                         ((((long long)(2 * I + (q >> 2)) << lgDf) + (2 * J + ((q >> 1) & 1))) << lgDf) +
-                         (2 * K + (q & 1));
-    s += gf.p[mf * gf.ld + gf.off + c];
+    const B8 v = ldf8(gf.p + (size_t)daughter(mc, lgDc, q) * gf.ld + gf.off + c);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) s.v[i] += v.v[i];
   }
-  gc.p[mc * gc.ld + gc.off + c] = s;
+  stf8(gc.p + (size_t)mc * gc.ld + gc.off + c, s);
 }
 
-// gradient of the pre-activation: g * (y > 0), to BF16, contiguous [M][C]
-__global__ void k_relu_bwd(FView g, TView y, int C, long long M, __nv_bfloat16* __restrict__ out) {
-  const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (t >= M * C) return;
-  const long long m = t / C;
-  const int c = (int)(t % C);
-  const float yy = __bfloat162float(y.p[m * y.ld + y.off + c]);
-  out[t] = __float2bfloat16(yy > 0.f ? g.p[m * g.ld + g.off + c] : 0.f);
+// gradient of the pre-activation: g * (y > 0), to BF16, contiguous [M][C], and
+// the bias gradient's partial sums over this block's voxels (of the BF16
+// values; part [block][C]).  The grid stride is a multiple of C/8, so a thread
+// keeps its channels; the block's threads of a channel group are added in a
+// fixed order.
+__global__ void __launch_bounds__(BS) k_relu_bwd(FView g, TView y, int lc8, long long n,
+                                                 __nv_bfloat16* __restrict__ out,
+                                                 float* __restrict__ part) {
+  __shared__ float red[8][BS];
+  float s[8] = {};
+  for (long long e = blockIdx.x * (long long)BS + threadIdx.x; e < n;
+       e += (long long)gridDim.x * BS) {
+    const size_t m = (size_t)(e >> lc8);
+    const int c = 8 * (int)(e & ((1 << lc8) - 1));
+    const B8 yy = ldb8(y.p + m * y.ld + y.off + c);
+    B8 gg = ldf8(g.p + m * g.ld + g.off + c);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      gg.v[i] = __bfloat162float(__float2bfloat16(yy.v[i] > 0.f ? gg.v[i] : 0.f));
+      s[i] += gg.v[i];
+    }
+    *reinterpret_cast<uint4*>(out + 8 * e) = packb8(gg.v);
+  }
+#pragma unroll
+  for (int i = 0; i < 8; ++i) red[i][threadIdx.x] = s[i];
+  __syncthreads();
+  const int ng = 1 << lc8;  // channel groups; group of thread t: t & (ng - 1)
+  for (int w = BS / 2; w >= ng; w >>= 1) {
+    if ((int)threadIdx.x < w)
+#pragma unroll
+      for (int i = 0; i < 8; ++i) red[i][threadIdx.x] += red[i][threadIdx.x + w];
+    __syncthreads();
+  }
+  if ((int)threadIdx.x < ng)
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+      part[(size_t)blockIdx.x * 8 * ng + 8 * threadIdx.x + i] = red[i][threadIdx.x];
 }
 
-__global__ void k_head_fwd(TView x, const float* __restrict__ w, long long M, float* __restrict__ out) {
+// db[c] = the blocks' partial sums, in order of the blocks within each of 32
+// lanes, then a fixed tree; one warp per channel
+__global__ void k_bias_parts(const float* __restrict__ part, int nb, int C,
+                             float* __restrict__ db) {
+  const int c = blockIdx.x, lane = threadIdx.x;
+  float s = 0.f;
+  for (int q = lane; q < nb; q += 32) s += part[(size_t)q * C + c];
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if (lane == 0) db[c] = s;
+}
+
+__global__ void __launch_bounds__(BS) k_head_fwd(TView x, const float* __restrict__ w, long long M,
+                                                 float* __restrict__ out) {
   const long long m = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (m >= M) return;
   float s = w[16];
-  for (int c = 0; c < 16; ++c) s = fmaf(w[c], __bfloat162float(x.p[m * x.ld + x.off + c]), s);
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const B8 v = ldb8(x.p + m * x.ld + x.off + 8 * h);
+#pragma unroll
+    for (int c = 0; c < 8; ++c) s = fmaf(w[8 * h + c], v.v[c], s);
+  }
   out[m] = s;
 }
 
@@ -157,16 +281,27 @@ __global__ void k_head_fwd(TView x, const float* __restrict__ w, long long M, fl
 // to ~10) have comparable weight in the loss.
 constexpr double U_SCALE = 0.01;
 
+// asinh(x): the FP32 value y, then one Newton step on sinh y = x with sinh y
+// from two FP64 exponentials (24 FP64 instructions against about 100); the
+// step's relative error 1e-7 leaves 1e-14
+__device__ __forceinline__ double asinh_lean(double x) {
+  const float yf = asinhf(f_from_double_bits(x));
+  if (!(fabsf(yf) < 80.f)) return asinh(x);
+  const double y = d_from_float_bits(yf), e = lean_exp(y), ei = lean_exp(-y);
+  const float d = f_from_double_bits(fma(0.5, ei - e, x));  // x - sinh y
+  return y + d_from_float_bits(d / coshf(yf));
+}
+
 // loss partials (in v) and d loss / d out = 2 (out - v) / M
 __global__ void k_mse(const float* __restrict__ out, const double* __restrict__ target, long long M,
-                      float* __restrict__ gout, double* __restrict__ partial) {
+                      double gscale, float* __restrict__ gout, double* __restrict__ partial) {
   __shared__ double red[BS];
   double s = 0.0;
   for (long long m = blockIdx.x * (long long)blockDim.x + threadIdx.x; m < M;
        m += (long long)gridDim.x * blockDim.x) {
-    const double d = (double)out[m] - asinh(target[m] / U_SCALE);
-    s += d * d;
-    gout[m] = (float)(2.0 * d / (double)M);
+    const double d = d_from_float_bits(out[m]) - asinh_lean(target[m] * (1.0 / U_SCALE));
+    s = fma(d, d, s);
+    gout[m] = f_from_double_bits(d * gscale);
   }
   red[threadIdx.x] = s;
   __syncthreads();
@@ -185,9 +320,16 @@ __global__ void k_head_bwd(TView x, const float* __restrict__ w, const float* __
   for (long long m = blockIdx.x * (long long)blockDim.x + threadIdx.x; m < M;
        m += (long long)gridDim.x * blockDim.x) {
     const float g = gout[m];
-    for (int c = 0; c < 16; ++c) {
-      acc[c] = fmaf(g, __bfloat162float(x.p[m * x.ld + x.off + c]), acc[c]);
-      gx.p[m * gx.ld + gx.off + c] = g * w[c];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const B8 v = ldb8(x.p + m * x.ld + x.off + 8 * h);
+      B8 o;
+#pragma unroll
+      for (int c = 0; c < 8; ++c) {
+        acc[8 * h + c] = fmaf(g, v.v[c], acc[8 * h + c]);
+        o.v[c] = g * w[8 * h + c];
+      }
+      stf8(gx.p + m * gx.ld + gx.off + 8 * h, o);
     }
     acc[16] += g;
   }
@@ -226,9 +368,30 @@ __global__ void k_adam(float* __restrict__ p, const float* __restrict__ g, float
   p[i] -= lr * (a / c1) / (sqrtf(b / c2) + eps);
 }
 
-__global__ void k_to_bf16(const float* __restrict__ x, __nv_bfloat16* __restrict__ y, long long n) {
-  const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (i < n) y[i] = __float2bfloat16(x[i]);
+// The BF16 copies of the 14 convolutions' weights: as they are, and packed for
+// the tensor-core forward and input gradient (nn_tc_pack's layouts); one launch
+// for all (42 launches took 140 us of a training step).
+struct PackTab {
+  long long woff[14], boff[15];  // FP32 parameters, BF16 offsets (boff[14]: the end)
+  int cin[14], cout[14];
+};
+__global__ void __launch_bounds__(BS) k_refresh(const float* __restrict__ P, PackTab T,
+                                                __nv_bfloat16* __restrict__ Wbf,
+                                                __nv_bfloat16* __restrict__ Wtf,
+                                                __nv_bfloat16* __restrict__ Wtd) {
+  const long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  if (e >= T.boff[14]) return;
+  int i = 0;
+#pragma unroll
+  for (int q = 1; q < 14; ++q) i += e >= T.boff[q] ? 1 : 0;
+  const unsigned r = (unsigned)(e - T.boff[i]), ci_n = T.cin[i], co_n = T.cout[i];
+  const unsigned co = r % co_n, ci = (r / co_n) % ci_n, t = r / (co_n * ci_n);
+  const __nv_bfloat16 v = __float2bfloat16(P[T.woff[i] + r]);
+  Wbf[e] = v;
+  const unsigned per = ci_n * co_n;
+  // forward: [t][ci / 8][co][ci & 7]; input gradient: [t][co / 8][ci][co & 7]
+  Wtf[T.boff[i] + t * per + ((ci >> 3) * co_n + co) * 8 + (ci & 7)] = v;
+  Wtd[T.boff[i] + t * per + ((co >> 3) * ci_n + ci) * 8 + (co & 7)] = v;
 }
 
 // u = U_SCALE sinh(v)
@@ -240,6 +403,14 @@ __global__ void k_out_to_double(const float* __restrict__ x, double* __restrict_
 }  // namespace
 
 // ============================================================================
+static int lg_of(int D) {
+  int lg = 0;
+  while ((1 << lg) < D) ++lg;
+  return lg;
+}
+
+constexpr int kBiasBlocks = 152 * 8;  // blocks of k_relu_bwd
+
 struct UNet {
   // parameter layout in one flat FP32 array: per conv W[27][cin][cout], b[cout]; head w[16], b
   long long woff[14], boff[14], head_off = 0, nparam = 0;
@@ -257,7 +428,8 @@ struct UNet {
   __nv_bfloat16 *X0, *E1a, *CAT1, *P1, *E2a, *CAT2, *P2, *E3a, *CAT3, *P3, *Ba, *Bb, *D3a, *D3b,
       *D2a, *D2b, *D1a, *D1b, *Gpre;
   float *OUT, *GOUT, *G_E1a, *G_CAT1, *G_P1, *G_E2a, *G_CAT2, *G_P2, *G_E3a, *G_CAT3, *G_P3, *G_Ba,
-      *G_Bb, *G_D3a, *G_D3b, *G_D2a, *G_D2b, *G_D1a, *G_D1b, *wpart;
+      *G_Bb, *G_D3a, *G_D3b, *G_D2a, *G_D2b, *G_D1a, *G_D1b, *wpart, *bpart;
+  __nv_bfloat16* ffr0 = nullptr;  // the feature log10|fR0| + 5 per sample
   double* fr0d = nullptr;
   double* lossp = nullptr;
   long long wpart_n = 0;
@@ -340,6 +512,8 @@ static mgfr_status unet_alloc(mgfr_ctx* c, UNet* U, int B, int lgD) {
                                nn_tc_wgrad_scratch(cs.cin, cs.cout)));
   U->wpart_n = wn;
   U->wpart = f(std::max(wn, 17LL * 1024));
+  U->bpart = f(128LL * kBiasBlocks);
+  U->ffr0 = bf(4096);
   void* p = nullptr;
   if (cudaMalloc(&p, sizeof(double) * 1024) != cudaSuccess) return set_err(c, MGFR_E_OOM, "unet");
   U->bufs.push_back(p);
@@ -413,12 +587,12 @@ static void forward(mgfr_ctx* c, UNet* U) {
   const long long M0 = (long long)B << (3 * g);
   auto launch_pool = [&](TView x, TView y, int C, int lgDc) {
     const long long Mc = (long long)B << (3 * lgDc);
-    k_pool<<<nblocks(Mc * C, BS), BS, 0, c->s>>>(x, y, C, lgDc, Mc);
+    k_pool<<<nblocks(Mc * C / 8, BS), BS, 0, c->s>>>(x, y, lg_of(C / 8), lgDc, Mc * C / 8);
     c->launches += 1;
   };
   auto launch_up = [&](TView x, TView y, int C, int lgDf) {
     const long long Mf = (long long)B << (3 * lgDf);
-    k_up<<<nblocks(Mf * C, BS), BS, 0, c->s>>>(x, y, C, lgDf, Mf);
+    k_up<<<nblocks(Mf * C / 8, BS), BS, 0, c->s>>>(x, y, lg_of(C / 8), lgDf, Mf * C / 8);
     c->launches += 1;
   };
   conv_fwd(c, U, 0, L[0]);
@@ -448,12 +622,15 @@ static void forward(mgfr_ctx* c, UNet* U) {
 static void conv_bwd(mgfr_ctx* c, UNet* U, int i, const LayerIO& L, int acc_in) {
   const ConvSpec& s = kConvs[i];
   const long long M = (long long)U->B << (3 * L.lgD);
-  k_relu_bwd<<<nblocks(M * s.cout, BS), BS, 0, c->s>>>(L.gy, L.y, s.cout, M, U->Gpre);
+  // the bias gradient comes out of the pass that forms the pre-activation's
+  const long long n8 = M * s.cout / 8;
+  const int nb = (int)std::min<long long>(kBiasBlocks, nblocks(n8, BS));
+  k_relu_bwd<<<nb, BS, 0, c->s>>>(L.gy, L.y, lg_of(s.cout / 8), n8, U->Gpre, U->bpart);
+  k_bias_parts<<<s.cout, 32, 0, c->s>>>(U->bpart, nb, s.cout, U->G + U->boff[i]);
   const TView g = tv(U->Gpre, s.cout);
-  if (!nn_tc_wgrad(L.x, s.cin, g, s.cout, U->G + U->woff[i], U->G + U->boff[i], U->wpart, U->B,
-                   L.lgD, U->tc_err, c->s))
-    nn_conv_wgrad(L.x, s.cin, g, s.cout, U->G + U->woff[i], U->G + U->boff[i], U->wpart, U->B,
-                  L.lgD, c->s);
+  if (!nn_tc_wgrad(L.x, s.cin, g, s.cout, U->G + U->woff[i], nullptr, U->wpart, U->B, L.lgD,
+                   U->tc_err, c->s))
+    nn_conv_wgrad(L.x, s.cin, g, s.cout, U->G + U->woff[i], nullptr, U->wpart, U->B, L.lgD, c->s);
   if (L.gx.p) {
     if (nn_tc_supported(s.cout, s.cin)) {
       TcArgs a{};
@@ -488,12 +665,12 @@ static void backward(mgfr_ctx* c, UNet* U) {
   c->launches += 2;
   auto up_bwd = [&](FView gf, FView gc, int C, int lgDc) {
     const long long Mc = (long long)B << (3 * lgDc);
-    k_up_bwd<<<nblocks(Mc * C, BS), BS, 0, c->s>>>(gf, gc, C, lgDc, Mc);
+    k_up_bwd<<<nblocks(Mc * C / 8, BS), BS, 0, c->s>>>(gf, gc, lg_of(C / 8), lgDc, Mc * C / 8);
     c->launches += 1;
   };
   auto pool_bwd = [&](FView gc, FView gf, int C, int lgDf) {
     const long long Mf = (long long)B << (3 * lgDf);
-    k_pool_bwd<<<nblocks(Mf * C, BS), BS, 0, c->s>>>(gc, gf, C, lgDf, Mf);
+    k_pool_bwd<<<nblocks(Mf * C / 8, BS), BS, 0, c->s>>>(gc, gf, lg_of(C / 8), lgDf, Mf * C / 8);
     c->launches += 1;
   };
   conv_bwd(c, U, 13, L[13], 0);                        // -> G_D1a
@@ -519,14 +696,16 @@ static void backward(mgfr_ctx* c, UNet* U) {
 }
 
 static void refresh_bf16(mgfr_ctx* c, UNet* U) {
+  PackTab T;
   for (int i = 0; i < 14; ++i) {
-    const ConvSpec& s = kConvs[i];
-    const long long n = 27LL * s.cin * s.cout;
-    k_to_bf16<<<nblocks(n, BS), BS, 0, c->s>>>(U->P + U->woff[i], U->Wbf + U->wbf_off[i], n);
-    nn_tc_pack(U->Wbf + U->wbf_off[i], s.cin, s.cout, 0, U->Wtf + U->wbf_off[i], c->s);
-    nn_tc_pack(U->Wbf + U->wbf_off[i], s.cin, s.cout, 1, U->Wtd + U->wbf_off[i], c->s);
-    c->launches += 3;
+    T.woff[i] = U->woff[i];
+    T.boff[i] = U->wbf_off[i];
+    T.cin[i] = kConvs[i].cin;
+    T.cout[i] = kConvs[i].cout;
   }
+  T.boff[14] = U->nwbf;
+  k_refresh<<<nblocks(U->nwbf, BS), BS, 0, c->s>>>(U->P, T, U->Wbf, U->Wtf, U->Wtd);
+  c->launches += 1;
 }
 
 // the tensor-core kernels' error word (read after the stream has synchronised)
@@ -583,12 +762,6 @@ static mgfr_status unet_make(mgfr_ctx* c, unsigned long long seed) {
   return MGFR_OK;
 }
 
-static int lg_of(int D) {
-  int lg = 0;
-  while ((1 << lg) < D) ++lg;
-  return lg;
-}
-
 static const char kUnetTag[9] = "MGFRUNT1";
 
 mgfr_status unet_predict_batch(mgfr_ctx* c, int B, int D, const double* x, double dscale,
@@ -604,8 +777,10 @@ mgfr_status unet_predict_batch(mgfr_ctx* c, int B, int D, const double* x, doubl
   const long long per = (long long)D * D * D, M0 = per * B;
   MG_CK(c, cudaMemcpyAsync(U->fr0d, fr0_host, sizeof(double) * B, cudaMemcpyHostToDevice, c->s));
   const Model mm = make_model(c->cfg, 1.0);
-  k_features<<<nblocks(M0, BS), BS, 0, c->s>>>(x, U->fr0d, per, M0, U->X0, c->cfg.omega_m / mm.Rt,
-                                               (double)(c->cfg.n + 1), dscale);
+  k_fr0_feature<<<nblocks(B, BS), BS, 0, c->s>>>(U->fr0d, B, U->ffr0);
+  k_features<<<nblocks(M0, BS), BS, 0, c->s>>>(x, U->ffr0, 3 * U->lgD, M0, U->X0,
+                                               c->cfg.omega_m / mm.Rt, (double)(c->cfg.n + 1),
+                                               dscale);
   forward(c, U);
   k_out_to_double<<<nblocks(M0, BS), BS, 0, c->s>>>(U->OUT, u_out, M0);
   c->launches += 2;
@@ -639,12 +814,13 @@ mgfr_status mgfr_unet_train_step(mgfr_ctx* c, int B, int D, const double* delta_
   MG_CK(c, cudaStreamWaitEvent(c->s, c->ev_in, 0));
   MG_CK(c, cudaMemcpyAsync(U->fr0d, fr0_host, sizeof(double) * B, cudaMemcpyHostToDevice, c->s));
   const Model mm = make_model(c->cfg, 1.0);
-  k_features<<<nblocks(M0, BS), BS, 0, c->s>>>(delta_dev, U->fr0d, (long long)D * D * D, M0, U->X0,
+  k_fr0_feature<<<nblocks(B, BS), BS, 0, c->s>>>(U->fr0d, B, U->ffr0);
+  k_features<<<nblocks(M0, BS), BS, 0, c->s>>>(delta_dev, U->ffr0, 3 * U->lgD, M0, U->X0,
                                                c->cfg.omega_m / mm.Rt, (double)(c->cfg.n + 1),
                                                1.0);
   forward(c, U);
   const int nb = 1024;
-  k_mse<<<nb, BS, 0, c->s>>>(U->OUT, u_target_dev, M0, U->GOUT, U->lossp);
+  k_mse<<<nb, BS, 0, c->s>>>(U->OUT, u_target_dev, M0, 2.0 / (double)M0, U->GOUT, U->lossp);
   backward(c, U);
   U->step += 1;
   const float b1 = 0.9f, b2 = 0.999f;
@@ -769,6 +945,108 @@ mgfr_status mgfr_unet_grads(mgfr_ctx* c, float* host) {
   return MGFR_OK;
 }
 
+}  // extern "C"
+
+// Scratch of mgfr_nn_conv3d (packed weights or partial sums, and the kernels'
+// error word), kept between calls: cudaMalloc and cudaFree took 0.2 ms of every
+// call.  A call owns its block from acquire to release, which come before and
+// after its work (the call waits for its stream), so blocks never serve two
+// streams or threads at once.  At most 4 blocks and 128 MB per device stay;
+// mgfr_destroy gives those of its device back.
+namespace {
+struct ConvScratch {
+  int dev = 0;
+  size_t bytes = 0;
+  void* p = nullptr;
+  int *err = nullptr, *err_h = nullptr;  // device word (0), page-locked copy
+};
+std::mutex g_scratch_mu;
+std::vector<ConvScratch> g_scratch;
+
+void scratch_drop(ConvScratch& b) {
+  if (b.p) cudaFree(b.p);
+  if (b.err) cudaFree(b.err);
+  if (b.err_h) cudaFreeHost(b.err_h);
+  b = ConvScratch();
+}
+
+bool scratch_acquire(size_t bytes, ConvScratch* out) {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return false;
+  {
+    std::lock_guard<std::mutex> lk(g_scratch_mu);
+    int best = -1;
+    for (size_t i = 0; i < g_scratch.size(); ++i)
+      if (g_scratch[i].dev == dev && g_scratch[i].bytes >= bytes &&
+          (best < 0 || g_scratch[i].bytes < g_scratch[best].bytes))
+        best = (int)i;
+    if (best >= 0) {
+      *out = g_scratch[best];
+      g_scratch.erase(g_scratch.begin() + best);
+      return true;
+    }
+  }
+  ConvScratch b;
+  b.dev = dev;
+  b.bytes = bytes;
+  if (cudaMalloc(&b.p, bytes) != cudaSuccess || cudaMalloc(&b.err, sizeof(int)) != cudaSuccess ||
+      cudaMallocHost(&b.err_h, sizeof(int)) != cudaSuccess ||
+      cudaMemset(b.err, 0, sizeof(int)) != cudaSuccess) {
+    (void)cudaGetLastError();
+    scratch_drop(b);
+    return false;
+  }
+  *out = b;
+  return true;
+}
+
+void scratch_release(ConvScratch& b) {
+  {
+    std::lock_guard<std::mutex> lk(g_scratch_mu);
+    size_t n = 0, sum = b.bytes;
+    for (const auto& q : g_scratch)
+      if (q.dev == b.dev) {
+        ++n;
+        sum += q.bytes;
+      }
+    if (n < 4 && sum <= (128u << 20)) {
+      g_scratch.push_back(b);
+      return;
+    }
+  }
+  scratch_drop(b);
+}
+
+// wait for the call's work, read the kernels' error word, give the block back
+mgfr_status scratch_finish(ConvScratch& b, cudaStream_t s) {
+  const bool ok =
+      cudaMemcpyAsync(b.err_h, b.err, sizeof(int), cudaMemcpyDeviceToHost, s) == cudaSuccess &&
+      cudaStreamSynchronize(s) == cudaSuccess && cudaGetLastError() == cudaSuccess;
+  if (!ok) {
+    scratch_drop(b);
+    return MGFR_E_CUDA;
+  }
+  const int e = *b.err_h;
+  if (e && cudaMemset(b.err, 0, sizeof(int)) != cudaSuccess) {
+    scratch_drop(b);
+    return MGFR_E_CUDA;
+  }
+  scratch_release(b);
+  return e ? MGFR_E_TIMEOUT : MGFR_OK;
+}
+}  // namespace
+
+void conv_scratch_trim(int dev) {
+  std::lock_guard<std::mutex> lk(g_scratch_mu);
+  for (size_t i = g_scratch.size(); i-- > 0;)
+    if (g_scratch[i].dev == dev) {
+      scratch_drop(g_scratch[i]);
+      g_scratch.erase(g_scratch.begin() + i);
+    }
+}
+
+extern "C" {
+
 // Convolution primitive on caller buffers (contiguous NDHWC, C multiples of 16):
 // op 0: y(bf16) = relu?(conv(x, W) + b); op 1: gx(FP32) = conv^T(g, W);
 // op 2: dW(FP32 [27][Cin][Cout]), db(FP32) from x and g.
@@ -783,21 +1061,16 @@ mgfr_status mgfr_nn_conv3d(int op, int B, int D, int Cin, int Cout, const void* 
   const bool tc = (op == 0 && nn_tc_supported(Cin, Cout)) || (op == 1 && nn_tc_supported(Cout, Cin));
   if (tc) {
     // pack the weights for the tensor-core kernel (scratch of this call)
-    __nv_bfloat16* wp = nullptr;
-    int* err = nullptr;
-    if (cudaMalloc(&wp, sizeof(__nv_bfloat16) * (size_t)nn_tc_packed_size(Cin, Cout)) != cudaSuccess)
+    ConvScratch sc;
+    if (!scratch_acquire(sizeof(__nv_bfloat16) * (size_t)nn_tc_packed_size(Cin, Cout), &sc))
       return MGFR_E_OOM;
-    if (cudaMalloc(&err, sizeof(int)) != cudaSuccess) {
-      cudaFree(wp);
-      return MGFR_E_OOM;
-    }
-    cudaMemsetAsync(err, 0, sizeof(int), s);
+    __nv_bfloat16* wp = (__nv_bfloat16*)sc.p;
     nn_tc_pack((const __nv_bfloat16*)w_bf16, Cin, Cout, op, wp, s);
     TcArgs a{};
     a.Wp = wp;
     a.lgD = lgD;
     a.Mtot = (long long)B << (3 * lgD);
-    a.err = err;
+    a.err = sc.err;
     if (op == 0) {
       a.x = (const __nv_bfloat16*)x_bf16;
       a.ldx = Cin;
@@ -812,13 +1085,7 @@ mgfr_status mgfr_nn_conv3d(int op, int B, int D, int Cin, int Cout, const void* 
       a.ldg = Cin;
     }
     nn_tc_conv(a, op == 0 ? Cin : Cout, op == 0 ? Cout : Cin, op == 1, s);
-    int e = 0;
-    const bool okc = cudaStreamSynchronize(s) == cudaSuccess &&
-                     cudaMemcpy(&e, err, sizeof(int), cudaMemcpyDeviceToHost) == cudaSuccess;
-    cudaFree(wp);
-    cudaFree(err);
-    if (!okc || cudaGetLastError() != cudaSuccess) return MGFR_E_CUDA;
-    return e ? MGFR_E_TIMEOUT : MGFR_OK;
+    return scratch_finish(sc, s);
   }
   if (op == 0) {
     nn_conv_fwd(TView{(__nv_bfloat16*)x_bf16, Cin, 0}, Cin, (const __nv_bfloat16*)w_bf16, bias,
@@ -828,25 +1095,14 @@ mgfr_status mgfr_nn_conv3d(int op, int B, int D, int Cin, int Cout, const void* 
                   FView{(float*)out, Cin, 0}, Cin, 0, B, lgD, s);
   } else if (op == 2) {
     const bool tcw = nn_tc_wgrad_supported(Cin, Cout);
-    float* part = nullptr;
-    int* err = nullptr;
     const long long np = tcw ? nn_tc_wgrad_scratch(Cin, Cout) : nn_wgrad_scratch(Cin, Cout);
-    if (cudaMalloc(&part, sizeof(float) * (size_t)np) != cudaSuccess) return MGFR_E_OOM;
-    if (cudaMalloc(&err, sizeof(int)) != cudaSuccess) {
-      cudaFree(part);
-      return MGFR_E_OOM;
-    }
-    cudaMemsetAsync(err, 0, sizeof(int), s);
+    ConvScratch sc;
+    if (!scratch_acquire(sizeof(float) * (size_t)np, &sc)) return MGFR_E_OOM;
+    float* part = (float*)sc.p;
     const TView xv{(__nv_bfloat16*)x_bf16, Cin, 0}, gv{(__nv_bfloat16*)g_bf16, Cout, 0};
-    if (!tcw || !nn_tc_wgrad(xv, Cin, gv, Cout, (float*)out, db, part, B, lgD, err, s))
+    if (!tcw || !nn_tc_wgrad(xv, Cin, gv, Cout, (float*)out, db, part, B, lgD, sc.err, s))
       nn_conv_wgrad(xv, Cin, gv, Cout, (float*)out, db, part, B, lgD, s);
-    int e = 0;
-    const bool okc = cudaStreamSynchronize(s) == cudaSuccess &&
-                     cudaMemcpy(&e, err, sizeof(int), cudaMemcpyDeviceToHost) == cudaSuccess;
-    cudaFree(part);
-    cudaFree(err);
-    if (!okc || cudaGetLastError() != cudaSuccess) return MGFR_E_CUDA;
-    if (e) return MGFR_E_TIMEOUT;
+    return scratch_finish(sc, s);
   } else {
     return MGFR_E_INVALID;
   }
