@@ -188,13 +188,23 @@ __global__ void __launch_bounds__(128) k_wgrad(const __nv_bfloat16* __restrict__
   }
 }
 
-__global__ void k_wgrad_reduce(const float* __restrict__ partials, int S, long long n,
-                               float* __restrict__ dW) {
-  const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (i >= n) return;
+// dW = the sum of the S partials: 32 elements x 8 segments of the partials per
+// block, each segment in order of its stride, then the segments in order
+__global__ void __launch_bounds__(256) k_wgrad_reduce(const float* __restrict__ partials, int S,
+                                                      long long n, float* __restrict__ dW) {
+  __shared__ float red[8][32];
+  const int l = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const long long i = blockIdx.x * 32LL + l;
   float s = 0.f;
-  for (int z = 0; z < S; ++z) s += partials[(long long)z * n + i];
-  dW[i] = s;
+  if (i < n)
+    for (int z = w; z < S; z += 8) s += partials[(long long)z * n + i];
+  red[w][l] = s;
+  __syncthreads();
+  if (w == 0 && i < n) {
+#pragma unroll
+    for (int q = 1; q < 8; ++q) s += red[q][l];
+    dW[i] = s;
+  }
 }
 
 // db[c] = sum over voxels of g[m][c].  Each thread sums 8 channels (16-byte
@@ -276,7 +286,7 @@ void nn_conv_dgrad(TView g, int Cout, const __nv_bfloat16* W, FView gx, int Cin,
 void nn_wgrad_finish(float* partials, int S, int Cin, int Cout, float* dW, TView g,
                      float* db, long long Mtot, cudaStream_t s) {
   const long long n = 27LL * Cin * Cout;
-  k_wgrad_reduce<<<nblocks(n, 256), 256, 0, s>>>(partials, S, n, dW);
+  k_wgrad_reduce<<<nblocks(n, 32), 256, 0, s>>>(partials, S, n, dW);
   if (!db) return;
   // the bias stages reuse the partials (read by k_wgrad_reduce before them on
   // this stream); they hold S * 27 * Cin * Cout >= 432 * Cout floats (Cin >= 16)

@@ -159,25 +159,68 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* v) {
   for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
 
-// neighbour voxel of m at offset (dx,dy,dz), periodic in each sample
-__device__ __forceinline__ long long tc_nbr(long long m, int lgD, int dx, int dy, int dz) {
-  const int D = 1 << lgD, M = D - 1;
-  const long long per = 1LL << (3 * lgD);
-  const long long b = m >> (3 * lgD), r = m & (per - 1);
-  const int i = (int)(r >> (2 * lgD)), j = (int)((r >> lgD) & M), k = (int)(r & M);
-  return b * per + ((((long long)((i + dx) & M) << lgD) + ((j + dy) & M)) << lgD) + ((k + dz) & M);
+// neighbour voxel of m at offset (dx,dy,dz), periodic in each sample (a tensor
+// of 2^32 voxels of 16 BF16 channels would fill 137 GB: 32-bit indices suffice)
+__device__ __forceinline__ unsigned tc_nbr(unsigned m, int lgD, int dx, int dy, int dz) {
+  const unsigned M = (1u << lgD) - 1;
+  const unsigned i = (m >> (2 * lgD)) & M, j = (m >> lgD) & M, k = m & M;
+  const unsigned b = m >> lgD >> lgD >> lgD;  // 3 lgD may reach 32
+  return (((((b << lgD) + ((i + dx) & M)) << lgD) + ((j + dy) & M)) << lgD) + ((k + dz) & M);
 }
 
 // KC: channels of an A row (the reduction per tap); NC: output columns.
 // DGRAD: the input-gradient form (mirrored tap, FP32 output, optional add).
+// threads of a convolution CTA: two warps per scheduler, because staging the
+// operands is a chain of address arithmetic and copies per 16-byte chunk (with
+// four warps the 96 -> 32 halo kernel spent 20 of 27 us per CTA there)
+constexpr int HT = 256;
+// stride between the 8-channel chunks of an A tile: the 128 rows and 16 bytes,
+// so that the chunks of a row, which neighbouring threads write, fall into
+// different banks
+constexpr uint32_t kALbo = TC_M * 16 + 16;
+constexpr int a_bytes(int kc) { return (kc / 8) * (int)kALbo; }
+
+// 16 accumulators of voxel m, columns n0..n0+15, to the output: BF16 with bias
+// and ReLU (forward), or FP32 (input gradient)
+template <bool DGRAD>
+__device__ __forceinline__ void store16(const float* v, long long m, int n0,
+                                        const float* __restrict__ bias, int relu,
+                                        __nv_bfloat16* __restrict__ y, int ldy, int offy,
+                                        float* __restrict__ gx, int ldg, int offg,
+                                        int accumulate) {
+  if (!DGRAD) {
+    __align__(16) __nv_bfloat16 o[16];
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+      float a = v[i] + (bias ? bias[n0 + i] : 0.f);
+      if (relu) a = fmaxf(a, 0.f);
+      o[i] = __float2bfloat16(a);
+    }
+    uint4* dst = reinterpret_cast<uint4*>(y + m * ldy + offy + n0);
+    dst[0] = reinterpret_cast<const uint4*>(o)[0];
+    dst[1] = reinterpret_cast<const uint4*>(o)[1];
+  } else {
+    float4* q = reinterpret_cast<float4*>(gx + m * ldg + offg + n0);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      float4 a = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
+      if (accumulate) {
+        const float4 p = q[i];
+        a = make_float4(p.x + a.x, p.y + a.y, p.z + a.z, p.w + a.w);
+      }
+      q[i] = a;
+    }
+  }
+}
+
 template <int KC, int NC, bool DGRAD>
-__global__ void __launch_bounds__(TC_THREADS) k_conv_tc(
+__global__ void __launch_bounds__(HT) k_conv_tc(
     const __nv_bfloat16* __restrict__ x, int ldx, int offx, const __nv_bfloat16* __restrict__ Wp,
     const float* __restrict__ bias, int relu, __nv_bfloat16* __restrict__ y, int ldy, int offy,
     float* __restrict__ gx, int ldg, int offg, int accumulate, int lgD, long long Mtot,
     int tmem_cols, int* __restrict__ err) {
-  constexpr int A_BYTES = TC_M * KC * 2, B_BYTES = NC * KC * 2;
-  constexpr uint32_t A_LBO = TC_M * 16, B_LBO = NC * 16, SBO = 128;
+  constexpr uint32_t A_LBO = kALbo, B_LBO = NC * 16, SBO = 128;
+  constexpr int A_BYTES = a_bytes(KC), B_BYTES = NC * KC * 2;
   constexpr uint32_t IDESC = idesc_bf16(TC_M, NC);
   extern __shared__ __align__(1024) unsigned char smem[];
   unsigned char* As = smem;                        // [2][A_BYTES]
@@ -210,12 +253,14 @@ __global__ void __launch_bounds__(TC_THREADS) k_conv_tc(
     const int sg = DGRAD ? -1 : 1;
     unsigned char* A = As + s * A_BYTES;
     constexpr int CH = KC / 8;  // 16-byte chunks per row
-    for (int e = tid; e < TC_M * CH; e += TC_THREADS) {
+    // consecutive threads take the chunks of a row (contiguous in memory)
+#pragma unroll 4
+    for (int e = tid; e < TC_M * CH; e += HT) {
       const int r = e / CH, c = e - r * CH;
       const long long m = m0 + r;
       const bool v = m < Mtot;
-      const long long src = v ? tc_nbr(m, lgD, sg * dx, sg * dy, sg * dz) : 0;
-      cp_async16(A + c * (TC_M * 16) + r * 16, x + src * ldx + offx + 8 * c, v);
+      const unsigned src = v ? tc_nbr((unsigned)m, lgD, sg * dx, sg * dy, sg * dz) : 0u;
+      cp_async16(A + c * A_LBO + r * 16, x + (size_t)src * ldx + offx + 8 * c, v);
     }
     cp_async_commit();
   };
@@ -273,31 +318,14 @@ __global__ void __launch_bounds__(TC_THREADS) k_conv_tc(
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   ok = __syncthreads_and(ok);
   if (ok) {
-    const int row = warp * 32 + (tid & 31);
+    const int row = (warp & 3) * 32 + (tid & 31);  // TMEM lanes of a warp: its quarter
     const long long m = m0 + row;
-    const uint32_t lane_addr = tbase + ((uint32_t)(warp * 32) << 16);
+    const uint32_t lane_addr = tbase + ((uint32_t)((warp & 3) * 32) << 16);
 #pragma unroll 1
-    for (int n0 = 0; n0 < NC; n0 += 16) {
+    for (int n0 = 16 * (warp >> 2); n0 < NC; n0 += 16 * (HT / 128)) {
       float v[16];
       tmem_ld16(lane_addr + n0, v);
-      if (m < Mtot) {
-        if (!DGRAD) {
-          __align__(16) __nv_bfloat16 o[16];
-#pragma unroll
-          for (int i = 0; i < 16; ++i) {
-            float a = v[i] + (bias ? bias[n0 + i] : 0.f);
-            if (relu) a = fmaxf(a, 0.f);
-            o[i] = __float2bfloat16(a);
-          }
-          uint4* dst = reinterpret_cast<uint4*>(y + m * ldy + offy + n0);
-          dst[0] = reinterpret_cast<const uint4*>(o)[0];
-          dst[1] = reinterpret_cast<const uint4*>(o)[1];
-        } else {
-          float* q = gx + m * ldg + offg + n0;
-#pragma unroll
-          for (int i = 0; i < 16; ++i) q[i] = accumulate ? q[i] + v[i] : v[i];
-        }
-      }
+      if (m < Mtot) store16<DGRAD>(v, m, n0, bias, relu, y, ldy, offy, gx, ldg, offg, accumulate);
     }
   } else {
     // a wait ran out: let the copies and MMAs still in flight finish (each
@@ -382,7 +410,7 @@ __global__ void __launch_bounds__(TC_THREADS) k_wgrad_tc(
       long long src = 0;
       if (ok_e) {
         const int dx = t / 9 - 1, dy = (t / 3) % 3 - 1, dz = t % 3 - 1;
-        src = tc_nbr(v, lgD, -dx, -dy, -dz) * ldg + offg + 8 * co8;
+        src = (long long)tc_nbr((unsigned)v, lgD, -dx, -dy, -dz) * ldg + offg + 8 * co8;
       }
       cp_async16(As + 16 * e, g + src, ok_e);
     }
@@ -510,14 +538,37 @@ void launch_wgrad(TView x, TView g, int lgD, long long Mtot, float* part, int* e
 // 8-channel groups one block-plane apart (LBO), the start shifted by the tap
 // offset.  So the block is read from global memory once instead of 27 times,
 // and a tile costs 27 (KC / 16) MMAs on shared-memory operands.
+// The halo block of a CTA: 8-channel chunk c8 of voxel (hx, hy, hz) lands at
+// c8 halo_plane + 16 ((hx HY + hy) HZ + hz); consecutive threads take the
+// chunks of a voxel (contiguous in memory; the plane stride's extra 16 bytes
+// put them into different banks)
+constexpr int HY = 18, HZ = 10;
+constexpr int halo_plane(int hx) { return hx * HY * HZ * 16 + 16; }
+
+template <int CH, int HX>
+__device__ __forceinline__ void load_halo(unsigned char* Hs, const __nv_bfloat16* __restrict__ x,
+                                          int ldx, int offx, unsigned sample, int x0, int y0,
+                                          int z0, int lgD, int tid) {
+  const int M = (1 << lgD) - 1;
+#pragma unroll 4
+  for (int e = tid; e < CH * HX * HY * HZ; e += HT) {
+    const int v = e / CH, c8 = e - v * CH;
+    const int r = v / HZ, hz = v - r * HZ;
+    const int hx = r / HY, hy = r - hx * HY;
+    const unsigned q = ((((sample << lgD) + ((x0 + hx - 1) & M)) << lgD) + ((y0 + hy - 1) & M));
+    const unsigned vox = (q << lgD) + ((z0 + hz - 1) & M);
+    cp_async16(Hs + c8 * halo_plane(HX) + 16 * v, x + (size_t)vox * ldx + offx + 8 * c8, true);
+  }
+}
+
 template <int KC, int NC, bool DGRAD, int TX>
-__global__ void __launch_bounds__(TC_THREADS) k_conv_halo(
+__global__ void __launch_bounds__(HT) k_conv_halo(
     const __nv_bfloat16* __restrict__ x, int ldx, int offx, const __nv_bfloat16* __restrict__ Wp,
     const float* __restrict__ bias, int relu, __nv_bfloat16* __restrict__ y, int ldy, int offy,
     float* __restrict__ gx, int ldg, int offg, int accumulate, int lgD, int tmem_cols,
     int* __restrict__ err) {
-  constexpr int HX = TX + 2, HY = 18, HZ = 10, CH = KC / 8;
-  constexpr int PLANE = HX * HY * HZ * 16;  // bytes of one 8-channel group
+  constexpr int HX = TX + 2, CH = KC / 8;
+  constexpr int PLANE = halo_plane(HX);  // bytes of one 8-channel group
   constexpr int H_BYTES = CH * PLANE;
   constexpr int W_BYTES = 27 * NC * KC * 2;
   constexpr uint32_t SBO = HZ * 16, B_LBO = NC * 16;
@@ -559,20 +610,7 @@ __global__ void __launch_bounds__(TC_THREADS) k_conv_halo(
   const uint32_t tbase = *tslot;
   bool ok = true;
   if (tid == 0) bulk_load(Ws, Wp, (uint32_t)W_BYTES, bars);
-  // the halo block: chunk e = ((c8 HX + hx) HY + hy) HZ + hz lands at 16 e
-  for (int e = tid; e < CH * HX * HY * HZ; e += TC_THREADS) {
-    int r = e;
-    const int hz = r % HZ;
-    r /= HZ;
-    const int hy = r % HY;
-    r /= HY;
-    const int hx = r % HX;
-    const int c8 = r / HX;
-    const long long v = sbase + ((((long long)((x0 + hx - 1) & M) << lgD) + ((y0 + hy - 1) & M))
-                                 << lgD) +
-                        ((z0 + hz - 1) & M);
-    cp_async16(Hs + 16 * e, x + v * ldx + offx + 8 * c8, true);
-  }
+  load_halo<CH, HX>(Hs, x, ldx, offx, (unsigned)b, x0, y0, z0, lgD, tid);
   cp_async_commit();
   cp_async_wait<0>();
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -608,33 +646,18 @@ __global__ void __launch_bounds__(TC_THREADS) k_conv_halo(
   ok = __syncthreads_and(ok);
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   if (ok) {
-    const int row = warp * 32 + (tid & 31);
+    // warp w reads TMEM lanes 32 (w & 3)..; the column chunks alternate between
+    // the two groups of four warps
+    const int row = (warp & 3) * 32 + (tid & 31);
     const int yy = row >> 3, zz = row & 7;
-    const uint32_t lane_addr = tbase + ((uint32_t)(warp * 32) << 16);
+    const uint32_t lane_addr = tbase + ((uint32_t)((warp & 3) * 32) << 16);
 #pragma unroll 1
-    for (int tx = 0; tx < TX; ++tx) {
+    for (int q = warp >> 2; q < TX * (NC / 16); q += HT / 128) {
+      const int tx = q / (NC / 16), n0 = 16 * (q - tx * (NC / 16));
       const long long m = sbase + ((((long long)(x0 + tx) << lgD) + (y0 + yy)) << lgD) + (z0 + zz);
-#pragma unroll 1
-      for (int n0 = 0; n0 < NC; n0 += 16) {
-        float v[16];
-        tmem_ld16(lane_addr + tx * NC + n0, v);
-        if (!DGRAD) {
-          __align__(16) __nv_bfloat16 o[16];
-#pragma unroll
-          for (int i = 0; i < 16; ++i) {
-            float a = v[i] + (bias ? bias[n0 + i] : 0.f);
-            if (relu) a = fmaxf(a, 0.f);
-            o[i] = __float2bfloat16(a);
-          }
-          uint4* dst = reinterpret_cast<uint4*>(y + m * ldy + offy + n0);
-          dst[0] = reinterpret_cast<const uint4*>(o)[0];
-          dst[1] = reinterpret_cast<const uint4*>(o)[1];
-        } else {
-          float* q = gx + m * ldg + offg + n0;
-#pragma unroll
-          for (int i = 0; i < 16; ++i) q[i] = accumulate ? q[i] + v[i] : v[i];
-        }
-      }
+      float v[16];
+      tmem_ld16(lane_addr + tx * NC + n0, v);
+      store16<DGRAD>(v, m, n0, bias, relu, y, ldy, offy, gx, ldg, offg, accumulate);
     }
   } else if (tid == 0) {
     // a wait ran out: the weights' copy and the MMAs in flight (each bounded)
@@ -651,7 +674,7 @@ __global__ void __launch_bounds__(TC_THREADS) k_conv_halo(
 
 template <int KC, int NC, bool DG, int TX>
 void launch_halo(const TcArgs& a, cudaStream_t s) {
-  constexpr int H_BYTES = (KC / 8) * (TX + 2) * 18 * 10 * 16, W_BYTES = 27 * NC * KC * 2;
+  constexpr int H_BYTES = (KC / 8) * halo_plane(TX + 2), W_BYTES = 27 * NC * KC * 2;
   const int cols0 = TX * NC;
   const int cols = cols0 <= 32 ? 32 : (cols0 <= 64 ? 64 : (cols0 <= 128 ? 128 : 256));
   const size_t need = (size_t)H_BYTES + W_BYTES + 2 * 8 + 16;
@@ -665,7 +688,7 @@ void launch_halo(const TcArgs& a, cudaStream_t s) {
     attr = true;
   }
   const long long tiles = a.Mtot / (TX * 16 * 8);
-  k_conv_halo<KC, NC, DG, TX><<<(unsigned)tiles, TC_THREADS, smem, s>>>(
+  k_conv_halo<KC, NC, DG, TX><<<(unsigned)tiles, HT, smem, s>>>(
       a.x, a.ldx, a.offx, a.Wp, a.bias, a.relu, a.y, a.ldy, a.offy, a.gx, a.ldg, a.offg,
       a.accumulate, a.lgD, cols, a.err);
 }
@@ -676,13 +699,13 @@ void launch_halo(const TcArgs& a, cudaStream_t s) {
 // alone loads the slices and issues the MMAs, so the loop over taps has no
 // block-wide synchronisation.
 template <int KC, int NC, bool DGRAD, int TX>
-__global__ void __launch_bounds__(TC_THREADS) k_conv_halo_s(
+__global__ void __launch_bounds__(HT) k_conv_halo_s(
     const __nv_bfloat16* __restrict__ x, int ldx, int offx, const __nv_bfloat16* __restrict__ Wp,
     const float* __restrict__ bias, int relu, __nv_bfloat16* __restrict__ y, int ldy, int offy,
     float* __restrict__ gx, int ldg, int offg, int accumulate, int lgD, int tmem_cols,
     int* __restrict__ err) {
-  constexpr int HX = TX + 2, HY = 18, HZ = 10, CH = KC / 8;
-  constexpr int PLANE = HX * HY * HZ * 16;
+  constexpr int HX = TX + 2, CH = KC / 8;
+  constexpr int PLANE = halo_plane(HX);
   constexpr int H_BYTES = CH * PLANE;
   constexpr int T_BYTES = NC * KC * 2;  // one tap's weight slice
   constexpr uint32_t SBO = HZ * 16, B_LBO = NC * 16;
@@ -726,19 +749,7 @@ __global__ void __launch_bounds__(TC_THREADS) k_conv_halo_s(
     bulk_load(Ws, Wp, (uint32_t)T_BYTES, bars);
     ++issued[0];
   }
-  for (int e = tid; e < CH * HX * HY * HZ; e += TC_THREADS) {
-    int r = e;
-    const int hz = r % HZ;
-    r /= HZ;
-    const int hy = r % HY;
-    r /= HY;
-    const int hx = r % HX;
-    const int c8 = r / HX;
-    const long long v = sbase + ((((long long)((x0 + hx - 1) & M) << lgD) + ((y0 + hy - 1) & M))
-                                 << lgD) +
-                        ((z0 + hz - 1) & M);
-    cp_async16(Hs + 16 * e, x + v * ldx + offx + 8 * c8, true);
-  }
+  load_halo<CH, HX>(Hs, x, ldx, offx, (unsigned)b, x0, y0, z0, lgD, tid);
   cp_async_commit();
   cp_async_wait<0>();
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -795,33 +806,18 @@ __global__ void __launch_bounds__(TC_THREADS) k_conv_halo_s(
   ok = __syncthreads_and(ok);
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   if (ok) {
-    const int row = warp * 32 + (tid & 31);
+    // warp w reads TMEM lanes 32 (w & 3)..; the column chunks alternate between
+    // the two groups of four warps
+    const int row = (warp & 3) * 32 + (tid & 31);
     const int yy = row >> 3, zz = row & 7;
-    const uint32_t lane_addr = tbase + ((uint32_t)(warp * 32) << 16);
+    const uint32_t lane_addr = tbase + ((uint32_t)((warp & 3) * 32) << 16);
 #pragma unroll 1
-    for (int tx = 0; tx < TX; ++tx) {
+    for (int q = warp >> 2; q < TX * (NC / 16); q += HT / 128) {
+      const int tx = q / (NC / 16), n0 = 16 * (q - tx * (NC / 16));
       const long long m = sbase + ((((long long)(x0 + tx) << lgD) + (y0 + yy)) << lgD) + (z0 + zz);
-#pragma unroll 1
-      for (int n0 = 0; n0 < NC; n0 += 16) {
-        float v[16];
-        tmem_ld16(lane_addr + tx * NC + n0, v);
-        if (!DGRAD) {
-          __align__(16) __nv_bfloat16 o[16];
-#pragma unroll
-          for (int i = 0; i < 16; ++i) {
-            float a = v[i] + (bias ? bias[n0 + i] : 0.f);
-            if (relu) a = fmaxf(a, 0.f);
-            o[i] = __float2bfloat16(a);
-          }
-          uint4* dst = reinterpret_cast<uint4*>(y + m * ldy + offy + n0);
-          dst[0] = reinterpret_cast<const uint4*>(o)[0];
-          dst[1] = reinterpret_cast<const uint4*>(o)[1];
-        } else {
-          float* q = gx + m * ldg + offg + n0;
-#pragma unroll
-          for (int i = 0; i < 16; ++i) q[i] = accumulate ? q[i] + v[i] : v[i];
-        }
-      }
+      float v[16];
+      tmem_ld16(lane_addr + tx * NC + n0, v);
+      store16<DGRAD>(v, m, n0, bias, relu, y, ldy, offy, gx, ldg, offg, accumulate);
     }
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -834,7 +830,7 @@ __global__ void __launch_bounds__(TC_THREADS) k_conv_halo_s(
 
 template <int KC, int NC, bool DG, int TX>
 void launch_halo_s(const TcArgs& a, cudaStream_t s) {
-  constexpr int H_BYTES = (KC / 8) * (TX + 2) * 18 * 10 * 16, T_BYTES = NC * KC * 2;
+  constexpr int H_BYTES = (KC / 8) * halo_plane(TX + 2), T_BYTES = NC * KC * 2;
   const int cols0 = TX * NC;
   const int cols = cols0 <= 32 ? 32 : (cols0 <= 64 ? 64 : (cols0 <= 128 ? 128 : 256));
   const size_t need = (size_t)H_BYTES + 2 * T_BYTES + 4 * 8 + 16;
@@ -848,9 +844,235 @@ void launch_halo_s(const TcArgs& a, cudaStream_t s) {
     attr = true;
   }
   const long long tiles = a.Mtot / (TX * 16 * 8);
-  k_conv_halo_s<KC, NC, DG, TX><<<(unsigned)tiles, TC_THREADS, smem, s>>>(
+  k_conv_halo_s<KC, NC, DG, TX><<<(unsigned)tiles, HT, smem, s>>>(
       a.x, a.ldx, a.offx, a.Wp, a.bias, a.relu, a.y, a.ldy, a.offy, a.gx, a.ldg, a.offg,
       a.accumulate, a.lgD, cols, a.err);
+}
+
+// ---- weight gradient from resident blocks (the layers of up to 32 output
+// channels, whose voxels are the most) --------------------------------------
+// dW[t][ci][co] = sum_u x[u][ci] g[u - d_t][co].  A stage holds PL x planes of
+// x over a 16 (y) x 8 (z) block with its one-voxel halo in y and z, and the
+// PL + 2 slices of g around them without a halo, both [plane][8-channel group]
+// [y][z] with 16 bytes per voxel.  Reduction = the block's 128 voxels, both
+// operands MN-major (core matrices of 8 z-consecutive voxels x 16 bytes of
+// channels, the next 8 voxels one y row on, the next 8 channels one group on):
+//   A: rows (slice s, co): the 16 groups from the first slice on, M = 128
+//      (rows of slices past PL + 2 are not used; they read what the stage holds);
+//   B: columns (plane p, ci), N = PL CI, started (dy, dz) into the halo.
+// One accumulator per (dy, dz) then holds the taps of every dx = p - s: each
+// operand is staged once instead of once per tap (the per-tap kernel spent its
+// time on the address arithmetic of that staging).  A CTA walks its range of
+// blocks with the next stages in flight and the ND accumulators in TMEM.  The
+// tensor core's FP32 accumulation truncates, an error that grows with the length
+// of the chain, so every kFlush voxels the accumulators are added, rounded to
+// nearest, to the CTA's partial dW in shared memory: relative error 4e-7 at
+// 96 -> 32 on 4 x 32^3 against 1.6e-6 of the per-tap kernel's chains (2.8e-6
+// without the flushes).
+template <int CI, int CO, int PL, int ND>
+struct WgHalo {
+  static constexpr int CI8 = CI / 8, CO8 = CO / 8, SL = 16 / CO8;
+  static constexpr int NG = PL + 2;                         // slices of g loaded
+  static constexpr int XG = HY * HZ * 16, GG = 16 * 8 * 16; // bytes of an 8-channel group
+  static constexpr int XB = PL * CI8 * XG, GB = NG * CO8 * GG, ST = XB + GB;
+  static constexpr int N = PL * CI, COLS = ND * N;
+  static constexpr int kFlush = 512, FL = kFlush / (128 * PL);  // voxels, blocks
+  static constexpr int ACC = 3 * ND * CI * CO * 4;               // bytes of a partial dW
+  static constexpr int STAGES = 3 * ST + ACC <= 226 * 1024 ? 3 : 2;
+  // the rows of slices past NG read on behind the last stage: into the partial dW
+  static constexpr int OVER = (SL - NG) * CO8 * GG;
+  static constexpr int TCOLS = COLS <= 256 ? 256 : 512;
+  static_assert(SL >= NG && N <= 256 && COLS <= 512 && OVER <= ACC &&
+                    STAGES * ST + ACC <= 226 * 1024, "tile");
+};
+
+template <int CI, int CO, int PL, int ND>
+__global__ void __launch_bounds__(HT) k_wgrad_halo(
+    const __nv_bfloat16* __restrict__ x, int ldx, int offx, const __nv_bfloat16* __restrict__ g,
+    int ldg, int offg, int lgD, int ntile, int chunk, float* __restrict__ part,
+    int* __restrict__ err) {
+  using W = WgHalo<CI, CO, PL, ND>;
+  constexpr uint32_t IDESC = idesc_bf16_mn(TC_M, W::N);
+  extern __shared__ __align__(1024) unsigned char smem[];
+  float* acc = reinterpret_cast<float*>(smem + W::STAGES * W::ST);  // [dx][q][ci][co]
+  uint64_t* done = reinterpret_cast<uint64_t*>(smem + W::STAGES * W::ST + W::ACC);
+  uint32_t* tslot = reinterpret_cast<uint32_t*>(done + W::STAGES);
+  const int tid = threadIdx.x, warp = tid >> 5;
+  const int dy0 = ND == 9 ? -1 : (int)blockIdx.x - 1;  // ND = 3: this CTA's dy
+  const int k0 = blockIdx.y * chunk, k1 = min(ntile, k0 + chunk);
+  const int nk = k1 > k0 ? k1 - k0 : 0;
+  const int D = 1 << lgD, M = D - 1, nz = D >> 3, ny = D >> 4;
+
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                     smem_u32(tslot)),
+                 "r"(W::TCOLS)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  if (tid == 0) {
+    for (int q = 0; q < W::STAGES; ++q) mbar_init(done + q, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const uint32_t tbase = *tslot;
+  bool ok = true;
+
+  auto load = [&](int k, int st) {
+    unsigned char* X = smem + st * W::ST;
+    unsigned char* Gs = X + W::XB;
+    int r = k0 + k;  // block: z, then y, then x planes, then sample
+    const int z0 = 8 * (r % nz);
+    r /= nz;
+    const int y0 = 16 * (r % ny);
+    r /= ny;
+    const int p0 = PL * (r % (D / PL));
+    const unsigned b = (unsigned)(r / (D / PL));
+#pragma unroll 4
+    for (int e = tid; e < W::CI8 * PL * HY * HZ; e += HT) {
+      const int v = e / W::CI8, c8 = e - v * W::CI8;
+      const int q = v / HZ, hz = v - q * HZ, p = q / HY, hy = q - p * HY;
+      const unsigned row = ((((b << lgD) + p0 + p) << lgD) + ((y0 + hy - 1) & M));
+      const unsigned vox = (row << lgD) + ((z0 + hz - 1) & M);
+      cp_async16(X + (p * W::CI8 + c8) * W::XG + 16 * (hy * HZ + hz),
+                 x + (size_t)vox * ldx + offx + 8 * c8, true);
+    }
+#pragma unroll 4
+    for (int e = tid; e < W::CO8 * W::NG * 128; e += HT) {
+      const int v = e / W::CO8, c8 = e - v * W::CO8;
+      const int z = v & 7, y = (v >> 3) & 15, s = v >> 7;
+      const unsigned row = ((((b << lgD) + ((p0 - 1 + s) & M)) << lgD) + y0 + y);
+      const unsigned vox = (row << lgD) + z0 + z;
+      cp_async16(Gs + (s * W::CO8 + c8) * W::GG + 16 * (v & 127),
+                 g + (size_t)vox * ldg + offg + 8 * c8, true);
+    }
+  };
+
+  float* out = part + (long long)blockIdx.y * 27 * CI * CO;
+  // Row (s, co) of accumulator (dy, dz), columns (p, ci): tap dx = p - s + 1 (s
+  // counted from the slice before plane 0).  The planes' terms of a tap lie in
+  // different rows, so the planes are added one after the other.
+  auto flush = [&](bool first) {
+    const int row = (warp & 3) * 32 + (tid & 31);
+    const int s = row / CO, co = row - s * CO;
+    const uint32_t lane_addr = tbase + ((uint32_t)((warp & 3) * 32) << 16);
+    for (int p = 0; p < PL; ++p) {
+      const int dx = p - s + 1;  // -1, 0 or 1 where this row contributes
+#pragma unroll 1
+      for (int e = warp >> 2; e < ND * (CI / 16); e += HT / 128) {
+        const int q = e / (CI / 16), n0 = 16 * (e - q * (CI / 16));
+        float v[16];
+        tmem_ld16(lane_addr + q * W::N + p * CI + n0, v);
+        if (dx >= -1 && dx <= 1) {
+          float* w = acc + (((dx + 1) * ND + q) * CI + n0) * CO + co;
+#pragma unroll
+          for (int i = 0; i < 16; ++i) w[i * CO] = first && p == 0 ? v[i] : w[i * CO] + v[i];
+        }
+        __syncwarp();
+      }
+      __syncthreads();
+    }
+  };
+
+  int commits[W::STAGES] = {}, last_commit = -1;
+  bool fresh = true, first = true;  // accumulators to be overwritten; no flush yet
+  for (int k = 0; k < W::STAGES - 1; ++k) {
+    if (k < nk) load(k, k);
+    cp_async_commit();
+  }
+  for (int k = 0; k < nk; ++k) {
+    const int st = k % W::STAGES, kn = k + W::STAGES - 1;
+    if (kn < nk) {
+      const int sn = kn % W::STAGES;  // last read by the MMAs of block k - 1
+      if (k >= 1 && tid == 0 &&
+          !mbar_wait(done + sn, (uint32_t)(((k - 1) / W::STAGES) & 1), err))
+        ok = false;
+      ok = __syncthreads_and(ok);
+      if (!ok) break;
+      load(kn, sn);
+    }
+    cp_async_commit();
+    cp_async_wait<W::STAGES - 1>();
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    __syncthreads();
+    if (tid == 0) {
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      const uint32_t x0 = smem_u32(smem + st * W::ST), g0 = x0 + W::XB;
+#pragma unroll 1
+      for (int q = 0; q < ND; ++q) {
+        const int dy = ND == 9 ? q / 3 - 1 : dy0, dz = q % 3 - 1;
+#pragma unroll
+        for (int kk = 0; kk < 8; ++kk) {  // 16 voxels: two y rows
+          const uint64_t ad = sdesc_mn(g0 + kk * 256, W::GG, 128);
+          const uint64_t bd =
+              sdesc_mn(x0 + ((2 * kk + dy + 1) * HZ + dz + 1) * 16, W::XG, HZ * 16);
+          mma_bf16(tbase + q * W::N, ad, bd, IDESC, (!fresh || kk > 0) ? 1u : 0u);
+        }
+      }
+      mma_commit(done + st);
+      ++commits[st];
+      last_commit = st;
+    }
+    fresh = false;
+    if ((k + 1) % W::FL == 0 || k + 1 == nk) {
+      if (tid == 0 && !mbar_wait(done + st, (uint32_t)((k / W::STAGES) & 1), err)) ok = false;
+      ok = __syncthreads_and(ok);
+      if (!ok) break;
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      flush(first);
+      // the reads are done before the next MMA overwrites the accumulators
+      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+      __syncthreads();
+      fresh = true;
+      first = false;
+    }
+  }
+  ok = __syncthreads_and(ok);
+  if (ok) {
+    // [dx][q][ci][co] -> the taps of this CTA's dy (all nine q: the whole dW)
+    for (int e = tid; e < 3 * ND * CI * CO; e += HT) {
+      const int dq = e / (CI * CO), dx = dq / ND, q = dq - dx * ND;
+      const int t = dx * 9 + (ND == 9 ? q : 3 * (int)blockIdx.x + q);
+      out[(long long)t * CI * CO + (e - dq * CI * CO)] = acc[e];
+    }
+  } else {
+    // a wait ran out: let the copies and MMAs in flight finish (bounded)
+    cp_async_wait<0>();
+    if (tid == 0 && last_commit >= 0)
+      mbar_wait(done + last_commit, (uint32_t)((commits[last_commit] - 1) & 1), err);
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  if (warp == 0)
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tbase),
+                 "r"(W::TCOLS)
+                 : "memory");
+}
+
+// ranges of blocks: one CTA per SM (its accumulators take the SM's TMEM)
+constexpr int WG_HALO_CTAS = 152;
+
+template <int CI, int CO, int PL, int ND>
+void launch_wgrad_halo(TView x, TView g, int B, int lgD, float* part, int* err, int* S_out,
+                       cudaStream_t s) {
+  using W = WgHalo<CI, CO, PL, ND>;
+  const size_t need = (size_t)W::STAGES * W::ST + W::ACC + W::STAGES * 8 + 16;
+  const size_t cap = 233472 / (512 / W::TCOLS + 1) - 1024 + 16;
+  const size_t smem = need > cap ? need : cap;
+  static bool attr = false;
+  if (!attr) {
+    cudaFuncSetAttribute(k_wgrad_halo<CI, CO, PL, ND>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         227 * 1024);
+    attr = true;
+  }
+  const int ntile = (B << (3 * lgD - 7)) / PL;
+  const int S0 = std::max(1, WG_HALO_CTAS / (9 / ND));
+  const int chunk = (ntile + S0 - 1) / S0, S = (ntile + chunk - 1) / chunk;
+  k_wgrad_halo<CI, CO, PL, ND><<<dim3(9 / ND, S), HT, smem, s>>>(
+      x.p, x.ld, x.off, g.p, g.ld, g.off, lgD, ntile, chunk, part, err);
+  *S_out = S;
 }
 
 // Packed weight slices.  Forward (N = Cout, K = Cin):
@@ -875,7 +1097,7 @@ __global__ void k_pack_tc(const __nv_bfloat16* __restrict__ W, int Cin, int Cout
 
 template <int KC, int NC, bool DG>
 void launch_tc(const TcArgs& a, cudaStream_t s) {
-  constexpr int A_BYTES = TC_M * KC * 2, B_BYTES = NC * KC * 2;
+  constexpr int A_BYTES = a_bytes(KC), B_BYTES = NC * KC * 2;
   const int cols = NC <= 32 ? 32 : (NC <= 64 ? 64 : (NC <= 128 ? 128 : 256));
   const size_t need = 2 * (size_t)A_BYTES + 2 * (size_t)B_BYTES + 4 * 8 + 16;
   // at most 512 / cols CTAs per SM may hold TMEM at once: pad the shared
@@ -891,7 +1113,7 @@ void launch_tc(const TcArgs& a, cudaStream_t s) {
     attr = true;
   }
   const unsigned grid = (unsigned)((a.Mtot + TC_M - 1) / TC_M);
-  k_conv_tc<KC, NC, DG><<<grid, TC_THREADS, smem, s>>>(
+  k_conv_tc<KC, NC, DG><<<grid, HT, smem, s>>>(
       a.x, a.ldx, a.offx, a.Wp, a.bias, a.relu, a.y, a.ldy, a.offy, a.gx, a.ldg, a.offg,
       a.accumulate, a.lgD, a.Mtot, cols, a.err);
 }
@@ -974,13 +1196,35 @@ bool nn_tc_wgrad_supported(int Cin, int Cout) {
 
 long long nn_tc_wgrad_scratch(int Cin, int Cout) {
   const int nt = (27 + TC_M / Cout - 1) / (TC_M / Cout);
-  return (long long)std::max(1, WG_CTAS / nt) * 27 * Cin * Cout;
+  return (long long)std::max(WG_HALO_CTAS, WG_CTAS / nt) * 27 * Cin * Cout;
 }
 
 bool nn_tc_wgrad(TView x, int Cin, TView g, int Cout, float* dW, float* db, float* partials,
                  int B, int lgD, int* err, cudaStream_t s) {
   const long long Mtot = (long long)B << (3 * lgD);
   int S = 0;
+  // up to 32 output channels on grids that hold the 16 x 8 blocks: resident
+  // blocks (16 -> 16 on 4 x 64^3 283 -> see below; smaller grids and 64 and more
+  // output channels, whose slices leave no room for the three dx, per tap)
+  if (lgD >= 4) {
+    bool done = true;
+    if (Cin == 16 && Cout == 16)
+      launch_wgrad_halo<16, 16, 2, 9>(x, g, B, lgD, partials, err, &S, s);
+    else if (Cin == 48 && Cout == 16)
+      launch_wgrad_halo<48, 16, 1, 9>(x, g, B, lgD, partials, err, &S, s);
+    else if (Cin == 16 && Cout == 32)
+      launch_wgrad_halo<16, 32, 2, 9>(x, g, B, lgD, partials, err, &S, s);
+    else if (Cin == 32 && Cout == 32)
+      launch_wgrad_halo<32, 32, 1, 9>(x, g, B, lgD, partials, err, &S, s);
+    else if (Cin == 96 && Cout == 32)
+      launch_wgrad_halo<96, 32, 1, 3>(x, g, B, lgD, partials, err, &S, s);
+    else
+      done = false;
+    if (done) {
+      nn_wgrad_finish(partials, S, Cin, Cout, dW, g, db, Mtot, s);
+      return true;
+    }
+  }
 #define WG_CASE(CI, CO)                                                  \
   if (Cin == CI && Cout == CO) {                                         \
     launch_wgrad<CI, CO>(x, g, lgD, Mtot, partials, err, &S, s);         \
