@@ -128,6 +128,28 @@ __host__ __device__ constexpr uint32_t idesc_bf16_mn(int M, int N) {
   return idesc_bf16(M, N) | (1u << 15) | (1u << 16);
 }
 
+// The MMA loops run in one whole warp, warp-uniform, and only the elected lane
+// issues: descriptors then stay in uniform registers (issued from inside an
+// `if (tid == 0)` each MMA cost about 100 clocks of moves and 64-bit shifts, more
+// than its work).
+__device__ __forceinline__ bool elect_one() {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "elect.sync _|p, 0xffffffff;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok));
+  return ok != 0;
+}
+__device__ __forceinline__ int warp_index() {
+  return __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0);
+}
+// a descriptor advanced by `bytes` (a multiple of 16, inside shared memory: the
+// address field does not overflow into its neighbour)
+__device__ __forceinline__ uint64_t desc_add(uint64_t d, uint32_t bytes) {
+  return d + (uint64_t)(bytes >> 4);
+}
+
 __device__ __forceinline__ void mma_bf16(uint32_t dtmem, uint64_t a, uint64_t b, uint32_t idesc,
                                          uint32_t acc) {
   asm volatile(
@@ -227,7 +249,7 @@ __global__ void __launch_bounds__(HT) k_conv_tc(
   unsigned char* Bs = smem + 2 * A_BYTES;          // [2][B_BYTES]
   uint64_t* bars = reinterpret_cast<uint64_t*>(Bs + 2 * B_BYTES);  // full[2], done[2]
   uint32_t* tslot = reinterpret_cast<uint32_t*>(bars + 4);
-  const int tid = threadIdx.x, warp = tid >> 5;
+  const int tid = threadIdx.x, warp = warp_index();
   const long long m0 = (long long)blockIdx.x * TC_M;
 
   if (warp == 0) {
@@ -292,21 +314,24 @@ __global__ void __launch_bounds__(HT) k_conv_tc(
     // tensor cores (async proxy) and to the issuing thread
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     __syncthreads();
-    if (tid == 0) {
+    if (warp == 0) {
       if (!mbar_wait(bars + s, (t >> 1) & 1, err)) {
         ok = false;
       } else {
         ++landed[s];
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const uint32_t a0 = smem_u32(As + s * A_BYTES), b0 = smem_u32(Bs + s * B_BYTES);
+        // K steps of 16 = two 8-channel chunks
+        const uint64_t ad = sdesc(smem_u32(As + s * A_BYTES), A_LBO, SBO);
+        const uint64_t bd = sdesc(smem_u32(Bs + s * B_BYTES), B_LBO, SBO);
+        const uint32_t acc = t > 0 ? 1u : 0u;
+        if (elect_one()) {
 #pragma unroll
-        for (int kk = 0; kk < KC / 16; ++kk) {
-          // K step of 16 = two 8-channel chunks
-          const uint64_t ad = sdesc(a0 + kk * 2 * A_LBO, A_LBO, SBO);
-          const uint64_t bd = sdesc(b0 + kk * 2 * B_LBO, B_LBO, SBO);
-          mma_bf16(tbase, ad, bd, IDESC, (t > 0 || kk > 0) ? 1u : 0u);
+          for (int kk = 0; kk < KC / 16; ++kk)
+            mma_bf16(tbase, desc_add(ad, kk * 2 * A_LBO), desc_add(bd, kk * 2 * B_LBO), IDESC,
+                     kk > 0 ? 1u : acc);
+          mma_commit(bars + 2 + s);
         }
-        mma_commit(bars + 2 + s);
+        __syncwarp();
         ++commits[s];
         last_commit = s;
       }
@@ -371,7 +396,7 @@ __global__ void __launch_bounds__(TC_THREADS) k_wgrad_tc(
   extern __shared__ __align__(1024) unsigned char smem[];
   uint64_t* done = reinterpret_cast<uint64_t*>(smem + WG_STAGES * ST_BYTES);
   uint32_t* tslot = reinterpret_cast<uint32_t*>(done + WG_STAGES);
-  const int tid = threadIdx.x, warp = tid >> 5;
+  const int tid = threadIdx.x, warp = warp_index();
   const int tile = blockIdx.x;
   const long long v0 = (long long)blockIdx.y * chunk;
   const long long v1 = v0 + chunk < Mtot ? v0 + chunk : Mtot;
@@ -443,16 +468,19 @@ __global__ void __launch_bounds__(TC_THREADS) k_wgrad_tc(
     cp_async_wait<WG_STAGES - 1>();
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     __syncthreads();
-    if (tid == 0) {
+    if (warp == 0) {
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       const uint32_t a0 = smem_u32(smem + st * ST_BYTES), b0 = a0 + A_BYTES;
+      const uint64_t ad = sdesc_mn(a0, 128, A_KSTR), bd = sdesc_mn(b0, 128, B_KSTR);
+      const uint32_t acc = k > 0 ? 1u : 0u;
+      if (elect_one()) {
 #pragma unroll
-      for (int kk = 0; kk < WG_KC / 16; ++kk) {
-        const uint64_t ad = sdesc_mn(a0 + 2 * kk * A_KSTR, 128, A_KSTR);
-        const uint64_t bd = sdesc_mn(b0 + 2 * kk * B_KSTR, 128, B_KSTR);
-        mma_bf16(tbase, ad, bd, IDESC, (k > 0 || kk > 0) ? 1u : 0u);
+        for (int kk = 0; kk < WG_KC / 16; ++kk)
+          mma_bf16(tbase, desc_add(ad, 2 * kk * A_KSTR), desc_add(bd, 2 * kk * B_KSTR), IDESC,
+                   kk > 0 ? 1u : acc);
+        mma_commit(done + st);
       }
-      mma_commit(done + st);
+      __syncwarp();
       ++commits[st];
       last_commit = st;
     }
@@ -578,7 +606,7 @@ __global__ void __launch_bounds__(HT) k_conv_halo(
   unsigned char* Ws = smem + H_BYTES;
   uint64_t* bars = reinterpret_cast<uint64_t*>(Ws + W_BYTES);  // weights, MMAs
   uint32_t* tslot = reinterpret_cast<uint32_t*>(bars + 2);
-  const int tid = threadIdx.x, warp = tid >> 5;
+  const int tid = threadIdx.x, warp = warp_index();
   const int D = 1 << lgD, M = D - 1;
   // tile coordinates: z blocks of 8, y blocks of 16, x blocks of TX, samples
   const int nz = D >> 3, ny = D >> 4, nx = D / TX;
@@ -616,28 +644,31 @@ __global__ void __launch_bounds__(HT) k_conv_halo(
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   __syncthreads();
   bool issued = false;
-  if (tid == 0) {
+  if (warp == 0) {
     if (!mbar_wait(bars, 0, err)) {
       ok = false;
     } else {
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      const uint32_t h0 = smem_u32(Hs), w0 = smem_u32(Ws);
       const int sg = DGRAD ? -1 : 1;
+      const uint64_t ad0 = sdesc(smem_u32(Hs), PLANE, SBO), bd0 = sdesc(smem_u32(Ws), B_LBO, 128);
+      const bool lead = elect_one();
 #pragma unroll 1
       for (int t = 0; t < 27; ++t) {
         const int dx = sg * (t / 9 - 1), dy = sg * ((t / 3) % 3 - 1), dz = sg * (t % 3 - 1);
-#pragma unroll 1
-        for (int tx = 0; tx < TX; ++tx) {
-          const uint32_t a_off = (uint32_t)((((tx + dx + 1) * HY + (dy + 1)) * HZ + (dz + 1)) * 16);
+        const uint64_t at = desc_add(ad0, (uint32_t)((((dx + 1) * HY + (dy + 1)) * HZ + (dz + 1)) * 16));
+        const uint64_t bt = desc_add(bd0, (uint32_t)(t * (NC * KC * 2)));
+        const uint32_t acc = t > 0 ? 1u : 0u;
+        if (lead) {
 #pragma unroll
-          for (int kk = 0; kk < KC / 16; ++kk) {
-            const uint64_t ad = sdesc(h0 + a_off + 2 * kk * PLANE, PLANE, SBO);
-            const uint64_t bd = sdesc(w0 + t * (NC * KC * 2) + 2 * kk * B_LBO, B_LBO, 128);
-            mma_bf16(tbase + tx * NC, ad, bd, IDESC, (t > 0 || kk > 0) ? 1u : 0u);
-          }
+          for (int kk = 0; kk < KC / 16; ++kk)
+#pragma unroll
+            for (int tx = 0; tx < TX; ++tx)  // consecutive MMAs into different accumulators
+              mma_bf16(tbase + tx * NC, desc_add(at, tx * (HY * HZ * 16) + 2 * kk * PLANE),
+                       desc_add(bt, 2 * kk * B_LBO), IDESC, kk > 0 ? 1u : acc);
         }
+        __syncwarp();
       }
-      mma_commit(bars + 1);
+      if (lead) mma_commit(bars + 1);
       issued = true;
     }
   }
@@ -695,9 +726,21 @@ void launch_halo(const TcArgs& a, cudaStream_t s) {
 
 // The same halo-tiled form for layers whose 27 weight slices do not fit beside
 // the input block: the block stays resident while the taps' weight slices
-// stream through two shared-memory stages (one bulk copy each).  Thread 0
-// alone loads the slices and issues the MMAs, so the loop over taps has no
-// block-wide synchronisation.
+// stream through NS shared-memory stages (one bulk copy each).  Thread 0 alone
+// loads the slices and issues the MMAs, so the loop over taps has no block-wide
+// synchronisation.  A tap's MMAs take about 0.3 us and a copy's latency is 1 us:
+// as many slices are in flight as the shared memory holds, up to 8 (with two,
+// 96 -> 32 waited for every slice: 110 us on 4 x 32^3).
+constexpr int halo_s_fit(int kc, int nc, int tx, int bytes) {
+  return (bytes - (kc / 8) * halo_plane(tx + 2)) / (nc * kc * 2);
+}
+// up to 8 where two CTAs share an SM with at least four each, else one CTA's room
+constexpr int halo_s_stages(int kc, int nc, int tx) {
+  const int two = halo_s_fit(kc, nc, tx, 112 * 1024), one = halo_s_fit(kc, nc, tx, 226 * 1024);
+  const int n = two >= 4 ? two : one;
+  return n > 8 ? 8 : n;
+}
+
 template <int KC, int NC, bool DGRAD, int TX>
 __global__ void __launch_bounds__(HT) k_conv_halo_s(
     const __nv_bfloat16* __restrict__ x, int ldx, int offx, const __nv_bfloat16* __restrict__ Wp,
@@ -708,14 +751,16 @@ __global__ void __launch_bounds__(HT) k_conv_halo_s(
   constexpr int PLANE = halo_plane(HX);
   constexpr int H_BYTES = CH * PLANE;
   constexpr int T_BYTES = NC * KC * 2;  // one tap's weight slice
+  constexpr int NS = halo_s_stages(KC, NC, TX);
+  static_assert(NS >= 2, "two weight slices beside the block");
   constexpr uint32_t SBO = HZ * 16, B_LBO = NC * 16;
   constexpr uint32_t IDESC = idesc_bf16(TC_M, NC);
   extern __shared__ __align__(1024) unsigned char smem[];
   unsigned char* Hs = smem;
-  unsigned char* Ws = smem + H_BYTES;  // [2][T_BYTES]
-  uint64_t* bars = reinterpret_cast<uint64_t*>(Ws + 2 * T_BYTES);  // full[2], done[2]
-  uint32_t* tslot = reinterpret_cast<uint32_t*>(bars + 4);
-  const int tid = threadIdx.x, warp = tid >> 5;
+  unsigned char* Ws = smem + H_BYTES;  // [NS][T_BYTES]
+  uint64_t* bars = reinterpret_cast<uint64_t*>(Ws + NS * T_BYTES);  // full[NS], done[NS]
+  uint32_t* tslot = reinterpret_cast<uint32_t*>(bars + 2 * NS);
+  const int tid = threadIdx.x, warp = warp_index();
   const int D = 1 << lgD, M = D - 1;
   const int nz = D >> 3, ny = D >> 4, nx = D / TX;
   long long bid = blockIdx.x;
@@ -736,18 +781,24 @@ __global__ void __launch_bounds__(HT) k_conv_halo_s(
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   if (tid == 0) {
-    for (int q = 0; q < 4; ++q) mbar_init(bars + q, 1);
+    for (int q = 0; q < 2 * NS; ++q) mbar_init(bars + q, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tbase = *tslot;
-  // thread 0's account of the copies and MMAs in flight
-  int issued[2] = {0, 0}, landed[2] = {0, 0}, commits[2] = {0, 0}, last_commit = -1;
-  if (tid == 0) {
-    bulk_load(Ws, Wp, (uint32_t)T_BYTES, bars);
-    ++issued[0];
+  int issued = 0, landed = 0, committed = 0;  // warp 0: slices copied, arrived, used
+  auto issue_w = [&](int q) {
+    bulk_load(Ws + (q % NS) * T_BYTES, Wp + (long long)q * NC * KC, (uint32_t)T_BYTES,
+              bars + q % NS);
+    ++issued;
+  };
+  if (warp == 0) {
+    const bool lead = elect_one();
+    for (int q = 0; q < NS - 1; ++q)
+      if (lead) issue_w(q); else ++issued;
+    __syncwarp();
   }
   load_halo<CH, HX>(Hs, x, ldx, offx, (unsigned)b, x0, y0, z0, lgD, tid);
   cp_async_commit();
@@ -755,52 +806,52 @@ __global__ void __launch_bounds__(HT) k_conv_halo_s(
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   __syncthreads();
   bool ok = true;
-  if (tid == 0) {
-    const uint32_t h0 = smem_u32(Hs), w0 = smem_u32(Ws);
+  if (warp == 0) {
     const int sg = DGRAD ? -1 : 1;
-    for (int t = 0; t < 27 && ok; ++t) {
-      const int st = t & 1;
-      if (t + 1 < 27) {
-        const int s1 = (t + 1) & 1;  // last read by the MMAs of tap t - 1
-        if (t >= 1 && !mbar_wait(bars + 2 + s1, ((t - 1) >> 1) & 1, err)) {
+    const uint64_t ad0 = sdesc(smem_u32(Hs), PLANE, SBO), bd0 = sdesc(smem_u32(Ws), B_LBO, 128);
+    const bool lead = elect_one();
+#pragma unroll 1
+    for (int t = 0; t < 27; ++t) {
+      const int st = t % NS, q = t + NS - 1;
+      if (q < 27) {
+        // its stage was last read by the MMAs of tap t - 1
+        if (t >= 1 && !mbar_wait(bars + NS + q % NS, ((t - 1) / NS) & 1, err)) {
           ok = false;
           break;
         }
-        bulk_load(Ws + s1 * T_BYTES, Wp + (long long)(t + 1) * NC * KC, (uint32_t)T_BYTES,
-                  bars + s1);
-        ++issued[s1];
+        if (lead) issue_w(q); else ++issued;
+        __syncwarp();
       }
-      if (!mbar_wait(bars + st, (t >> 1) & 1, err)) {
+      if (!mbar_wait(bars + st, (t / NS) & 1, err)) {
         ok = false;
         break;
       }
-      ++landed[st];
+      ++landed;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       const int dx = sg * (t / 9 - 1), dy = sg * ((t / 3) % 3 - 1), dz = sg * (t % 3 - 1);
-#pragma unroll 1
-      for (int tx = 0; tx < TX; ++tx) {
-        const uint32_t a_off = (uint32_t)((((tx + dx + 1) * HY + (dy + 1)) * HZ + (dz + 1)) * 16);
+      const uint64_t at = desc_add(ad0, (uint32_t)((((dx + 1) * HY + (dy + 1)) * HZ + (dz + 1)) * 16));
+      const uint64_t bt = desc_add(bd0, (uint32_t)(st * T_BYTES));
+      const uint32_t acc = t > 0 ? 1u : 0u;
+      if (lead) {
 #pragma unroll
-        for (int kk = 0; kk < KC / 16; ++kk) {
-          const uint64_t ad = sdesc(h0 + a_off + 2 * kk * PLANE, PLANE, SBO);
-          const uint64_t bd = sdesc(w0 + st * T_BYTES + 2 * kk * B_LBO, B_LBO, 128);
-          mma_bf16(tbase + tx * NC, ad, bd, IDESC, (t > 0 || kk > 0) ? 1u : 0u);
-        }
+        for (int kk = 0; kk < KC / 16; ++kk)
+#pragma unroll
+          for (int tx = 0; tx < TX; ++tx)  // consecutive MMAs into different accumulators
+            mma_bf16(tbase + tx * NC, desc_add(at, tx * (HY * HZ * 16) + 2 * kk * PLANE),
+                     desc_add(bt, 2 * kk * B_LBO), IDESC, kk > 0 ? 1u : acc);
+        mma_commit(bars + NS + st);
       }
-      mma_commit(bars + 2 + st);
-      ++commits[st];
-      last_commit = st;
+      __syncwarp();
+      ++committed;
     }
-    if (ok && !mbar_wait(bars + 2 + (26 & 1), (26 >> 1) & 1, err)) ok = false;
+    if (ok && !mbar_wait(bars + NS + 26 % NS, (26 / NS) & 1, err)) ok = false;
     if (!ok) {
       // a wait ran out: the copies and MMAs in flight (each wait bounded)
-      for (int q = 0; q < 2; ++q)
-        while (landed[q] < issued[q]) {
-          if (!mbar_wait(bars + q, (uint32_t)(landed[q] & 1), err)) break;
-          ++landed[q];
-        }
-      if (last_commit >= 0)
-        mbar_wait(bars + 2 + last_commit, (uint32_t)((commits[last_commit] - 1) & 1), err);
+      __syncwarp();
+      for (; landed < issued; ++landed)
+        if (!mbar_wait(bars + landed % NS, (uint32_t)((landed / NS) & 1), err)) break;
+      if (committed > 0)
+        mbar_wait(bars + NS + (committed - 1) % NS, (uint32_t)(((committed - 1) / NS) & 1), err);
     }
   }
   ok = __syncthreads_and(ok);
@@ -833,7 +884,8 @@ void launch_halo_s(const TcArgs& a, cudaStream_t s) {
   constexpr int H_BYTES = (KC / 8) * halo_plane(TX + 2), T_BYTES = NC * KC * 2;
   const int cols0 = TX * NC;
   const int cols = cols0 <= 32 ? 32 : (cols0 <= 64 ? 64 : (cols0 <= 128 ? 128 : 256));
-  const size_t need = (size_t)H_BYTES + 2 * T_BYTES + 4 * 8 + 16;
+  constexpr int NS = halo_s_stages(KC, NC, TX);
+  const size_t need = (size_t)H_BYTES + NS * T_BYTES + 2 * NS * 8 + 16;
   const int k = 512 / cols;
   const size_t cap = 233472 / (k + 1) - 1024 + 16;
   const size_t smem = need > cap ? need : cap;
@@ -897,7 +949,7 @@ __global__ void __launch_bounds__(HT) k_wgrad_halo(
   float* acc = reinterpret_cast<float*>(smem + W::STAGES * W::ST);  // [dx][q][ci][co]
   uint64_t* done = reinterpret_cast<uint64_t*>(smem + W::STAGES * W::ST + W::ACC);
   uint32_t* tslot = reinterpret_cast<uint32_t*>(done + W::STAGES);
-  const int tid = threadIdx.x, warp = tid >> 5;
+  const int tid = threadIdx.x, warp = warp_index();
   const int dy0 = ND == 9 ? -1 : (int)blockIdx.x - 1;  // ND = 3: this CTA's dy
   const int k0 = blockIdx.y * chunk, k1 = min(ntile, k0 + chunk);
   const int nk = k1 > k0 ? k1 - k0 : 0;
@@ -997,21 +1049,25 @@ __global__ void __launch_bounds__(HT) k_wgrad_halo(
     cp_async_wait<W::STAGES - 1>();
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     __syncthreads();
-    if (tid == 0) {
+    if (warp == 0) {
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      const uint32_t x0 = smem_u32(smem + st * W::ST), g0 = x0 + W::XB;
+      const uint32_t x0 = smem_u32(smem + st * W::ST);
+      const uint64_t ad = sdesc_mn(x0 + W::XB, W::GG, 128), bd0 = sdesc_mn(x0, W::XG, HZ * 16);
+      const bool lead = elect_one();
 #pragma unroll 1
       for (int q = 0; q < ND; ++q) {
         const int dy = ND == 9 ? q / 3 - 1 : dy0, dz = q % 3 - 1;
+        const uint64_t bd = desc_add(bd0, (uint32_t)(((dy + 1) * HZ + dz + 1) * 16));
+        const uint32_t acc0 = fresh ? 0u : 1u;
+        if (lead) {
 #pragma unroll
-        for (int kk = 0; kk < 8; ++kk) {  // 16 voxels: two y rows
-          const uint64_t ad = sdesc_mn(g0 + kk * 256, W::GG, 128);
-          const uint64_t bd =
-              sdesc_mn(x0 + ((2 * kk + dy + 1) * HZ + dz + 1) * 16, W::XG, HZ * 16);
-          mma_bf16(tbase + q * W::N, ad, bd, IDESC, (!fresh || kk > 0) ? 1u : 0u);
+          for (int kk = 0; kk < 8; ++kk)  // 16 voxels: two y rows
+            mma_bf16(tbase + q * W::N, desc_add(ad, kk * 256), desc_add(bd, 2 * kk * HZ * 16),
+                     IDESC, kk > 0 ? 1u : acc0);
         }
+        __syncwarp();
       }
-      mma_commit(done + st);
+      if (lead) mma_commit(done + st);
       ++commits[st];
       last_commit = st;
     }
