@@ -23,7 +23,8 @@
 
 #include "amr.cuh"
 #include "colour_split.cuh"
-#include "dfloat.cuh"
+#include "lean_fp64.cuh"
+#include "mg32_dev.cuh"
 
 namespace {
 
@@ -642,11 +643,82 @@ __global__ void __launch_bounds__(64) k_dlin_coarse(float* __restrict__ eg, cons
   eg[t] = e[t];
 }
 
-__global__ void k_zero32(float* __restrict__ x, long long n) {
-  const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (i < n) x[i] = 0.f;
+// ---- deviation cycle (FP64 form): L(u + e) - L(u) = r in FP32 ---------------------
+// The masked V-cycle of the level in the deviation e from the FP64 iterate u
+// (mg32.cuh, MG_DEV), in the arrays of the linear cycle: u (FP32 copy), r, e.
+PF pf32(const MT<float>& m, float cap) { return PF{m.aRt, m.aRt_np1, m.inv_np1, cap}; }
+
+__global__ void __launch_bounds__(BS) k_ddev_sweep_list(float* __restrict__ e,
+                                                        const float* __restrict__ r,
+                                                        const float* __restrict__ u, int lg,
+                                                        const int* __restrict__ list, long long n,
+                                                        PF m, float ih2) {
+  const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  if (t >= n) return;
+  const unsigned c = (unsigned)list[t];
+  const int M = (1 << lg) - 1;
+  const int k = (int)(c & M), j = (int)((c >> lg) & M), i = (int)(c >> (2 * lg));
+  float un[6], en[6];
+  dnb_x(u, i, j, k, lg, un);
+  dnb_x(e, i, j, k, lg, en);
+  e[c] = point_update<MG_DEV>(e[c], en, u[c], un, r[c], m, ih2, 0.f);
 }
 
+__global__ void __launch_bounds__(BS) k_ddev_restrict(const float* __restrict__ e,
+                                                      const float* __restrict__ r,
+                                                      const float* __restrict__ u, int lgf,
+                                                      float* __restrict__ rc, float* __restrict__ uc,
+                                                      float* __restrict__ ec, PF m, float ih2,
+                                                      const unsigned char* __restrict__ act) {
+  const int lgc = lgf - 1, Nc = 1 << lgc;
+  const unsigned t = blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= (1u << (3 * lgc))) return;
+  const int K = (int)(t & (Nc - 1)), J = (int)((t >> lgc) & (Nc - 1)), I = (int)(t >> (2 * lgc));
+  float su = 0.f, sr = 0.f;
+  for (int q = 0; q < 8; ++q) {
+    const int i = 2 * I + (q >> 2), j = 2 * J + ((q >> 1) & 1), k = 2 * K + (q & 1);
+    const unsigned c = cidx(i, j, k, lgf);
+    su += u[c] + e[c];
+    if (!act || act[c]) {
+      float un[6], en[6];
+      dnb_x(u, i, j, k, lgf, un);
+      dnb_x(e, i, j, k, lgf, en);
+      sr += r[c] - point_apply<MG_DEV>(e[c], en, u[c], un, m, ih2);
+    }
+  }
+  uc[t] = 0.125f * su;
+  rc[t] = 0.125f * sr;
+  ec[t] = 0.f;
+}
+
+__global__ void __launch_bounds__(64) k_ddev_coarse(float* __restrict__ eg,
+                                                    const float* __restrict__ rg,
+                                                    const float* __restrict__ ug, PF m, float ih2,
+                                                    int sweeps,
+                                                    const unsigned char* __restrict__ act) {
+  __shared__ float e[64];
+  const int t = threadIdx.x;
+  const bool active = !act || act[t];
+  const int i = t >> 4, j = (t >> 2) & 3, k = t & 3, colour = (i + j + k) & 1;
+  const int q[6] = {(((i + 3) & 3) << 4) | (j << 2) | k, (((i + 1) & 3) << 4) | (j << 2) | k,
+                    (i << 4) | (((j + 3) & 3) << 2) | k, (i << 4) | (((j + 1) & 3) << 2) | k,
+                    (i << 4) | (j << 2) | ((k + 3) & 3), (i << 4) | (j << 2) | ((k + 1) & 3)};
+  float un[6];
+  for (int d = 0; d < 6; ++d) un[d] = ug[q[d]];
+  const float uc = ug[t], rc = rg[t];
+  e[t] = eg[t];
+  __syncthreads();
+  for (int s = 0; s < sweeps; ++s)
+    for (int col = 0; col < 2; ++col) {
+      if (colour == col && active) {
+        float en[6];
+        for (int d = 0; d < 6; ++d) en[d] = e[q[d]];
+        e[t] = point_update<MG_DEV>(e[t], en, uc, un, rc, m, ih2, 0.f);
+      }
+      __syncthreads();
+    }
+  eg[t] = e[t];
+}
 
 // ---- FP32 storage of oct levels -------------------------------------------
 // The FP32 arrays of an oct level (u, f or r, e) are stored by colour
@@ -1084,6 +1156,156 @@ __global__ void __launch_bounds__(BS) k_oprolong32(long long n, const int* __res
     U.v[ch] += v;
   }
   st8(u, o, no, U);
+}
+
+// ---- thread-per-oct kernels of the deviation cycle ------------------------------
+// the values of x (colour-split) on the four cells across each face of oct o, by
+// face cell (face_q); `gh`: the ghost values (NULL: zero)
+struct Faces {
+  float v[6][4];
+};
+__device__ __forceinline__ Faces oct_faces(const float* __restrict__ x, const int* nb,
+                                           const float* __restrict__ gh, long long no) {
+  Faces F;
+#pragma unroll
+  for (int d = 0; d < 6; ++d) {
+    const int a = d >> 1, plus = d & 1;
+    if (nb[d] >= 0) {
+      const Oct8 N = ld8(x, nb[d], no);
+#pragma unroll
+      for (int ch = 0; ch < 8; ++ch)
+        if (((ch >> (2 - a)) & 1) == plus) F.v[d][face_q(ch, a)] = N.v[ch ^ (1 << (2 - a))];
+    } else if (gh) {
+      const float4 g = *reinterpret_cast<const float4*>(gh + 4LL * (-nb[d] - 1));
+      F.v[d][0] = g.x;
+      F.v[d][1] = g.y;
+      F.v[d][2] = g.z;
+      F.v[d][3] = g.w;
+    } else {
+      F.v[d][0] = F.v[d][1] = F.v[d][2] = F.v[d][3] = 0.f;
+    }
+  }
+  return F;
+}
+// the six neighbours of cell ch
+__device__ __forceinline__ void oct_six(const Oct8& X, const Faces& F, int ch, float* o) {
+#pragma unroll
+  for (int d = 0; d < 6; ++d) {
+    const int a = d >> 1, plus = d & 1;
+    o[d] = ((ch >> (2 - a)) & 1) != plus ? X.v[ch ^ (1 << (2 - a))] : F.v[d][face_q(ch, a)];
+  }
+}
+
+template <int COL>
+__global__ void __launch_bounds__(BS) k_oct_dev_sweep(
+    const float* __restrict__ u, float* __restrict__ e, const float* __restrict__ r,
+    const int* __restrict__ nbr, const float* __restrict__ gh,
+    const unsigned char* __restrict__ act, long long n, const int* __restrict__ olist,
+    long long no, PF m, float ih2) {
+  const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  if (t >= n) return;
+  const long long o = olist ? olist[t] : t;
+  constexpr int CC[2][4] = {{0, 3, 5, 6}, {1, 2, 4, 7}};
+  int nb[6];
+#pragma unroll
+  for (int d = 0; d < 6; ++d) nb[d] = __ldg(nbr + 6 * o + d);
+  const Oct8 U = ld8(u, o, no), X = ld8(e, o, no);
+  const Faces FU = oct_faces(u, nb, gh, no), FX = oct_faces(e, nb, nullptr, no);
+  const float4 R4 = ldc(r, o, no, COL);
+  float out[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const int ch = CC[COL][q];
+    float un[6], xn[6];
+    oct_six(U, FU, ch, un);
+    oct_six(X, FX, ch, xn);
+    out[q] = !act || act[8 * o + ch]
+                 ? point_update<MG_DEV>(X.v[ch], xn, U.v[ch], un, f4(R4, q), m, ih2, 0.f)
+                 : X.v[ch];
+  }
+  stc(e, o, no, COL, make_float4(out[0], out[1], out[2], out[3]));
+}
+
+// r_c = R(r - D(e)) over relaxed cells, u_c = R(u + e), e_c = 0
+__global__ void __launch_bounds__(BS) k_oct_dev_restrict(
+    const float* __restrict__ e, const float* __restrict__ r, const float* __restrict__ u,
+    const int* __restrict__ nbr, const float* __restrict__ gh,
+    const unsigned char* __restrict__ act, long long n, const int* __restrict__ olist,
+    long long no, const int* __restrict__ pcell, long long pno, PF m, float ih2,
+    float* __restrict__ rc, float* __restrict__ uc, float* __restrict__ ec) {
+  const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  if (t >= n) return;
+  const long long o = olist ? olist[t] : t;
+  int nb[6];
+#pragma unroll
+  for (int d = 0; d < 6; ++d) nb[d] = __ldg(nbr + 6 * o + d);
+  const Oct8 U = ld8(u, o, no), X = ld8(e, o, no), R = ld8(r, o, no);
+  const Faces FU = oct_faces(u, nb, gh, no), FX = oct_faces(e, nb, nullptr, no);
+  float su = 0.f, sr = 0.f;
+#pragma unroll
+  for (int ch = 0; ch < 8; ++ch) {
+    su += U.v[ch] + X.v[ch];
+    if (!act || act[8 * o + ch]) {
+      float un[6], xn[6];
+      oct_six(U, FU, ch, un);
+      oct_six(X, FX, ch, xn);
+      sr += R.v[ch] - point_apply<MG_DEV>(X.v[ch], xn, U.v[ch], un, m, ih2);
+    }
+  }
+  const long long p = pidx(pcell[o], pno);
+  uc[p] = 0.125f * su;
+  rc[p] = 0.125f * sr;
+  ec[p] = 0.f;
+}
+
+// The FP64 residual of the level: its norms (as k_onorm<double>) and the
+// deviation problem, r32 = r, u32 = u
+__global__ void __launch_bounds__(BS) k_oresid_dev(const double* __restrict__ u,
+                                                   const double* __restrict__ E,
+                                                   const double* __restrict__ f,
+                                                   const int* __restrict__ nbr,
+                                                   const double* __restrict__ gh,
+                                                   const double* __restrict__ ghE, long long ncell,
+                                                   MT<double> m, double ih2h,
+                                                   float* __restrict__ r32, float* __restrict__ u32,
+                                                   double* __restrict__ partials) {
+  double ss = 0.0, fs = 0.0;
+  long long mx = 0;  // bits of max |r|
+  const long long no = ncell >> 3;
+  for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < ncell;
+       c += (long long)gridDim.x * blockDim.x) {
+    const long long o = c >> 3;
+    const int ch = (int)(c & 7);
+    const double uc = u[c], Ec = E[c], fc = f[c];
+    double s = 0.0;
+#pragma unroll
+    for (int d = 0; d < 6; ++d) {
+      const NB<double> nb = onb(u, E, nbr, gh, ghE, o, ch, d);
+      s = fma(nb.E + Ec, nb.u - uc, s);
+    }
+    const double sN = m.n == 1 ? lean_rsqrt(Ec) : lean_exp(-uc * m.inv_np1);
+    const double r = fc - fma(s, ih2h, m.aRt * (1.0 - sN));
+    const long long q = pidx(c, no);
+    r32[q] = f_from_double_bits(r);
+    u32[q] = f_from_double_bits(uc);
+    ss = fma(r, r, ss);
+    fs = fma(fc, fc, fs);
+    const long long b = __double_as_longlong(r) & 0x7fffffffffffffffLL;
+    mx = b > mx ? b : mx;
+  }
+  block_partials3(ss, __longlong_as_double(mx), fs, partials);
+}
+
+// w += sign e (where finite), wE = e^w
+__global__ void __launch_bounds__(BS) k_oapply_dev(double* __restrict__ w, double* __restrict__ wE,
+                                                   const float* __restrict__ e, long long ncell,
+                                                   float sign) {
+  const long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  if (c >= ncell) return;
+  const float x = e[pidx(c, ncell >> 3)];
+  const double v = w[c] + (isfinite(x) ? d_from_float_bits(sign * x) : 0.0);
+  w[c] = v;
+  wE[c] = lean_exp(v);
 }
 
 // ---- phase B in double-float (mixed form) ---------------------------------
@@ -1809,50 +2031,80 @@ mgfr_status build_oct_list(mgfr_ctx* c, AmrWork* A, AmrLevel& P, float mthr) {
   return MGFR_OK;
 }
 
-// ---- linear masked V-cycle (phase B of the mixed form) -------------------------
-// level arrays: u = w32 (linearisation point), E = wE32, r = wf32, e = wold32;
-// dense levels below the base: u = u32, E = e32, r = r32, e = uold32.
-void lin_relax(SolveCtx& S, int l, int sweeps) {
+// ---- correction V-cycles on e: linear (phase B of the mixed form) or in the
+// deviation (DEV: the FP64 form) -----------------------------------------------------
+// level arrays: u = w32 (linearisation point), r = wf32, e = wold32; dense levels
+// below the base: u = u32, r = r32, e = uold32.
+template <bool DEV>
+void corr_relax(SolveCtx& S, int l, int sweeps) {
   mgfr_ctx* c = S.c;
   AmrLevel& L = S.A->L[l];
   const MT<float> m = mt<float>(S.m);
+  const PF p = pf32(m, (float)c->cfg.step_cap);
   for (int s = 0; s < sweeps; ++s) {
     for (int col = 0; col < 2; ++col) {
       if (l >= 1) {
         const unsigned char* mk = l == S.L ? nullptr : L.act;
         const ORange R = orange(S, L, l);
         if (R.n == 0) continue;
-        if (l == S.L) prof_begin(c, 4, L.ncell);
-        if (col == 0)
-          k_oct_sweep32<true, 0><<<nblocks(R.n, BS), BS, 0, c->s>>>(
-              L.w32, L.wold32, L.wf32, L.nbr, L.ghost32, mk, R.n, R.list, L.n_oct, m,
-              (float)L.ih2, 0.f);
-        else
-          k_oct_sweep32<true, 1><<<nblocks(R.n, BS), BS, 0, c->s>>>(
-              L.w32, L.wold32, L.wf32, L.nbr, L.ghost32, mk, R.n, R.list, L.n_oct, m,
-              (float)L.ih2, 0.f);
+        if (l == S.L) prof_begin(c, DEV ? 3 : 4, L.ncell);
+        if constexpr (DEV) {
+          (col == 0 ? k_oct_dev_sweep<0> : k_oct_dev_sweep<1>)<<<nblocks(R.n, BS), BS, 0, c->s>>>(
+              L.w32, L.wold32, L.wf32, L.nbr, L.ghost32, mk, R.n, R.list, L.n_oct, p,
+              (float)L.ih2);
+        } else {
+          (col == 0 ? k_oct_sweep32<true, 0> : k_oct_sweep32<true, 1>)
+              <<<nblocks(R.n, BS), BS, 0, c->s>>>(L.w32, L.wold32, L.wf32, L.nbr, L.ghost32, mk,
+                                                  R.n, R.list, L.n_oct, m, (float)L.ih2, 0.f);
+        }
         if (l == S.L) prof_end(c);
       } else {
         const long long nl = S.A->dlist_n[0][col];
         if (nl == 0) continue;
-        k_dlin_sweep_list<<<nblocks(nl, BS), BS, 0, c->s>>>(
-            L.wold32, L.wf32, L.w32, L.wE32, L.lgN, S.A->dlist[0] + col * (L.ncell / 2), nl, m,
-            (float)L.ih2);
+        const int* list = S.A->dlist[0] + col * (L.ncell / 2);
+        if constexpr (DEV)
+          k_ddev_sweep_list<<<nblocks(nl, BS), BS, 0, c->s>>>(L.wold32, L.wf32, L.w32, L.lgN, list,
+                                                              nl, p, (float)L.ih2);
+        else
+          k_dlin_sweep_list<<<nblocks(nl, BS), BS, 0, c->s>>>(L.wold32, L.wf32, L.w32, L.wE32,
+                                                              L.lgN, list, nl, m, (float)L.ih2);
       }
       c->launches += 1;
     }
   }
+  (DEV ? S.updates : S.lin_updates) += (long long)sweeps * L.relaxed;
 }
 
-void lin_vcycle_dense(SolveCtx& S, int k) {
+// restriction of dense arrays (u, r, e) of level lgf to the dense level C
+template <bool DEV>
+void corr_drestrict(SolveCtx& S, const float* e, const float* r, const float* u, const float* E,
+                    int lgf, double ih2, const unsigned char* act, DenseLevel& C) {
+  mgfr_ctx* c = S.c;
+  const MT<float> m = mt<float>(S.m);
+  if constexpr (DEV)
+    k_ddev_restrict<<<nblocks(C.n, BS), BS, 0, c->s>>>(e, r, u, lgf, C.r32, C.u32, C.uold32,
+                                                       pf32(m, (float)c->cfg.step_cap),
+                                                       (float)ih2, act);
+  else
+    k_dlin_restrict<<<nblocks(C.n, BS), BS, 0, c->s>>>(e, r, u, E, lgf, C.r32, C.u32, C.e32,
+                                                       C.uold32, m, (float)ih2, act);
+  c->launches += 1;
+}
+
+template <bool DEV>
+void corr_vcycle_dense(SolveCtx& S, int k) {
   mgfr_ctx* c = S.c;
   const mgfr_config& g = c->cfg;
   DenseHier& H = c->dh;
   DenseLevel& F = H.L[k];
   const unsigned char* mk = S.A->dact[k];
   const MT<float> m = mt<float>(S.m);
+  const PF p = pf32(m, (float)g.step_cap);
   if (F.N <= 4) {
-    k_dlin_coarse<<<1, 64, 0, c->s>>>(F.uold32, F.r32, F.u32, F.e32, m, (float)F.ih2, 20, mk);
+    if constexpr (DEV)
+      k_ddev_coarse<<<1, 64, 0, c->s>>>(F.uold32, F.r32, F.u32, p, (float)F.ih2, 20, mk);
+    else
+      k_dlin_coarse<<<1, 64, 0, c->s>>>(F.uold32, F.r32, F.u32, F.e32, m, (float)F.ih2, 20, mk);
     c->launches += 1;
     return;
   }
@@ -1861,20 +2113,21 @@ void lin_vcycle_dense(SolveCtx& S, int k) {
       for (int col = 0; col < 2; ++col) {
         const long long nl = S.A->dlist_n[k][col];
         if (nl == 0) continue;
-        k_dlin_sweep_list<<<nblocks(nl, BS), BS, 0, c->s>>>(F.uold32, F.r32, F.u32, F.e32, F.lg,
-                                                            S.A->dlist[k] + col * (F.n / 2), nl,
-                                                            m, (float)F.ih2);
+        const int* list = S.A->dlist[k] + col * (F.n / 2);
+        if constexpr (DEV)
+          k_ddev_sweep_list<<<nblocks(nl, BS), BS, 0, c->s>>>(F.uold32, F.r32, F.u32, F.lg, list,
+                                                              nl, p, (float)F.ih2);
+        else
+          k_dlin_sweep_list<<<nblocks(nl, BS), BS, 0, c->s>>>(F.uold32, F.r32, F.u32, F.e32, F.lg,
+                                                              list, nl, m, (float)F.ih2);
         c->launches += 1;
       }
   };
   sweep(sweeps_of(S, -1, g.n_pre));
   if (k + 1 <= S.kmax) {
     DenseLevel& C = H.L[k + 1];
-    k_dlin_restrict<<<nblocks(C.n, BS), BS, 0, c->s>>>(F.uold32, F.r32, F.u32, F.e32, F.lg,
-                                                       C.r32, C.u32, C.e32, C.uold32, m,
-                                                       (float)F.ih2, mk);
-    c->launches += 1;
-    lin_vcycle_dense(S, k + 1);
+    corr_drestrict<DEV>(S, F.uold32, F.r32, F.u32, F.e32, F.lg, F.ih2, mk, C);
+    corr_vcycle_dense<DEV>(S, k + 1);
     const CList cf = clist(S, k);
     if (cl_threads(cf, F.n) > 0)
       k_dlin_prolong<<<nblocks(cl_threads(cf, F.n), BS), BS, 0, c->s>>>(
@@ -1884,26 +2137,31 @@ void lin_vcycle_dense(SolveCtx& S, int k) {
   sweep(sweeps_of(S, -1, g.n_post));
 }
 
-void lin_vcycle_tree(SolveCtx& S, int l) {
+template <bool DEV>
+void corr_vcycle_tree(SolveCtx& S, int l) {
   mgfr_ctx* c = S.c;
   AmrWork* A = S.A;
   const mgfr_config& g = c->cfg;
   const MT<float> m = mt<float>(S.m);
   AmrLevel& F = A->L[l];
-  const int npre = sweeps_of(S, l, g.n_pre), npost = sweeps_of(S, l, g.n_post);
-  lin_relax(S, l, npre);
-  S.lin_updates += (long long)npre * F.relaxed;
+  corr_relax<DEV>(S, l, sweeps_of(S, l, g.n_pre));
   const unsigned char* fmask = l == S.L ? nullptr : F.act;
   if (l >= 1 && has_coarse(S, l)) {
     AmrLevel& P = A->L[l - 1];
     const ORange R = orange(S, F, l);
     const long long pno = l - 1 >= 1 ? P.n_oct : 0;  // FP32 parent layout (0: dense)
-    if (R.n > 0)
-      k_olin_restrict32<<<nblocks(R.n, BS), BS, 0, c->s>>>(
-          F.wold32, F.wf32, F.w32, F.nbr, F.ghost32, fmask, R.n, R.list, F.n_oct, F.pcell, pno,
-          m, (float)F.ih2, P.wf32, P.w32, P.wold32);
+    if (R.n > 0) {
+      if constexpr (DEV)
+        k_oct_dev_restrict<<<nblocks(R.n, BS), BS, 0, c->s>>>(
+            F.wold32, F.wf32, F.w32, F.nbr, F.ghost32, fmask, R.n, R.list, F.n_oct, F.pcell, pno,
+            pf32(m, (float)g.step_cap), (float)F.ih2, P.wf32, P.w32, P.wold32);
+      else
+        k_olin_restrict32<<<nblocks(R.n, BS), BS, 0, c->s>>>(
+            F.wold32, F.wf32, F.w32, F.nbr, F.ghost32, fmask, R.n, R.list, F.n_oct, F.pcell, pno,
+            m, (float)F.ih2, P.wf32, P.w32, P.wold32);
+    }
     c->launches += 1;
-    lin_vcycle_tree(S, l - 1);
+    corr_vcycle_tree<DEV>(S, l - 1);
     if (R.n > 0)
       k_oprolong32<true><<<nblocks(R.n, BS), BS, 0, c->s>>>(R.n, R.list, F.n_oct, F.pcell,
                                                            F.pnbr, pno, P.wold32, nullptr, fmask,
@@ -1912,19 +2170,30 @@ void lin_vcycle_tree(SolveCtx& S, int l) {
   } else if (l == 0 && S.kmax >= 1) {
     DenseHier& H = c->dh;
     DenseLevel& C = H.L[1];
-    k_dlin_restrict<<<nblocks(C.n, BS), BS, 0, c->s>>>(F.wold32, F.wf32, F.w32, F.wE32, F.lgN,
-                                                       C.r32, C.u32, C.e32, C.uold32, m,
-                                                       (float)F.ih2, F.act);
-    c->launches += 1;
-    lin_vcycle_dense(S, 1);
+    corr_drestrict<DEV>(S, F.wold32, F.wf32, F.w32, F.wE32, F.lgN, F.ih2, F.act, C);
+    corr_vcycle_dense<DEV>(S, 1);
     const CList c0 = clist(S, 0);
     if (cl_threads(c0, F.ncell) > 0)
       k_dlin_prolong<<<nblocks(cl_threads(c0, F.ncell), BS), BS, 0, c->s>>>(
           F.wold32, C.uold32, F.lgN, g.prolong_linear, F.act, c0);
     c->launches += 1;
   }
-  lin_relax(S, l, npost);
-  S.lin_updates += (long long)npost * F.relaxed;
+  corr_relax<DEV>(S, l, sweeps_of(S, l, g.n_post));
+}
+
+// FP64 residual of level L -> hs[0..2] and the deviation problem (FP64 form)
+mgfr_status dev_resid(SolveCtx& S, double* hs) {
+  mgfr_ctx* c = S.c;
+  AmrLevel& L = S.A->L[S.L];
+  DenseHier& H = c->dh;
+  const int nparts = (int)std::min<long long>(H.nparts / 2, nblocks(L.ncell, BS));
+  k_oresid_dev<<<nparts, BS, 0, c->s>>>(L.w, L.wE, L.wf, L.nbr, L.ghost, L.ghostE, L.ncell,
+                                        mt<double>(S.m), 0.5 * L.ih2, L.wf32, L.w32, H.partials);
+  k_finish3<<<1, 256, 0, c->s>>>(H.partials, nparts, H.scal + 8);
+  c->launches += 2;
+  MG_CK(c, cudaMemcpyAsync(hs, H.scal + 8, 3 * sizeof(double), cudaMemcpyDeviceToHost, c->s));
+  MG_CK(c, cudaStreamSynchronize(c->s));
+  return MGFR_OK;
 }
 
 // FP64 residual of level L with the linear system set up for phase B
@@ -2004,8 +2273,8 @@ mgfr_status amr_solve_level(mgfr_ctx* c, AmrWork* A, int Lv, const Model& m, mgf
     c->launches += 1;
   }
   F.relaxed = F.ncell;
-  // FP64 work copies of the coarser levels: set up front in the FP64 form; in
-  // the mixed form only the FP64 fallback V-cycles below need them
+  // FP64 work copies of the coarser levels: only the V-cycles in FP64 throughout
+  // need them
   auto fp64_coarse = [&]() -> mgfr_status {
     for (int l = Lv - 1; l >= 0; --l) {
       AmrLevel& P = A->L[l];
@@ -2019,15 +2288,15 @@ mgfr_status amr_solve_level(mgfr_ctx* c, AmrWork* A, int Lv, const Model& m, mgf
     }
     return MGFR_OK;
   };
-  if (!mixed) TRY(fp64_coarse());
   for (int l = Lv - 1; l >= 0; --l) {
     AmrLevel& P = A->L[l];
     const double* uu = l == 0 ? H.L[0].u : P.u;
-    if (mixed) {
-      const long long pno = l >= 1 ? P.n_oct : 0;  // FP32 layout (0: dense)
+    const long long pno = l >= 1 ? P.n_oct : 0;  // FP32 layout (0: dense)
+    if (mixed)
       k_d2f2<<<nblocks(P.ncell, BS), BS, 0, c->s>>>(uu, P.w32, P.wold32, P.ncell, pno);
-      c->launches += 1;
-    }
+    else
+      k_d2f<<<nblocks(P.ncell, BS), BS, 0, c->s>>>(uu, P.w32, P.ncell, pno);
+    c->launches += 1;
     MG_CK(c, cudaMemsetAsync(P.mask, 0, sizeof(float) * (size_t)P.ncell, c->s));
     AmrLevel& Ch = A->L[l + 1];
     k_mask_up<<<nblocks(Ch.n_oct, BS), BS, 0, c->s>>>(Ch.mask, Ch.n_oct, Ch.pcell, P.mask);
@@ -2065,12 +2334,20 @@ mgfr_status amr_solve_level(mgfr_ctx* c, AmrWork* A, int Lv, const Model& m, mgf
   if (mixed)
     TRY(level_norm<float>(S, hs));
   else
-    TRY(level_norm<double>(S, hs));
+    TRY(dev_resid(S, hs));
   const double fn = std::sqrt(hs[2]), r0 = std::sqrt(hs[0]);
   const double ref = fn > 0.0 ? fn : r0;
   const double target = g.tol_rel * ref;
   double r = r0;
   int it = 0, it32 = 0;
+  // e = 0 on the coarser levels (cells that are never relaxed keep it)
+  auto zero_corr = [&]() -> mgfr_status {
+    for (int l = Lv - 1; l >= 0; --l)
+      MG_CK(c, cudaMemsetAsync(A->L[l].wold32, 0, sizeof(float) * (size_t)A->L[l].ncell, c->s));
+    for (int k = 1; k < H.nlev; ++k)
+      MG_CK(c, cudaMemsetAsync(H.L[k].uold32, 0, sizeof(float) * (size_t)H.L[k].n, c->s));
+    return MGFR_OK;
+  };
   if (mixed && r > target) {
     // FP32 V-cycles until mixed_switch or a stall
     double prev = -1.0;
@@ -2088,15 +2365,7 @@ mgfr_status amr_solve_level(mgfr_ctx* c, AmrWork* A, int Lv, const Model& m, mgf
     w_df = true;
     // phase B: FP64-accurate residual (double-float), FP32 linear masked
     // V-cycles on J(u) e = r, u += e
-    for (int l = Lv - 1; l >= 0; --l) {
-      AmrLevel& P = A->L[l];
-      k_zero32<<<nblocks(P.ncell, BS), BS, 0, c->s>>>(P.wold32, P.ncell);
-      c->launches += 1;
-    }
-    for (int k = 1; k < H.nlev; ++k) {
-      k_zero32<<<nblocks(H.L[k].n, BS), BS, 0, c->s>>>(H.L[k].uold32, H.L[k].n);
-      c->launches += 1;
-    }
+    TRY(zero_corr());
     c->capturing = 3;
     TRY(lin_resid(S, hs));
     c->capturing = -1;
@@ -2105,7 +2374,7 @@ mgfr_status amr_solve_level(mgfr_ctx* c, AmrWork* A, int Lv, const Model& m, mgf
     int inner = g.mixed_inner;
     while (r > target && it < g.max_vcycles) {
       c->capturing = 3;
-      for (int q = 0; q < inner; ++q) lin_vcycle_tree(S, Lv);
+      for (int q = 0; q < inner; ++q) corr_vcycle_tree<false>(S, Lv);
       k_apply_df<<<nblocks(F.ncell, BS), BS, 0, c->s>>>(reinterpret_cast<dfl*>(F.w),
                                                         reinterpret_cast<dfl*>(F.wE), F.wold32,
                                                         F.n_oct, F.ncell, (float)g.step_cap);
@@ -2153,11 +2422,42 @@ mgfr_status amr_solve_level(mgfr_ctx* c, AmrWork* A, int Lv, const Model& m, mgf
     gh_df = false;
     TRY(fp64_coarse());
   }
+  // FP64 form: V-cycles with the correction in FP32 (as the base level's; 33% of a
+  // solve was in the FP64 oct sweeps alone), in FP64 throughout while the residual
+  // is beyond kDevMax ||f|| and from the first FP32 cycle that gains nothing
+  constexpr double kDevMax = 2.0;
+  bool dev_ok = !mixed, coarse64 = mixed;
+  if (dev_ok && r > target) TRY(zero_corr());
   while (r > target && it < g.max_vcycles) {
+    if (dev_ok && r <= kDevMax * ref) {
+      MG_CK(c, cudaMemsetAsync(F.wold32, 0, sizeof(float) * (size_t)F.ncell, c->s));
+      c->capturing = 3;
+      corr_vcycle_tree<true>(S, Lv);
+      c->capturing = -1;
+      k_oapply_dev<<<nblocks(F.ncell, BS), BS, 0, c->s>>>(F.w, F.wE, F.wold32, F.ncell, 1.f);
+      c->launches += 1;
+      TRY(dev_resid(S, hs));
+      prof_collect(c, 3, st);
+      const double rn = std::sqrt(hs[0]);
+      if (!(rn < r)) {
+        k_oapply_dev<<<nblocks(F.ncell, BS), BS, 0, c->s>>>(F.w, F.wE, F.wold32, F.ncell, -1.f);
+        c->launches += 1;
+        dev_ok = false;
+        continue;
+      }
+      r = rn;
+      ++it;
+      continue;
+    }
+    if (!coarse64) {
+      TRY(fp64_coarse());
+      coarse64 = true;
+    }
     TRY(run_vcycle<double>(S, st, hs));
     r = std::sqrt(hs[0]);
     ++it;
     if (!std::isfinite(r)) break;
+    if (dev_ok && r <= kDevMax * ref && r > target) TRY(dev_resid(S, hs));
   }
   if (w_df) {
     k_df2d<<<nblocks(F.ncell, BS), BS, 0, c->s>>>(reinterpret_cast<const dfl*>(F.w), F.u,

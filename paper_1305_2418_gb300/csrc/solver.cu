@@ -243,10 +243,8 @@ static mgfr_status ensure_dense(mgfr_ctx* c, int N, bool mixed) {
     MG_CK(c, cudaMalloc(&L.u32, b4));
     MG_CK(c, cudaMalloc(&L.e32, b4));
     MG_CK(c, cudaMalloc(&L.r32, b4));
-    if (mixed) {
-      MG_CK(c, cudaMalloc(&L.f32, b4));
-      if (l > 0) MG_CK(c, cudaMalloc(&L.uold32, b4));
-    }
+    if (l > 0) MG_CK(c, cudaMalloc(&L.uold32, b4));
+    if (mixed) MG_CK(c, cudaMalloc(&L.f32, b4));
   }
   H.nparts = 152 * 8;
   if (mixed) MG_CK(c, cudaMalloc(&H.fdf, sizeof(double) * (size_t)H.L[0].n));

@@ -112,3 +112,35 @@ def test_batch_in_both_precisions(dev, tol):
         scale = float(ref["acc"].abs().max())
         assert float((o["acc"] - ref["acc"]).abs().max()) <= 1e3 * tol * scale
     s.close()
+
+
+@pytest.mark.parametrize("sig,fr0,levels,kw", [
+    (1.5, 1e-5, 2, {}),
+    (2.0, 1e-6, 3, dict(n_pre=1, n_post=2)),
+    (1.0, 1e-4, 1, dict(n=2, prolong_linear=0)),
+])
+def test_refined_levels_in_fp64_with_fp32_corrections(dev, sig, fr0, levels, kw):
+    """The FP64 form of the refined levels: a tolerance far below FP32's rounding
+    is reached on every level, and f_R there agrees with the oracle's sweeps."""
+    import oracle
+    N0, box = 16, 50.0
+    pos = synth.poisson_particles(synth.lognormal_delta(N0, box, sig, 90), box, 2.0, 91)
+    s = mgfr.Solver(0, fr0_abs=fr0, max_level=levels, tol_rel=1e-12, max_vcycles=300, **kw)
+    out = s.solve_particles(torch.from_numpy(pos).to(dev), N0, box)
+    st = out["stats"]
+    nlev = st["n_levels"]
+    assert nlev >= 2 and max(st["level_res"][1:nlev]) <= 1e-12
+    A = oracle.AMR(pos, N0, box, levels, 8)
+    A.deposit()
+    A.set_model(fr0, n=kw.get("n", 1))
+    rc, _ = A.solve(tol=1e-12, max_vcycles=400, prolong_linear=bool(kw.get("prolong_linear", 1)))
+    assert rc == 0
+    for l in range(nlev):
+        fr = s.level_field(l, mgfr.FIELD_FR)
+        ref, _ = A.level_force(l, bool(kw.get("prolong_linear", 1)))
+        if l > 0:
+            perm = np.argsort(s.level_keys(l), kind="stable")
+            fr = fr[(8 * perm[:, None] + np.arange(8)[None, :]).ravel()]
+        # both at 1e-12 of ||f||; 1e3 for the operator's inverse
+        assert np.abs(fr / ref - 1.0).max() <= 1e-9, l
+    s.close()
