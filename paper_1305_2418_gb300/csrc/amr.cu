@@ -93,8 +93,8 @@ __global__ void k_count(const double* __restrict__ pos, long long Np, double inv
   const P3 t = particle_t(pos, p, inv, N0);
   int lev;
   const int sh = QB - l;  // X >> (52 - l) = floor(t 2^l)
-  const long long c =
-      find_cell(T, l, qfix(t.x) >> sh, qfix(t.y) >> sh, qfix(t.z) >> sh, &lev);
+  const unsigned c = find_cell(T, l, (unsigned)(qfix(t.x) >> sh), (unsigned)(qfix(t.y) >> sh),
+                               (unsigned)(qfix(t.z) >> sh), &lev);
   if (lev == l) atomicAdd(count + c, 1);
 }
 
@@ -103,13 +103,13 @@ __global__ void k_flag(const int* __restrict__ count, long long ncell, int thr, 
                        unsigned char* __restrict__ refined) {
   const long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (c >= ncell || count[c] <= thr) return;
-  long long I, J, K;
-  cell_coords(T, l, c, &I, &J, &K);
+  unsigned I, J, K;
+  cell_coords(T, l, (unsigned)c, &I, &J, &K);
   for (int a = -1; a <= 1; ++a)
     for (int b = -1; b <= 1; ++b)
       for (int d = -1; d <= 1; ++d) {
         int lev;
-        const long long nb = find_cell(T, l, I + a, J + b, K + d, &lev);
+        const unsigned nb = find_cell(T, l, I + a, J + b, K + d, &lev);
         if (lev == l) refined[nb] = 1;
       }
 }
@@ -224,8 +224,8 @@ __global__ void k_make_octs(const int* __restrict__ son, long long ncell, int l,
   if (c >= ncell) return;
   const int o = son[c];
   if (o < 0) return;
-  long long I, J, K;
-  cell_coords(T, l, c, &I, &J, &K);
+  unsigned I, J, K;
+  cell_coords(T, l, (unsigned)c, &I, &J, &K);
   pcell[o] = (int)c;
   opos[o] = make_int4((int)I, (int)J, (int)K, 0);
 }
@@ -238,7 +238,7 @@ __global__ void k_oct_nbrs(long long n_oct, int l, TreeView T, int* __restrict__
   const int dd[6][3] = {{-1, 0, 0}, {1, 0, 0}, {0, -1, 0}, {0, 1, 0}, {0, 0, -1}, {0, 0, 1}};
   for (int d = 0; d < 6; ++d) {
     int lev;
-    const long long q = find_cell(T, l - 1, p.x + dd[d][0], p.y + dd[d][1], p.z + dd[d][2], &lev);
+    const unsigned q = find_cell(T, l - 1, p.x + dd[d][0], p.y + dd[d][1], p.z + dd[d][2], &lev);
     nbr[6 * o + d] = lev == l - 1 ? T.son[l - 1][q] : -1;
   }
 }
@@ -406,81 +406,124 @@ __device__ bool visit_particle(const TreeView& T, const P3& t, LevelPtrs& D, con
   const bool rec = !GATHER && D.rec_idx;
   bool split = false;
   const long long X[3] = {qfix(t.x), qfix(t.y), qfix(t.z)};
-  // leaf level lam of the particle and the oct holding its leaf cell
-  int lam = 0, own = -1;
-  long long c = ((((X[0] >> QB) << T.lg0) + (X[1] >> QB)) << T.lg0) + (X[2] >> QB);
-  for (int m = 1; m < T.nlev; ++m) {
-    const int o = T.son[m - 1][c];
-    if (o < 0) break;
-    const int sh = QB - m;
-    c = 8LL * o + (((X[0] >> sh) & 1) << 2) + (((X[1] >> sh) & 1) << 1) + ((X[2] >> sh) & 1);
-    lam = m;
-    own = o;
+  // floor(t 2^8): its upper bits are the cell at every level
+  constexpr int LM = AMR_MAXL - 1;
+  unsigned xi[3];
+#pragma unroll
+  for (int a = 0; a < 3; ++a) xi[a] = (unsigned)(X[a] >> (QB - LM));
+  // leaf level lam of the particle
+  int lam = 0;
+  {
+    unsigned c = ((((xi[0] >> LM) << T.lg0) + (xi[1] >> LM)) << T.lg0) + (xi[2] >> LM);
+    for (int m = 1; m < T.nlev; ++m) {
+      const int o = T.son[m - 1][c];
+      if (o < 0) break;
+      const int sh = LM - m;
+      c = 8u * (unsigned)o + (((xi[0] >> sh) & 1) << 2) + (((xi[1] >> sh) & 1) << 1) +
+          ((xi[2] >> sh) & 1);
+      lam = m;
+    }
   }
-  // the cube: side one level-lam cell, centred on the particle: [cl, cl + 2^F)
+  // the cube: side one level-lam cell, centred on the particle: [cl, cl + 2^F),
+  // per axis 2^F - fr of it in cell i0 and fr in i0 + 1
   const int F = QB - lam;
   const long long one = 1LL << F;
-  long long cl[3], i0[3], edge[3];
+  const unsigned M = (1u << (T.lg0 + lam)) - 1u;
+  long long cl[3], fr[3];
+  unsigned kc[3][2];  // level-lam coordinates of the two cells, wrapped
   W Lw[3][2];
   // fixed-point volume -> fraction of the cube
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
     cl[a] = X[a] - (one >> 1);
-    i0[a] = cl[a] >> F;
-    edge[a] = (i0[a] + 1) * one;  // boundary between the two cells the cube spans
+    fr[a] = cl[a] & (one - 1);
+    const unsigned i0 = (unsigned)(cl[a] >> F);
+    kc[a][0] = i0 & M;
+    kc[a][1] = (i0 + 1u) & M;
     // the fraction of the cube (scale) enters through axis 0
-    Lw[a][0] = a == 0 ? Wt<W>::len_scaled(edge[a] - cl[a], F) : Wt<W>::len(edge[a] - cl[a], F);
-    Lw[a][1] = a == 0 ? Wt<W>::len_scaled(cl[a] + one - edge[a], F)
-                      : Wt<W>::len(cl[a] + one - edge[a], F);
+    Lw[a][0] = a == 0 ? Wt<W>::len_scaled(one - fr[a], F) : Wt<W>::len(one - fr[a], F);
+    Lw[a][1] = a == 0 ? Wt<W>::len_scaled(fr[a], F) : Wt<W>::len(fr[a], F);
   }
   // x-y products of the corner weights, shared by the two z pieces
   W Lxy[4];
 #pragma unroll
   for (int b = 0; b < 4; ++b) Lxy[b] = Lw[0][b >> 1] * Lw[1][b & 1];
-  StackEnt st[48];
-  int sp = 0;
-  for (int q = 0; q < 8; ++q) {
-    const int bits[3] = {(q >> 2) & 1, (q >> 1) & 1, q & 1};
-    if ((bits[0] && edge[0] == cl[0] + one) || (bits[1] && edge[1] == cl[1] + one) ||
-        (bits[2] && edge[2] == cl[2] + one)) {
-      if (rec) ri[q] = kRecSkip;
-      continue;  // zero-width piece
-    }
-    const long long K[3] = {i0[0] + bits[0], i0[1] + bits[1], i0[2] + bits[2]};
-    int lev;
-    long long cq;
-    if (lam > 0 && (K[0] >> 1) == (X[0] >> (F + 1)) && (K[1] >> 1) == (X[1] >> (F + 1)) &&
-        (K[2] >> 1) == (X[2] >> (F + 1))) {
-      // same oct as the particle's leaf cell
-      cq = 8LL * own + ((K[0] & 1) << 2) + ((K[1] & 1) << 1) + (K[2] & 1);
-      lev = lam;
-    } else {
-      cq = find_cell(T, lam, K[0], K[1], K[2], &lev);
-    }
-    const bool refined = lev == lam && lam + 1 < T.nlev && T.son[lam][cq] >= 0;
-    if (!refined) {
-      if (MODE != kVisitSplit) {
-        const W w = Lxy[(bits[0] << 1) | bits[1]] * Lw[2][bits[2]];
-        touch<GATHER, W>(lev, cq, w, D, G, out);
-        if (rec) ri[q] = ((unsigned)lev << D.rb) | (unsigned)cq;
-      }
-      continue;
-    }
-    split = true;
-    if (rec) ri[q] = kRecSkip;
-    if (MODE == kVisitUnsplit) continue;
-    long long lo[3], hi[3];
+  // The cells of the eight corners, level by level: the eight look-ups of a level
+  // do not depend on each other and are in flight together (corner by corner the
+  // walk waited 5000 clocks for one chain of loads after the other).
+  unsigned cc[8];
+  unsigned on = 0xffu;      // corners whose path still goes down
+  unsigned levs = 0u;       // their levels, four bits each
 #pragma unroll
-    for (int a = 0; a < 3; ++a) {
-      lo[a] = bits[a] ? edge[a] : cl[a];
-      hi[a] = bits[a] ? cl[a] + one : edge[a];
+  for (int q = 0; q < 8; ++q)
+    cc[q] = (((kc[0][q >> 2] >> lam) << T.lg0) + (kc[1][(q >> 1) & 1] >> lam) << T.lg0) +
+            (kc[2][q & 1] >> lam);
+  for (int m = 1; m <= lam; ++m) {
+    const int sh = lam - m;
+    int o[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) o[q] = (on >> q) & 1 ? T.son[m - 1][cc[q]] : -1;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      if (o[q] >= 0) {
+        cc[q] = 8u * (unsigned)o[q] + (((kc[0][q >> 2] >> sh) & 1) << 2) +
+                (((kc[1][(q >> 1) & 1] >> sh) & 1) << 1) + ((kc[2][q & 1] >> sh) & 1);
+        levs += 1u << (4 * q);
+      } else {
+        on &= ~(1u << q);
+      }
     }
-    split_q<GATHER, W, 2>(T, lam, cq, lo, hi, F, D, G, out, st, sp, err);
   }
-  // pieces refined three or more levels below the particle's leaf
-  while (sp > 0) {
-    const StackEnt e = st[--sp];
-    split_q<GATHER, W, 1>(T, e.l, e.c, e.lo, e.hi, F, D, G, out, st, sp, err);
+  unsigned refined = 0u;    // corners whose cell is refined again
+  if (lam + 1 < T.nlev) {
+#pragma unroll
+    for (int q = 0; q < 8; ++q)
+      if ((on >> q) & 1 && T.son[lam][cc[q]] >= 0) refined |= 1u << q;
+  }
+  // corners of zero width
+  const unsigned empty = (fr[0] == 0 ? 0xf0u : 0u) | (fr[1] == 0 ? 0xccu : 0u) |
+                         (fr[2] == 0 ? 0xaau : 0u);
+  split = (refined & ~empty) != 0u;
+  if constexpr (MODE == kVisitUnsplit) {
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      const bool keep = !((empty | refined) >> q & 1u);
+      const int lev = (int)(levs >> (4 * q) & 15u);
+      if (keep) touch<GATHER, W>(lev, cc[q], Lxy[q >> 1] * Lw[2][q & 1], D, G, out);
+      if (rec) ri[q] = keep ? ((unsigned)lev << D.rb) | cc[q] : kRecSkip;
+    }
+  } else {
+    StackEnt st[48];
+    int sp = 0;
+    for (int q = 0; q < 8; ++q) {
+      if ((empty >> q) & 1u) {
+        if (rec) ri[q] = kRecSkip;
+        continue;
+      }
+      const int lev = (int)(levs >> (4 * q) & 15u);
+      if (!((refined >> q) & 1u)) {
+        if (MODE != kVisitSplit) {
+          touch<GATHER, W>(lev, cc[q], Lxy[q >> 1] * Lw[2][q & 1], D, G, out);
+          if (rec) ri[q] = ((unsigned)lev << D.rb) | cc[q];
+        }
+        continue;
+      }
+      if (rec) ri[q] = kRecSkip;
+      long long lo[3], hi[3];
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+        const bool up = (q >> (2 - a)) & 1;
+        const long long edge = cl[a] - fr[a] + one;  // between the two cells
+        lo[a] = up ? edge : cl[a];
+        hi[a] = up ? cl[a] + one : edge;
+      }
+      split_q<GATHER, W, 2>(T, lam, cc[q], lo, hi, F, D, G, out, st, sp, err);
+    }
+    // pieces refined three or more levels below the particle's leaf
+    while (sp > 0) {
+      const StackEnt e = st[--sp];
+      split_q<GATHER, W, 1>(T, e.l, e.c, e.lo, e.hi, F, D, G, out, st, sp, err);
+    }
   }
   if (rec && split) ri[0] = kRecSplit;
   return split;
@@ -728,8 +771,8 @@ __global__ void k_eff_pm(int l, int lpm, TreeView T, const double* __restrict__ 
   }
   if (l <= lpm) {
     if (!leaf) return;
-    long long I, J, K;
-    cell_coords(T, l, c, &I, &J, &K);
+    unsigned I, J, K;
+    cell_coords(T, l, (unsigned)c, &I, &J, &K);
     const long long Npm = 1LL << (T.lg0 + lpm);
     const long long s = 1LL << (lpm - l);
     for (long long a = 0; a < s; ++a)
@@ -839,7 +882,7 @@ __global__ void k_oct_pnbrs(long long n_oct, int l, TreeView T, int* __restrict_
   const int dd[6][3] = {{-1, 0, 0}, {1, 0, 0}, {0, -1, 0}, {0, 1, 0}, {0, 0, -1}, {0, 0, 1}};
   for (int d = 0; d < 6; ++d) {
     int lev;
-    const long long q = find_cell(T, l - 1, p.x + dd[d][0], p.y + dd[d][1], p.z + dd[d][2], &lev);
+    const unsigned q = find_cell(T, l - 1, p.x + dd[d][0], p.y + dd[d][1], p.z + dd[d][2], &lev);
     pnbr[6 * o + d] = lev == l - 1 ? (int)q : -1;
   }
 }

@@ -56,15 +56,17 @@ struct TreeView {
 };
 
 // ---- tree lookups ----------------------------------------------------------
+// 32-bit throughout: coordinates stay below 2^10 2^8, and a level's cells below
+// 2^32 (its 6 n_oct faces fit 31 bits, checked where the level is built).
 // Cell at level l with level-l coordinates (I,J,K) (wrapped).  Returns the
 // cell index at the deepest level m <= l that exists on the path, m in *lev.
-static __device__ __forceinline__ long long find_cell(const TreeView& T, int l, long long I, long long J,
-                                               long long K, int* lev) {
-  const long long Nl = 1LL << (T.lg0 + l);
-  I &= Nl - 1;
-  J &= Nl - 1;
-  K &= Nl - 1;
-  long long c = (((I >> l) << T.lg0) + (J >> l) << T.lg0) + (K >> l);
+static __device__ __forceinline__ unsigned find_cell(const TreeView& T, int l, unsigned I,
+                                                     unsigned J, unsigned K, int* lev) {
+  const unsigned M = (1u << (T.lg0 + l)) - 1u;
+  I &= M;
+  J &= M;
+  K &= M;
+  unsigned c = (((I >> l) << T.lg0) + (J >> l) << T.lg0) + (K >> l);
   for (int m = 1; m <= l; ++m) {
     const int o = T.son[m - 1][c];
     if (o < 0) {
@@ -72,26 +74,26 @@ static __device__ __forceinline__ long long find_cell(const TreeView& T, int l, 
       return c;
     }
     const int sh = l - m;
-    c = 8LL * o + (((I >> sh) & 1) << 2) + (((J >> sh) & 1) << 1) + ((K >> sh) & 1);
+    c = 8u * (unsigned)o + (((I >> sh) & 1) << 2) + (((J >> sh) & 1) << 1) + ((K >> sh) & 1);
   }
   *lev = l;
   return c;
 }
 
-static __device__ __forceinline__ void cell_coords(const TreeView& T, int l, long long c, long long* I,
-                                            long long* J, long long* K) {
+static __device__ __forceinline__ void cell_coords(const TreeView& T, int l, unsigned c, unsigned* I,
+                                            unsigned* J, unsigned* K) {
   if (l == 0) {
-    const long long M = (1LL << T.lg0) - 1;
+    const unsigned M = (1u << T.lg0) - 1;
     *K = c & M;
     *J = (c >> T.lg0) & M;
     *I = c >> (2 * T.lg0);
     return;
   }
   const int4 p = T.opos[l][c >> 3];
-  const int ch = (int)(c & 7);
-  *I = 2LL * p.x + ((ch >> 2) & 1);
-  *J = 2LL * p.y + ((ch >> 1) & 1);
-  *K = 2LL * p.z + (ch & 1);
+  const unsigned ch = c & 7;
+  *I = 2u * p.x + ((ch >> 2) & 1);
+  *J = 2u * p.y + ((ch >> 1) & 1);
+  *K = 2u * p.z + (ch & 1);
 }
 
 

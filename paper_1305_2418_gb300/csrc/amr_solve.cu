@@ -1484,40 +1484,61 @@ __global__ void k_d2df(const double* __restrict__ x, dfl* __restrict__ y, long l
 
 // ---- set-up kernels --------------------------------------------------------
 // initial guess of level L from the converged level L-1 (linear
-// reconstruction with the parent's neighbours), FP64 and FP32 copies
-__global__ void k_init_level(long long ncell, const int* __restrict__ pcell,
-                             const int* __restrict__ pnbr, const double* __restrict__ up,
-                             int linear, double* __restrict__ w, double* __restrict__ wE,
-                             float* __restrict__ w32, long long no) {
-  const long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (c >= ncell) return;
-  const long long o = c >> 3;
-  const int ch = (int)(c & 7);
-  if (w32) {
-    // mixed form: an FP32 guess (the FP64 iterate is taken from w32 later),
-    // with the parent values converted on the integer pipes
-    float v = f_from_double_bits(up[pcell[o]]);
-    if (linear) {
-      for (int ax = 0; ax < 3; ++ax) {
-        const int pm = pnbr[6 * o + 2 * ax], pp = pnbr[6 * o + 2 * ax + 1];
-        if (pm < 0 || pp < 0) continue;
-        v = fmaf(((ch >> (2 - ax)) & 1) ? 0.125f : -0.125f,
-                 f_from_double_bits(up[pp]) - f_from_double_bits(up[pm]), v);
-      }
+// reconstruction with the parent's neighbours), one thread per oct: FP64 (w, wE),
+// or in the mixed form FP32 only (w32; the FP64 iterate is taken from it later)
+// with the parent values converted on the integer pipes
+__global__ void __launch_bounds__(BS) k_init_level(const int* __restrict__ pcell,
+                                                   const int* __restrict__ pnbr,
+                                                   const double* __restrict__ up, int linear,
+                                                   double* __restrict__ w, double* __restrict__ wE,
+                                                   float* __restrict__ w32, long long no) {
+  const long long o = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  if (o >= no) return;
+  int pm[3] = {-1, -1, -1}, pp[3] = {-1, -1, -1};
+  if (linear) {
+    const int2* nb = reinterpret_cast<const int2*>(pnbr) + 3 * o;
+#pragma unroll
+    for (int ax = 0; ax < 3; ++ax) {
+      const int2 q = __ldg(nb + ax);
+      pm[ax] = q.x;
+      pp[ax] = q.y;
     }
-    w32[pidx(c, no)] = v;
+  }
+  if (w32) {
+    const float v0 = f_from_double_bits(up[pcell[o]]);
+    float g[3] = {0.f, 0.f, 0.f};
+    bool have[3];
+#pragma unroll
+    for (int ax = 0; ax < 3; ++ax) {
+      have[ax] = pm[ax] >= 0 && pp[ax] >= 0;
+      if (have[ax]) g[ax] = f_from_double_bits(up[pp[ax]]) - f_from_double_bits(up[pm[ax]]);
+    }
+    Oct8 V;
+#pragma unroll
+    for (int ch = 0; ch < 8; ++ch) {
+      float v = v0;
+#pragma unroll
+      for (int ax = 0; ax < 3; ++ax)
+        if (have[ax]) v = fmaf(((ch >> (2 - ax)) & 1) ? 0.125f : -0.125f, g[ax], v);
+      V.v[ch] = v;
+    }
+    st8(w32, o, no, V);
     return;
   }
-  double v = up[pcell[o]];
-  if (linear) {
-    for (int ax = 0; ax < 3; ++ax) {
-      const int pm = pnbr[6 * o + 2 * ax], pp = pnbr[6 * o + 2 * ax + 1];
-      if (pm < 0 || pp < 0) continue;
-      v += (((ch >> (2 - ax)) & 1) ? 0.125 : -0.125) * (up[pp] - up[pm]);
-    }
+  const double v0 = up[pcell[o]];
+  double g[3] = {0.0, 0.0, 0.0};
+#pragma unroll
+  for (int ax = 0; ax < 3; ++ax)
+    if (pm[ax] >= 0 && pp[ax] >= 0) g[ax] = up[pp[ax]] - up[pm[ax]];
+#pragma unroll
+  for (int ch = 0; ch < 8; ++ch) {
+    double v = v0;
+#pragma unroll
+    for (int ax = 0; ax < 3; ++ax)
+      if (pm[ax] >= 0 && pp[ax] >= 0) v += (((ch >> (2 - ax)) & 1) ? 0.125 : -0.125) * g[ax];
+    w[8 * o + ch] = v;
+    wE[8 * o + ch] = lean_exp(v);
   }
-  w[c] = v;
-  wE[c] = exp(v);
 }
 
 // Start of level L from the previous particle solve where its octs persist
@@ -1557,16 +1578,17 @@ __global__ void k_warm_level(const int4* __restrict__ opos, long long n_oct,
 // (Sec. 3.3), one thread per ghost value: slot s = t / 4 (its face 6 o + d
 // from gface), qi = t % 4 the face cell.  The face's four outside cells are
 // daughters of one level-(l-1) cell P, the oct's parent shifted along the face
-// normal; the four threads of a face look up P and its six neighbours (the
-// same addresses).  A ghost is P's value plus, per axis, s (c+ - c-)/8,
+// normal; the four threads of a face share the look-ups of P and its six
+// neighbours.  A ghost is P's value plus, per axis, s (c+ - c-)/8,
 // s = +1 or -1 for the ghost's high or low daughter position in P (a
 // component is 0 where one of P's neighbours does not exist).  Written as
 // (u, e^u) in FP64 (double-float pairs in the mixed form) and FP32 u.
 __global__ void k_ghosts(long long n_gslot, int l, TreeView T, const unsigned* __restrict__ gface,
                          const double* __restrict__ up, int linear, double* __restrict__ ghost,
                          double* __restrict__ ghostE, float* __restrict__ g32, int dfmode) {
-  const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (t >= 4 * n_gslot) return;
+  const long long t0 = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  const bool live = t0 < 4 * n_gslot;  // the others repeat the last face (shuffles)
+  const long long t = live ? t0 : 4 * n_gslot - 4 + (t0 & 3);
   const unsigned f = gface[t >> 2];
   const int qi = (int)(t & 3);
   const unsigned o = f / 6u;
@@ -1574,25 +1596,34 @@ __global__ void k_ghosts(long long n_gslot, int l, TreeView T, const unsigned* _
   const int ax = d >> 1, plus = d & 1;
   const int t1 = ax == 0 ? 1 : 0;  // the first tangential axis
   const int4 p = T.opos[l][o];
-  const long long P0 = p.x + (ax == 0 ? (plus ? 1 : -1) : 0);
-  const long long P1 = p.y + (ax == 1 ? (plus ? 1 : -1) : 0);
-  const long long P2 = p.z + (ax == 2 ? (plus ? 1 : -1) : 0);
-  int lev;
-  const long long pc = find_cell(T, l - 1, P0, P1, P2, &lev);
-  // per axis, the indices of P's two neighbours (-1: no gradient)
-  long long cm[3] = {-1, -1, -1}, cp[3] = {-1, -1, -1};
-  if (lev == l - 1 && linear) {
+  const unsigned P0 = p.x + (ax == 0 ? (plus ? 1 : -1) : 0);
+  const unsigned P1 = p.y + (ax == 1 ? (plus ? 1 : -1) : 0);
+  const unsigned P2 = p.z + (ax == 2 ? (plus ? 1 : -1) : 0);
+  // P and its neighbours (+x, -x, +y, -y, +z, -z) as look-ups 0..6: lane qi of the
+  // face's four does qi and qi + 4, the others get them by shuffle (-1: not there)
+  int own[2] = {-1, -1};
 #pragma unroll
-    for (int a = 0; a < 3; ++a) {
-      int lp, lm;
-      const long long qp = find_cell(T, l - 1, P0 + (a == 0), P1 + (a == 1), P2 + (a == 2), &lp);
-      const long long qm = find_cell(T, l - 1, P0 - (a == 0), P1 - (a == 1), P2 - (a == 2), &lm);
-      if (lp == l - 1 && lm == l - 1) {
-        cp[a] = qp;
-        cm[a] = qm;
-      }
-    }
+  for (int h = 0; h < 2; ++h) {
+    const int j = qi + 4 * h;
+    if (j > 6 || (j > 0 && !linear)) continue;
+    const int a = (j - 1) >> 1, s = j & 1 ? 1 : -1;
+    int lev;
+    const unsigned q = find_cell(T, l - 1, P0 + (j > 0 && a == 0 ? s : 0),
+                                 P1 + (j > 0 && a == 1 ? s : 0), P2 + (j > 0 && a == 2 ? s : 0),
+                                 &lev);
+    if (lev == l - 1) own[h] = (int)q;
   }
+  const int pc = __shfl_sync(0xffffffffu, own[0], 0, 4);
+  // per axis, the indices of P's two neighbours (-1: no gradient)
+  int cm[3], cp[3];
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    const int jp = 2 * a + 1, jm = 2 * a + 2;
+    cp[a] = __shfl_sync(0xffffffffu, own[jp >> 2], jp & 3, 4);
+    cm[a] = __shfl_sync(0xffffffffu, own[jm >> 2], jm & 3, 4);
+    if (cp[a] < 0 || cm[a] < 0 || pc < 0) cp[a] = cm[a] = -1;
+  }
+  if (!live) return;
   // daughter bit of the ghost along axis a inside P: along the normal the
   // side facing the oct, tangentially the oct cell's own bits (qi's two bits)
   auto hbit = [&](int a) { return a == ax ? 1 - plus : a == t1 ? (qi >> 1) & 1 : qi & 1; };
@@ -1601,7 +1632,7 @@ __global__ void k_ghosts(long long n_gslot, int l, TreeView T, const unsigned* _
     // values converted on the integer pipes, the stencil and e^v on the FP32
     // pipes
     dfl V{0.f, 0.f};
-    if (lev == l - 1) V = df_from_double_bits(up[pc]);
+    if (pc >= 0) V = df_from_double_bits(up[pc]);
 #pragma unroll
     for (int a = 0; a < 3; ++a)
       if (cp[a] >= 0) {
@@ -1615,7 +1646,7 @@ __global__ void k_ghosts(long long n_gslot, int l, TreeView T, const unsigned* _
     g32[t] = V.hi;
     return;
   }
-  double v = lev == l - 1 ? up[pc] : 0.0;
+  double v = pc >= 0 ? up[pc] : 0.0;
 #pragma unroll
   for (int a = 0; a < 3; ++a)
     if (cp[a] >= 0) v += (hbit(a) ? 0.125 : -0.125) * (up[cp[a]] - up[cm[a]]);
@@ -2250,9 +2281,8 @@ mgfr_status amr_solve_level(mgfr_ctx* c, AmrWork* A, int Lv, const Model& m, mgf
                                                           g.prolong_linear, F.ghost, F.ghostE,
                                                           F.ghost32, mixed ? 1 : 0);
   c->launches += 1;
-  k_init_level<<<nblocks(F.ncell, BS), BS, 0, c->s>>>(F.ncell, F.pcell, F.pnbr, up,
-                                                      g.prolong_linear, F.w, F.wE,
-                                                      mixed ? F.w32 : nullptr, F.n_oct);
+  k_init_level<<<nblocks(F.n_oct, BS), BS, 0, c->s>>>(F.pcell, F.pnbr, up, g.prolong_linear, F.w,
+                                                      F.wE, mixed ? F.w32 : nullptr, F.n_oct);
   if (g.start == MGFR_START_PREVIOUS_ALL && Lv < A->prev_nlev && A->prev_N0 == A->N0 &&
       A->prev_box == A->box && A->prev_noct[Lv] > 0 && F.n_oct > 0) {
     k_warm_level<<<nblocks(F.n_oct, BS), BS, 0, c->s>>>(F.opos, F.n_oct, A->prev_key[Lv],
