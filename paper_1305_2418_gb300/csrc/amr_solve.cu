@@ -773,8 +773,16 @@ __device__ __forceinline__ int face_q(int ch, int ax) {
 //   LIN = true : Gauss-Seidel on J(u) e = r  (u fixed; e updated)
 //   LIN = false: Newton-Gauss-Seidel on L(u) = f (u updated)
 // no: octs of the level (plane stride); n, olist: the octs visited.
+//
+// Bound by the latency of two dependent loads (the neighbour table, then six
+// scattered vectors).  With all face loads issued before any arithmetic and 64
+// registers a linear half-sweep of the solved level of 16.8 M particles takes 61-63 us
+// (40 registers, the faces loaded one after the other, 24 resident warps more: 70-71), a
+// nonlinear one 42-44 (47-48); blocks of 64 leave the smallest gap when a block's
+// slowest warp ends (256: 44 and 66).
+constexpr int SWB = 64;
 template <bool LIN, int COL>
-__global__ void __launch_bounds__(BS, 6) k_oct_sweep32(
+__global__ void __launch_bounds__(SWB, 16) k_oct_sweep32(
     float* __restrict__ u, float* __restrict__ e, const float* __restrict__ rf,
     const int* __restrict__ nbr, const float* __restrict__ gh,
     const unsigned char* __restrict__ act, long long n, const int* __restrict__ olist,
@@ -789,6 +797,25 @@ __global__ void __launch_bounds__(BS, 6) k_oct_sweep32(
   const float4* __restrict__ uo = u4 + OC * no;  // the other colour's plane
   const float4* __restrict__ e4 = reinterpret_cast<const float4*>(e);
   const float4* __restrict__ g4 = reinterpret_cast<const float4*>(gh);
+  // the six face neighbours as three 8-byte loads (6 o ints: 8-byte aligned)
+  const int2* nb2 = reinterpret_cast<const int2*>(nbr) + 3 * o;
+  const int2 n01 = __ldg(nb2), n23 = __ldg(nb2 + 1), n45 = __ldg(nb2 + 2);
+  const int nbv[6] = {n01.x, n01.y, n23.x, n23.y, n45.x, n45.y};
+  // what lies across the faces: the neighbouring oct's other colour, or the ghost face
+  float4 NUv[6], NXv[6];
+#pragma unroll
+  for (int d = 0; d < 6; ++d) {
+    const int nb = nbv[d];
+    NXv[d] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (!LIN) {
+      NUv[d] = nb >= 0 ? uo[nb] : g4[-nb - 1];  // one load, no divergent branch
+    } else if (nb >= 0) {
+      NUv[d] = uo[nb];
+      NXv[d] = e4[OC * no + nb];
+    } else {
+      NUv[d] = g4[-nb - 1];
+    }
+  }
   const float4 a0 = u4[o], a1 = u4[no + o];
   Oct8 U;
   U.v[0] = a0.x; U.v[3] = a0.y; U.v[5] = a0.z; U.v[6] = a0.w;
@@ -800,14 +827,10 @@ __global__ void __launch_bounds__(BS, 6) k_oct_sweep32(
   // LIN: corrections of the other colour (the in-oct neighbours)
   const float4 XO = LIN ? e4[OC * no + o] : make_float4(0.f, 0.f, 0.f, 0.f);
   bool on[4];
-  float s1[4], s2[4], s3[4];  // LIN: (sum off*e, diag sum, -); NL: (sum b du, sum du, sum b)
+  float s1[4], s2[4], s3[4];  // LIN: (sum off*e, diag sum, -); NL: (sum 2 b du, sum du, sum 2 b)
   // the oct's eight relax flags in one 8-byte load
   const unsigned long long a8 = act ? __ldg(reinterpret_cast<const unsigned long long*>(act) + o)
                                     : ~0ULL;
-  // the six face neighbours as three 8-byte loads (6 o ints: 8-byte aligned)
-  const int2* nb2 = reinterpret_cast<const int2*>(nbr) + 3 * o;
-  const int2 n01 = __ldg(nb2), n23 = __ldg(nb2 + 1), n45 = __ldg(nb2 + 2);
-  const int nbv[6] = {n01.x, n01.y, n23.x, n23.y, n45.x, n45.y};
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
     const int ch = CC[COL][q];
@@ -823,28 +846,19 @@ __global__ void __launch_bounds__(BS, 6) k_oct_sweep32(
                      s1[q]);
         s2[q] += fmaf(EE.v[ch], du, -EE.v[ch] - EE.v[cn]);
       } else {
-        const float b = 0.5f * (EE.v[cn] + EE.v[ch]);
+        const float b = EE.v[cn] + EE.v[ch];
         s1[q] = fmaf(b, du, s1[q]);
         s2[q] += du;
         s3[q] += b;
       }
     }
   }
-  // faces: the neighbouring oct's other colour, or the ghost face
+  // across the faces
 #pragma unroll
   for (int d = 0; d < 6; ++d) {
     const int a = d >> 1, plus = d & 1;
-    const int nb = nbv[d];
-    const bool has = nb >= 0;
-    float4 NU, NX = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (!LIN) {
-      NU = has ? uo[nb] : g4[-nb - 1];  // one load, no divergent branch
-    } else if (has) {
-      NU = uo[nb];
-      NX = e4[OC * no + nb];
-    } else {
-      NU = g4[-nb - 1];
-    }
+    const bool has = nbv[d] >= 0;
+    const float4 NU = NUv[d], NX = NXv[d];
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
       const int ch = CC[COL][q];
@@ -858,7 +872,7 @@ __global__ void __launch_bounds__(BS, 6) k_oct_sweep32(
         s1[q] = fmaf(0.5f * ih2 * fmaf(En, du, EE.v[ch] + En), xn, s1[q]);
         s2[q] += fmaf(EE.v[ch], du, -EE.v[ch] - En);
       } else {
-        const float b = 0.5f * (En + EE.v[ch]);
+        const float b = En + EE.v[ch];
         s1[q] = fmaf(b, du, s1[q]);
         s2[q] += du;
         s3[q] += b;
@@ -879,8 +893,8 @@ __global__ void __launch_bounds__(BS, 6) k_oct_sweep32(
       const float diag = s2[q] * 0.5f * ih2 + m.aRt_np1 * sN;
       res[q] = __fdividef(f4(R4, q) - s1[q], diag);
     } else {
-      const float L = s1[q] * ih2 + m.aRt * (1.f - sN);
-      const float dL = (0.5f * EE.v[ch] * s2[q] - s3[q]) * ih2 + m.aRt_np1 * sN;
+      const float L = s1[q] * (0.5f * ih2) + m.aRt * (1.f - sN);
+      const float dL = (EE.v[ch] * s2[q] - s3[q]) * (0.5f * ih2) + m.aRt_np1 * sN;
       float step = __fdividef(L - f4(R4, q), dL);
       step = fminf(fmaxf(step, -cap), cap);
       res[q] = U.v[ch] - step;
@@ -991,7 +1005,7 @@ __device__ __forceinline__ void block_partials3(double ss, double mx, double fs,
 
 // FP32 residual norms of the solved level (sum r^2, max |r|, sum f^2), one
 // thread per oct; the oct's eight terms are summed in FP32, the octs in FP64.
-__global__ void __launch_bounds__(BS) k_onorm32(const float* __restrict__ u,
+__global__ void __launch_bounds__(BS, 4) k_onorm32(const float* __restrict__ u,
                                                 const float* __restrict__ f,
                                                 const int* __restrict__ nbr,
                                                 const float* __restrict__ gh, long long n_oct,
@@ -1048,7 +1062,7 @@ __global__ void __launch_bounds__(BS) k_ofas32(const float* __restrict__ u, floa
 // FAS restriction of one oct to its parent (FP32): u average, average of the
 // residual f - L(u) over the oct's relaxed cells.  pno: octs of the parent
 // level (0: dense).
-__global__ void __launch_bounds__(BS) k_orestrict32(
+__global__ void __launch_bounds__(BS, 4) k_orestrict32(
     const float* __restrict__ u, const float* __restrict__ f, const int* __restrict__ nbr,
     const float* __restrict__ gh, const unsigned char* __restrict__ act, long long n,
     const int* __restrict__ olist, long long no, const int* __restrict__ pcell, long long pno,
@@ -1079,7 +1093,7 @@ __global__ void __launch_bounds__(BS) k_orestrict32(
 
 // Linear-phase restriction of one oct: r_c = R(r - J e) over relaxed cells,
 // u_c = R(u), e_c = 0.
-__global__ void __launch_bounds__(BS) k_olin_restrict32(
+__global__ void __launch_bounds__(BS, 4) k_olin_restrict32(
     const float* __restrict__ e, const float* __restrict__ r, const float* __restrict__ u,
     const int* __restrict__ nbr, const float* __restrict__ gh,
     const unsigned char* __restrict__ act, long long n, const int* __restrict__ olist,
@@ -1851,11 +1865,11 @@ void relax(SolveCtx& S, int l, int sweeps) {
         if constexpr (std::is_same<T, float>::value) {
           const unsigned char* mk = l == S.L ? nullptr : L.act;
           if (col == 0)
-            k_oct_sweep32<false, 0><<<nblocks(R.n, BS), BS, 0, c->s>>>(
+            k_oct_sweep32<false, 0><<<nblocks(R.n, SWB), SWB, 0, c->s>>>(
                 L.w32, nullptr, L.wf32, L.nbr, L.ghost32, mk, R.n, R.list, L.n_oct, m,
                 (float)L.ih2, (float)g.step_cap);
           else
-            k_oct_sweep32<false, 1><<<nblocks(R.n, BS), BS, 0, c->s>>>(
+            k_oct_sweep32<false, 1><<<nblocks(R.n, SWB), SWB, 0, c->s>>>(
                 L.w32, nullptr, L.wf32, L.nbr, L.ghost32, mk, R.n, R.list, L.n_oct, m,
                 (float)L.ih2, (float)g.step_cap);
         } else {
@@ -2085,7 +2099,7 @@ void corr_relax(SolveCtx& S, int l, int sweeps) {
               (float)L.ih2);
         } else {
           (col == 0 ? k_oct_sweep32<true, 0> : k_oct_sweep32<true, 1>)
-              <<<nblocks(R.n, BS), BS, 0, c->s>>>(L.w32, L.wold32, L.wf32, L.nbr, L.ghost32, mk,
+              <<<nblocks(R.n, SWB), SWB, 0, c->s>>>(L.w32, L.wold32, L.wf32, L.nbr, L.ghost32, mk,
                                                   R.n, R.list, L.n_oct, m, (float)L.ih2, 0.f);
         }
         if (l == S.L) prof_end(c);
