@@ -303,6 +303,12 @@ __host__ __device__ __forceinline__ dfl df_rsqrt(dfl a) {
 #endif
   const dfl y2 = df_two_prod(y, y);
   const dfl ay2 = df_mul(a, y2);
-  const dfl d = df_add_f(df_neg(ay2), 1.f);  // 1 - a y^2, small
-  return df_two_sum(y, DF_MUL(DF_MUL(0.5f, y), d.hi));
+  const float d = DF_SUB(DF_SUB(1.f, ay2.hi), ay2.lo);  // 1 - a y^2: the first exact
+  return df_two_sum(y, DF_MUL(DF_MUL(0.5f, y), d));
+}
+
+// (Ea + Eb)(ua - ub), twice the flux through the face between two cells; exchanging a
+// and b changes its sign and nothing else
+__host__ __device__ __forceinline__ dfl df_face(dfl Ea, dfl Eb, dfl ua, dfl ub) {
+  return df_mul(df_add_abs(Ea, Eb), df_add_abs(ua, df_neg(ub)));
 }
