@@ -86,11 +86,13 @@ __device__ __forceinline__ void block_partial(double ss, float mx, double* __res
   }
 }
 
-// residual norm of the nonlinear FP32 iterate; a thread sums the squares of
+// residual norm of the FP32 iterate x (MG_DEV: of the deviation x from w); a thread sums the squares of
 // four cells in FP32, the vectors are summed in FP64 (an FP64 addition per
 // cell made this the slowest kernel of the cycle: 860 us on 512^3)
+template <int OP>
 __global__ void __launch_bounds__(BS) k_vnorm(const float* __restrict__ x,
-                                              const float* __restrict__ f, int lg, PF m, float ih2,
+                                              const float* __restrict__ f,
+                                              const float* __restrict__ w, int lg, PF m, float ih2,
                                               double* __restrict__ partials) {
   const unsigned half = 1u << (3 * lg - 1), nv = 1u << (3 * lg - 2);
   const int M = (1 << lg) - 1;
@@ -103,12 +105,19 @@ __global__ void __launch_bounds__(BS) k_vnorm(const float* __restrict__ x,
     const Rows R = rows_at(i, j, kh0, p, lg);
     const Nb4 xn = load_nb(x + (1 - colour) * half, R, p);
     const V4 xv = ld4(x + colour * half + R.c), fv = ld4(f + colour * half + R.c);
+    V4 wv{};
+    Nb4 wn{};
+    if (OP == MG_DEV) {
+      wn = load_nb(w + (1 - colour) * half, R, p);
+      wv = ld4(w + colour * half + R.c);
+    }
     float s4 = 0.f;
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-      float a[6];
+      float a[6], b[6];
       xn.get(q, a);
-      const float r = fv.v[q] - point_apply<MG_NL>(xv.v[q], a, 0.f, a, m, ih2);
+      wn.get(q, b);
+      const float r = fv.v[q] - point_apply<OP>(xv.v[q], a, wv.v[q], b, m, ih2);
       s4 = fmaf(r, r, s4);
       mx = fmaxf(mx, fabsf(r));
     }
@@ -552,11 +561,11 @@ long long mg32_cycle(Mg32Op op, const Mg32Level* L, int nlev, const Mg32Par& p, 
   }
 }
 
-void mg32_norm(const Mg32Level& L, const Mg32Par& p, double* partials, int nparts, double* out,
-               cudaStream_t s) {
+void mg32_norm(Mg32Op op, const Mg32Level& L, const Mg32Par& p, double* partials, int nparts,
+               double* out, cudaStream_t s) {
   const long long nv = 1LL << (3 * L.lg - 2);
   const int nb = (int)std::min<long long>(nparts, nblocks(nv, BS));
-  k_vnorm<<<nb, BS, 0, s>>>(L.x, L.r, L.lg, PF{p.aRt, p.aRt_np1, p.inv_np1, p.cap}, L.ih2,
-                            partials);
+  (op == MG_DEV ? k_vnorm<MG_DEV> : k_vnorm<MG_NL>)<<<nb, BS, 0, s>>>(
+      L.x, L.r, L.w, L.lg, PF{p.aRt, p.aRt_np1, p.inv_np1, p.cap}, L.ih2, partials);
   k_finish2<<<1, 256, 0, s>>>(partials, nb, out);
 }

@@ -37,9 +37,9 @@ struct Mg32Hook {      // called around every half-sweep of the finest level
 // half-sweep pairs' cell updates (the 4^3 grid not counted).
 long long mg32_cycle(Mg32Op op, const Mg32Level* L, int nlev, const Mg32Par& p, cudaStream_t s,
                      const Mg32Hook* hook = nullptr);
-// Residual norm of the nonlinear operator (sum r^2, max |r|) into out[0..1]
+// Norm of the residual of op's equation, MG_NL or MG_DEV (sum, max |.|), into out[0..1]
 // (device), per-block partial sums in `partials` (2 nparts doubles).
-void mg32_norm(const Mg32Level& L, const Mg32Par& p, double* partials, int nparts, double* out,
+void mg32_norm(Mg32Op op, const Mg32Level& L, const Mg32Par& p, double* partials, int nparts, double* out,
                cudaStream_t s);
 // raise the cluster kernels' launch limits once per device (before a capture)
 mgfr_status mg32_prepare(mgfr_ctx* c);

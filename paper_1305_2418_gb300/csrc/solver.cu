@@ -395,12 +395,26 @@ static long long cycle32(mgfr_ctx* c, Mg32Op op, const Model& m, int fam, int n_
   return upd;
 }
 
-static void norm32(mgfr_ctx* c, const Model& m) {
+static void norm32(mgfr_ctx* c, Mg32Op op, const Model& m) {
   DenseHier& H = c->dh;
   const DenseLevel& D = H.L[0];
-  const Mg32Level L{D.lg, (float)D.ih2, (float)(D.h * D.h), D.u32, D.f32, nullptr};
-  mg32_norm(L, mg32_par(m, c->cfg, MG_NL), H.partials, H.nparts, H.scal, c->s);
+  const bool dev = op == MG_DEV;
+  const Mg32Level L{D.lg, (float)D.ih2, (float)(D.h * D.h), dev ? D.e32 : D.u32,
+                    dev ? D.r32 : D.f32, dev ? D.u32 : nullptr};
+  mg32_norm(op, L, mg32_par(m, c->cfg, op), H.partials, H.nparts, H.scal, c->s);
 }
+
+// FP64 form.  FP64 arithmetic is 2 FMA per SM and clock: the FP64 update of u and e^u and
+// the residual take 190 of a cycle's 430 us on 128^3.  Two FP32 cycles that certainly both
+// stay above the target share them: the first one's norm is formed from the deviation in
+// FP32 (15 us), and the second goes on from the same deviation.  They are the same
+// cycles but for the FP32 rounding of the first correction where the second one's is
+// added to it; that rounding's residual, on grid-scale waves 12 2^-24 (N / 2 pi)^2 of the
+// first one's, stays below 1.5e-3 up to kPairMax, against the 1e-2 that two cycles leave,
+// and the cycle that follows takes it out.  128^3: 3.43 -> 3.00 ms, 256^3 18.1 -> 14.1;
+// below kPairMin the norm and its read-back cost what they save (32^3 0.61 -> 0.65 ms, 64^3
+// 1.04 -> 1.06).
+constexpr int kPairMin = 128, kPairMax = 256;
 
 // FP64 base-level solve on the already-filled hierarchy (f on level 0, u/E
 // initialised).  Fills stats (vcycles, updates, norms).
@@ -425,12 +439,15 @@ mgfr_status dense_solve64(mgfr_ctx* c, const Model& m, double box, mgfr_stats* s
   // deviation from the iterate, which FP32 resolves to its own relative
   // accuracy (the iterate, e^u, the residual and the test stay in FP64)
   make_key(key, sizeof(key), "dev", H.N, box, m, g);
-  auto bodydev = [&]() {
-    cudaMemsetAsync(L0.e32, 0, sizeof(float) * (size_t)L0.n, c->s);
-    updates_per = cycle32(c, MG_DEV, m, 0);
+  const bool pairs = H.N >= kPairMin && H.N <= kPairMax;
+  auto fp64_dev = [&]() {
     f64::apply_dev(L0, 1.f, c->s);
     f64::resid_dev(L0, m, H.partials, H.nparts, H.scal, c->s);
-    cudaMemcpyAsync(hs, H.scal, 2 * sizeof(double), cudaMemcpyDeviceToHost, c->s);
+  };
+  auto bodydev = [&]() {
+    if (!pairs) cudaMemsetAsync(L0.e32, 0, sizeof(float) * (size_t)L0.n, c->s);
+    updates_per = cycle32(c, MG_DEV, m, 0);
+    if (!pairs) fp64_dev();
   };
   if (!c->g_dev || std::strcmp(key, c->keydev) != 0) {
     if (c->g_dev) cudaGraphExecDestroy(c->g_dev);
@@ -453,41 +470,75 @@ mgfr_status dense_solve64(mgfr_ctx* c, const Model& m, double box, mgfr_stats* s
   };
   const double ref = fn > 0.0 ? fn : r0;
   bool dev_ok = true;
-  double r = r0;
+  double r = r0, rho = 0.0;  // rho: reduction of the last cycle
   int it = 0;
   long long updates = 0;
+  auto cycle_dev = [&](bool fresh, bool fp64) -> mgfr_status {
+    if (pairs && fresh) cudaMemsetAsync(L0.e32, 0, sizeof(float) * (size_t)L0.n, c->s);
+    const mgfr_status is = issue(c, 4, c->g_dev, bodydev);
+    if (is != MGFR_OK) return is;
+    if (pairs) {
+      if (fp64)
+        fp64_dev();
+      else
+        norm32(c, MG_DEV, m);
+      c->launches += fp64 ? 3 : 2;
+    }
+    updates += c->updates_dev;
+    MG_CK(c, cudaMemcpyAsync(hs, H.scal, 2 * sizeof(double), cudaMemcpyDeviceToHost, c->s));
+    const mgfr_status ss = sync_read(c);
+    prof_collect(c, 4, st);
+    return ss;
+  };
   while (r > target && it < g.max_vcycles) {
     const bool dev = dev_ok && r <= kDevMax * ref;
-    if (!dev) {
-      make_key(key, sizeof(key), "v64", H.N, box, m, g);
-      if (!c->g_v64 || std::strcmp(key, c->graph_key) != 0) {
-        if (c->g_v64) cudaGraphExecDestroy(c->g_v64);
-        c->g_v64 = nullptr;
-        if ((rs = capture(c, 0, &c->g_v64, body64)) != MGFR_OK) return rs;
-        std::strcpy(c->graph_key, key);
-        c->updates_v64 = updates_per;
+    if (dev) {
+      int n = 1;
+      // expected above the target after two cycles, from the last one's reduction
+      const bool pair = pairs && it + 3 <= g.max_vcycles &&
+                        r * (rho > 0.0 ? rho * rho : 1e-3) > 2.0 * target;
+      if ((rs = cycle_dev(true, !pair)) != MGFR_OK) return rs;
+      if (pair) {
+        const double r1 = std::sqrt(hs[0]);
+        if (r1 < r && r1 * (r1 / r) > 2.0 * target) {
+          n = 2;
+          if ((rs = cycle_dev(false, true)) != MGFR_OK) return rs;
+        } else {
+          fp64_dev();
+          c->launches += 3;
+          MG_CK(c, cudaMemcpyAsync(hs, H.scal, 2 * sizeof(double), cudaMemcpyDeviceToHost, c->s));
+          if ((rs = sync_read(c)) != MGFR_OK) return rs;
+        }
       }
-      rs = issue(c, 0, c->g_v64, body64);
-    } else {
-      rs = issue(c, 4, c->g_dev, bodydev);
-    }
-    if (rs != MGFR_OK) return rs;
-    rs = sync_read(c);
-    if (rs != MGFR_OK) return rs;
-    prof_collect(c, dev ? 4 : 0, st);
-    const double rn = std::sqrt(hs[0]);
-    updates += dev ? c->updates_dev : c->updates_v64;
-    if (dev && !(rn < r)) {
-      f64::apply_dev(L0, -1.f, c->s);
-      c->launches += 1;
-      dev_ok = false;
+      const double rn = std::sqrt(hs[0]);
+      if (!(rn < r)) {
+        f64::apply_dev(L0, -1.f, c->s);
+        c->launches += 1;
+        dev_ok = false;
+        continue;
+      }
+      it += n;
+      rho = n == 2 ? std::sqrt(rn / r) : rn / r;
+      r = rn;
       continue;
     }
+    make_key(key, sizeof(key), "v64", H.N, box, m, g);
+    if (!c->g_v64 || std::strcmp(key, c->graph_key) != 0) {
+      if (c->g_v64) cudaGraphExecDestroy(c->g_v64);
+      c->g_v64 = nullptr;
+      if ((rs = capture(c, 0, &c->g_v64, body64)) != MGFR_OK) return rs;
+      std::strcpy(c->graph_key, key);
+      c->updates_v64 = updates_per;
+    }
+    if ((rs = issue(c, 0, c->g_v64, body64)) != MGFR_OK) return rs;
+    if ((rs = sync_read(c)) != MGFR_OK) return rs;
+    prof_collect(c, 0, st);
+    r = std::sqrt(hs[0]);
+    updates += c->updates_v64;
     ++it;
-    r = rn;
     if (!std::isfinite(r)) break;
     // the deviation cycle starts from u32 and r32 of this iterate
-    if (!dev && dev_ok && r <= kDevMax * ref) {
+    if (dev_ok && r <= kDevMax * ref) {
       f64::resid_dev(L0, m, H.partials, H.nparts, H.scal, c->s);
       c->launches += 2;
     }
@@ -523,7 +574,7 @@ mgfr_status dense_solve_mixed(mgfr_ctx* c, const Model& m, double box, mgfr_stat
   f64::norm(L0.f, L0.n, H.partials, H.nparts, H.scal + 2, c->s);
   f32::from64(L0.f, L0.f32, L0, c->s);
   f32::from64(L0.u, L0.u32, L0, c->s);
-  norm32(c, m);
+  norm32(c, MG_NL, m);
   c->launches += 6;
   MG_CK(c, cudaMemcpyAsync(hs, H.scal, 4 * sizeof(double), cudaMemcpyDeviceToHost, c->s));
   mgfr_status rs = sync_read(c);
@@ -542,7 +593,7 @@ mgfr_status dense_solve_mixed(mgfr_ctx* c, const Model& m, double box, mgfr_stat
   long long upd = 0;
   auto body32 = [&]() {
     upd = cycle32(c, MG_NL, m, 0);
-    norm32(c, m);
+    norm32(c, MG_NL, m);
     cudaMemcpyAsync(hs, H.scal, 2 * sizeof(double), cudaMemcpyDeviceToHost, c->s);
   };
   if (!c->g_v32 || std::strcmp(key, c->key32) != 0) {
