@@ -753,47 +753,64 @@ __global__ void k_eff_level(const double* __restrict__ mass, const double* __res
 // contrast as a density (plain stores: leaves do not overlap); a leaf at
 // l > lpm lies in one PM cell and adds its contrast 8^-(l-lpm) (atomics).
 // The contrast is delta_eff (what 0), delta (what 1) or delta + delta_eff
-// (what 2, the right-hand side of Eq. (30)).  FP64 pipe bound; the eight
-// daughters of an oct beyond lpm fall into one PM cell, so their lanes add up
-// first and the oct costs one atomic instead of eight (78 M cells of a 256^3
-// base with two levels took 4.1 ms with an FP64 exponential and an atomic per
-// leaf).
+// (what 2, the right-hand side of Eq. (30)).  FP64 pipe bound, 9 instructions of it per
+// leaf: levels above lpm below, levels beyond it per oct.
+__device__ __forceinline__ double eff_leaf(double mass, double u, double E, const EffPar& q,
+                                           int what) {
+  const double d = fma(mass, q.scale, -1.0);
+  if (what == 1) return d;
+  const double eff = eff_density(d, u, E, q);
+  return what == 2 ? eff + d : eff;
+}
+
 __global__ void k_eff_pm(int l, int lpm, TreeView T, const double* __restrict__ mass,
                          const double* __restrict__ u, const double* __restrict__ E, long long n,
                          EffPar q, int what, double* __restrict__ out) {
   const long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  const bool leaf = c < n && T.son[l][c] < 0;
-  double eff = 0.0;
-  if (leaf) {
-    const double d = fma(mass[c], q.scale, -1.0);
-    eff = what == 1 ? d : eff_density(d, q.n == 1 ? 0.0 : u[c], q.n == 1 ? E[c] : 1.0, q);
-    if (what == 2) eff += d;
+  if (c >= n || T.son[l][c] >= 0) return;
+  const double eff = eff_leaf(mass[c], q.n == 1 ? 0.0 : u[c], q.n == 1 ? E[c] : 1.0, q, what);
+  unsigned I, J, K;
+  cell_coords(T, l, (unsigned)c, &I, &J, &K);
+  const long long Npm = 1LL << (T.lg0 + lpm);
+  const long long s = 1LL << (lpm - l);
+  for (long long a = 0; a < s; ++a)
+    for (long long b = 0; b < s; ++b)
+      for (long long e = 0; e < s; ++e)
+        out[((I * s + a) * Npm + (J * s + b)) * Npm + (K * s + e)] = eff;
+}
+
+// The eight daughters of an oct beyond lpm fall into one PM cell: one thread per oct adds
+// its leaves and makes one atomic.  Every FP64 instruction of a warp then serves 32
+// cells (one cell per thread summed the octs by shuffles, three FP64 additions and a
+// division per cell for all lanes: 1.73 ms on 42.9 M cells, here 0.88).
+__global__ void __launch_bounds__(128) k_eff_pm_oct(int l, int lpm, TreeView T,
+                                                    const double* __restrict__ mass,
+                                                    const double* __restrict__ u,
+                                                    const double* __restrict__ E, long long n_oct,
+                                                    EffPar q, int what, double* __restrict__ out) {
+  const long long o = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  if (o >= n_oct) return;
+  const int4* sp = reinterpret_cast<const int4*>(T.son[l]) + 2 * o;
+  const int4 sa = sp[0], sb = sp[1];
+  const int son[8] = {sa.x, sa.y, sa.z, sa.w, sb.x, sb.y, sb.z, sb.w};
+  if ((sa.x | sa.y | sa.z | sa.w | sb.x | sb.y | sb.z | sb.w) >= 0) return;  // no leaf
+  const double2* mp = reinterpret_cast<const double2*>(mass) + 4 * o;
+  const double2* xp = reinterpret_cast<const double2*>(q.n == 1 ? E : u) + 4 * o;
+  double e[8];
+#pragma unroll
+  for (int p = 0; p < 4; ++p) {
+    const double2 m2 = mp[p], x2 = xp[p];
+    const double ea = eff_leaf(m2.x, x2.x, x2.x, q, what), eb = eff_leaf(m2.y, x2.y, x2.y, q, what);
+    e[2 * p] = son[2 * p] < 0 ? ea : 0.0;
+    e[2 * p + 1] = son[2 * p + 1] < 0 ? eb : 0.0;
   }
-  if (l <= lpm) {
-    if (!leaf) return;
-    unsigned I, J, K;
-    cell_coords(T, l, (unsigned)c, &I, &J, &K);
-    const long long Npm = 1LL << (T.lg0 + lpm);
-    const long long s = 1LL << (lpm - l);
-    for (long long a = 0; a < s; ++a)
-      for (long long b = 0; b < s; ++b)
-        for (long long e = 0; e < s; ++e)
-          out[((I * s + a) * Npm + (J * s + b)) * Npm + (K * s + e)] = eff;
-    return;
-  }
-  // whole warps reach here (l >= 1: cells come in octs of 8 lanes)
-  unsigned any = __ballot_sync(0xffffffffu, leaf);
-  any = (any >> (threadIdx.x & 24)) & 0xffu;
-  if (any == 0u) return;
-  const unsigned oct = 0xffu << (threadIdx.x & 24);
-  for (int o = 4; o > 0; o >>= 1) eff += __shfl_xor_sync(oct, eff, o);
-  if (threadIdx.x & 7) return;
-  const int4 p = T.opos[l][c >> 3];  // the parent at level l - 1 >= lpm
+  const double sum = ((e[0] + e[4]) + (e[2] + e[6])) + ((e[1] + e[5]) + (e[3] + e[7]));
+  const int4 p = T.opos[l][o];  // the parent at level l - 1 >= lpm
   const int sh = l - lpm;
   const long long Npm = 1LL << (T.lg0 + lpm);
   atomicAdd(out + ((long long)(p.x >> (sh - 1)) * Npm + (p.y >> (sh - 1))) * Npm +
                 (p.z >> (sh - 1)),
-            eff / (double)(1LL << (3 * sh)));
+            sum * dfrombits((unsigned long long)(1023 - 3 * sh) << 52));  // 8^-sh
 }
 
 __global__ void k_nan_check(const double* __restrict__ x, long long n,
@@ -1565,8 +1582,12 @@ mgfr_status amr_density_pm(mgfr_ctx* c, int lpm, int what, double* out_dev, int*
     AmrLevel& L = A->L[l];
     const double* u = l == 0 ? c->dh.L[0].u : L.u;
     const double* E = l == 0 ? c->dh.L[0].E : L.E;
-    k_eff_pm<<<nblocks(L.ncell, BS), BS, 0, c->s>>>(l, lpm, T, L.mass, u, E, L.ncell,
-                                                    eff_par(A, l), what, out_dev);
+    if (l <= lpm)
+      k_eff_pm<<<nblocks(L.ncell, BS), BS, 0, c->s>>>(l, lpm, T, L.mass, u, E, L.ncell,
+                                                      eff_par(A, l), what, out_dev);
+    else
+      k_eff_pm_oct<<<nblocks(L.n_oct, 128), 128, 0, c->s>>>(l, lpm, T, L.mass, u, E, L.n_oct,
+                                                            eff_par(A, l), what, out_dev);
     c->launches += 1;
   }
   return MGFR_OK;
