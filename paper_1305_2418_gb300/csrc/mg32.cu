@@ -565,7 +565,7 @@ void mg32_norm(Mg32Op op, const Mg32Level& L, const Mg32Par& p, double* partials
                double* out, cudaStream_t s) {
   const long long nv = 1LL << (3 * L.lg - 2);
   const int nb = (int)std::min<long long>(nparts, nblocks(nv, BS));
-  (op == MG_DEV ? k_vnorm<MG_DEV> : k_vnorm<MG_NL>)<<<nb, BS, 0, s>>>(
+  (op == MG_DEV ? k_vnorm<MG_DEV> : op == MG_POI ? k_vnorm<MG_POI> : k_vnorm<MG_NL>)<<<nb, BS, 0, s>>>(
       L.x, L.r, L.w, L.lg, PF{p.aRt, p.aRt_np1, p.inv_np1, p.cap}, L.ih2, partials);
   k_finish2<<<1, 256, 0, s>>>(partials, nb, out);
 }

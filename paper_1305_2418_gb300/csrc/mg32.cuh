@@ -33,11 +33,32 @@ struct Mg32Hook {      // called around every half-sweep of the finest level
   void* arg = nullptr;
 };
 
+// Pairs of cycles.  What follows a cycle at the accuracy of the iterate costs a good part of
+// it (FP64 form: the update of u and e^u and the residual, 190 of 430 us on 128^3, FP64
+// arithmetic being 2 FMA per SM and clock; Poisson: 130 of 400 on 256^3).  Two FP32 cycles
+// that certainly both stay above the target share it: the first one's norm is formed from
+// the correction in FP32, and the second goes on from the same correction.  They are the
+// same cycles but for the FP32 rounding of the first correction where the second one's is
+// added to it; that rounding's residual, on grid-scale waves 12 2^-24 (N / 2 pi)^2 of the
+// first one's, stays below 1.5e-3 up to kPairMax, against the 1e-2 that two cycles leave,
+// and the cycle that follows takes it out.  FP64 form: 128^3 3.43 -> 3.00 ms, 256^3 18.1 ->
+// 14.1; below kPairMin the norm and its read-back cost what they save (32^3 0.61 -> 0.65
+// ms, 64^3 1.04 -> 1.06).
+constexpr int kPairMin = 128, kPairMax = 256;
+// whether to try a pair at residual norm r, rho the last cycle's reduction (0: none yet),
+// and whether to go on after its first cycle left r1: both above the target
+inline bool pair_start(double r, double rho, double target) {
+  return r * (rho > 0.0 ? rho * rho : 1e-3) > 2.0 * target;
+}
+inline bool pair_on(double r, double r1, double target) {
+  return r1 < r && r1 * (r1 / r) > 2.0 * target;
+}
+
 // One V-cycle over levels L[0] (finest) .. L[nlev - 1] (4^3); returns the
 // half-sweep pairs' cell updates (the 4^3 grid not counted).
 long long mg32_cycle(Mg32Op op, const Mg32Level* L, int nlev, const Mg32Par& p, cudaStream_t s,
                      const Mg32Hook* hook = nullptr);
-// Norm of the residual of op's equation, MG_NL or MG_DEV (sum, max |.|), into out[0..1]
+// Norm of the residual of op's equation (not MG_LIN; sum of squares, max |.|), into out[0..1]
 // (device), per-block partial sums in `partials` (2 nparts doubles).
 void mg32_norm(Mg32Op op, const Mg32Level& L, const Mg32Par& p, double* partials, int nparts, double* out,
                cudaStream_t s);

@@ -316,7 +316,7 @@ mgfr_status pm_alloc(mgfr_ctx* c, PmWork* P, int lg, double box) {
       MG_CK(c, cudaMalloc(&P->r[l], sizeof(float) * nl));
     }
     P->nparts = 152 * 8;
-    MG_CK(c, cudaMalloc(&P->part, sizeof(double) * P->nparts));
+    MG_CK(c, cudaMalloc(&P->part, sizeof(double) * (2 * P->nparts + 2)));
     MG_CK(c, cudaMallocHost(&P->part_h, sizeof(double) * P->nparts));
     P->lg = lg;
   }
@@ -392,18 +392,36 @@ static mgfr_status pm_solve(mgfr_ctx* c, int lpm, int what, double* phi_out_dev,
   par.linear = 1;
   par.coarse_sweeps = 60;
   const double fn = std::sqrt(sq), target = g.tol_rel * fn;
-  double r = fn;
+  double r = fn, rho = 0.0;  // rho: reduction of the last cycle
   int it = 0;
   long long updates = 0;
-  while (r > target && it < g.max_vcycles) {
-    MG_CK(c, cudaMemsetAsync(P->e[0], 0, sizeof(float) * (size_t)P->n, c->s));
+  const bool pairs = (1 << lg) >= kPairMin && (1 << lg) <= kPairMax;
+  auto cycle = [&]() {
     updates += mg32_cycle(MG_POI, L, P->nlev, par, c->s) + 60 * 64;
     c->launches += 10 * std::max(0, lg - 5) + 1;
+  };
+  while (r > target && it < g.max_vcycles) {
+    MG_CK(c, cudaMemsetAsync(P->e[0], 0, sizeof(float) * (size_t)P->n, c->s));
+    const double rp = r;
+    int n = 1;
+    cycle();
+    if (pairs && it + 3 <= g.max_vcycles && pair_start(r, rho, target)) {
+      mg32_norm(MG_POI, L[0], par, P->part, P->nparts, P->part + 2 * P->nparts, c->s);
+      c->launches += 2;
+      MG_CK(c, cudaMemcpyAsync(P->part_h, P->part + 2 * P->nparts, sizeof(double),
+                               cudaMemcpyDeviceToHost, c->s));
+      MG_CK(c, cudaStreamSynchronize(c->s));
+      if (pair_on(r, std::sqrt(P->part_h[0]), target)) {
+        cycle();
+        n = 2;
+      }
+    }
     k_pm_update<<<nb8, BS, 0, c->s>>>(P->phi, P->e[0], P->r[0], P->rlo, lg, df_from_double(ih2),
                                       P->part);
     if ((rs = pm_total(c, P, nb8, &sq)) != MGFR_OK) return rs;
     r = std::sqrt(sq);
-    ++it;
+    it += n;
+    rho = n == 2 ? std::sqrt(r / rp) : r / rp;
     if (!std::isfinite(r)) break;
     if (r <= target) {
       // the residual carried along says converged: the FP64 one decides

@@ -404,18 +404,6 @@ static void norm32(mgfr_ctx* c, Mg32Op op, const Model& m) {
   mg32_norm(op, L, mg32_par(m, c->cfg, op), H.partials, H.nparts, H.scal, c->s);
 }
 
-// FP64 form.  FP64 arithmetic is 2 FMA per SM and clock: the FP64 update of u and e^u and
-// the residual take 190 of a cycle's 430 us on 128^3.  Two FP32 cycles that certainly both
-// stay above the target share them: the first one's norm is formed from the deviation in
-// FP32 (15 us), and the second goes on from the same deviation.  They are the same
-// cycles but for the FP32 rounding of the first correction where the second one's is
-// added to it; that rounding's residual, on grid-scale waves 12 2^-24 (N / 2 pi)^2 of the
-// first one's, stays below 1.5e-3 up to kPairMax, against the 1e-2 that two cycles leave,
-// and the cycle that follows takes it out.  128^3: 3.43 -> 3.00 ms, 256^3 18.1 -> 14.1;
-// below kPairMin the norm and its read-back cost what they save (32^3 0.61 -> 0.65 ms, 64^3
-// 1.04 -> 1.06).
-constexpr int kPairMin = 128, kPairMax = 256;
-
 // FP64 base-level solve on the already-filled hierarchy (f on level 0, u/E
 // initialised).  Fills stats (vcycles, updates, norms).
 mgfr_status dense_solve64(mgfr_ctx* c, const Model& m, double box, mgfr_stats* st) {
@@ -494,13 +482,11 @@ mgfr_status dense_solve64(mgfr_ctx* c, const Model& m, double box, mgfr_stats* s
     const bool dev = dev_ok && r <= kDevMax * ref;
     if (dev) {
       int n = 1;
-      // expected above the target after two cycles, from the last one's reduction
-      const bool pair = pairs && it + 3 <= g.max_vcycles &&
-                        r * (rho > 0.0 ? rho * rho : 1e-3) > 2.0 * target;
+      const bool pair = pairs && it + 3 <= g.max_vcycles && pair_start(r, rho, target);
       if ((rs = cycle_dev(true, !pair)) != MGFR_OK) return rs;
       if (pair) {
         const double r1 = std::sqrt(hs[0]);
-        if (r1 < r && r1 * (r1 / r) > 2.0 * target) {
+        if (pair_on(r, r1, target)) {
           n = 2;
           if ((rs = cycle_dev(false, true)) != MGFR_OK) return rs;
         } else {

@@ -49,3 +49,35 @@ def test_same_cycles_as_single_ones(dev, tol, sig, fr0, kw):
         else:
             assert out["status"] == mgfr.MGFR_E_NOCONVERGE
         s.close()
+
+
+@pytest.mark.parametrize("tol", [1e-6, 1e-8, 1e-10])
+def test_poisson_pairs(dev, tol):
+    """The particle-mesh potential on 128^3 (csrc/pm.cu): the cycles needed are the
+    smallest limit that suffices, and the forces are those of a solve to 1e-12 within the
+    tolerance (||r|| <= tol ||rhs||; 10 for the force of smooth modes over their source)."""
+    N0, box = 64, 100.0
+    pos = synth.poisson_particles(synth.lognormal_delta(32, box, 1.5, 411), box, 8.0, 412)
+    p = torch.from_numpy(np.ascontiguousarray(pos)).to(dev)
+
+    def accel(tol, most, fails=False):
+        s = mgfr.Solver(0, fr0_abs=1e-5, max_level=1, tol_rel=1e-3, max_vcycles=50)
+        s.solve_particles(p, N0, box)
+        s.set_config(tol_rel=tol, max_vcycles=most)
+        try:
+            if fails:
+                with pytest.raises(mgfr.MGFRError):
+                    s.pm_accel(p, 1)
+                return None, None
+            return s.pm_accel(p, 1)
+        finally:
+            s.close()
+
+    exact, _ = accel(1e-12, 100)
+    acc, st = accel(tol, 100)
+    again, st2 = accel(tol, st["vcycles"])
+    assert st2["vcycles"] == st["vcycles"]
+    accel(tol, st["vcycles"] - 1, fails=True)
+    scale = float(exact.abs().max())
+    assert float((acc - exact).abs().max()) <= 10 * tol * scale
+    assert float((again - acc).abs().max()) <= 10 * tol * scale
