@@ -188,23 +188,43 @@ __global__ void __launch_bounds__(128) k_wgrad(const __nv_bfloat16* __restrict__
   }
 }
 
-// dW = the sum of the S partials: 32 elements x 8 segments of the partials per
-// block, each segment in order of its stride, then the segments in order
+// dW = the sum of the S partials in order (one chain per element, so that the result does
+// not depend on the launch shape): a block's eight warps fetch 128 partials of 32
+// elements at a time, one warp adds them.  (One thread per element fetching its own
+// chain stood on the latency of S dependent steps: 78 us for 16 -> 16 on 4 x 64^3.)
+// Up to WR_FEW partials, where the elements are many, a thread fetches its own.
+constexpr int WR_Z = 128, WR_FEW = 32;
+__global__ void __launch_bounds__(256) k_wgrad_reduce_few(const float* __restrict__ partials,
+                                                          int S, long long n,
+                                                          float* __restrict__ dW) {
+  const long long i = blockIdx.x * 256LL + threadIdx.x;
+  if (i >= n) return;
+  float s = 0.f;
+#pragma unroll 8
+  for (int z = 0; z < S; ++z) s += partials[(long long)z * n + i];
+  dW[i] = s;
+}
 __global__ void __launch_bounds__(256) k_wgrad_reduce(const float* __restrict__ partials, int S,
                                                       long long n, float* __restrict__ dW) {
-  __shared__ float red[8][32];
+  __shared__ float v[WR_Z][32];
   const int l = threadIdx.x & 31, w = threadIdx.x >> 5;
   const long long i = blockIdx.x * 32LL + l;
   float s = 0.f;
-  if (i < n)
-    for (int z = w; z < S; z += 8) s += partials[(long long)z * n + i];
-  red[w][l] = s;
-  __syncthreads();
-  if (w == 0 && i < n) {
+  for (int z0 = 0; z0 < S; z0 += WR_Z) {
+    const int nz = S - z0 < WR_Z ? S - z0 : WR_Z;
+    if (i < n) {
 #pragma unroll
-    for (int q = 1; q < 8; ++q) s += red[q][l];
-    dW[i] = s;
+      for (int q = 0; q < WR_Z / 8; ++q)
+        if (w + 8 * q < nz) v[w + 8 * q][l] = partials[(long long)(z0 + w + 8 * q) * n + i];
+    }
+    __syncthreads();
+    if (w == 0) {
+#pragma unroll 8
+      for (int z = 0; z < nz; ++z) s += v[z][l];
+    }
+    __syncthreads();
   }
+  if (w == 0 && i < n) dW[i] = s;
 }
 
 // db[c] = sum over voxels of g[m][c].  Each thread sums 8 channels (16-byte
@@ -286,7 +306,10 @@ void nn_conv_dgrad(TView g, int Cout, const __nv_bfloat16* W, FView gx, int Cin,
 void nn_wgrad_finish(float* partials, int S, int Cin, int Cout, float* dW, TView g,
                      float* db, long long Mtot, cudaStream_t s) {
   const long long n = 27LL * Cin * Cout;
-  k_wgrad_reduce<<<nblocks(n, 32), 256, 0, s>>>(partials, S, n, dW);
+  if (S <= WR_FEW)
+    k_wgrad_reduce_few<<<nblocks(n, 256), 256, 0, s>>>(partials, S, n, dW);
+  else
+    k_wgrad_reduce<<<nblocks(n, 32), 256, 0, s>>>(partials, S, n, dW);
   if (!db) return;
   // the bias stages reuse the partials (read by k_wgrad_reduce before them on
   // this stream); they hold S * 27 * Cin * Cout >= 432 * Cout floats (Cin >= 16)

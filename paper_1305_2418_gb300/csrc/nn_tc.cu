@@ -6,7 +6,7 @@
 // input block with its one-voxel halo staged once per CTA, each tap a shifted
 // descriptor into it) and the weight gradient (k_wgrad_tc).
 //
-// Implicit GEMM per CTA (128 threads): rows = an M tile of 128 consecutive
+// Implicit GEMM per CTA: rows = an M tile of 128 consecutive
 // voxels, columns = all N output channels (N <= 256), reduction = 27 taps x
 // the K input channels.  Per tap:
 //   A (128 x K): each row the channel vector of the row voxel's neighbour at
@@ -164,6 +164,15 @@ __device__ __forceinline__ void mma_commit(uint64_t* bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
                    smem_u32(bar))
                : "memory");
+}
+
+// 16 columns of the warp's 32 lanes set to zero
+__device__ __forceinline__ void tmem_zero16(uint32_t taddr) {
+  asm volatile(
+      "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], "
+      "{%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1};" ::"r"(taddr),
+      "r"(0)
+      : "memory");
 }
 
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* v) {
@@ -560,12 +569,26 @@ void launch_wgrad(TView x, TView g, int lgD, long long Mtot, float* part, int* e
 // M = 128 tile per slice (row m = 8 y + z).  It stages the input once as a
 // (TX + 2) x 18 x 10 voxel block with its one-voxel periodic halo, laid out
 // [8-channel group][x][y][z] with 16 bytes per voxel, and all 27 taps'
-// packed weights by one bulk copy.  The A operand of tap (dx, dy, dz) is then
-// a K-major no-swizzle view of the halo block: core matrices of 8 z-
+// packed weights.  The A operand of tap (dy, dz) on an input slice is
+// then a K-major no-swizzle view of the halo block: core matrices of 8 z-
 // consecutive voxels x 16 bytes, 8-row groups (y) 10 x 16 bytes apart (SBO),
 // 8-channel groups one block-plane apart (LBO), the start shifted by the tap
-// offset.  So the block is read from global memory once instead of 27 times,
-// and a tile costs 27 (KC / 16) MMAs on shared-memory operands.
+// offset.
+//
+// An MMA of M = 128, K = 16 takes 39 clocks at N = 16, 44 at 48, 56 at 96 (measured): the
+// A operand's 4 KB set the time.  The three taps dx of an input slice are therefore one
+// MMA: the accumulators of neighbouring output slices lie side by side in TMEM, and B holds
+// the three taps' weights side by side, so that its columns add to the output slices
+// before, at and after the input slice.  (TX + 2) 9 (KC / 16) MMAs instead of
+// TX 27 (KC / 16), each output's terms in the same order.  The accumulators start at
+// zero, since one MMA meets slices at different stages.
+// A CTA stays for many tiles: its weights and tensor memory are set up once, and the next
+// tile's block arrives while the results of this one are stored.
+// 256^3: 16 -> 16 433 us (a CTA per tile, one MMA per tap: 536), 48 -> 16 2023 (2025, now
+// bound by the block's arrival: two CTAs per SM hold one block each); 128^3: 32 -> 32 210
+// (251), 16 -> 32 97 (117); input gradient on 4 x 64^3: 16 -> 48 89 (113), 16 -> 16 40
+// (54).  TX = 8 for 16 channels: 25% more than the tile read against 50% at 4 (356 against
+// 437 us).
 // The halo block of a CTA: 8-channel chunk c8 of voxel (hx, hy, hz) lands at
 // c8 halo_plane + 16 ((hx HY + hy) HZ + hz); consecutive threads take the
 // chunks of a voxel (contiguous in memory; the plane stride's extra 16 bytes
@@ -593,33 +616,44 @@ template <int KC, int NC, bool DGRAD, int TX>
 __global__ void __launch_bounds__(HT) k_conv_halo(
     const __nv_bfloat16* __restrict__ x, int ldx, int offx, const __nv_bfloat16* __restrict__ Wp,
     const float* __restrict__ bias, int relu, __nv_bfloat16* __restrict__ y, int ldy, int offy,
-    float* __restrict__ gx, int ldg, int offg, int accumulate, int lgD, int tmem_cols,
+    float* __restrict__ gx, int ldg, int offg, int accumulate, int lgD, int tiles, int tmem_cols,
     int* __restrict__ err) {
   constexpr int HX = TX + 2, CH = KC / 8;
   constexpr int PLANE = halo_plane(HX);  // bytes of one 8-channel group
   constexpr int H_BYTES = CH * PLANE;
   constexpr int W_BYTES = 27 * NC * KC * 2;
-  constexpr uint32_t SBO = HZ * 16, B_LBO = NC * 16;
-  constexpr uint32_t IDESC = idesc_bf16(TC_M, NC);
+  constexpr uint32_t SBO = HZ * 16, B_LBO = 3 * NC * 16;
   extern __shared__ __align__(1024) unsigned char smem[];
   unsigned char* Hs = smem;
-  unsigned char* Ws = smem + H_BYTES;
-  uint64_t* bars = reinterpret_cast<uint64_t*>(Ws + W_BYTES);  // weights, MMAs
-  uint32_t* tslot = reinterpret_cast<uint32_t*>(bars + 2);
+  unsigned char* Ws = smem + H_BYTES;  // [dy, dz][8-channel group][slot][NC rows]
+  uint64_t* bar = reinterpret_cast<uint64_t*>(Ws + W_BYTES);  // the MMAs
+  uint32_t* tslot = reinterpret_cast<uint32_t*>(bar + 1);
   const int tid = threadIdx.x, warp = warp_index();
-  const int D = 1 << lgD, M = D - 1;
   // tile coordinates: z blocks of 8, y blocks of 16, x blocks of TX, samples
-  const int nz = D >> 3, ny = D >> 4, nx = D / TX;
-  long long bid = blockIdx.x;
-  const int bz = (int)(bid % nz);
-  bid /= nz;
-  const int by = (int)(bid % ny);
-  bid /= ny;
-  const int bx = (int)(bid % nx);
-  const long long b = bid / nx;
-  const int x0 = bx * TX, y0 = by * 16, z0 = bz * 8;
-  const long long sbase = b << (3 * lgD);
-
+  const int lz = lgD - 3, ly = lgD - 4, nx = (1 << lgD) / TX;
+  auto coords = [&](int t, int* x0, int* y0, int* z0) {
+    *z0 = (t & ((1 << lz) - 1)) * 8;
+    t >>= lz;
+    *y0 = (t & ((1 << ly) - 1)) * 16;
+    t >>= ly;
+    const int b = t / nx;
+    *x0 = (t - b * nx) * TX;
+    return b;  // the sample
+  };
+  auto load = [&](int t) {
+    int x0, y0, z0;
+    const int b = coords(t, &x0, &y0, &z0);
+    load_halo<CH, HX>(Hs, x, ldx, offx, (unsigned)b, x0, y0, z0, lgD, tid);
+    cp_async_commit();
+  };
+  // the copies run while the CTA gets its tensor memory
+#pragma unroll 4
+  for (int e = tid; e < 27 * CH * NC; e += HT) {  // 16 bytes: row n of tap t's group c
+    const int n = e % NC, tc = e / NC, t = tc / CH, c = tc - t * CH;
+    const int dx = t / 9, q = DGRAD ? dx : 2 - dx;
+    cp_async16(Ws + ((((t - 9 * dx) * CH + c) * 3 + q) * NC + n) * 16, Wp + 8 * (size_t)e, true);
+  }
+  load((int)blockIdx.x);
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
                      smem_u32(tslot)),
@@ -628,73 +662,80 @@ __global__ void __launch_bounds__(HT) k_conv_halo(
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   if (tid == 0) {
-    mbar_init(bars, 1);
-    mbar_init(bars + 1, 1);
+    mbar_init(bar, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tbase = *tslot;
-  bool ok = true;
-  if (tid == 0) bulk_load(Ws, Wp, (uint32_t)W_BYTES, bars);
-  load_halo<CH, HX>(Hs, x, ldx, offx, (unsigned)b, x0, y0, z0, lgD, tid);
-  cp_async_commit();
-  cp_async_wait<0>();
-  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-  __syncthreads();
-  bool issued = false;
-  if (warp == 0) {
-    if (!mbar_wait(bars, 0, err)) {
-      ok = false;
-    } else {
+  // warp w reads TMEM lanes 32 (w & 3)..; the column chunks alternate between
+  // the two groups of four warps
+  const uint32_t lane_addr = tbase + ((uint32_t)((warp & 3) * 32) << 16);
+#pragma unroll 1
+  for (int q = warp >> 2; q < TX * (NC / 16); q += HT / 128) tmem_zero16(lane_addr + 16 * q);
+  uint32_t parity = 0;
+#pragma unroll 1
+  for (int tile = (int)blockIdx.x; tile < tiles; tile += (int)gridDim.x, parity ^= 1u) {
+    asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+    cp_async_wait<0>();
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    if (warp == 0) {
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       const int sg = DGRAD ? -1 : 1;
       const uint64_t ad0 = sdesc(smem_u32(Hs), PLANE, SBO), bd0 = sdesc(smem_u32(Ws), B_LBO, 128);
       const bool lead = elect_one();
 #pragma unroll 1
-      for (int t = 0; t < 27; ++t) {
-        const int dx = sg * (t / 9 - 1), dy = sg * ((t / 3) % 3 - 1), dz = sg * (t % 3 - 1);
-        const uint64_t at = desc_add(ad0, (uint32_t)((((dx + 1) * HY + (dy + 1)) * HZ + (dz + 1)) * 16));
-        const uint64_t bt = desc_add(bd0, (uint32_t)(t * (NC * KC * 2)));
-        const uint32_t acc = t > 0 ? 1u : 0u;
-        if (lead) {
+      for (int h = 0; h < HX; ++h) {
+        const int hx = DGRAD ? HX - 1 - h : h;  // input slice x0 - 1 + hx: dx ascends per output
+        // its slots in the tile; slot q is the output slice x0 + hx - 2 + q, its tap dx = 1 - q
+        // (input gradient: q - 1)
+        const int q0 = hx < 2 ? 2 - hx : 0, q1 = hx >= TX ? TX + 1 - hx : 2;
+        const uint32_t dcol = tbase + (hx - 2 + q0) * NC;
+        const uint32_t idesc = idesc_bf16(TC_M, (q1 - q0 + 1) * NC);
+        const uint64_t bh = desc_add(bd0, (uint32_t)(q0 * NC * 16));
+#pragma unroll 1
+        for (int t = 0; t < 9; ++t) {
+          const int dy = sg * (t / 3 - 1), dz = sg * (t % 3 - 1);
+          const uint64_t at = desc_add(ad0, (uint32_t)(((hx * HY + (dy + 1)) * HZ + (dz + 1)) * 16));
+          const uint64_t bt = desc_add(bh, (uint32_t)(t * (3 * NC * KC * 2)));
+          if (lead) {
 #pragma unroll
-          for (int kk = 0; kk < KC / 16; ++kk)
-#pragma unroll
-            for (int tx = 0; tx < TX; ++tx)  // consecutive MMAs into different accumulators
-              mma_bf16(tbase + tx * NC, desc_add(at, tx * (HY * HZ * 16) + 2 * kk * PLANE),
-                       desc_add(bt, 2 * kk * B_LBO), IDESC, kk > 0 ? 1u : acc);
+            for (int kk = 0; kk < KC / 16; ++kk)
+              mma_bf16(dcol, desc_add(at, 2 * kk * PLANE), desc_add(bt, 2 * kk * B_LBO), idesc, 1u);
+          }
+          __syncwarp();
         }
-        __syncwarp();
       }
-      if (lead) mma_commit(bars + 1);
-      issued = true;
+      if (lead) mma_commit(bar);
     }
-  }
-  ok = __syncthreads_and(ok);
-  if (ok && tid == 0 && !mbar_wait(bars + 1, 0, err)) ok = false;
-  ok = __syncthreads_and(ok);
-  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  if (ok) {
-    // warp w reads TMEM lanes 32 (w & 3)..; the column chunks alternate between
-    // the two groups of four warps
+    const bool ok = __syncthreads_and(tid != 0 || mbar_wait(bar, parity, err));
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    if (!ok) {  // the wait ran out: the MMAs in flight (bounded)
+      if (tid == 0) mbar_wait(bar, parity, err);
+      break;
+    }
+    // the next tile's block arrives while this one's results are stored
+    if (tile + (int)gridDim.x < tiles) load(tile + (int)gridDim.x);
+    int x0, y0, z0;
+    const long long b = coords(tile, &x0, &y0, &z0);
     const int row = (warp & 3) * 32 + (tid & 31);
-    const int yy = row >> 3, zz = row & 7;
-    const uint32_t lane_addr = tbase + ((uint32_t)((warp & 3) * 32) << 16);
+    const long long m0 =
+        (b << (3 * lgD)) + ((((long long)x0 << lgD) + (y0 + (row >> 3))) << lgD) + (z0 + (row & 7));
 #pragma unroll 1
     for (int q = warp >> 2; q < TX * (NC / 16); q += HT / 128) {
       const int tx = q / (NC / 16), n0 = 16 * (q - tx * (NC / 16));
-      const long long m = sbase + ((((long long)(x0 + tx) << lgD) + (y0 + yy)) << lgD) + (z0 + zz);
       float v[16];
-      tmem_ld16(lane_addr + tx * NC + n0, v);
-      store16<DGRAD>(v, m, n0, bias, relu, y, ldy, offy, gx, ldg, offg, accumulate);
+      tmem_ld16(lane_addr + 16 * q, v);
+      tmem_zero16(lane_addr + 16 * q);
+      store16<DGRAD>(v, m0 + ((long long)tx << (2 * lgD)), n0, bias, relu, y, ldy, offy, gx, ldg,
+                     offg, accumulate);
     }
-  } else if (tid == 0) {
-    // a wait ran out: the weights' copy and the MMAs in flight (each bounded)
-    if (issued) mbar_wait(bars + 1, 0, err);
-    else mbar_wait(bars, 0, err);
   }
+  cp_async_wait<0>();
+  asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   if (warp == 0)
@@ -706,22 +747,25 @@ __global__ void __launch_bounds__(HT) k_conv_halo(
 template <int KC, int NC, bool DG, int TX>
 void launch_halo(const TcArgs& a, cudaStream_t s) {
   constexpr int H_BYTES = (KC / 8) * halo_plane(TX + 2), W_BYTES = 27 * NC * KC * 2;
-  const int cols0 = TX * NC;
-  const int cols = cols0 <= 32 ? 32 : (cols0 <= 64 ? 64 : (cols0 <= 128 ? 128 : 256));
-  const size_t need = (size_t)H_BYTES + W_BYTES + 2 * 8 + 16;
-  const int k = 512 / cols;
-  const size_t cap = 233472 / (k + 1) - 1024 + 16;
-  const size_t smem = need > cap ? need : cap;
+  constexpr int cols0 = TX * NC;
+  constexpr int cols = cols0 <= 32 ? 32 : (cols0 <= 64 ? 64 : (cols0 <= 128 ? 128 : 256));
+  // CTAs per SM: by shared memory (1 KB reserved for each) and by tensor memory; the
+  // shared memory is padded so that no more are resident (tcgen05.alloc would wait)
+  constexpr int need = H_BYTES + W_BYTES + 8 + 16;
+  constexpr int fit = 233472 / (need + 1024), mem = 512 / cols;
+  constexpr int per_sm = fit < mem ? fit : mem;
+  constexpr int cap = 233472 / (per_sm + 1) - 1024 + 16, smem = need > cap ? need : cap;
+  static_assert(per_sm >= 1 && smem <= 227 * 1024, "one CTA fits");
   static bool attr = false;
   if (!attr) {
     cudaFuncSetAttribute(k_conv_halo<KC, NC, DG, TX>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          227 * 1024);
     attr = true;
   }
-  const long long tiles = a.Mtot / (TX * 16 * 8);
-  k_conv_halo<KC, NC, DG, TX><<<(unsigned)tiles, HT, smem, s>>>(
+  const int tiles = (int)(a.Mtot / (TX * 16 * 8));
+  k_conv_halo<KC, NC, DG, TX><<<(unsigned)std::min(tiles, 152 * per_sm), HT, smem, s>>>(
       a.x, a.ldx, a.offx, a.Wp, a.bias, a.relu, a.y, a.ldy, a.offy, a.gx, a.ldg, a.offg,
-      a.accumulate, a.lgD, cols, a.err);
+      a.accumulate, a.lgD, tiles, cols, a.err);
 }
 
 // The same halo-tiled form for layers whose 27 weight slices do not fit beside
@@ -1198,15 +1242,16 @@ bool nn_tc_supported(int K, int N) {
 bool nn_tc_conv(const TcArgs& a, int K, int N, bool dgrad, cudaStream_t s) {
   // the layers of the two finest levels whose input block and 27 weight
   // slices fit one CTA's shared memory run on the halo-tiled kernel when the
-  // grid holds its tiles (16^3 and more)
+  // grid holds its tiles (16^3 and more); the slices per tile (fourth argument) are
+  // the fastest of 1, 2, 4 and 8 on 128^3 and 256^3 that fit
   if (a.lgD >= 4 && a.lgD <= 10) {
 #define HALO_CASE(KK, NN, TXF, TXD)                                                       \
   if (K == KK && N == NN) {                                                             \
     if (dgrad) launch_halo<KK, NN, true, TXD>(a, s); else launch_halo<KK, NN, false, TXF>(a, s); \
     return true;                                                                        \
   }
-    HALO_CASE(16, 16, 4, 4) HALO_CASE(16, 32, 4, 4) HALO_CASE(32, 32, 2, 2)
-    HALO_CASE(32, 16, 2, 2)
+    HALO_CASE(16, 16, 8, 8) HALO_CASE(16, 32, 8, 8) HALO_CASE(32, 32, 2, 2)
+    HALO_CASE(32, 16, 4, 4)
 #undef HALO_CASE
     // larger channel counts: the weight slices stream beside the resident block
 #define HALO_S(KK, NN, TXX, DGR)                           \
@@ -1224,7 +1269,7 @@ bool nn_tc_conv(const TcArgs& a, int K, int N, bool dgrad, cudaStream_t s) {
       return true;
     }
     if (dgrad && K == 16 && N == 48) {
-      launch_halo<16, 48, true, 2>(a, s);
+      launch_halo<16, 48, true, 4>(a, s);
       return true;
     }
   }
@@ -1260,8 +1305,9 @@ bool nn_tc_wgrad(TView x, int Cin, TView g, int Cout, float* dW, float* db, floa
   const long long Mtot = (long long)B << (3 * lgD);
   int S = 0;
   // up to 32 output channels on grids that hold the 16 x 8 blocks: resident
-  // blocks (16 -> 16 on 4 x 64^3 283 -> see below; smaller grids and 64 and more
-  // output channels, whose slices leave no room for the three dx, per tap)
+  // blocks (on 4 x 64^3: 16 -> 16 109 us, per tap 279; 48 -> 16 217, 513; smaller grids
+  // and 64 and more output channels, whose slices leave no room for the three dx, per
+  // tap)
   if (lgD >= 4) {
     bool done = true;
     if (Cin == 16 && Cout == 16)
