@@ -358,7 +358,7 @@ typedef struct {
  * one gives up; the context stays usable).  per_solve (nullable) receives one
  * mgfr_stats per item, in item order.  The launch shape (threads per block,
  * blocks per SM) comes from mgfr_batch_autotune for the same list of sizes,
- * else 512 x 2.
+ * else from the number of cells; no more blocks than there is work for.
  */
 mgfr_status mgfr_batch_solve(mgfr_ctx* ctx, int nsolves, const mgfr_batch_item* items,
                              mgfr_stats* per_solve);

@@ -668,8 +668,9 @@ void batch_free(mgfr_ctx* c) {
   c->batch = nullptr;
 }
 
+// at most `blocks` blocks
 static mgfr_status launch_batch(mgfr_ctx* c, BatchWork* B, const BArgs& A, int threads, int bpsm,
-                                bool use_graph) {
+                                long long blocks, bool use_graph) {
   int dev = c->device, nsm = 0;
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   int occ = 0;
@@ -678,7 +679,7 @@ static mgfr_status launch_batch(mgfr_ctx* c, BatchWork* B, const BArgs& A, int t
   void* kern = A.tol >= 1e-10 ? (void*)k_batch<true> : (void*)k_batch<false>;
   MG_CK(c, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, threads, 0));
   if (occ < 1) return set_err(c, MGFR_E_UNSUPPORTED, "batched kernel cannot be resident");
-  const int grid = nsm * std::min(bpsm, occ);
+  const int grid = (int)std::min((long long)nsm * std::min(bpsm, occ), blocks);
   MG_CK(c, cudaMemsetAsync(B->bar, 0, 2 * sizeof(unsigned), c->s));
   MG_CK(c, cudaMemsetAsync(B->err, 0, 2 * sizeof(int), c->s));
   BArgs a = A;
@@ -848,16 +849,30 @@ mgfr_status mgfr_batch_solve(mgfr_ctx* c, int nsolves, const mgfr_batch_item* it
   A.bar_gen = B->bar + 1;
   A.err = B->err;
   A.max_spins = g.max_spins;
-  // launch shape: tuned choice for this signature, else 512 threads x 2 per SM
-  // (96 solves of 32^3..128^3: 45.0 ms; 256 x 2 54.5, 256 x 4 46.9, 128 x 8 50.3)
-  int threads = 512, bpsm = 2;
+  // Launch shape: the tuned choice for this signature, else by the work items of a
+  // half-sweep of the finest grids (four cells each).  Beyond 2^20 the device is full
+  // either way and 512 threads x 2 per SM are the fastest (96 solves of 32^3..128^3, ms:
+  // 45.0; 256 x 2 54.5, 256 x 3 47.1, 128 x 8 50.3), below it smaller blocks spread the
+  // items better (one 64^3 1.68 for 1.82, one 128^3 3.46 for 3.64).  A batch of few items is
+  // little but barriers, whose time grows with the blocks that arrive at them: no more
+  // blocks than there are items for (and one per solve, for the 4^3 grids), up to 16384
+  // items (one 32^3: 4096) small blocks on many SMs: one 32^3 1.39 ms (on a full grid of
+  // 512 x 2 1.53, of 256 x 2 with one cell per thread 1.45), one 8^3 0.39 (0.46).
+  long long vecs = 0;
+  for (const BSolve& S : hs) vecs += 1LL << (3 * S.lg - 3);
+  int threads = vecs > (1 << 20) ? 512 : (vecs > 16384 || vecs <= 1024 ? 256 : 128);
+  int bpsm = threads == 512 ? 2 : 3;
   auto itc = B->tuned.find(sig);
-  if (itc != B->tuned.end()) {
+  const bool tuned = itc != B->tuned.end();
+  if (tuned) {
     threads = itc->second.first;
     bpsm = itc->second.second;
   }
+  long long blocks = (vecs + threads - 1) / threads;
+  if (!tuned && threads == 128) blocks = std::max(blocks, std::min(128LL, vecs / 64));
+  blocks = std::max(blocks, (long long)nsolves);
   MG_CK(c, cudaEventRecord(c->t0, c->s));
-  mgfr_status rs = launch_batch(c, B, A, threads, bpsm, true);
+  mgfr_status rs = launch_batch(c, B, A, threads, bpsm, blocks, true);
   if (rs != MGFR_OK) return rs;
   MG_CK(c, cudaEventRecord(c->t1, c->s));
   std::vector<BState> st(nsolves);
