@@ -1295,9 +1295,19 @@ bool nn_tc_wgrad_supported(int Cin, int Cout) {
   return false;
 }
 
+// the pairs with a resident-block kernel (launch_wgrad_halo below), whose partials are
+// one per CTA
+static bool wgrad_halo_pair(int Cin, int Cout) {
+  return (Cout == 16 && (Cin == 16 || Cin == 48)) ||
+         (Cout == 32 && (Cin == 16 || Cin == 32 || Cin == 96));
+}
+
+// (counting a partial per CTA for every pair took 128 -> 128 to 269 MB, above what a
+// conv3d call's kept scratch may hold, and so to an allocation per call: 0.73 ms for the three ops on 8^3, now 0.32)
 long long nn_tc_wgrad_scratch(int Cin, int Cout) {
-  const int nt = (27 + TC_M / Cout - 1) / (TC_M / Cout);
-  return (long long)std::max(WG_HALO_CTAS, WG_CTAS / nt) * 27 * Cin * Cout;
+  const int nt = (27 + TC_M / Cout - 1) / (TC_M / Cout), tap = WG_CTAS / nt;
+  const int parts = wgrad_halo_pair(Cin, Cout) ? std::max(WG_HALO_CTAS, tap) : tap;
+  return (long long)parts * 27 * Cin * Cout;
 }
 
 bool nn_tc_wgrad(TView x, int Cin, TView g, int Cout, float* dW, float* db, float* partials,
@@ -1308,8 +1318,7 @@ bool nn_tc_wgrad(TView x, int Cin, TView g, int Cout, float* dW, float* db, floa
   // blocks (on 4 x 64^3: 16 -> 16 109 us, per tap 279; 48 -> 16 217, 513; smaller grids
   // and 64 and more output channels, whose slices leave no room for the three dx, per
   // tap)
-  if (lgD >= 4) {
-    bool done = true;
+  if (lgD >= 4 && wgrad_halo_pair(Cin, Cout)) {
     if (Cin == 16 && Cout == 16)
       launch_wgrad_halo<16, 16, 2, 9>(x, g, B, lgD, partials, err, &S, s);
     else if (Cin == 48 && Cout == 16)
@@ -1318,14 +1327,10 @@ bool nn_tc_wgrad(TView x, int Cin, TView g, int Cout, float* dW, float* db, floa
       launch_wgrad_halo<16, 32, 2, 9>(x, g, B, lgD, partials, err, &S, s);
     else if (Cin == 32 && Cout == 32)
       launch_wgrad_halo<32, 32, 1, 9>(x, g, B, lgD, partials, err, &S, s);
-    else if (Cin == 96 && Cout == 32)
-      launch_wgrad_halo<96, 32, 1, 3>(x, g, B, lgD, partials, err, &S, s);
     else
-      done = false;
-    if (done) {
-      nn_wgrad_finish(partials, S, Cin, Cout, dW, g, db, Mtot, s);
-      return true;
-    }
+      launch_wgrad_halo<96, 32, 1, 3>(x, g, B, lgD, partials, err, &S, s);
+    nn_wgrad_finish(partials, S, Cin, Cout, dW, g, db, Mtot, s);
+    return true;
   }
 #define WG_CASE(CI, CO)                                                  \
   if (Cin == CI && Cout == CO) {                                         \
