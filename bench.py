@@ -68,21 +68,16 @@ FAMILY_BOUND = {0: "hbm", 1: "hbm", 2: "alu", 3: "hbm", 4: "hbm"}
 # launch by its cells (family 3: 343.6 MB over the 24.8 M cells of a level-1
 # launch of that sample, 12124 x 256 threads, one per oct).
 TRAFFIC_PER_CELL = {3: 343.59e6 / (12124 * 256 * 8)}
-KERNEL_NAMES = {0: "k_sweep32 (FP32 NGS half-sweep, base level)",
-                1: "k_lin_sweep (FP32 linear GS half-sweep, base level)",
+KERNEL_NAMES = {0: "k_vsweep<MG_NL> (FP32 NGS half-sweep, base level)",
+                1: "k_vsweep<MG_LIN> (FP32 linear GS half-sweep, base level)",
                 2: "k_resid_df / k_oresid_df (FP64-accurate residual in double-float)",
                 3: "k_oct_sweep32<false> (FP32 NGS half-sweep on the octs of the refined level)",
                 4: "k_oct_sweep32<true> (FP32 linear GS half-sweep on the octs of the refined level)"}
-# FP64 form: FP64 operations per NGS point update counted from the kernels
-# (6 faces x (E sum, half, difference, FMA as 2, two running sums) = 42; L and
-# dL/du 10; step, clamp, update 4) = 56, plus one rsqrt (n = 1), one division
-# and one exponential, which the FP64 pipe also executes but are not counted.
-FP64_FLOPS_PER_UPDATE = 56.0
-FP64_KERNEL_NAMES = {0: "k_sweep (FP64 NGS half-sweep, base level)",
-                     3: "k_osweep<double> (FP64 NGS half-sweep on the octs of the refined level)"}
-# GB300 FP64: 1.25 TFLOP/s nominal (about 2 FP64 FMA per clock per SM at
-# 2.07 GHz on 152 SMs); no measured figure is available on this machine.
-FP64_PEAK_TFLOPS = 1.25
+# FP64 form: its half-sweeps relax the deviation from the FP64 iterate in FP32 (u and e
+# read, r and e of the active colour, e written: 12 bytes per level cell).
+FP64_FORM_BYTES = 12.0
+FP64_FORM_NAMES = {0: "k_vsweep<MG_DEV> (FP32 NGS half-sweep on the deviation, base level)",
+                   3: "k_oct_dev_sweep (FP32 NGS half-sweep on the deviation, octs)"}
 
 
 def peaks():
@@ -733,18 +728,18 @@ def main():
             "kernel_share_of_step": kern_ms[fam] / ms_prof,
             "profiled_ms_per_step": ms_prof / ksteps,
             "families": family_table(kern_ms, kern_n, kern_cells, ksteps, peak)}
-    fp64 = {"bound": "fp64", "peak_tflops": FP64_PEAK_TFLOPS, "peak_source": "nominal",
-            "flops_per_update": FP64_FLOPS_PER_UPDATE, "families": []}
+    fp64 = {"bound": "hbm", "peak": peak, "peak_source": peak_kind, "unit": "GB/s",
+            "alg_bytes_per_cell": FP64_FORM_BYTES, "families": []}
     for q in (0, 3):
         if st64["kern_launches"][q] == 0:
             continue
         a_ms = st64["kern_ms"][q] / st64["kern_launches"][q]
         cells = st64["kern_cells"][q] / st64["kern_launches"][q]
-        tfl = FP64_FLOPS_PER_UPDATE * cells / 2 / (a_ms / 1e3) / 1e12  # half the cells update
-        fp64["families"].append({"kernel": FP64_KERNEL_NAMES[q],
+        gbs = FP64_FORM_BYTES * cells / (a_ms / 1e3) / 1e9
+        fp64["families"].append({"kernel": FP64_FORM_NAMES[q],
                                  "launches": st64["kern_launches"][q],
-                                 "avg_launch_us": 1e3 * a_ms, "achieved_tflops": tfl,
-                                 "frac": tfl / FP64_PEAK_TFLOPS,
+                                 "avg_launch_us": 1e3 * a_ms, "achieved": gbs,
+                                 "frac": gbs / peak,
                                  "ms_per_solve": st64["kern_ms"][q]})
 
     cpu = None if (args.no_cpu_baseline or world > 1) else cpu_baseline_sample()

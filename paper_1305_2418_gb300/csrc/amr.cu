@@ -935,7 +935,7 @@ static AmrWork* W(mgfr_ctx* c) { return (AmrWork*)c->amr; }
 static void free_level(AmrLevel& L) {
   void* ps[] = {L.son,  L.refined, L.count,  L.opos, L.pcell,   L.nbr,     L.mass,
                 L.w,    L.wE,      L.wf,     L.wold, L.mask,    L.ghost,   L.ghostE,
-                L.acc,  L.pnbr,    L.w32,    L.wE32, L.wf32,    L.wold32,  L.ghost32, L.gface,
+                L.acc,  L.pnbr,    L.w32,    L.wf32,    L.wold32,  L.ghost32, L.gface,
                 L.olist,  L.acc32, L.act};
   for (void* p : ps)
     if (p) cudaFree(p);
@@ -1054,7 +1054,7 @@ static void drop_level(AmrWork* A, int l) {
   L.son = nullptr; L.refined = nullptr; L.count = nullptr; L.opos = nullptr; L.pcell = nullptr;
   L.nbr = nullptr; L.mass = nullptr; L.w = nullptr; L.wE = nullptr; L.wf = nullptr;
   L.wold = nullptr; L.mask = nullptr; L.ghost = nullptr; L.ghostE = nullptr; L.acc = nullptr;
-  L.pnbr = nullptr; L.w32 = nullptr; L.wE32 = nullptr; L.wf32 = nullptr; L.wold32 = nullptr;
+  L.pnbr = nullptr; L.w32 = nullptr; L.wf32 = nullptr; L.wold32 = nullptr;
   L.ghost32 = nullptr; L.olist = nullptr; L.acc32 = nullptr; L.act = nullptr; L.gface = nullptr;
   if (l > 0) {
     if (L.u) cudaFree(L.u);
@@ -1079,7 +1079,6 @@ static mgfr_status grow_level(mgfr_ctx* c, AmrWork* A, int l, long long n, long 
   TRY(grow(c, &L.mask, n));
   TRY(grow(c, &L.act, n));
   TRY(grow(c, &L.w32, n));
-  TRY(grow(c, &L.wE32, n));
   TRY(grow(c, &L.wf32, n));
   TRY(grow(c, &L.wold32, n));
   if (l > 0) {

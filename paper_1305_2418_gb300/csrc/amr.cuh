@@ -36,7 +36,7 @@ struct AmrLevel {
   float4* acc32 = nullptr;            // [ncell] FP32 force for the mixed-form gather
   int* pnbr = nullptr;                // [n_oct*6] parent's face-neighbour cells (-1: none)
   // FP32 work arrays (mixed precision phase of the level solves)
-  float *w32 = nullptr, *wE32 = nullptr, *wf32 = nullptr, *wold32 = nullptr;
+  float *w32 = nullptr, *wf32 = nullptr, *wold32 = nullptr;
   float* ghost32 = nullptr;           // [n_gslot*4] FP32 ghost u (e^u recomputed)
   unsigned* gface = nullptr;          // [n_gslot] face 6 o + d of each ghost slot
   long long relaxed = 0;              // cells relaxed in the current level solve

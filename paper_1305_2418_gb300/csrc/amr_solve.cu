@@ -10,8 +10,10 @@
 // converged coarse solution (or the restriction of their daughters), so the
 // coarse solutions themselves are never modified.
 //
-// Kernels are templated on the working precision T.  The FP64 form runs FP64
-// V-cycles to the tolerance.  The mixed form first runs FP32 V-cycles (u in
+// The FP64 form holds u, e^u and the residual in FP64 and forms each V-cycle's
+// correction in FP32, in the deviation from the FP64 iterate (mg32.cuh, MG_DEV); it
+// runs in FP64 throughout (the templates with T = double) while the residual is too far
+// from f for FP32, and after a cycle that gains nothing.  The mixed form first runs FP32 V-cycles (u in
 // FP32, e^u recomputed by the SFU) until the FP32 residual reaches
 // mixed_switch or stalls (phase A), then corrects the defect (phase B): the
 // residual r = f - L(u) of the level in double-float (FP64-accurate, on the
@@ -1782,7 +1784,7 @@ TA<double> tarr<double>(AmrLevel& L) {
 }
 template <>
 TA<float> tarr<float>(AmrLevel& L) {
-  return TA<float>{L.w32, L.wE32, L.wf32, L.wold32, L.ghost32, nullptr};
+  return TA<float>{L.w32, nullptr, L.wf32, L.wold32, L.ghost32, nullptr};
 }
 
 // work arrays of dense level k of the hierarchy below the base (k >= 1)
@@ -2109,7 +2111,7 @@ void corr_relax(SolveCtx& S, int l, int sweeps) {
           k_ddev_sweep_list<<<nblocks(nl, BS), BS, 0, c->s>>>(L.wold32, L.wf32, L.w32, L.lgN, list,
                                                               nl, p, (float)L.ih2);
         else
-          k_dlin_sweep_list<<<nblocks(nl, BS), BS, 0, c->s>>>(L.wold32, L.wf32, L.w32, L.wE32,
+          k_dlin_sweep_list<<<nblocks(nl, BS), BS, 0, c->s>>>(L.wold32, L.wf32, L.w32, nullptr,
                                                               L.lgN, list, nl, m, (float)L.ih2);
       }
       c->launches += 1;
@@ -2213,7 +2215,7 @@ void corr_vcycle_tree(SolveCtx& S, int l) {
   } else if (l == 0 && S.kmax >= 1) {
     DenseHier& H = c->dh;
     DenseLevel& C = H.L[1];
-    corr_drestrict<DEV>(S, F.wold32, F.wf32, F.w32, F.wE32, F.lgN, F.ih2, F.act, C);
+    corr_drestrict<DEV>(S, F.wold32, F.wf32, F.w32, nullptr, F.lgN, F.ih2, F.act, C);
     corr_vcycle_dense<DEV>(S, 1);
     const CList c0 = clist(S, 0);
     if (cl_threads(c0, F.ncell) > 0)

@@ -4,7 +4,9 @@
 // Layout: level of size N = 2^lg, C order index ((i*N)+j)*N+k, k along z
 // (fastest).  Each level keeps u and E = e^u side by side so a point update
 // needs one exponential (its own new E) instead of seven; on GB300 the FP64
-// pipe, not HBM, bounds these kernels.
+// pipe, not HBM, bounds these kernels.  The FP64 form's V-cycles form their correction
+// in FP32 (mg32.cuh, MG_DEV) between k_resid_dev and k_apply_dev; the sweeps and
+// transfers here run where FP32 cannot resolve the residual against f.
 #include <algorithm>
 
 #include "colour_split.cuh"

@@ -3,8 +3,9 @@
 // FP32 accumulator in tensor memory (TMEM), BF16 operands in shared memory.
 // Three forms: the per-tap kernel (k_conv_tc, below), the halo-tiled kernels
 // of the full- and second-resolution layers (k_conv_halo, k_conv_halo_s: the
-// input block with its one-voxel halo staged once per CTA, each tap a shifted
-// descriptor into it) and the weight gradient (k_wgrad_tc).
+// input block with its one-voxel halo staged once per tile, each tap a shifted
+// descriptor into it) and the weight gradient (k_wgrad_tc per tap; k_wgrad_halo from
+// resident blocks for up to 32 output channels).
 //
 // Implicit GEMM per CTA: rows = an M tile of 128 consecutive
 // voxels, columns = all N output channels (N <= 256), reduction = 27 taps x
@@ -17,7 +18,7 @@
 // Both tiles use the canonical K-major layout without swizzle: core matrices
 // of 8 rows x 16 bytes; for each 8-channel chunk the rows are contiguous (so
 // the 8-row groups are 128 B apart: SBO), and the chunks follow each other one
-// tile-height apart (LBO).  Thread 0 issues the tap's MMAs (K = 16 each) and
+// tile-height apart (LBO).  An elected lane issues the tap's MMAs (K = 16 each) and
 // commits them to the stage's mbarrier; two stages overlap the copies of tap
 // t+1 with the MMAs of tap t.  The epilogue reads the accumulator with
 // tcgen05.ld (warp w its 32 TMEM lanes = rows 32w..32w+31).
