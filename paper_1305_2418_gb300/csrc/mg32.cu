@@ -55,6 +55,24 @@ __global__ void __launch_bounds__(BS) k_vrestrict(const float* __restrict__ x,
 }
 
 template <int OP>
+__global__ void __launch_bounds__(128) k_vrestrict_rows(
+    const float* __restrict__ x, const float* __restrict__ r, const float* __restrict__ w,
+    int lgf, float* __restrict__ xc, float* __restrict__ rc, float* __restrict__ wc, PF m,
+    float ih2) {
+  const unsigned t = blockIdx.x * blockDim.x + threadIdx.x;
+  if (t < (1u << (3 * lgf - 3))) vec_restrict_rows<OP>(t, x, r, w, lgf, xc, rc, wc, m, ih2);
+}
+
+template <int OP>
+__global__ void __launch_bounds__(128) k_vprolong_rows(float* __restrict__ x,
+                                                       const float* __restrict__ xc,
+                                                       const float* __restrict__ wc, int lgf,
+                                                       int linear) {
+  const unsigned t = blockIdx.x * blockDim.x + threadIdx.x;
+  if (t < (1u << (3 * lgf - 3))) vec_prolong<OP, 1>(t, x, xc, wc, lgf, linear);
+}
+
+template <int OP>
 __global__ void __launch_bounds__(BS) k_vprolong(float* __restrict__ x, const float* __restrict__ xc,
                                                  const float* __restrict__ wc, int lgf,
                                                  int linear) {
@@ -155,6 +173,11 @@ __global__ void k_finish2(const double* __restrict__ partials, int nparts, doubl
 // also the 8^3 and 4^3 levels whole.
 constexpr int BT = 512;
 constexpr int kBotMaxLg = 5;
+// Transfers from levels up to 2^kRowsMax take four lanes per group of four coarse cells,
+// larger ones one thread: on 64^3 the 8192 threads of the latter stand on the latency of
+// their four rows (restriction in the deviation 15.7 us, 7.5 by rows; prolongation 6.9,
+// 4.5), on 128^3 both take the same (21; 7.5), on 256^3 the rows cost more (46 and 70).
+constexpr int kRowsMax = 6;
 
 struct BotArgs {
   int lg;             // the finest level held, 3..5
@@ -508,8 +531,12 @@ long long cycle(const Mg32Level* L, int nlev, const Mg32Par& p, cudaStream_t s,
     const Mg32Level &F = L[l], &C = L[l + 1];
     const long long nc = 1LL << (3 * C.lg);
     relax(l, p.n_pre);
-    k_vrestrict<OP><<<nblocks(nc / 4, BS), BS, 0, s>>>(F.x, F.r, F.w, F.lg, C.x, C.r, C.w, m,
-                                                       F.ih2);
+    if (F.lg <= kRowsMax)
+      k_vrestrict_rows<OP><<<nblocks(nc, 128), 128, 0, s>>>(F.x, F.r, F.w, F.lg, C.x, C.r, C.w, m,
+                                                            F.ih2);
+    else
+      k_vrestrict<OP><<<nblocks(nc / 4, BS), BS, 0, s>>>(F.x, F.r, F.w, F.lg, C.x, C.r, C.w, m,
+                                                         F.ih2);
     if (OP == MG_NL) k_vfas<<<nblocks(nc / 4, BS), BS, 0, s>>>(C.x, C.r, C.lg, m, C.ih2);
   }
   BotArgs A{};
@@ -530,8 +557,11 @@ long long cycle(const Mg32Level* L, int nlev, const Mg32Par& p, cudaStream_t s,
   launch_bottom<OP>(A, s);
   for (int l = lb - 1; l >= 0; --l) {
     const Mg32Level &F = L[l], &C = L[l + 1];
-    k_vprolong<OP><<<nblocks((1LL << (3 * C.lg)) / 4, BS), BS, 0, s>>>(F.x, C.x, C.w, F.lg,
-                                                                       p.linear);
+    const long long nc = 1LL << (3 * C.lg);
+    if (F.lg <= kRowsMax)
+      k_vprolong_rows<OP><<<nblocks(nc, 128), 128, 0, s>>>(F.x, C.x, C.w, F.lg, p.linear);
+    else
+      k_vprolong<OP><<<nblocks(nc / 4, BS), BS, 0, s>>>(F.x, C.x, C.w, F.lg, p.linear);
     relax(l, p.n_post);
   }
   return upd;

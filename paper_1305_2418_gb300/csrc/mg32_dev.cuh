@@ -317,12 +317,90 @@ __device__ __forceinline__ void vec_restrict(unsigned t, const float* __restrict
   }
 }
 
-// x += P(c) with c = xc - wc (NL) or xc: four coarse cells, their 32 daughters
+// 4 x 4 values of four consecutive lanes transposed: lane q's v[a] becomes lane a's v[q]
+__device__ __forceinline__ void transpose4(float* v) {
+  const unsigned lane = threadIdx.x & 31, grp = 0xfu << (lane & 28);
+#pragma unroll
+  for (int b = 1; b <= 2; b <<= 1)
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      if (r & b) continue;
+      const bool hi = lane & b;
+      const float got = __shfl_xor_sync(grp, hi ? v[r] : v[r | b], b);
+      if (hi)
+        v[r] = got;
+      else
+        v[r | b] = got;
+    }
+}
+
+// The same by four consecutive lanes, t = 4 (group) + lane: a lane forms the eight
+// daughters of one fine row, then takes the sums of one coarse cell, in the same order
 template <int OP>
+__device__ __forceinline__ void vec_restrict_rows(unsigned t, const float* __restrict__ x,
+                                                  const float* __restrict__ r,
+                                                  const float* __restrict__ w, int lgf,
+                                                  float* __restrict__ xc, float* __restrict__ rc,
+                                                  float* __restrict__ wc, PF m, float ih2) {
+  const int lgc = lgf - 1, Mc = (1 << lgc) - 1;
+  const int ab = (int)(t & 3);
+  t >>= 2;
+  const int K0 = 4 * (int)(t & ((1u << (lgc - 2)) - 1));
+  const int J = (int)((t >> (lgc - 2)) & Mc), I = (int)(t >> (2 * lgc - 2));
+  const unsigned half = 1u << (3 * lgf - 1);
+  const int i = 2 * I + (ab >> 1), j = 2 * J + (ab & 1);
+  const int qe = (i + j) & 1;  // the plane of the row's even k
+  V4 res[2], val[2];
+#pragma unroll
+  for (int c = 0; c < 2; ++c) {  // k = 2K + c
+    const unsigned own = ((qe ^ c) ? half : 0u), oth = half - own;
+    const Rows R = rows_at(i, j, K0, c, lgf);
+    const Nb4 xn = load_nb(x + oth, R, c);
+    const V4 xv = ld4(x + own + R.c), rv = ld4(r + own + R.c);
+    V4 wv{};
+    Nb4 wn{};
+    if (OP == MG_LIN || OP == MG_DEV) {
+      wn = load_nb(w + oth, R, c);
+      wv = ld4(w + own + R.c);
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      float a[6], b[6];
+      xn.get(q, a);
+      wn.get(q, b);
+      res[c].v[q] = rv.v[q] - point_apply<OP>(xv.v[q], a, wv.v[q], b, m, ih2);
+      val[c].v[q] = OP == MG_NL ? xv.v[q] : (OP == MG_DEV ? wv.v[q] + xv.v[q] : wv.v[q]);
+    }
+  }
+  float sr = 0.f, su = 0.f;
+  transpose4(res[0].v);
+  transpose4(res[1].v);
+  if (OP != MG_POI) {
+    transpose4(val[0].v);
+    transpose4(val[1].v);
+  }
+#pragma unroll
+  for (int a = 0; a < 4; ++a)
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+      sr += res[c].v[a];
+      su += val[c].v[a];
+    }
+  const unsigned p = pdx(I, J, K0 + ab, lgc);
+  rc[p] = 0.125f * sr;
+  xc[p] = OP == MG_NL ? 0.125f * su : 0.f;
+  if (OP != MG_POI) wc[p] = 0.125f * su;
+}
+
+// x += P(c) with c = xc - wc (NL) or xc: four coarse cells, their 32 daughters
+// (ROWS 4: one thread; 1: four consecutive lanes, a fine row each)
+template <int OP, int ROWS = 4>
 __device__ __forceinline__ void vec_prolong(unsigned t, float* __restrict__ x, const float* __restrict__ xc,
                                                  const float* __restrict__ wc, int lgf,
                                                  int linear) {
   const int lgc = lgf - 1, Mc = (1 << lgc) - 1, hmc = Mc >> 1;
+  const int row = (int)(t & 3);
+  if (ROWS == 1) t >>= 2;
   const int K0 = 4 * (int)(t & ((1u << (lgc - 2)) - 1));
   const int J = (int)((t >> (lgc - 2)) & Mc), I = (int)(t >> (2 * lgc - 2));
   const unsigned halfc = 1u << (3 * lgc - 1);
@@ -365,7 +443,8 @@ __device__ __forceinline__ void vec_prolong(unsigned t, float* __restrict__ x, c
   }
   const unsigned half = 1u << (3 * lgf - 1);
 #pragma unroll
-  for (int ab = 0; ab < 4; ++ab) {
+  for (int ab0 = 0; ab0 < ROWS; ++ab0) {
+    const int ab = ROWS == 1 ? row : ab0;
     const int i = 2 * I + (ab >> 1), j = 2 * J + (ab & 1);
     const unsigned rw = prow(i, j, lgf) + K0;
     const int qe = (i + j) & 1;
