@@ -650,7 +650,11 @@ __global__ void __launch_bounds__(64) k_dlin_coarse(float* __restrict__ eg, cons
 // (mg32.cuh, MG_DEV), in the arrays of the linear cycle: u (FP32 copy), r, e.
 PF pf32(const MT<float>& m, float cap) { return PF{m.aRt, m.aRt_np1, m.inv_np1, cap}; }
 
-__global__ void __launch_bounds__(BS) k_ddev_sweep_list(float* __restrict__ e,
+// Blocks of 128: the levels of the FP64 form are often a few thousand octs, and smaller
+// blocks spread them over more SMs (100 half-sweeps of a 64^3 base's two levels: 681 us with
+// 256, 631 with 128, 641 with 64; restriction 10.6, 9.4, 9.5 us).
+constexpr int DVB = 128;
+__global__ void __launch_bounds__(DVB) k_ddev_sweep_list(float* __restrict__ e,
                                                         const float* __restrict__ r,
                                                         const float* __restrict__ u, int lg,
                                                         const int* __restrict__ list, long long n,
@@ -1213,7 +1217,7 @@ __device__ __forceinline__ void oct_six(const Oct8& X, const Faces& F, int ch, f
 }
 
 template <int COL>
-__global__ void __launch_bounds__(BS) k_oct_dev_sweep(
+__global__ void __launch_bounds__(DVB) k_oct_dev_sweep(
     const float* __restrict__ u, float* __restrict__ e, const float* __restrict__ r,
     const int* __restrict__ nbr, const float* __restrict__ gh,
     const unsigned char* __restrict__ act, long long n, const int* __restrict__ olist,
@@ -1243,7 +1247,7 @@ __global__ void __launch_bounds__(BS) k_oct_dev_sweep(
 }
 
 // r_c = R(r - D(e)) over relaxed cells, u_c = R(u + e), e_c = 0
-__global__ void __launch_bounds__(BS) k_oct_dev_restrict(
+__global__ void __launch_bounds__(DVB) k_oct_dev_restrict(
     const float* __restrict__ e, const float* __restrict__ r, const float* __restrict__ u,
     const int* __restrict__ nbr, const float* __restrict__ gh,
     const unsigned char* __restrict__ act, long long n, const int* __restrict__ olist,
@@ -2094,7 +2098,7 @@ void corr_relax(SolveCtx& S, int l, int sweeps) {
         if (R.n == 0) continue;
         if (l == S.L) prof_begin(c, DEV ? 3 : 4, L.ncell);
         if constexpr (DEV) {
-          (col == 0 ? k_oct_dev_sweep<0> : k_oct_dev_sweep<1>)<<<nblocks(R.n, BS), BS, 0, c->s>>>(
+          (col == 0 ? k_oct_dev_sweep<0> : k_oct_dev_sweep<1>)<<<nblocks(R.n, DVB), DVB, 0, c->s>>>(
               L.w32, L.wold32, L.wf32, L.nbr, L.ghost32, mk, R.n, R.list, L.n_oct, p,
               (float)L.ih2);
         } else {
@@ -2108,7 +2112,7 @@ void corr_relax(SolveCtx& S, int l, int sweeps) {
         if (nl == 0) continue;
         const int* list = S.A->dlist[0] + col * (L.ncell / 2);
         if constexpr (DEV)
-          k_ddev_sweep_list<<<nblocks(nl, BS), BS, 0, c->s>>>(L.wold32, L.wf32, L.w32, L.lgN, list,
+          k_ddev_sweep_list<<<nblocks(nl, DVB), DVB, 0, c->s>>>(L.wold32, L.wf32, L.w32, L.lgN, list,
                                                               nl, p, (float)L.ih2);
         else
           k_dlin_sweep_list<<<nblocks(nl, BS), BS, 0, c->s>>>(L.wold32, L.wf32, L.w32, nullptr,
@@ -2160,7 +2164,7 @@ void corr_vcycle_dense(SolveCtx& S, int k) {
         if (nl == 0) continue;
         const int* list = S.A->dlist[k] + col * (F.n / 2);
         if constexpr (DEV)
-          k_ddev_sweep_list<<<nblocks(nl, BS), BS, 0, c->s>>>(F.uold32, F.r32, F.u32, F.lg, list,
+          k_ddev_sweep_list<<<nblocks(nl, DVB), DVB, 0, c->s>>>(F.uold32, F.r32, F.u32, F.lg, list,
                                                               nl, p, (float)F.ih2);
         else
           k_dlin_sweep_list<<<nblocks(nl, BS), BS, 0, c->s>>>(F.uold32, F.r32, F.u32, F.e32, F.lg,
@@ -2197,7 +2201,7 @@ void corr_vcycle_tree(SolveCtx& S, int l) {
     const long long pno = l - 1 >= 1 ? P.n_oct : 0;  // FP32 parent layout (0: dense)
     if (R.n > 0) {
       if constexpr (DEV)
-        k_oct_dev_restrict<<<nblocks(R.n, BS), BS, 0, c->s>>>(
+        k_oct_dev_restrict<<<nblocks(R.n, DVB), DVB, 0, c->s>>>(
             F.wold32, F.wf32, F.w32, F.nbr, F.ghost32, fmask, R.n, R.list, F.n_oct, F.pcell, pno,
             pf32(m, (float)g.step_cap), (float)F.ih2, P.wf32, P.w32, P.wold32);
       else
