@@ -124,12 +124,14 @@ __global__ void __launch_bounds__(128) k_conv(const __nv_bfloat16* __restrict__ 
   }
 }
 
-// weight gradient partials: block (tap, 16-row ci tile, voxel chunk z)
+// weight gradient partials: block (tap, 16-row ci tile and group of NT 8 output
+// channels, voxel chunk z); ncol: the groups (Cout = 8 NT ncol)
 template <int NT>
 __global__ void __launch_bounds__(128) k_wgrad(const __nv_bfloat16* __restrict__ x, int ldx, int offx,
                                                int Cin, const __nv_bfloat16* __restrict__ g, int ldg,
-                                               int offg, int Cout, float* __restrict__ partials,
-                                               long long Mtot, long long chunk, int lgD) {
+                                               int offg, int Cout, int ncol,
+                                               float* __restrict__ partials, long long Mtot,
+                                               long long chunk, int lgD) {
   constexpr int MC = 64;  // voxels per staging step
   constexpr int STAGE_BYTES = (16 + NT * 8) * (MC + KPAD) * 2;
   constexpr int RED_BYTES = 4 * 16 * NT * 8 * 4;
@@ -137,7 +139,8 @@ __global__ void __launch_bounds__(128) k_wgrad(const __nv_bfloat16* __restrict__
   auto Xs = reinterpret_cast<__nv_bfloat16(*)[MC + KPAD]>(raw);
   auto Gs = reinterpret_cast<__nv_bfloat16(*)[MC + KPAD]>(raw + 16 * (MC + KPAD) * 2);
   auto red = reinterpret_cast<float(*)[16 * NT * 8]>(raw);
-  const int tap = blockIdx.x, ci0 = blockIdx.y * 16;
+  const int tap = blockIdx.x, ci0 = ((int)blockIdx.y / ncol) * 16;
+  const int co0 = ((int)blockIdx.y % ncol) * NT * 8;
   const int dx = tap / 9 - 1, dy = (tap / 3) % 3 - 1, dz = tap % 3 - 1;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, gid = lane >> 2, tig = lane & 3;
   float acc[NT][4];
@@ -156,7 +159,7 @@ __global__ void __launch_bounds__(128) k_wgrad(const __nv_bfloat16* __restrict__
     for (int e = threadIdx.x; e < NT * 8 * MC; e += blockDim.x) {
       const int mm = e / (NT * 8), co = e % (NT * 8);
       const long long m = mb + mm;
-      Gs[co][mm] = m < mend ? g[m * ldg + offg + co] : __float2bfloat16(0.f);
+      Gs[co][mm] = m < mend ? g[m * ldg + offg + co0 + co] : __float2bfloat16(0.f);
     }
     __syncthreads();
     const int k0 = warp * 16;
@@ -184,7 +187,7 @@ __global__ void __launch_bounds__(128) k_wgrad(const __nv_bfloat16* __restrict__
   for (int e = threadIdx.x; e < 16 * NT * 8; e += blockDim.x) {
     const float v = red[0][e] + red[1][e] + red[2][e] + red[3][e];
     const int row = e / (NT * 8), col = e % (NT * 8);
-    partials[(((long long)blockIdx.z * 27 + tap) * Cin + ci0 + row) * Cout + col] = v;
+    partials[(((long long)blockIdx.z * 27 + tap) * Cin + ci0 + row) * Cout + co0 + col] = v;
   }
 }
 
@@ -327,12 +330,14 @@ void nn_conv_wgrad(TView x, int Cin, TView g, int Cout, float* dW, float* db, fl
   const long long Mtot = (long long)B << (3 * lgD);
   const int S = std::max(1, WG_S_TARGET / (27 * (Cin / 16)));
   const long long chunk = ((Mtot + S - 1) / S + 63) / 64 * 64;
-  dim3 grid(27, Cin / 16, S);
-  // Cout in {16, 32, 64, 128}: one launch covers all output channels
-#define LAUNCH_W(NT)                                                                            \
-  k_wgrad<NT><<<grid, 128, 0, s>>>(x.p, x.ld, x.off, Cin, g.p, g.ld, g.off, Cout, partials, Mtot, \
-                                   chunk, lgD)
-  switch (Cout / 8) {
+  // 16, 32, 64 and 128 output channels in one group, others in groups of the largest of
+  // 16 and 32 that divides them
+  const int nt = Cout == 128 ? 16 : pick_nt(Cout), ncol = Cout / (nt * 8);
+  dim3 grid(27, (Cin / 16) * ncol, S);
+#define LAUNCH_W(NT)                                                                          \
+  k_wgrad<NT><<<grid, 128, 0, s>>>(x.p, x.ld, x.off, Cin, g.p, g.ld, g.off, Cout, ncol,       \
+                                   partials, Mtot, chunk, lgD)
+  switch (nt) {
     case 2: LAUNCH_W(2); break;
     case 4: LAUNCH_W(4); break;
     case 8: LAUNCH_W(8); break;
