@@ -431,6 +431,10 @@ mgfr_status mgfr_unet_grads(mgfr_ctx* ctx, float* host);
  *   op 1: out (FP32 [B D^3][Cin])  = gradient w.r.t. x for output gradient g
  *   op 2: out (FP32 [27][Cin][Cout]) = gradient w.r.t. W, db (FP32 [Cout],
  *         nullable) = gradient w.r.t. the bias; allocates its own scratch.
+ * Alignment: for the network's (Cin, Cout) pairs (in ops 0 and 1 also with the two
+ * exchanged) x and g, and out of ops 0 and 1, lie on 16-byte boundaries; for other pairs x, g
+ * and out on 4-byte boundaries, x and g of op 2 on their own 2 bytes.  MGFR_E_INVALID
+ * otherwise.
  * Runs on `stream` and returns when done. */
 mgfr_status mgfr_nn_conv3d(int op, int B, int D, int Cin, int Cout, const void* x_bf16,
                            const void* w_bf16, const float* bias, int relu, const void* g_bf16,

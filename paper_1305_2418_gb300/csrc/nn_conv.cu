@@ -14,6 +14,7 @@
 // these serve the others.  nn_wgrad_finish (the reduction of the partial dW
 // and the bias gradient) serves both.
 #include <algorithm>
+#include <cstdint>
 
 #include "nn_kernels.cuh"
 
@@ -234,10 +235,12 @@ __global__ void __launch_bounds__(256) k_wgrad_reduce(const float* __restrict__ 
 // loads) of its voxels, the block's threads of a channel group are added in
 // order, and the blocks' sums in order by one warp per channel: fixed orders,
 // short chains (one thread per (slot, channel) with 4096-element chains took
-// 78 us per full-resolution layer; this is bound by reading g).
+// 78 us per full-resolution layer; this is bound by reading g).  VEC: g lies on a 16-byte
+// boundary and the loads are of 16 bytes; else of one value (a caller's view).
 constexpr int BG_BLOCKS = 152;
 constexpr int BG_BS = 256;
 
+template <bool VEC>
 __global__ void __launch_bounds__(BG_BS) k_bias_part(const __nv_bfloat16* __restrict__ g, int ldg,
                                                      int offg, long long Mtot, int Cout,
                                                      float* __restrict__ part) {
@@ -247,12 +250,18 @@ __global__ void __launch_bounds__(BG_BS) k_bias_part(const __nv_bfloat16* __rest
   float s[8] = {};
   if (vo < vpb)
     for (long long m = (long long)blockIdx.x * vpb + vo; m < Mtot; m += (long long)gridDim.x * vpb) {
-      const uint4 q = *reinterpret_cast<const uint4*>(g + m * ldg + offg + 8 * c8);
-      const unsigned w[4] = {q.x, q.y, q.z, q.w};
+      const __nv_bfloat16* p = g + m * ldg + offg + 8 * c8;
+      if (VEC) {
+        const uint4 q = *reinterpret_cast<const uint4*>(p);
+        const unsigned w[4] = {q.x, q.y, q.z, q.w};
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        s[2 * i] += __uint_as_float(w[i] << 16);
-        s[2 * i + 1] += __uint_as_float(w[i] & 0xffff0000u);
+        for (int i = 0; i < 4; ++i) {
+          s[2 * i] += __uint_as_float(w[i] << 16);
+          s[2 * i + 1] += __uint_as_float(w[i] & 0xffff0000u);
+        }
+      } else {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) s[i] += __bfloat162float(p[i]);
       }
     }
 #pragma unroll
@@ -316,7 +325,9 @@ void nn_wgrad_finish(float* partials, int S, int Cin, int Cout, float* dW, TView
   if (!db) return;
   // the bias stages reuse the partials (read by k_wgrad_reduce before them on
   // this stream); they hold S * 27 * Cin * Cout >= 432 * Cout floats (Cin >= 16)
-  k_bias_part<<<BG_BLOCKS, BG_BS, 0, s>>>(g.p, g.ld, g.off, Mtot, Cout, partials);
+  const bool vec = (uintptr_t)(g.p + g.off) % 16 == 0 && g.ld % 8 == 0;
+  (vec ? k_bias_part<true> : k_bias_part<false>)<<<BG_BLOCKS, BG_BS, 0, s>>>(g.p, g.ld, g.off,
+                                                                            Mtot, Cout, partials);
   k_bias_sum<<<Cout, 32, 0, s>>>(partials, BG_BLOCKS, Cout, db);
 }
 

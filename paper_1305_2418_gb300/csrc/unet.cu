@@ -18,6 +18,7 @@
 // of 32 to 512 cells per side at the cell size it was trained on.
 #include <algorithm>
 #include <cmath>
+#include <cstdint>
 #include <cstdio>
 #include <cstring>
 #include <mutex>
@@ -1058,8 +1059,16 @@ mgfr_status mgfr_nn_conv3d(int op, int B, int D, int Cin, int Cout, const void* 
     return MGFR_E_INVALID;
   cudaStream_t s = (cudaStream_t)stream;
   const int lgD = lg_of(D);
-  const bool tc = (op == 0 && nn_tc_supported(Cin, Cout)) || (op == 1 && nn_tc_supported(Cout, Cin));
-  if (tc) {
+  const bool tc = (op == 0 && nn_tc_supported(Cin, Cout)) ||
+                  (op == 1 && nn_tc_supported(Cout, Cin)) ||
+                  (op == 2 && nn_tc_wgrad_supported(Cin, Cout));
+  // the tcgen05 kernels move 16 bytes of a voxel's channels at a time (in, and for ops 0 and
+  // 1 out), the mma.sync ones 4 in ops 0 and 1 and single values in op 2
+  auto on = [](const void* p, unsigned b) { return (uintptr_t)p % b == 0; };
+  const unsigned bi = tc ? 16 : (op == 2 ? 2 : 4), bo = tc && op != 2 ? 16 : 4;
+  if ((op != 1 && !on(x_bf16, bi)) || (op != 0 && !on(g_bf16, bi)) || !on(out, bo))
+    return MGFR_E_INVALID;
+  if (tc && op != 2) {
     // pack the weights for the tensor-core kernel (scratch of this call)
     ConvScratch sc;
     if (!scratch_acquire(sizeof(__nv_bfloat16) * (size_t)nn_tc_packed_size(Cin, Cout), &sc))
@@ -1094,13 +1103,12 @@ mgfr_status mgfr_nn_conv3d(int op, int B, int D, int Cin, int Cout, const void* 
     nn_conv_dgrad(TView{(__nv_bfloat16*)g_bf16, Cout, 0}, Cout, (const __nv_bfloat16*)w_bf16,
                   FView{(float*)out, Cin, 0}, Cin, 0, B, lgD, s);
   } else if (op == 2) {
-    const bool tcw = nn_tc_wgrad_supported(Cin, Cout);
-    const long long np = tcw ? nn_tc_wgrad_scratch(Cin, Cout) : nn_wgrad_scratch(Cin, Cout);
+    const long long np = tc ? nn_tc_wgrad_scratch(Cin, Cout) : nn_wgrad_scratch(Cin, Cout);
     ConvScratch sc;
     if (!scratch_acquire(sizeof(float) * (size_t)np, &sc)) return MGFR_E_OOM;
     float* part = (float*)sc.p;
     const TView xv{(__nv_bfloat16*)x_bf16, Cin, 0}, gv{(__nv_bfloat16*)g_bf16, Cout, 0};
-    if (!tcw || !nn_tc_wgrad(xv, Cin, gv, Cout, (float*)out, db, part, B, lgD, sc.err, s))
+    if (!tc || !nn_tc_wgrad(xv, Cin, gv, Cout, (float*)out, db, part, B, lgD, sc.err, s))
       nn_conv_wgrad(xv, Cin, gv, Cout, (float*)out, db, part, B, lgD, s);
     return scratch_finish(sc, s);
   } else {

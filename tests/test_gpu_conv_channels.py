@@ -55,3 +55,45 @@ def test_weight_gradient_of_any_channel_count(dev, B, D, ci, co):
         assert rel(got[:, :, c:c + 16], want_gw[:, :, c:c + 16]) <= 1e-5, c
     assert rel(db[:co], want_db) <= 1e-5
     assert bool((gw[nw:] == 7.0).all()) and bool((db[co:] == 7.0).all())
+
+
+def at_offset(t, values):
+    """The same values `values` elements off a fresh buffer's start (256-byte aligned)."""
+    flat = torch.empty(t.numel() + values, dtype=t.dtype, device=t.device)
+    v = flat[values:].view(t.shape)
+    v.copy_(t)
+    return v
+
+
+@pytest.mark.parametrize("off", [1, 2, 3, 7, 8])
+@pytest.mark.parametrize("ci,co", [(80, 32), (16, 48), (48, 64)])
+def test_gradients_of_views_at_any_element(dev, off, ci, co):
+    """Op 2 outside the network's pairs reads x and g value by value: views at any element
+    are accepted, and give what the aligned tensors give, bit by bit."""
+    r = torch.Generator(device=dev).manual_seed(off + co)
+    x = torch.randn((2, 8, 8, 8, ci), generator=r, device=dev).to(torch.bfloat16)
+    g = torch.randn((2, 8, 8, 8, co), generator=r, device=dev).to(torch.bfloat16)
+    w = torch.zeros((27, ci, co), dtype=torch.bfloat16, device=dev)
+    want_db, db = torch.empty(co, device=dev), torch.empty(co, device=dev)
+    want = mgfr.conv3d(2, x, w, g=g, db=want_db)
+    got = mgfr.conv3d(2, at_offset(x, off), w, g=at_offset(g, off), db=db)
+    assert torch.equal(got, want) and torch.equal(db, want_db)
+    assert rel(db, g.double().reshape(-1, co).sum(0)) <= 1e-5
+
+
+@pytest.mark.parametrize("ci,co,need", [(16, 16, 8), (96, 32, 8), (80, 32, 2)])
+def test_misaligned_tensors_are_refused(dev, ci, co, need):
+    """`need`: the elements of BF16 that the kernels load at a time."""
+    x = torch.zeros((1, 16, 16, 16, ci), dtype=torch.bfloat16, device=dev)
+    g = torch.zeros((1, 16, 16, 16, co), dtype=torch.bfloat16, device=dev)
+    w = torch.zeros((27, ci, co), dtype=torch.bfloat16, device=dev)
+    for off in (1, need // 2, need - 1):
+        for call in (lambda: mgfr.conv3d(0, at_offset(x, off), w),
+                     lambda: mgfr.conv3d(1, x, w, g=at_offset(g, off))):
+            with pytest.raises(mgfr.MGFRError):
+                call()
+        if need == 8:
+            for a, b in ((at_offset(x, off), g), (x, at_offset(g, off))):
+                with pytest.raises(mgfr.MGFRError):
+                    mgfr.conv3d(2, a, w, g=b)
+    assert float(mgfr.conv3d(0, at_offset(x, need), w).abs().max()) == 0.0
