@@ -952,14 +952,15 @@ mgfr_status mgfr_unet_grads(mgfr_ctx* c, float* host) {
 // error word), kept between calls: cudaMalloc and cudaFree took 0.2 ms of every
 // call.  A call owns its block from acquire to release, which come before and
 // after its work (the call waits for its stream), so blocks never serve two
-// streams or threads at once.  At most 4 blocks and 128 MB per device stay;
+// streams or threads at once; it clears the error word on its own stream, with
+// which no other stream is in order.  At most 4 blocks and 128 MB per device stay;
 // mgfr_destroy gives those of its device back.
 namespace {
 struct ConvScratch {
   int dev = 0;
   size_t bytes = 0;
   void* p = nullptr;
-  int *err = nullptr, *err_h = nullptr;  // device word (0), page-locked copy
+  int *err = nullptr, *err_h = nullptr;  // device word, page-locked copy
 };
 std::mutex g_scratch_mu;
 std::vector<ConvScratch> g_scratch;
@@ -971,9 +972,10 @@ void scratch_drop(ConvScratch& b) {
   b = ConvScratch();
 }
 
-bool scratch_acquire(size_t bytes, ConvScratch* out) {
+mgfr_status scratch_acquire(size_t bytes, cudaStream_t s, ConvScratch* out) {
   int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) return false;
+  if (cudaGetDevice(&dev) != cudaSuccess) return MGFR_E_CUDA;
+  ConvScratch b;
   {
     std::lock_guard<std::mutex> lk(g_scratch_mu);
     int best = -1;
@@ -982,23 +984,27 @@ bool scratch_acquire(size_t bytes, ConvScratch* out) {
           (best < 0 || g_scratch[i].bytes < g_scratch[best].bytes))
         best = (int)i;
     if (best >= 0) {
-      *out = g_scratch[best];
+      b = g_scratch[best];
       g_scratch.erase(g_scratch.begin() + best);
-      return true;
     }
   }
-  ConvScratch b;
-  b.dev = dev;
-  b.bytes = bytes;
-  if (cudaMalloc(&b.p, bytes) != cudaSuccess || cudaMalloc(&b.err, sizeof(int)) != cudaSuccess ||
-      cudaMallocHost(&b.err_h, sizeof(int)) != cudaSuccess ||
-      cudaMemset(b.err, 0, sizeof(int)) != cudaSuccess) {
+  if (!b.p) {
+    b.dev = dev;
+    b.bytes = bytes;
+    if (cudaMalloc(&b.p, bytes) != cudaSuccess || cudaMalloc(&b.err, sizeof(int)) != cudaSuccess ||
+        cudaMallocHost(&b.err_h, sizeof(int)) != cudaSuccess) {
+      (void)cudaGetLastError();
+      scratch_drop(b);
+      return MGFR_E_OOM;
+    }
+  }
+  if (cudaMemsetAsync(b.err, 0, sizeof(int), s) != cudaSuccess) {
     (void)cudaGetLastError();
     scratch_drop(b);
-    return false;
+    return MGFR_E_CUDA;
   }
   *out = b;
-  return true;
+  return MGFR_OK;
 }
 
 void scratch_release(ConvScratch& b) {
@@ -1028,10 +1034,6 @@ mgfr_status scratch_finish(ConvScratch& b, cudaStream_t s) {
     return MGFR_E_CUDA;
   }
   const int e = *b.err_h;
-  if (e && cudaMemset(b.err, 0, sizeof(int)) != cudaSuccess) {
-    scratch_drop(b);
-    return MGFR_E_CUDA;
-  }
   scratch_release(b);
   return e ? MGFR_E_TIMEOUT : MGFR_OK;
 }
@@ -1071,8 +1073,9 @@ mgfr_status mgfr_nn_conv3d(int op, int B, int D, int Cin, int Cout, const void* 
   if (tc && op != 2) {
     // pack the weights for the tensor-core kernel (scratch of this call)
     ConvScratch sc;
-    if (!scratch_acquire(sizeof(__nv_bfloat16) * (size_t)nn_tc_packed_size(Cin, Cout), &sc))
-      return MGFR_E_OOM;
+    const mgfr_status rs =
+        scratch_acquire(sizeof(__nv_bfloat16) * (size_t)nn_tc_packed_size(Cin, Cout), s, &sc);
+    if (rs != MGFR_OK) return rs;
     __nv_bfloat16* wp = (__nv_bfloat16*)sc.p;
     nn_tc_pack((const __nv_bfloat16*)w_bf16, Cin, Cout, op, wp, s);
     TcArgs a{};
@@ -1105,7 +1108,8 @@ mgfr_status mgfr_nn_conv3d(int op, int B, int D, int Cin, int Cout, const void* 
   } else if (op == 2) {
     const long long np = tc ? nn_tc_wgrad_scratch(Cin, Cout) : nn_wgrad_scratch(Cin, Cout);
     ConvScratch sc;
-    if (!scratch_acquire(sizeof(float) * (size_t)np, &sc)) return MGFR_E_OOM;
+    const mgfr_status rs = scratch_acquire(sizeof(float) * (size_t)np, s, &sc);
+    if (rs != MGFR_OK) return rs;
     float* part = (float*)sc.p;
     const TView xv{(__nv_bfloat16*)x_bf16, Cin, 0}, gv{(__nv_bfloat16*)g_bf16, Cout, 0};
     if (!tc || !nn_tc_wgrad(xv, Cin, gv, Cout, (float*)out, db, part, B, lgD, sc.err, s))
