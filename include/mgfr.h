@@ -430,7 +430,10 @@ mgfr_status mgfr_unet_grads(mgfr_ctx* ctx, float* host);
  *   op 0: out (BF16 [B D^3][Cout]) = relu?(conv(x) + bias)   (bias nullable)
  *   op 1: out (FP32 [B D^3][Cin])  = gradient w.r.t. x for output gradient g
  *   op 2: out (FP32 [27][Cin][Cout]) = gradient w.r.t. W, db (FP32 [Cout],
- *         nullable) = gradient w.r.t. the bias; allocates its own scratch.
+ *         nullable) = gradient w.r.t. the bias.
+ * Scratch (packed weights, partial sums) comes from blocks that the library keeps between
+ * calls, at most 4 and 128 MB per device; destroying a context gives those of its device
+ * back.
  * Alignment: for the network's (Cin, Cout) pairs (in ops 0 and 1 also with the two
  * exchanged) x and g, and out of ops 0 and 1, lie on 16-byte boundaries; for other pairs x, g
  * and out on 4-byte boundaries, x and g of op 2 on their own 2 bytes.  MGFR_E_INVALID

@@ -48,3 +48,30 @@ def test_error_word_is_in_the_callers_stream_order(dev, empty_scratch):
     torch.cuda.synchronize()
     for a, b in zip(want, got):
         assert all(torch.equal(p, q) for p, q in zip(a, b))
+
+
+def test_largest_blocks_are_kept(dev, empty_scratch):
+    """Calls in ascending size: the block that stays is the one that serves them all, so a
+    repeated call of the largest allocates nothing.  192 -> 64 sums its weight gradient
+    over 43 partials of 27 x 192 x 64 (57 MB), beside four smaller blocks."""
+    small = [(16, 16), (16, 32), (32, 32), (32, 64)]
+    for ci, co in small:
+        x, w, _ = layer(dev, ci, co)
+        mgfr.conv3d(0, x, w)
+    x, w, g = layer(dev, 192, 64)
+    mgfr.conv3d(2, x, w, g=g)
+    torch.cuda.synchronize()
+    big = 43 * 27 * 192 * 64 * 4
+    free0 = torch.cuda.mem_get_info(dev)[0]
+    mgfr.Solver(0).close()  # what it gives back was kept
+    kept = torch.cuda.mem_get_info(dev)[0] - free0
+    assert kept >= big
+    # and the limits hold over many sizes, two of them above half of the limit
+    for ci, co in small + [(192, 64), (128, 128), (64, 128), (192, 64), (96, 32), (48, 16)]:
+        x, w, g = layer(dev, ci, co)
+        mgfr.conv3d(2, x, w, g=g)
+    torch.cuda.synchronize()
+    free1 = torch.cuda.mem_get_info(dev)[0]
+    mgfr.Solver(0).close()
+    kept = torch.cuda.mem_get_info(dev)[0] - free1
+    assert big <= kept <= (128 << 20) + 8 * (2 << 20)  # 2 MB: an allocation's granularity
