@@ -952,13 +952,14 @@ mgfr_status mgfr_unet_grads(mgfr_ctx* c, float* host) {
 // error word), kept between calls: cudaMalloc and cudaFree took 0.2 ms of every
 // call.  A call owns its block from acquire to release, which come before and
 // after its work (the call waits for its stream), so blocks never serve two
-// streams or threads at once; it clears the error word on its own stream, with
-// which no other stream is in order.  At most 4 blocks and 128 MB per device stay,
-// the largest ones (a block serves every call that needs no more, so one caller's calls
-// come to rest on the largest of their sizes, at most 57 MB); mgfr_destroy gives those
-// of its device back.  (When the first four blocks stayed, a call larger than they
-// allocated and freed its own each time: weight gradients on 16^3 after four small layers
-// 225-260 us, now 44-64.)
+// streams or threads at once; it clears an error word that is not known to be 0
+// on its own stream, with which no other stream is in order.  At most 4 blocks
+// and 128 MB per device stay, the largest ones (a block serves every call that
+// needs no more, so one caller's calls come to rest on the largest of their
+// sizes, at most 57 MB); mgfr_destroy gives those of its device back.  (When the
+// first four blocks stayed, a call larger than they allocated and freed its own
+// each time: weight gradients on 16^3 after four small layers 225-260 us, now
+// 44-64.)
 namespace {
 constexpr size_t kScratchBlocks = 4, kScratchBytes = (size_t)128 << 20;
 struct ConvScratch {
@@ -966,6 +967,7 @@ struct ConvScratch {
   size_t bytes = 0;
   void* p = nullptr;
   int *err = nullptr, *err_h = nullptr;  // device word, page-locked copy
+  bool clear = false;                    // the word was last read as 0 (kernels only set it)
 };
 std::mutex g_scratch_mu;
 std::vector<ConvScratch> g_scratch;
@@ -1003,7 +1005,7 @@ mgfr_status scratch_acquire(size_t bytes, cudaStream_t s, ConvScratch* out) {
       return MGFR_E_OOM;
     }
   }
-  if (cudaMemsetAsync(b.err, 0, sizeof(int), s) != cudaSuccess) {
+  if (!b.clear && cudaMemsetAsync(b.err, 0, sizeof(int), s) != cudaSuccess) {
     (void)cudaGetLastError();
     scratch_drop(b);
     return MGFR_E_CUDA;
@@ -1044,6 +1046,7 @@ mgfr_status scratch_finish(ConvScratch& b, cudaStream_t s) {
     return MGFR_E_CUDA;
   }
   const int e = *b.err_h;
+  b.clear = e == 0;
   scratch_release(b);
   return e ? MGFR_E_TIMEOUT : MGFR_OK;
 }
