@@ -689,9 +689,11 @@ static mgfr_status launch_batch(mgfr_ctx* c, BatchWork* B, const BArgs& A, int t
     c->launches += 1;
     return MGFR_OK;
   }
+  // the launch and its settings; the sizes are the workspace's (batch_release drops the
+  // graph with it)
   char key[512];
-  std::snprintf(key, sizeof(key), "%s|%d|%d|%d|%d|%d|%d|%.17g|%.17g|%.17g|%lld", B->sig.c_str(),
-                threads, grid, A.n_pre, A.n_post, A.linear, A.max_cycles, (double)A.cap32, A.tol, A.sw,
+  std::snprintf(key, sizeof(key), "%d|%d|%d|%d|%d|%d|%.17g|%.17g|%.17g|%lld", threads, grid,
+                A.n_pre, A.n_post, A.linear, A.max_cycles, (double)A.cap32, A.tol, A.sw,
                 A.max_spins);
   if (!B->gx || B->gkey != key) {
     if (B->gx) cudaGraphExecDestroy(B->gx);

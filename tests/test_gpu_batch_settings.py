@@ -15,7 +15,7 @@ def dev():
     return torch.device("cuda:0")
 
 
-@pytest.mark.parametrize("N,count", [(8, 200), (16, 130), (32, 1)])
+@pytest.mark.parametrize("N,count", [(8, 400), (16, 180), (32, 1)])
 def test_settings_of_a_call_are_its_own(dev, N, count):
     """A tolerance, and a limit on the cycles, set between two calls on the same sizes,
     however many, hold for the next: each solve meets the tolerance asked for, by the
@@ -34,6 +34,12 @@ def test_settings_of_a_call_are_its_own(dev, N, count):
         for d, o in list(zip(ds, outs))[::37]:
             r, f = residual(o["u"], d, box, fr0)
             assert r <= 1.01 * tol * f + 1e-13 * f * (N / 6.28) ** 2
+    # other smoothing: not the cycle counts of before
+    s.set_config(tol_rel=1e-9, n_pre=1, n_post=1)
+    less, st = s.batch_solve(ds, [box] * count, [fr0] * count)
+    assert st == mgfr.MGFR_OK
+    assert sum(o["stats"]["vcycles"] + o["stats"]["outer_iters"] for o in less) \
+        > sum(o["stats"]["vcycles"] + o["stats"]["outer_iters"] for o in outs)
     s.set_config(tol_rel=1e-12, max_vcycles=2)
     outs, st = s.batch_solve(ds, [box] * count, [fr0] * count, allow_noconverge=True)
     assert st == mgfr.MGFR_E_NOCONVERGE
