@@ -478,9 +478,12 @@ __global__ void __launch_bounds__(512, 2) k_batch(BArgs A) {
         const double rm = __longlong_as_double((long long)q.acc_max);
         q.acc_ss = 0.0;
         q.acc_max = 0ULL;
+        // at the limit on the cycles a solve in mode A still goes through the transition,
+        // which makes its FP32 iterate the result and forms that one's residual
         if (q.mode == BM_A) {
           q.cyclesA++;
-          if (!(r == r) || r <= A.sw * q.ref || (q.rprev > 0.0 && r > 0.7 * q.rprev))
+          if (!(r == r) || r <= A.sw * q.ref || (q.rprev > 0.0 && r > 0.7 * q.rprev) ||
+              q.cyclesA + q.cyclesB >= A.max_cycles)
             q.mode = BM_TRANS;
           q.rprev = r;
         } else if (q.mode == BM_B) {
@@ -488,14 +491,13 @@ __global__ void __launch_bounds__(512, 2) k_batch(BArgs A) {
           const bool rose = !(r < q.r);
           q.r = r;
           q.rmax = rm;
-          if (r <= q.target) {
+          if (r <= q.target || q.cyclesA + q.cyclesB >= A.max_cycles) {
             q.mode = BM_DONE;
           } else if (rose) {
             q.mode = BM_A;  // back to nonlinear FP32 cycles from u32 = fp32(u)
             q.rprev = -1.0;
           }
         }
-        if (q.mode != BM_DONE && q.cyclesA + q.cyclesB >= A.max_cycles) q.mode = BM_DONE;
       }
     }
     if (!gsync(A)) return;
@@ -524,7 +526,7 @@ __global__ void __launch_bounds__(512, 2) k_batch(BArgs A) {
           const double r = sqrt(q.acc_ss);
           q.r = r;
           q.rmax = __longlong_as_double((long long)q.acc_max);
-          q.mode = r <= q.target ? BM_DONE : BM_B;
+          q.mode = r <= q.target || q.cyclesA + q.cyclesB >= A.max_cycles ? BM_DONE : BM_B;
           q.acc_ss = 0.0;
           q.acc_max = 0ULL;
         }

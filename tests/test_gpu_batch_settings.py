@@ -47,6 +47,45 @@ def test_settings_of_a_call_are_its_own(dev, N, count):
     s.close()
 
 
+@pytest.mark.parametrize("tol", [1e-9, 1e-12])  # pairs of floats, FP64
+@pytest.mark.parametrize("most", [1, 2, 3, 5, 6])
+def test_a_solve_at_its_limit_returns_its_last_iterate(dev, tol, most):
+    """max_vcycles reached in the FP32 cycles (the first five or so) or after them: u, f_R and
+    the residual belong to each other, the residual falls with the cycles, and the verdict
+    is the residual's."""
+    box, fr0, N = 100.0, [1e-4, 1e-5, 1e-6], 32
+    ds = [torch.from_numpy(synth.lognormal_delta(N, box, 1.5, 900 + i)).to(dev) for i in range(3)]
+    s = mgfr.Solver(0, precision=mgfr.PREC_MIXED, tol_rel=tol, max_vcycles=most)
+    outs, st = s.batch_solve(ds, [box] * 3, fr0, want_u=True, allow_noconverge=True)
+    s.close()
+    met = []
+    for d, q, o in zip(ds, fr0, outs):
+        t = o["stats"]
+        r, f = residual(o["u"], d, box, q)
+        assert t["vcycles"] + t["outer_iters"] <= most
+        assert t["f_l2"] == pytest.approx(f, rel=1e-12)
+        # the stored residual is FP32's rounding of an FP64 (48-bit) one
+        assert t["res_l2_final"] == pytest.approx(r, rel=1e-5, abs=1e-13 * f * (N / 6.28) ** 2)
+        assert float((o["fr"] / (-q * torch.exp(o["u"])) - 1.0).abs().max()) <= 1e-12
+        assert float(o["u"].abs().max()) > 0.0 and t["res_l2_final"] < 0.3 ** most * t["res_l2_init"]
+        met.append(t["res_l2_final"] <= tol * t["f_l2"])
+    assert st == (mgfr.MGFR_OK if all(met) else mgfr.MGFR_E_NOCONVERGE)
+
+
+def test_a_loose_tolerance_met_in_the_last_cycle_allowed(dev):
+    """Met by the FP32 cycles alone, at the limit."""
+    box, N = 100.0, 32
+    d = torch.from_numpy(synth.lognormal_delta(N, box, 1.5, 900)).to(dev)
+    s = mgfr.Solver(0, precision=mgfr.PREC_MIXED, tol_rel=0.1)
+    for most in (1, 2, 3):
+        s.set_config(max_vcycles=most)
+        outs, st = s.batch_solve([d], [box], [1e-5], want_u=True, allow_noconverge=True)
+        r, f = residual(outs[0]["u"], d, box, 1e-5)
+        assert (st == mgfr.MGFR_OK) == (r <= 0.1 * f)
+    assert st == mgfr.MGFR_OK  # three cycles leave less than a tenth
+    s.close()
+
+
 def residual(u, delta, box, fr0, om=0.3):
     """(||f - L(u)||, ||f||) of the discrete equation for n = 1, a = 1 in FP64."""
     N = u.shape[0]
