@@ -40,9 +40,22 @@
 #include <algorithm>
 #include <cstdint>
 
+#include "device_once.h"
 #include "nn_kernels.cuh"
 
 namespace {
+
+// opt in to 227 KB of shared memory per CTA, once per device and kernel; a launch on a
+// device that refused fails, and its caller reads the error
+template <class K>
+void smem_opt_in(DeviceOnce& once, K kernel) {
+  int dev = -1;
+  cudaGetDevice(&dev);
+  once(dev, [&] {
+    return (int)cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     227 * 1024);
+  });
+}
 
 constexpr int TC_THREADS = 128;
 constexpr int TC_M = 128;
@@ -550,12 +563,8 @@ void launch_wgrad(TView x, TView g, int lgD, long long Mtot, float* part, int* e
   const int k = 512 / cols;
   const size_t cap = 233472 / (k + 1) - 1024 + 16;
   const size_t smem = need > cap ? need : cap;
-  static bool attr = false;
-  if (!attr) {
-    cudaFuncSetAttribute(k_wgrad_tc<CI, CO>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         227 * 1024);
-    attr = true;
-  }
+  static DeviceOnce once;
+  smem_opt_in(once, k_wgrad_tc<CI, CO>);
   int S;
   long long chunk;
   wgrad_split(CO, Mtot, &S, &chunk);
@@ -757,12 +766,8 @@ void launch_halo(const TcArgs& a, cudaStream_t s) {
   constexpr int per_sm = fit < mem ? fit : mem;
   constexpr int cap = 233472 / (per_sm + 1) - 1024 + 16, smem = need > cap ? need : cap;
   static_assert(per_sm >= 1 && smem <= 227 * 1024, "one CTA fits");
-  static bool attr = false;
-  if (!attr) {
-    cudaFuncSetAttribute(k_conv_halo<KC, NC, DG, TX>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         227 * 1024);
-    attr = true;
-  }
+  static DeviceOnce once;
+  smem_opt_in(once, k_conv_halo<KC, NC, DG, TX>);
   const int tiles = (int)(a.Mtot / (TX * 16 * 8));
   k_conv_halo<KC, NC, DG, TX><<<(unsigned)std::min(tiles, 152 * per_sm), HT, smem, s>>>(
       a.x, a.ldx, a.offx, a.Wp, a.bias, a.relu, a.y, a.ldy, a.offy, a.gx, a.ldg, a.offg,
@@ -934,12 +939,8 @@ void launch_halo_s(const TcArgs& a, cudaStream_t s) {
   const int k = 512 / cols;
   const size_t cap = 233472 / (k + 1) - 1024 + 16;
   const size_t smem = need > cap ? need : cap;
-  static bool attr = false;
-  if (!attr) {
-    cudaFuncSetAttribute(k_conv_halo_s<KC, NC, DG, TX>,
-                         cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
-    attr = true;
-  }
+  static DeviceOnce once;
+  smem_opt_in(once, k_conv_halo_s<KC, NC, DG, TX>);
   const long long tiles = a.Mtot / (TX * 16 * 8);
   k_conv_halo_s<KC, NC, DG, TX><<<(unsigned)tiles, HT, smem, s>>>(
       a.x, a.ldx, a.offx, a.Wp, a.bias, a.relu, a.y, a.ldy, a.offy, a.gx, a.ldg, a.offg,
@@ -1162,12 +1163,8 @@ void launch_wgrad_halo(TView x, TView g, int B, int lgD, float* part, int* err, 
   const size_t need = (size_t)W::STAGES * W::ST + W::ACC + W::STAGES * 8 + 16;
   const size_t cap = 233472 / (512 / W::TCOLS + 1) - 1024 + 16;
   const size_t smem = need > cap ? need : cap;
-  static bool attr = false;
-  if (!attr) {
-    cudaFuncSetAttribute(k_wgrad_halo<CI, CO, PL, ND>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         227 * 1024);
-    attr = true;
-  }
+  static DeviceOnce once;
+  smem_opt_in(once, k_wgrad_halo<CI, CO, PL, ND>);
   const int ntile = (B << (3 * lgD - 7)) / PL;
   const int S0 = std::max(1, WG_HALO_CTAS / (9 / ND));
   const int chunk = (ntile + S0 - 1) / S0, S = (ntile + chunk - 1) / chunk;
@@ -1207,12 +1204,8 @@ void launch_tc(const TcArgs& a, cudaStream_t s) {
   const int k = 512 / cols;
   const size_t cap = 233472 / (k + 1) - 1024 + 16;
   const size_t smem = need > cap ? need : cap;
-  static bool attr = false;
-  if (!attr) {
-    cudaFuncSetAttribute(k_conv_tc<KC, NC, DG>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         227 * 1024);
-    attr = true;
-  }
+  static DeviceOnce once;
+  smem_opt_in(once, k_conv_tc<KC, NC, DG>);
   const unsigned grid = (unsigned)((a.Mtot + TC_M - 1) / TC_M);
   k_conv_tc<KC, NC, DG><<<grid, HT, smem, s>>>(
       a.x, a.ldx, a.offx, a.Wp, a.bias, a.relu, a.y, a.ldy, a.offy, a.gx, a.ldg, a.offg,
