@@ -764,7 +764,10 @@ mgfr_status mgfr_batch_solve(mgfr_ctx* c, int nsolves, const mgfr_batch_item* it
   auto buf = [&](size_t bytes) -> void* {
     if (bi < B->bufs.size()) return B->bufs[bi++];
     void* p = nullptr;
-    if (cudaMalloc(&p, bytes) != cudaSuccess) return nullptr;
+    if (cudaMalloc(&p, bytes) != cudaSuccess) {
+      (void)cudaGetLastError();
+      return nullptr;
+    }
     B->bufs.push_back(p);
     ++bi;
     return p;

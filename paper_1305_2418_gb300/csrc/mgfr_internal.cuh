@@ -186,9 +186,11 @@ void pm_free(mgfr_ctx* c);
 #define MG_CK(ctx, call)                                                                  \
   do {                                                                                    \
     cudaError_t e_ = (call);                                                              \
-    if (e_ != cudaSuccess)                                                                \
+    if (e_ != cudaSuccess) {                                                              \
+      (void)cudaGetLastError(); /* reported here: not by a later call again */            \
       return set_err((ctx), e_ == cudaErrorMemoryAllocation ? MGFR_E_OOM : MGFR_E_CUDA,   \
                      std::string(#call) + ": " + cudaGetErrorString(e_));                 \
+    }                                                                                     \
   } while (0)
 
 static inline unsigned nblocks(long long n, int bs) { return (unsigned)((n + bs - 1) / bs); }

@@ -215,18 +215,9 @@ static void drop_graphs(mgfr_ctx* c) {
   for (int g = 0; g < 5; ++g) prof_clear(c, g);
 }
 
-// Allocate the dense hierarchy N, N/2, ..., 4 (FP64 arrays always; FP32 ones
-// for the mixed form).
-static mgfr_status ensure_dense(mgfr_ctx* c, int N, bool mixed) {
-  DenseHier& H = c->dh;
-  if (H.N == N && (H.mixed || !mixed)) return MGFR_OK;
-  mgfr_status ps = mg32_prepare(c);
-  if (ps != MGFR_OK) return ps;
-  drop_graphs(c);
-  free_dense(H);
-  c->u_prev_N = 0;
-  H.N = N;
-  H.mixed = mixed;
+// The arrays of the dense hierarchy N, N/2, ..., 4 (f and the double-float copy
+// of it for the mixed form only).
+static mgfr_status alloc_dense(mgfr_ctx* c, DenseHier& H, int N, bool mixed) {
   int lg = 0;
   while ((1 << lg) < N) ++lg;
   H.nlev = lg - 1;  // N ... 4
@@ -250,7 +241,22 @@ static mgfr_status ensure_dense(mgfr_ctx* c, int N, bool mixed) {
   if (mixed) MG_CK(c, cudaMalloc(&H.fdf, sizeof(double) * (size_t)H.L[0].n));
   MG_CK(c, cudaMalloc(&H.partials, sizeof(double) * 2 * H.nparts));
   MG_CK(c, cudaMalloc(&H.scal, sizeof(double) * 16));
+  H.N = N;
+  H.mixed = mixed;
   return MGFR_OK;
+}
+
+static mgfr_status ensure_dense(mgfr_ctx* c, int N, bool mixed) {
+  DenseHier& H = c->dh;
+  if (H.N == N && (H.mixed || !mixed)) return MGFR_OK;
+  mgfr_status ps = mg32_prepare(c);
+  if (ps != MGFR_OK) return ps;
+  drop_graphs(c);
+  free_dense(H);
+  c->u_prev_N = 0;
+  const mgfr_status rs = alloc_dense(c, H, N, mixed);
+  if (rs != MGFR_OK) free_dense(H);  // the next call must not take a part for the whole
+  return rs;
 }
 
 static void set_spacing(DenseHier& H, double box) {

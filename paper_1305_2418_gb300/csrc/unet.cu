@@ -457,18 +457,15 @@ static mgfr_status unet_alloc(mgfr_ctx* c, UNet* U, int B, int lgD) {
   if (U->B == B && U->lgD == lgD) return MGFR_OK;
   unet_free_bufs(U);
   const long long M0 = (long long)B << (3 * lgD), M1 = M0 >> 3, M2 = M1 >> 3, M3 = M2 >> 3;
-  auto bf = [&](long long n) -> __nv_bfloat16* {
+  bool ok = true;
+  auto bytes = [&](size_t n) -> void* {
     void* p = nullptr;
-    if (cudaMalloc(&p, sizeof(__nv_bfloat16) * (size_t)n) != cudaSuccess) return nullptr;
-    U->bufs.push_back(p);
-    return (__nv_bfloat16*)p;
+    ok = ok && cudaMalloc(&p, n) == cudaSuccess;
+    if (p) U->bufs.push_back(p);
+    return p;
   };
-  auto f = [&](long long n) -> float* {
-    void* p = nullptr;
-    if (cudaMalloc(&p, sizeof(float) * (size_t)n) != cudaSuccess) return nullptr;
-    U->bufs.push_back(p);
-    return (float*)p;
-  };
+  auto bf = [&](long long n) { return (__nv_bfloat16*)bytes(sizeof(__nv_bfloat16) * (size_t)n); };
+  auto f = [&](long long n) { return (float*)bytes(sizeof(float) * (size_t)n); };
   U->X0 = bf(M0 * 16);
   U->E1a = bf(M0 * 16);
   U->CAT1 = bf(M0 * 48);
@@ -515,15 +512,13 @@ static mgfr_status unet_alloc(mgfr_ctx* c, UNet* U, int B, int lgD) {
   U->wpart = f(std::max(wn, 17LL * 1024));
   U->bpart = f(128LL * kBiasBlocks);
   U->ffr0 = bf(4096);
-  void* p = nullptr;
-  if (cudaMalloc(&p, sizeof(double) * 1024) != cudaSuccess) return set_err(c, MGFR_E_OOM, "unet");
-  U->bufs.push_back(p);
-  U->lossp = (double*)p;
-  if (cudaMalloc(&p, sizeof(double) * 4096) != cudaSuccess) return set_err(c, MGFR_E_OOM, "unet");
-  U->bufs.push_back(p);
-  U->fr0d = (double*)p;
-  for (void* q : U->bufs)
-    if (!q) return set_err(c, MGFR_E_OOM, "U-Net activation allocation failed");
+  U->lossp = (double*)bytes(sizeof(double) * 1024);
+  U->fr0d = (double*)bytes(sizeof(double) * 4096);
+  if (!ok) {
+    (void)cudaGetLastError();
+    unet_free_bufs(U);
+    return set_err(c, MGFR_E_OOM, "U-Net activation allocation failed");
+  }
   U->B = B;
   U->lgD = lgD;
   return MGFR_OK;
@@ -720,10 +715,7 @@ static mgfr_status tc_check(mgfr_ctx* c, UNet* U) {
   return MGFR_OK;
 }
 
-static mgfr_status unet_make(mgfr_ctx* c, unsigned long long seed) {
-  unet_free(c);
-  UNet* U = new UNet();
-  c->unet = U;
+static mgfr_status unet_fill(mgfr_ctx* c, UNet* U, unsigned long long seed) {
   long long off = 0, boff = 0;
   for (int i = 0; i < 14; ++i) {
     U->woff[i] = off;
@@ -761,6 +753,15 @@ static mgfr_status unet_make(mgfr_ctx* c, unsigned long long seed) {
   refresh_bf16(c, U);
   MG_CK(c, cudaStreamSynchronize(c->s));
   return MGFR_OK;
+}
+
+static mgfr_status unet_make(mgfr_ctx* c, unsigned long long seed) {
+  unet_free(c);
+  UNet* U = new UNet();
+  c->unet = U;
+  const mgfr_status rs = unet_fill(c, U, seed);
+  if (rs != MGFR_OK) unet_free(c);  // no network rather than a part of one
+  return rs;
 }
 
 static const char kUnetTag[9] = "MGFRUNT1";
