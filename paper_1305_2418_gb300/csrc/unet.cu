@@ -709,9 +709,26 @@ static mgfr_status tc_check(mgfr_ctx* c, UNet* U) {
   int e = 0;
   MG_CK(c, cudaMemcpy(&e, U->tc_err, sizeof(int), cudaMemcpyDeviceToHost));
   if (e) {
-    MG_CK(c, cudaMemset(U->tc_err, 0, sizeof(int)));
+    MG_CK(c, cudaMemsetAsync(U->tc_err, 0, sizeof(int), c->s));
     return set_err(c, MGFR_E_TIMEOUT, "a bounded wait in a tensor-core convolution gave up");
   }
+  return MGFR_OK;
+}
+
+// The parameters (nparam floats) from the host, with Adam's moments at zero where
+// `fresh`, and the BF16 copies; on the context's stream, whose kernels are in no order
+// with the legacy default stream's copies and memsets.  Waits for it.
+static mgfr_status unet_set(mgfr_ctx* c, UNet* U, const float* host, bool fresh) {
+  const size_t bytes = sizeof(float) * (size_t)U->nparam;
+  MG_CK(c, cudaSetDevice(c->device));
+  MG_CK(c, cudaMemcpyAsync(U->P, host, bytes, cudaMemcpyHostToDevice, c->s));
+  if (fresh) {
+    MG_CK(c, cudaMemsetAsync(U->M1, 0, bytes, c->s));
+    MG_CK(c, cudaMemsetAsync(U->M2, 0, bytes, c->s));
+    U->step = 0;
+  }
+  refresh_bf16(c, U);
+  MG_CK(c, cudaStreamSynchronize(c->s));
   return MGFR_OK;
 }
 
@@ -737,7 +754,7 @@ static mgfr_status unet_fill(mgfr_ctx* c, UNet* U, unsigned long long seed) {
   MG_CK(c, cudaMalloc(&U->Wtf, sizeof(__nv_bfloat16) * boff));
   MG_CK(c, cudaMalloc(&U->Wtd, sizeof(__nv_bfloat16) * boff));
   MG_CK(c, cudaMalloc(&U->tc_err, sizeof(int)));
-  MG_CK(c, cudaMemset(U->tc_err, 0, sizeof(int)));
+  MG_CK(c, cudaMemsetAsync(U->tc_err, 0, sizeof(int), c->s));
   // He-normal initialisation from a seeded generator (host), zero biases
   std::vector<float> h((size_t)off, 0.f);
   std::mt19937_64 rng(seed);
@@ -747,12 +764,7 @@ static mgfr_status unet_fill(mgfr_ctx* c, UNet* U, unsigned long long seed) {
   }
   // the head starts at zero: the first prediction is u = 0 (the zero start),
   // so early steps do not push the network into saturation
-  MG_CK(c, cudaMemcpy(U->P, h.data(), sizeof(float) * off, cudaMemcpyHostToDevice));
-  MG_CK(c, cudaMemset(U->M1, 0, sizeof(float) * off));
-  MG_CK(c, cudaMemset(U->M2, 0, sizeof(float) * off));
-  refresh_bf16(c, U);
-  MG_CK(c, cudaStreamSynchronize(c->s));
-  return MGFR_OK;
+  return unet_set(c, U, h.data(), true);
 }
 
 static mgfr_status unet_make(mgfr_ctx* c, unsigned long long seed) {
@@ -916,13 +928,7 @@ mgfr_status mgfr_unet_load(mgfr_ctx* c, const char* path) {
   }
   std::fclose(f);
   if (!ok) return set_err(c, MGFR_E_INVALID, "truncated network parameter file");
-  MG_CK(c, cudaMemcpy(U->P, h.data(), sizeof(float) * h.size(), cudaMemcpyHostToDevice));
-  MG_CK(c, cudaMemset(U->M1, 0, sizeof(float) * h.size()));
-  MG_CK(c, cudaMemset(U->M2, 0, sizeof(float) * h.size()));
-  U->step = 0;
-  refresh_bf16(c, U);
-  MG_CK(c, cudaStreamSynchronize(c->s));
-  return MGFR_OK;
+  return unet_set(c, U, h.data(), true);
 }
 
 mgfr_status mgfr_unet_params(mgfr_ctx* c, int set, float* host, long long* count) {
@@ -930,13 +936,8 @@ mgfr_status mgfr_unet_params(mgfr_ctx* c, int set, float* host, long long* count
   UNet* U = (UNet*)c->unet;
   if (count) *count = U->nparam;
   if (!host) return MGFR_OK;
-  if (set) {
-    MG_CK(c, cudaMemcpy(U->P, host, sizeof(float) * U->nparam, cudaMemcpyHostToDevice));
-    refresh_bf16(c, U);
-    MG_CK(c, cudaStreamSynchronize(c->s));
-  } else {
-    MG_CK(c, cudaMemcpy(host, U->P, sizeof(float) * U->nparam, cudaMemcpyDeviceToHost));
-  }
+  if (set) return unet_set(c, U, host, false);
+  MG_CK(c, cudaMemcpy(host, U->P, sizeof(float) * U->nparam, cudaMemcpyDeviceToHost));
   return MGFR_OK;
 }
 
