@@ -28,7 +28,13 @@
  *    [Np][3].
  *  - Memory: every pointer named *_dev is device memory owned by the caller;
  *    it must stay valid until the call returns.  The library allocates its
- *    own workspaces inside the context (freed by mgfr_destroy).  Work runs on
+ *    own workspaces inside the context (freed by mgfr_destroy): a dense grid
+ *    takes 43 bytes per cell in the FP64 form and 55 in the mixed form, a
+ *    particle-mesh potential 29 per cell of its grid and its force 32 more.  The
+ *    arrays of refined levels (about 140 bytes per cell) are kept from one
+ *    particle solve to the next while they are at most twice too large, and made
+ *    1/16 larger than asked for; where an allocation of the same context finds
+ *    no memory this reserve is given back first.  Work runs on
  *    the context's stream (given at mgfr_create; 0 = legacy default stream)
  *    and every solve call returns only after its results are written.
  *  - Errors: every call returns an mgfr_status and never aborts; the text of

@@ -22,6 +22,7 @@
 #include <cmath>
 #include <cstring>
 #include <type_traits>
+#include <type_traits>
 #include <vector>
 
 #include "amr.cuh"
@@ -932,27 +933,33 @@ __global__ void k_oct_force(const double* __restrict__ E, const int* __restrict_
 
 static AmrWork* W(mgfr_ctx* c) { return (AmrWork*)c->amr; }
 
-static void free_level(AmrLevel& L) {
-  void* ps[] = {L.son,  L.refined, L.count,  L.opos, L.pcell,   L.nbr,     L.mass,
-                L.w,    L.wE,      L.wf,     L.wold, L.mask,    L.ghost,   L.ghostE,
-                L.acc,  L.pnbr,    L.w32,    L.wf32,    L.wold32,  L.ghost32, L.gface,
-                L.olist,  L.acc32, L.act};
-  for (void* p : ps)
+// f(array, elements) for every array of level l with n cells, no octs and ng ghost faces
+// (u, E and f of level 0 are the dense workspace's)
+template <class F>
+static void level_arrays(AmrLevel& L, int l, long long n, long long no, long long ng, F f) {
+  f(L.son, n), f(L.refined, n), f(L.count, n), f(L.mass, n);
+  f(L.w, n), f(L.wE, n), f(L.wf, n), f(L.wold, n), f(L.mask, n), f(L.act, n);
+  f(L.w32, n), f(L.wf32, n), f(L.wold32, n);
+  if (l == 0) return;
+  f(L.pnbr, 6 * no), f(L.olist, no), f(L.opos, no), f(L.pcell, no), f(L.nbr, 6 * no);
+  f(L.acc, 3 * n), f(L.acc32, n), f(L.u, n), f(L.E, n), f(L.f, n);
+  f(L.ghost, 4 * ng), f(L.ghostE, 4 * ng), f(L.ghost32, 4 * ng), f(L.gface, ng);
+}
+
+static void drop_level(AmrWork* A, int l) {
+  AmrLevel& L = A->L[l];
+  level_arrays(L, l, 0, 0, 0, [](auto*& p, long long) {
     if (p) cudaFree(p);
-  // u, E, f of level >= 1 are owned here too
+    p = nullptr;
+  });
+  L.gcap = 0;
+  A->cap_cells[l] = A->cap_oct[l] = 0;
 }
 
 void amr_free(mgfr_ctx* c) {
   AmrWork* A = W(c);
   if (!A) return;
-  for (int l = 0; l < AMR_MAXL; ++l) {
-    free_level(A->L[l]);
-    if (l > 0) {
-      if (A->L[l].u) cudaFree(A->L[l].u);
-      if (A->L[l].E) cudaFree(A->L[l].E);
-      if (A->L[l].f) cudaFree(A->L[l].f);
-    }
-  }
+  for (int l = 0; l < AMR_MAXL; ++l) drop_level(A, l);
   for (int l = 0; l < MGFR_MAX_DENSE; ++l) {
     if (A->dmask[l]) cudaFree(A->dmask[l]);
     if (A->dact[l]) cudaFree(A->dact[l]);
@@ -1048,51 +1055,12 @@ static mgfr_status grow(mgfr_ctx* c, T** p, long long n, long long* cap_unused =
     if (s_ != MGFR_OK) return s_;            \
   } while (0)
 
-static void drop_level(AmrWork* A, int l) {
-  AmrLevel& L = A->L[l];
-  free_level(L);
-  L.son = nullptr; L.refined = nullptr; L.count = nullptr; L.opos = nullptr; L.pcell = nullptr;
-  L.nbr = nullptr; L.mass = nullptr; L.w = nullptr; L.wE = nullptr; L.wf = nullptr;
-  L.wold = nullptr; L.mask = nullptr; L.ghost = nullptr; L.ghostE = nullptr; L.acc = nullptr;
-  L.pnbr = nullptr; L.w32 = nullptr; L.wf32 = nullptr; L.wold32 = nullptr;
-  L.ghost32 = nullptr; L.olist = nullptr; L.acc32 = nullptr; L.act = nullptr; L.gface = nullptr;
-  if (l > 0) {
-    if (L.u) cudaFree(L.u);
-    if (L.E) cudaFree(L.E);
-    if (L.f) cudaFree(L.f);
-    L.u = L.E = L.f = nullptr;
-  }
-  L.gcap = 0;
-  A->cap_cells[l] = A->cap_oct[l] = 0;
-}
-
 static mgfr_status grow_level(mgfr_ctx* c, AmrWork* A, int l, long long n, long long no) {
-  AmrLevel& L = A->L[l];
-  TRY(grow(c, &L.son, n));
-  TRY(grow(c, &L.refined, n));
-  TRY(grow(c, &L.count, n));
-  TRY(grow(c, &L.mass, n));
-  TRY(grow(c, &L.w, n));
-  TRY(grow(c, &L.wE, n));
-  TRY(grow(c, &L.wf, n));
-  TRY(grow(c, &L.wold, n));
-  TRY(grow(c, &L.mask, n));
-  TRY(grow(c, &L.act, n));
-  TRY(grow(c, &L.w32, n));
-  TRY(grow(c, &L.wf32, n));
-  TRY(grow(c, &L.wold32, n));
-  if (l > 0) {
-    TRY(grow(c, &L.pnbr, 6 * no));
-    TRY(grow(c, &L.olist, no));
-    TRY(grow(c, &L.opos, no));
-    TRY(grow(c, &L.pcell, no));
-    TRY(grow(c, &L.nbr, 6 * no));
-    TRY(grow(c, &L.acc, 3 * n));
-    TRY(grow(c, &L.acc32, n));
-    TRY(grow(c, &L.u, n));
-    TRY(grow(c, &L.E, n));
-    TRY(grow(c, &L.f, n));
-  }
+  mgfr_status rs = MGFR_OK;
+  level_arrays(A->L[l], l, n, no, 0, [&](auto*& p, long long k) {
+    if (rs == MGFR_OK) rs = grow(c, &p, k);
+  });
+  if (rs != MGFR_OK) return rs;
   A->cap_cells[l] = n;
   A->cap_oct[l] = no;
   return MGFR_OK;
@@ -1100,20 +1068,20 @@ static mgfr_status grow_level(mgfr_ctx* c, AmrWork* A, int l, long long n, long 
 
 // Arrays of level l for its ncell cells and n_oct octs.  A refined level's size
 // changes with every set of particles: its arrays are kept while they are
-// large enough (and at most four times too large) and made 1/16 larger than
-// asked for, where the device has the room, so that the steps of a simulation
-// do not free and allocate them each time (67 GB at 512^3 particles: 70 ms of a
-// 580 ms call, 8 of 53 ms at 256^3).
+// large enough (and at most twice too large) and made 1/16 larger than
+// asked for, so that the steps of a simulation do not free and allocate them each time
+// (67 GB at 512^3 particles: 70 ms of a 580 ms call, 8 of 53 ms at 256^3).  Where the
+// device has no room for it they are made as large as asked for; where that fails,
+// the caller starts again with every refined level so (solve_particles).
 static mgfr_status alloc_level(mgfr_ctx* c, AmrWork* A, int l) {
   AmrLevel& L = A->L[l];
   const long long n = L.ncell, no = L.n_oct;
-  if (L.son && n <= A->cap_cells[l] && no <= A->cap_oct[l] && 4 * n >= A->cap_cells[l])
+  if (L.son && n <= A->cap_cells[l] && no <= A->cap_oct[l] && 2 * n >= A->cap_cells[l])
     return MGFR_OK;
   drop_level(A, l);
-  if (l > 0) {
+  if (l > 0 && !A->exact) {
     const long long ro = no + no / 16;
     if (grow_level(c, A, l, 8 * ro, ro) == MGFR_OK) return MGFR_OK;
-    (void)cudaGetLastError();
     c->err.clear();
     drop_level(A, l);
   }
@@ -1128,6 +1096,53 @@ static mgfr_status grow_ghosts(mgfr_ctx* c, AmrLevel& L, long long ng) {
   TRY(grow(c, &L.gface, ng));
   L.gcap = ng;
   return MGFR_OK;
+}
+
+// Memory that the refined levels hold beyond need: whole levels that the hierarchy of
+// the last particle solve does not have, and the reserve of those that it has, their
+// arrays copied one by one into exact ones (as far as there is room for the copies).
+static bool give_back_levels(mgfr_ctx* c) {
+  AmrWork* A = W(c);
+  bool any = false;
+  if (!A) return any;
+  for (int l = 1; l < AMR_MAXL; ++l) {
+    AmrLevel& L = A->L[l];
+    if (l >= A->nlev) {
+      any = any || L.son;
+      drop_level(A, l);
+      continue;
+    }
+    const bool cells = A->cap_cells[l] > L.ncell || A->cap_oct[l] > L.n_oct;
+    if (!cells && L.gcap <= L.n_gslot) continue;
+    level_arrays(L, l, L.ncell, L.n_oct, L.n_gslot, [&](auto*& p, long long k) {
+      if (!p || k <= 0) return;
+      const size_t bytes = sizeof(*p) * (size_t)k;
+      void* q = nullptr;
+      if (cudaMalloc(&q, bytes) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return;
+      }
+      if (cudaMemcpyAsync(q, p, bytes, cudaMemcpyDeviceToDevice, c->s) != cudaSuccess ||
+          cudaStreamSynchronize(c->s) != cudaSuccess) {
+        cudaFree(q);
+        return;
+      }
+      cudaFree(p);
+      p = static_cast<std::remove_reference_t<decltype(p)>>(q);
+      any = true;
+    });
+    A->cap_cells[l] = L.ncell;
+    A->cap_oct[l] = L.n_oct;
+    L.gcap = L.n_gslot;
+  }
+  return any;
+}
+
+cudaError_t dev_malloc_bytes(mgfr_ctx* c, void** p, size_t bytes) {
+  const cudaError_t e = cudaMalloc(p, bytes);
+  if (e != cudaErrorMemoryAllocation || !give_back_levels(c)) return e;
+  (void)cudaGetLastError();
+  return cudaMalloc(p, bytes);
 }
 
 static mgfr_status scan_flags(mgfr_ctx* c, AmrWork* A, const unsigned char* flags, long long n,
@@ -1195,8 +1210,7 @@ static mgfr_status build_structure(mgfr_ctx* c, AmrWork* A, const double* pos) {
     k_face_flags<<<nblocks(6 * N.n_oct, BS), BS, 0, c->s>>>(N.nbr, 6 * N.n_oct, N.refined);
     TRY(scan_flags(c, A, N.refined, 6 * N.n_oct, 0, N.son, &N.n_gslot));
     if (N.n_gslot > N.gcap) {
-      if (grow_ghosts(c, N, N.n_gslot + N.n_gslot / 16) != MGFR_OK) {
-        (void)cudaGetLastError();
+      if (A->exact || grow_ghosts(c, N, N.n_gslot + N.n_gslot / 16) != MGFR_OK) {
         c->err.clear();
         TRY(grow_ghosts(c, N, N.n_gslot));
       }
@@ -1287,11 +1301,10 @@ static mgfr_status check_particle_args(mgfr_ctx* c, const double* pos, long long
   return MGFR_OK;
 }
 
-static mgfr_status solve_particles(mgfr_ctx* c, const double* pos, long long Np, int N0, double box,
-                                   double a, const double* u_init, double* fr_out,
-                                   double* acc_out, double* acc_host, mgfr_stats* st) {
-  if (!c) return MGFR_E_INVALID;
-  TRY(check_particle_args(c, pos, Np, N0, box, a));
+static mgfr_status solve_particles_once(mgfr_ctx* c, const double* pos, long long Np, int N0,
+                                        double box, double a, const double* u_init,
+                                        double* fr_out, double* acc_out, double* acc_host,
+                                        mgfr_stats* st) {
   const mgfr_config& g = c->cfg;
   MG_CK(c, cudaSetDevice(c->device));
   if (st) std::memset(st, 0, sizeof(*st));
@@ -1491,6 +1504,28 @@ static mgfr_status solve_particles(mgfr_ctx* c, const double* pos, long long Np,
   return worst;
 }
 
+// Where the device's memory runs out, once more from the start with all refined levels
+// given back and made exactly as large as they have to be.
+static mgfr_status solve_particles(mgfr_ctx* c, const double* pos, long long Np, int N0, double box,
+                                   double a, const double* u_init, double* fr_out,
+                                   double* acc_out, double* acc_host, mgfr_stats* st) {
+  if (!c) return MGFR_E_INVALID;
+  TRY(check_particle_args(c, pos, Np, N0, box, a));
+  const mgfr_status rs =
+      solve_particles_once(c, pos, Np, N0, box, a, u_init, fr_out, acc_out, acc_host, st);
+  if (rs != MGFR_E_OOM || !c->amr) return rs;
+  AmrWork* A = W(c);
+  MG_CK(c, cudaStreamSynchronize(c->s));
+  amr_invalidate(c);
+  if (!give_back_levels(c)) return rs;
+  c->err.clear();
+  A->exact = true;
+  const mgfr_status again =
+      solve_particles_once(c, pos, Np, N0, box, a, u_init, fr_out, acc_out, acc_host, st);
+  A->exact = false;
+  return again;
+}
+
 mgfr_status mgfr_solve_particles(mgfr_ctx* c, const double* pos, long long Np, int N0, double box,
                                  double a, const double* u_init, double* fr_out, double* acc_out,
                                  mgfr_stats* st) {
@@ -1516,8 +1551,8 @@ mgfr_status mgfr_solve_particles_host(mgfr_ctx* c, const double* pos_host, long 
     if (A->acc_dev) cudaFree(A->acc_dev);
     A->pos_dev = A->acc_dev = nullptr;
     A->pio_cap = 0;
-    MG_CK(c, cudaMalloc(&A->pos_dev, sizeof(double) * 3 * (size_t)Np));
-    MG_CK(c, cudaMalloc(&A->acc_dev, sizeof(double) * 3 * (size_t)Np));
+    MG_CK(c, dev_malloc(c, &A->pos_dev, sizeof(double) * 3 * (size_t)Np));
+    MG_CK(c, dev_malloc(c, &A->acc_dev, sizeof(double) * 3 * (size_t)Np));
     A->pio_cap = Np;
   }
   // in the caller's stream order

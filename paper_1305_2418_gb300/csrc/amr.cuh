@@ -128,6 +128,7 @@ struct AmrWork {
   bool rec_on = false;                            // the last deposit recorded
   long long cap_cells[AMR_MAXL] = {}; // allocated capacity per level (cells)
   long long cap_oct[AMR_MAXL] = {};
+  bool exact = false;                 // refined levels without reserve (memory ran out)
   // the refined levels of the previous particle solve made with start =
   // MGFR_START_PREVIOUS_ALL: per level, the Morton keys of the octs' parent
   // cells (increasing: the storage order) and the converged u of their cells

@@ -619,7 +619,7 @@ static mgfr_status batch_learned_start(mgfr_ctx* c, BatchWork* B, const mgfr_bat
     if (B->lrn_out) cudaFree(B->lrn_out);
     B->lrn_out = nullptr;
     B->lrn_out_cap = 0;
-    MG_CK(c, cudaMalloc(&B->lrn_out, sizeof(double) * (size_t)total));
+    MG_CK(c, dev_malloc(c, &B->lrn_out, sizeof(double) * (size_t)total));
     B->lrn_out_cap = total;
   }
   long long off = 0;
@@ -647,7 +647,7 @@ static mgfr_status batch_learned_start(mgfr_ctx* c, BatchWork* B, const mgfr_bat
       if (B->lrn_in) cudaFree(B->lrn_in);
       B->lrn_in = nullptr;
       B->lrn_in_cap = 0;
-      MG_CK(c, cudaMalloc(&B->lrn_in, sizeof(double) * (size_t)need));
+      MG_CK(c, dev_malloc(c, &B->lrn_in, sizeof(double) * (size_t)need));
       B->lrn_in_cap = need;
     }
     for (size_t k = 0; k < grp.size(); ++k)
@@ -764,7 +764,7 @@ mgfr_status mgfr_batch_solve(mgfr_ctx* c, int nsolves, const mgfr_batch_item* it
   auto buf = [&](size_t bytes) -> void* {
     if (bi < B->bufs.size()) return B->bufs[bi++];
     void* p = nullptr;
-    if (cudaMalloc(&p, bytes) != cudaSuccess) {
+    if (dev_malloc(c, &p, bytes) != cudaSuccess) {
       (void)cudaGetLastError();
       return nullptr;
     }
@@ -823,10 +823,10 @@ mgfr_status mgfr_batch_solve(mgfr_ctx* c, int nsolves, const mgfr_batch_item* it
     S.acc_out = it.acc_out_dev;
     S.u_out = it.u_out_dev;
   }
-  if (!B->dS) MG_CK(c, cudaMalloc(&B->dS, sizeof(BSolve) * nsolves));
-  if (!B->dst) MG_CK(c, cudaMalloc(&B->dst, sizeof(BState) * nsolves));
-  if (!B->bar) MG_CK(c, cudaMalloc(&B->bar, 2 * sizeof(unsigned)));
-  if (!B->err) MG_CK(c, cudaMalloc(&B->err, 2 * sizeof(int)));
+  if (!B->dS) MG_CK(c, dev_malloc(c, &B->dS, sizeof(BSolve) * nsolves));
+  if (!B->dst) MG_CK(c, dev_malloc(c, &B->dst, sizeof(BState) * nsolves));
+  if (!B->bar) MG_CK(c, dev_malloc(c, &B->bar, 2 * sizeof(unsigned)));
+  if (!B->err) MG_CK(c, dev_malloc(c, &B->err, 2 * sizeof(int)));
   MG_CK(c, cudaEventRecord(c->ev_in, c->user));
   MG_CK(c, cudaStreamWaitEvent(c->s, c->ev_in, 0));
   if (g.start == MGFR_START_LEARNED) {

@@ -178,6 +178,14 @@ void prof_clear(mgfr_ctx* c, int graph);
 mgfr_status set_err(mgfr_ctx* c, mgfr_status st, const std::string& msg);
 // Range checks of a configuration (false and the reason in why if invalid).
 bool validate_cfg(const mgfr_config* c, std::string& why);
+// cudaMalloc for a context's workspaces: where memory runs out, once more after the
+// refined levels of the context have given back what they hold beyond need (amr.cu).
+// Not for the arrays of a hierarchy that is being built.
+cudaError_t dev_malloc_bytes(mgfr_ctx* c, void** p, size_t bytes);
+template <class T>
+cudaError_t dev_malloc(mgfr_ctx* c, T** p, size_t bytes) {
+  return dev_malloc_bytes(c, reinterpret_cast<void**>(p), bytes);
+}
 void batch_free(mgfr_ctx* c);
 void unet_free(mgfr_ctx* c);
 // give back the convolution primitive's scratch on this device (unet.cu)

@@ -307,16 +307,16 @@ mgfr_status pm_alloc(mgfr_ctx* c, PmWork* P, int lg, double box) {
     if (ps != MGFR_OK) return ps;
     P->nlev = lg - 1;  // N ... 4
     P->n = 1LL << (3 * lg);
-    MG_CK(c, cudaMalloc(&P->phi, sizeof(double) * (size_t)P->n));
-    MG_CK(c, cudaMalloc(&P->rhs, sizeof(double) * (size_t)P->n));
-    MG_CK(c, cudaMalloc(&P->rlo, sizeof(float) * (size_t)P->n));
+    MG_CK(c, dev_malloc(c, &P->phi, sizeof(double) * (size_t)P->n));
+    MG_CK(c, dev_malloc(c, &P->rhs, sizeof(double) * (size_t)P->n));
+    MG_CK(c, dev_malloc(c, &P->rlo, sizeof(float) * (size_t)P->n));
     for (int l = 0; l < P->nlev; ++l) {
       const size_t nl = (size_t)1 << (3 * (lg - l));
-      MG_CK(c, cudaMalloc(&P->e[l], sizeof(float) * nl));
-      MG_CK(c, cudaMalloc(&P->r[l], sizeof(float) * nl));
+      MG_CK(c, dev_malloc(c, &P->e[l], sizeof(float) * nl));
+      MG_CK(c, dev_malloc(c, &P->r[l], sizeof(float) * nl));
     }
     P->nparts = 152 * 8;
-    MG_CK(c, cudaMalloc(&P->part, sizeof(double) * (2 * P->nparts + 2)));
+    MG_CK(c, dev_malloc(c, &P->part, sizeof(double) * (2 * P->nparts + 2)));
     MG_CK(c, cudaMallocHost(&P->part_h, sizeof(double) * P->nparts));
     P->lg = lg;
   }
@@ -487,7 +487,7 @@ extern "C" mgfr_status mgfr_pm_accel(mgfr_ctx* c, int lpm, int what, const doubl
   PmWork* P = nullptr;
   mgfr_status rs = pm_solve(c, lpm, what, nullptr, nullptr, st, &P);
   if (rs != MGFR_OK && rs != MGFR_E_NOCONVERGE) return rs;
-  if (!P->grad) MG_CK(c, cudaMalloc(&P->grad, 2 * sizeof(float4) * (size_t)P->n));
+  if (!P->grad) MG_CK(c, dev_malloc(c, &P->grad, 2 * sizeof(float4) * (size_t)P->n));
   k_pm_grad<<<nblocks(P->n, BS), BS, 0, c->s>>>(P->phi, P->lg, df_from_double(0.5 / P->h), P->grad);
   k_pm_cic<<<nblocks(Np, BS), BS, 0, c->s>>>(pos_dev, Np, P->lg, 1.0 / P->h, P->grad, acc_out_dev);
   c->launches += 2;

@@ -183,7 +183,7 @@ mgfr_status start_guess(mgfr_ctx* c, int N, const double* x, double dscale, cons
     if (c->u_learn) cudaFree(c->u_learn);
     c->u_learn = nullptr;
     c->u_learn_cap = 0;
-    MG_CK(c, cudaMalloc(&c->u_learn, sizeof(double) * (size_t)n));
+    MG_CK(c, dev_malloc(c, &c->u_learn, sizeof(double) * (size_t)n));
     c->u_learn_cap = n;
   }
   const double fr0 = c->cfg.fr0_abs;
@@ -227,20 +227,20 @@ static mgfr_status alloc_dense(mgfr_ctx* c, DenseHier& H, int N, bool mixed) {
     L.N = 1 << L.lg;
     L.n = 1LL << (3 * L.lg);
     size_t b8 = sizeof(double) * (size_t)L.n, b4 = sizeof(float) * (size_t)L.n;
-    MG_CK(c, cudaMalloc(&L.u, b8));
-    MG_CK(c, cudaMalloc(&L.E, b8));
-    MG_CK(c, cudaMalloc(&L.f, b8));
-    if (l > 0) MG_CK(c, cudaMalloc(&L.uold, b8));
-    MG_CK(c, cudaMalloc(&L.u32, b4));
-    MG_CK(c, cudaMalloc(&L.e32, b4));
-    MG_CK(c, cudaMalloc(&L.r32, b4));
-    if (l > 0) MG_CK(c, cudaMalloc(&L.uold32, b4));
-    if (mixed) MG_CK(c, cudaMalloc(&L.f32, b4));
+    MG_CK(c, dev_malloc(c, &L.u, b8));
+    MG_CK(c, dev_malloc(c, &L.E, b8));
+    MG_CK(c, dev_malloc(c, &L.f, b8));
+    if (l > 0) MG_CK(c, dev_malloc(c, &L.uold, b8));
+    MG_CK(c, dev_malloc(c, &L.u32, b4));
+    MG_CK(c, dev_malloc(c, &L.e32, b4));
+    MG_CK(c, dev_malloc(c, &L.r32, b4));
+    if (l > 0) MG_CK(c, dev_malloc(c, &L.uold32, b4));
+    if (mixed) MG_CK(c, dev_malloc(c, &L.f32, b4));
   }
   H.nparts = 152 * 8;
-  if (mixed) MG_CK(c, cudaMalloc(&H.fdf, sizeof(double) * (size_t)H.L[0].n));
-  MG_CK(c, cudaMalloc(&H.partials, sizeof(double) * 2 * H.nparts));
-  MG_CK(c, cudaMalloc(&H.scal, sizeof(double) * 16));
+  if (mixed) MG_CK(c, dev_malloc(c, &H.fdf, sizeof(double) * (size_t)H.L[0].n));
+  MG_CK(c, dev_malloc(c, &H.partials, sizeof(double) * 2 * H.nparts));
+  MG_CK(c, dev_malloc(c, &H.scal, sizeof(double) * 16));
   H.N = N;
   H.mixed = mixed;
   return MGFR_OK;

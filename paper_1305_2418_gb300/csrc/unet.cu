@@ -460,7 +460,7 @@ static mgfr_status unet_alloc(mgfr_ctx* c, UNet* U, int B, int lgD) {
   bool ok = true;
   auto bytes = [&](size_t n) -> void* {
     void* p = nullptr;
-    ok = ok && cudaMalloc(&p, n) == cudaSuccess;
+    ok = ok && dev_malloc(c, &p, n) == cudaSuccess;
     if (p) U->bufs.push_back(p);
     return p;
   };
@@ -746,14 +746,14 @@ static mgfr_status unet_fill(mgfr_ctx* c, UNet* U, unsigned long long seed) {
   off += 17;
   U->nparam = off;
   U->nwbf = boff;
-  MG_CK(c, cudaMalloc(&U->P, sizeof(float) * off));
-  MG_CK(c, cudaMalloc(&U->G, sizeof(float) * off));
-  MG_CK(c, cudaMalloc(&U->M1, sizeof(float) * off));
-  MG_CK(c, cudaMalloc(&U->M2, sizeof(float) * off));
-  MG_CK(c, cudaMalloc(&U->Wbf, sizeof(__nv_bfloat16) * boff));
-  MG_CK(c, cudaMalloc(&U->Wtf, sizeof(__nv_bfloat16) * boff));
-  MG_CK(c, cudaMalloc(&U->Wtd, sizeof(__nv_bfloat16) * boff));
-  MG_CK(c, cudaMalloc(&U->tc_err, sizeof(int)));
+  MG_CK(c, dev_malloc(c, &U->P, sizeof(float) * off));
+  MG_CK(c, dev_malloc(c, &U->G, sizeof(float) * off));
+  MG_CK(c, dev_malloc(c, &U->M1, sizeof(float) * off));
+  MG_CK(c, dev_malloc(c, &U->M2, sizeof(float) * off));
+  MG_CK(c, dev_malloc(c, &U->Wbf, sizeof(__nv_bfloat16) * boff));
+  MG_CK(c, dev_malloc(c, &U->Wtf, sizeof(__nv_bfloat16) * boff));
+  MG_CK(c, dev_malloc(c, &U->Wtd, sizeof(__nv_bfloat16) * boff));
+  MG_CK(c, dev_malloc(c, &U->tc_err, sizeof(int)));
   MG_CK(c, cudaMemsetAsync(U->tc_err, 0, sizeof(int), c->s));
   // He-normal initialisation from a seeded generator (host), zero biases
   std::vector<float> h((size_t)off, 0.f);

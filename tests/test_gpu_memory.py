@@ -98,3 +98,68 @@ def mgfr_solver(**kw):
         yield s
     finally:
         s.close()
+
+
+# ---- the refined levels' reserve ------------------------------------------------
+N0, BOX = 64, 100.0
+
+
+def particles(dev, n, part, seed):
+    """n particles, uniform in the first `part` of the box along x: at 100 and more per base
+    cell two levels are refined wherever there are particles."""
+    r = torch.Generator(device=dev).manual_seed(seed)
+    p = torch.rand((n, 3), generator=r, device=dev, dtype=torch.float64) * BOX
+    p[:, 0] *= part
+    return p
+
+
+def held(dev, call):
+    """Device memory that stays taken after the call, beside torch's."""
+    gc.collect()
+    torch.cuda.empty_cache()
+    before = free_bytes(dev)
+    call()
+    torch.cuda.empty_cache()
+    return before - free_bytes(dev)
+
+
+def rel(a, b):
+    return float((a - b).norm() / b.norm())
+
+
+def test_a_kept_level_does_not_take_a_later_solves_memory(dev):
+    """All of the box refined, then 0.6 of it with more particles: the second solve gets the
+    memory that it takes by itself, which is less than what it needs beside the first
+    one's level arrays (1 GB more).  The same hierarchy and forces as by itself; the
+    masses are summed by atomics, whose order may flip FP32 roundings (6e-8 each)."""
+    first, second = particles(dev, 33_000_000, 1.0, 1), particles(dev, 55_000_000, 0.6, 2)
+    cfg = dict(precision=mgfr.PREC_MIXED, max_level=2, tol_rel=1e-5)
+    own = second.numel() * 8 + (8 << 20)  # the force array and f_R, torch's
+    with mgfr_solver(**cfg) as s:
+        need = held(dev, lambda: s.solve_particles(second, N0, BOX))
+        want = s.solve_particles(second, N0, BOX)["acc"].cpu()
+        levels = [s.level_info(l) for l in range(3)]
+        pm_need = held(dev, lambda: s.pm_accel(second, 2))
+        want_pm = s.pm_accel(second, 2)[0].cpu()
+    with mgfr_solver(**cfg) as s:
+        has = held(dev, lambda: s.solve_particles(first, N0, BOX))
+        assert s.level_info(2)[1] > 1.5 * levels[2][1]
+        with only(dev, need - has + own + (256 << 20)):
+            got = s.solve_particles(second, N0, BOX)["acc"].cpu()
+            assert [s.level_info(l) for l in range(3)] == levels
+        assert rel(got, want) <= 1e-6
+        # and again with room, on the arrays that it now has
+        assert rel(s.solve_particles(second, N0, BOX)["acc"].cpu(), want) <= 1e-6
+    # a particle-mesh force after it, the levels still holding more than they need
+    with mgfr_solver(**cfg) as s:
+        s.solve_particles(first, N0, BOX)
+        s.solve_particles(second, N0, BOX, want_acc=False)
+        d0 = s.effective_density(2)
+        with only(dev, pm_need + own - (256 << 20)):
+            got = s.pm_accel(second, 2)[0].cpu()
+        assert rel(got, want_pm) <= 1e-6
+        # the hierarchy is still there, its fields as they were
+        assert torch.equal(s.effective_density(2), d0)
+        assert [s.level_info(l) for l in range(3)] == levels
+        fr = s.level_field(2, mgfr.FIELD_FR)
+        assert np.isfinite(fr).all() and (fr < 0.0).all()
