@@ -369,10 +369,11 @@ typedef struct {
 mgfr_status mgfr_batch_solve(mgfr_ctx* ctx, int nsolves, const mgfr_batch_item* items,
                              mgfr_stats* per_solve);
 
-/* Time the candidate launch shapes (128/256/512 threads x 1/2/4 blocks per
- * SM) on this batch, keep the fastest for batches with the same sizes (and
- * append it to the file named by the environment variable MGFR_TUNE_CACHE,
- * when set).  Runs the batch 9 times; outputs are overwritten. */
+/* Time the launch shape that the batch has untuned and the candidates that
+ * launch differently (128/256/512 threads x 1/2/4 blocks per SM), keep the
+ * fastest for batches with the same sizes (and append it to the file named by
+ * the environment variable MGFR_TUNE_CACHE, when set).  Runs the batch twice
+ * per shape, at most 20 times; outputs are overwritten. */
 mgfr_status mgfr_batch_autotune(mgfr_ctx* ctx, int nsolves, const mgfr_batch_item* items,
                                 int* best_threads, int* best_blocks_per_sm);
 

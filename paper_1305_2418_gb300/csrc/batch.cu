@@ -23,6 +23,7 @@
 #include <string>
 #include <vector>
 
+#include "batch_shape.h"
 #include "lean_fp64.cuh"
 #include "mg32_dev.cuh"
 
@@ -575,7 +576,7 @@ struct BatchWork {
   unsigned* bar = nullptr;  // [0] count, [1] generation
   int* err = nullptr;
   std::vector<int> order;
-  std::map<std::string, std::pair<int, int>> tuned;  // signature -> (threads, blocks/SM)
+  std::map<std::string, BatchShape> tuned;  // by the sizes
   cudaGraphExec_t gx = nullptr;
   std::string gkey;
   // learned start: network input staging and the predicted initial guesses
@@ -670,9 +671,17 @@ void batch_free(mgfr_ctx* c) {
   c->batch = nullptr;
 }
 
+// work items of a half-sweep of the finest grids
+static long long batch_vecs(int nsolves, const mgfr_batch_item* items) {
+  long long v = 0;
+  for (int i = 0; i < nsolves; ++i) v += (long long)items[i].N * items[i].N * items[i].N / 8;
+  return v;
+}
+
 // at most `blocks` blocks
-static mgfr_status launch_batch(mgfr_ctx* c, BatchWork* B, const BArgs& A, int threads, int bpsm,
+static mgfr_status launch_batch(mgfr_ctx* c, BatchWork* B, const BArgs& A, BatchShape shape,
                                 long long blocks, bool use_graph) {
+  const int threads = shape.threads;
   int dev = c->device, nsm = 0;
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   int occ = 0;
@@ -681,7 +690,7 @@ static mgfr_status launch_batch(mgfr_ctx* c, BatchWork* B, const BArgs& A, int t
   void* kern = A.tol >= 1e-10 ? (void*)k_batch<true> : (void*)k_batch<false>;
   MG_CK(c, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, threads, 0));
   if (occ < 1) return set_err(c, MGFR_E_UNSUPPORTED, "batched kernel cannot be resident");
-  const int grid = (int)std::min((long long)nsm * std::min(bpsm, occ), blocks);
+  const int grid = (int)std::min((long long)nsm * std::min(shape.per_sm, occ), blocks);
   MG_CK(c, cudaMemsetAsync(B->bar, 0, 2 * sizeof(unsigned), c->s));
   MG_CK(c, cudaMemsetAsync(B->err, 0, 2 * sizeof(int), c->s));
   BArgs a = A;
@@ -722,11 +731,7 @@ static mgfr_status launch_batch(mgfr_ctx* c, BatchWork* B, const BArgs& A, int t
   return MGFR_OK;
 }
 
-extern "C" {
-
-mgfr_status mgfr_batch_solve(mgfr_ctx* c, int nsolves, const mgfr_batch_item* items,
-                             mgfr_stats* per_solve) {
-  if (!c) return MGFR_E_INVALID;
+static mgfr_status check_items(mgfr_ctx* c, int nsolves, const mgfr_batch_item* items) {
   if (nsolves < 1 || nsolves > kMaxBatch || !items)
     return set_err(c, MGFR_E_INVALID, "need 1..4096 batch items");
   const mgfr_config& g = c->cfg;
@@ -742,18 +747,37 @@ mgfr_status mgfr_batch_solve(mgfr_ctx* c, int nsolves, const mgfr_batch_item* it
     if (g.start == MGFR_START_PREVIOUS || g.start == MGFR_START_PREVIOUS_ALL)
       return set_err(c, MGFR_E_INVALID, "start = previous is not available for batches");
   }
+  return MGFR_OK;
+}
+
+// The sizes in descending order; order (if not NULL): the items so sorted, where the
+// participants of a size form a prefix
+static std::string batch_signature(int nsolves, const mgfr_batch_item* items,
+                                   std::vector<int>* order) {
+  std::vector<int> o(nsolves);
+  for (int i = 0; i < nsolves; ++i) o[i] = i;
+  std::stable_sort(o.begin(), o.end(), [&](int x, int y) { return items[x].N > items[y].N; });
+  std::string sig;
+  for (int i : o) sig += std::to_string(items[i].N) + ",";
+  if (order) *order = o;
+  return sig;
+}
+
+extern "C" {
+
+mgfr_status mgfr_batch_solve(mgfr_ctx* c, int nsolves, const mgfr_batch_item* items,
+                             mgfr_stats* per_solve) {
+  if (!c) return MGFR_E_INVALID;
+  const mgfr_status args = check_items(c, nsolves, items);
+  if (args != MGFR_OK) return args;
+  const mgfr_config& g = c->cfg;
   auto w0 = std::chrono::steady_clock::now();
   MG_CK(c, cudaSetDevice(c->device));
   c->launches = 0;
   if (!c->batch) c->batch = new BatchWork();
   BatchWork* B = (BatchWork*)c->batch;
-  // solves sorted by N (descending): participants of a size form a prefix
-  std::vector<int> order(nsolves);
-  for (int i = 0; i < nsolves; ++i) order[i] = i;
-  std::stable_sort(order.begin(), order.end(),
-                   [&](int x, int y) { return items[x].N > items[y].N; });
-  std::string sig;
-  for (int i : order) sig += std::to_string(items[i].N) + ",";
+  std::vector<int> order;
+  const std::string sig = batch_signature(nsolves, items, &order);
   if (sig != B->sig) {
     batch_release(B);
     B->sig = sig;
@@ -856,30 +880,15 @@ mgfr_status mgfr_batch_solve(mgfr_ctx* c, int nsolves, const mgfr_batch_item* it
   A.bar_gen = B->bar + 1;
   A.err = B->err;
   A.max_spins = g.max_spins;
-  // Launch shape: the tuned choice for this signature, else by the work items of a
-  // half-sweep of the finest grids (four cells each).  Beyond 2^20 the device is full
-  // either way and 512 threads x 2 per SM are the fastest (96 solves of 32^3..128^3, ms:
-  // 45.0; 256 x 2 54.5, 256 x 3 47.1, 128 x 8 50.3), below it smaller blocks spread the
-  // items better (one 64^3 1.68 for 1.82, one 128^3 3.46 for 3.64).  A batch of few items is
-  // little but barriers, whose time grows with the blocks that arrive at them: no more
-  // blocks than there are items for (and one per solve, for the 4^3 grids), up to 16384
-  // items (one 32^3: 4096) small blocks on many SMs: one 32^3 1.39 ms (on a full grid of
-  // 512 x 2 1.53, of 256 x 2 with one cell per thread 1.45), one 8^3 0.39 (0.46).
-  long long vecs = 0;
-  for (const BSolve& S : hs) vecs += 1LL << (3 * S.lg - 3);
-  int threads = vecs > (1 << 20) ? 512 : (vecs > 16384 || vecs <= 1024 ? 256 : 128);
-  int bpsm = threads == 512 ? 2 : 3;
+  // the tuned launch shape for these sizes, else by the amount of work (batch_shape.h)
+  const long long vecs = batch_vecs(nsolves, items);
+  int nsm = 0;
+  MG_CK(c, cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, c->device));
+  BatchShape shape = batch_rule(vecs, nsolves, nsm);
   auto itc = B->tuned.find(sig);
-  const bool tuned = itc != B->tuned.end();
-  if (tuned) {
-    threads = itc->second.first;
-    bpsm = itc->second.second;
-  }
-  long long blocks = (vecs + threads - 1) / threads;
-  if (!tuned && threads == 128) blocks = std::max(blocks, std::min(128LL, vecs / 64));
-  blocks = std::max(blocks, (long long)nsolves);
+  if (itc != B->tuned.end()) shape = itc->second;
   MG_CK(c, cudaEventRecord(c->t0, c->s));
-  mgfr_status rs = launch_batch(c, B, A, threads, bpsm, blocks, true);
+  mgfr_status rs = launch_batch(c, B, A, shape, batch_blocks(shape.threads, vecs, nsolves), true);
   if (rs != MGFR_OK) return rs;
   MG_CK(c, cudaEventRecord(c->t1, c->s));
   std::vector<BState> st(nsolves);
@@ -924,53 +933,48 @@ mgfr_status mgfr_batch_solve(mgfr_ctx* c, int nsolves, const mgfr_batch_item* it
   return MGFR_OK;
 }
 
-// Time every candidate launch shape on this batch and keep the fastest for
-// batches of the same size signature (persisted in the file named by
-// MGFR_TUNE_CACHE when set).
+// Time every candidate launch shape on this batch (its second run: the first
+// captures the launch between the events) and keep the fastest for batches of the same
+// size signature (persisted in the file named by MGFR_TUNE_CACHE when set).
 mgfr_status mgfr_batch_autotune(mgfr_ctx* c, int nsolves, const mgfr_batch_item* items,
                                 int* best_threads, int* best_blocks_per_sm) {
   if (!c) return MGFR_E_INVALID;
-  const int cand_t[] = {128, 256, 512};
-  const int cand_b[] = {1, 2, 4};
-  float best = 1e30f;
-  int bt = 256, bb = 2;
-  mgfr_config saved = c->cfg;
-  for (int t : cand_t)
-    for (int b : cand_b) {
-      if (!c->batch) c->batch = new BatchWork();
-      BatchWork* B = (BatchWork*)c->batch;
-      // force this shape through the tuned map for the current signature
-      std::vector<int> order(nsolves);
-      for (int i = 0; i < nsolves; ++i) order[i] = i;
-      std::stable_sort(order.begin(), order.end(),
-                       [&](int x, int y) { return items[x].N > items[y].N; });
-      std::string sig;
-      for (int i : order) sig += std::to_string(items[i].N) + ",";
-      B->tuned[sig] = {t, b};
-      mgfr_status rs = mgfr_batch_solve(c, nsolves, items, nullptr);
+  const mgfr_status args = check_items(c, nsolves, items);
+  if (args != MGFR_OK) return args;
+  if (!c->batch) c->batch = new BatchWork();
+  BatchWork* B = (BatchWork*)c->batch;
+  const std::string sig = batch_signature(nsolves, items, nullptr);
+  const long long vecs = batch_vecs(nsolves, items);
+  int nsm = 0;
+  MG_CK(c, cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, c->device));
+  BatchShape cand[10], best{};
+  const int n = batch_candidates(vecs, nsolves, nsm, cand);
+  float best_ms = 1e30f;
+  for (int i = 0; i < n; ++i) {
+    B->tuned[sig] = cand[i];
+    float ms = 0.f;
+    for (int rep = 0; rep < 2; ++rep) {
+      const mgfr_status rs = mgfr_batch_solve(c, nsolves, items, nullptr);
       if (rs != MGFR_OK && rs != MGFR_E_NOCONVERGE) {
-        c->cfg = saved;
+        B->tuned.erase(sig);
         return rs;
       }
-      float ms = 0.f;
-      cudaEventElapsedTime(&ms, c->t0, c->t1);
-      if (ms < best) {
-        best = ms;
-        bt = t;
-        bb = b;
-      }
     }
-  c->cfg = saved;
-  BatchWork* B = (BatchWork*)c->batch;
-  B->tuned[B->sig] = {bt, bb};
+    cudaEventElapsedTime(&ms, c->t0, c->t1);
+    if (ms < best_ms) {
+      best_ms = ms;
+      best = cand[i];
+    }
+  }
+  B->tuned[sig] = best;
   if (const char* path = std::getenv("MGFR_TUNE_CACHE")) {
     if (FILE* f = std::fopen(path, "a")) {
-      std::fprintf(f, "%s %d %d %.4f\n", B->sig.c_str(), bt, bb, best);
+      std::fprintf(f, "%s %d %d %.4f\n", sig.c_str(), best.threads, best.per_sm, best_ms);
       std::fclose(f);
     }
   }
-  if (best_threads) *best_threads = bt;
-  if (best_blocks_per_sm) *best_blocks_per_sm = bb;
+  if (best_threads) *best_threads = best.threads;
+  if (best_blocks_per_sm) *best_blocks_per_sm = best.per_sm;
   return MGFR_OK;
 }
 
