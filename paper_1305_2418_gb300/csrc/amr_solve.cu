@@ -537,12 +537,14 @@ __device__ __forceinline__ JR jrow(float uc, float Ec, const NB<float>* nb, cons
   return J;
 }
 
+// the FP32 form keeps no e^u: Eat and dnb form it from u
+constexpr const float* kNoE = nullptr;
+
 // masked Gauss-Seidel half-sweep on J(u) e = r of a dense level, one thread per
 // relaxed cell of the colour (list of C-order indices)
 __global__ void __launch_bounds__(BS) k_dlin_sweep_list(float* __restrict__ e,
                                                         const float* __restrict__ r,
-                                                        const float* __restrict__ u,
-                                                        const float* __restrict__ E, int lg,
+                                                        const float* __restrict__ u, int lg,
                                                         const int* __restrict__ list,
                                                         long long n, MT<float> m, float ih2) {
   const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
@@ -551,8 +553,8 @@ __global__ void __launch_bounds__(BS) k_dlin_sweep_list(float* __restrict__ e,
   const int M = (1 << lg) - 1;
   const int k = (int)(c & M), j = (int)((c >> lg) & M), i = (int)(c >> (2 * lg));
   NB<float> nb[6];
-  dnb(u, E, i, j, k, lg, nb);
-  const JR J = jrow(u[c], Eat(E, u, c), nb, m, ih2);
+  dnb(u, kNoE, i, j, k, lg, nb);
+  const JR J = jrow(u[c], Eat(kNoE, u, c), nb, m, ih2);
   float en[6];
   dnb_x(e, i, j, k, lg, en);
   float acc = r[c];
@@ -563,11 +565,9 @@ __global__ void __launch_bounds__(BS) k_dlin_sweep_list(float* __restrict__ e,
 
 __global__ void __launch_bounds__(BS) k_dlin_restrict(const float* __restrict__ e,
                                                       const float* __restrict__ r,
-                                                      const float* __restrict__ u,
-                                                      const float* __restrict__ E, int lgf,
+                                                      const float* __restrict__ u, int lgf,
                                                       float* __restrict__ rc, float* __restrict__ uc,
-                                                      float* __restrict__ Ec, float* __restrict__ ec,
-                                                      MT<float> m, float ih2,
+                                                      float* __restrict__ ec, MT<float> m, float ih2,
                                                       const unsigned char* __restrict__ act) {
   const int lgc = lgf - 1, Nc = 1 << lgc;
   const unsigned t = blockIdx.x * blockDim.x + threadIdx.x;
@@ -581,17 +581,16 @@ __global__ void __launch_bounds__(BS) k_dlin_restrict(const float* __restrict__ 
     if (!act || act[c]) {
       NB<float> nb[6];
       float en[6];
-      dnb(u, E, i, j, k, lgf, nb);
+      dnb(u, kNoE, i, j, k, lgf, nb);
       dnb_x(e, i, j, k, lgf, en);
-      const JR J = jrow(u[c], Eat(E, u, c), nb, m, ih2);
+      const JR J = jrow(u[c], Eat(kNoE, u, c), nb, m, ih2);
       float Je = J.diag * e[c];
 #pragma unroll
       for (int d = 0; d < 6; ++d) Je = fmaf(J.off[d], en[d], Je);
       sr += r[c] - Je;
     }
   }
-  const float um = 0.125f * su;
-  uc[t] = um;
+  uc[t] = 0.125f * su;
   rc[t] = 0.125f * sr;
   ec[t] = 0.f;
 }
@@ -616,8 +615,7 @@ __global__ void __launch_bounds__(BS) k_dlin_prolong(float* __restrict__ e, cons
 }
 
 __global__ void __launch_bounds__(64) k_dlin_coarse(float* __restrict__ eg, const float* __restrict__ rg,
-                                                    const float* __restrict__ ug,
-                                                    const float* __restrict__ Eg, MT<float> m,
+                                                    const float* __restrict__ ug, MT<float> m,
                                                     float ih2, int sweeps,
                                                     const unsigned char* __restrict__ act) {
   __shared__ float e[64];
@@ -628,8 +626,8 @@ __global__ void __launch_bounds__(64) k_dlin_coarse(float* __restrict__ eg, cons
                     (i << 4) | (((j + 3) & 3) << 2) | k, (i << 4) | (((j + 1) & 3) << 2) | k,
                     (i << 4) | (j << 2) | ((k + 3) & 3), (i << 4) | (j << 2) | ((k + 1) & 3)};
   NB<float> nb[6];
-  for (int d = 0; d < 6; ++d) nb[d] = NB<float>{ug[q[d]], Eat(Eg, ug, q[d])};
-  const JR J = jrow(ug[t], Eat(Eg, ug, t), nb, m, ih2);
+  for (int d = 0; d < 6; ++d) nb[d] = NB<float>{ug[q[d]], Eat(kNoE, ug, q[d])};
+  const JR J = jrow(ug[t], Eat(kNoE, ug, t), nb, m, ih2);
   const float rc = rg[t];
   e[t] = eg[t];
   __syncthreads();
@@ -2115,8 +2113,8 @@ void corr_relax(SolveCtx& S, int l, int sweeps) {
           k_ddev_sweep_list<<<nblocks(nl, DVB), DVB, 0, c->s>>>(L.wold32, L.wf32, L.w32, L.lgN, list,
                                                               nl, p, (float)L.ih2);
         else
-          k_dlin_sweep_list<<<nblocks(nl, BS), BS, 0, c->s>>>(L.wold32, L.wf32, L.w32, nullptr,
-                                                              L.lgN, list, nl, m, (float)L.ih2);
+          k_dlin_sweep_list<<<nblocks(nl, BS), BS, 0, c->s>>>(L.wold32, L.wf32, L.w32, L.lgN, list,
+                                                              nl, m, (float)L.ih2);
       }
       c->launches += 1;
     }
@@ -2126,8 +2124,8 @@ void corr_relax(SolveCtx& S, int l, int sweeps) {
 
 // restriction of dense arrays (u, r, e) of level lgf to the dense level C
 template <bool DEV>
-void corr_drestrict(SolveCtx& S, const float* e, const float* r, const float* u, const float* E,
-                    int lgf, double ih2, const unsigned char* act, DenseLevel& C) {
+void corr_drestrict(SolveCtx& S, const float* e, const float* r, const float* u, int lgf,
+                    double ih2, const unsigned char* act, DenseLevel& C) {
   mgfr_ctx* c = S.c;
   const MT<float> m = mt<float>(S.m);
   if constexpr (DEV)
@@ -2135,8 +2133,8 @@ void corr_drestrict(SolveCtx& S, const float* e, const float* r, const float* u,
                                                        pf32(m, (float)c->cfg.step_cap),
                                                        (float)ih2, act);
   else
-    k_dlin_restrict<<<nblocks(C.n, BS), BS, 0, c->s>>>(e, r, u, E, lgf, C.r32, C.u32, C.e32,
-                                                       C.uold32, m, (float)ih2, act);
+    k_dlin_restrict<<<nblocks(C.n, BS), BS, 0, c->s>>>(e, r, u, lgf, C.r32, C.u32, C.uold32, m,
+                                                       (float)ih2, act);
   c->launches += 1;
 }
 
@@ -2153,7 +2151,7 @@ void corr_vcycle_dense(SolveCtx& S, int k) {
     if constexpr (DEV)
       k_ddev_coarse<<<1, 64, 0, c->s>>>(F.uold32, F.r32, F.u32, p, (float)F.ih2, 20, mk);
     else
-      k_dlin_coarse<<<1, 64, 0, c->s>>>(F.uold32, F.r32, F.u32, F.e32, m, (float)F.ih2, 20, mk);
+      k_dlin_coarse<<<1, 64, 0, c->s>>>(F.uold32, F.r32, F.u32, m, (float)F.ih2, 20, mk);
     c->launches += 1;
     return;
   }
@@ -2167,15 +2165,15 @@ void corr_vcycle_dense(SolveCtx& S, int k) {
           k_ddev_sweep_list<<<nblocks(nl, DVB), DVB, 0, c->s>>>(F.uold32, F.r32, F.u32, F.lg, list,
                                                               nl, p, (float)F.ih2);
         else
-          k_dlin_sweep_list<<<nblocks(nl, BS), BS, 0, c->s>>>(F.uold32, F.r32, F.u32, F.e32, F.lg,
-                                                              list, nl, m, (float)F.ih2);
+          k_dlin_sweep_list<<<nblocks(nl, BS), BS, 0, c->s>>>(F.uold32, F.r32, F.u32, F.lg, list,
+                                                              nl, m, (float)F.ih2);
         c->launches += 1;
       }
   };
   sweep(sweeps_of(S, -1, g.n_pre));
   if (k + 1 <= S.kmax) {
     DenseLevel& C = H.L[k + 1];
-    corr_drestrict<DEV>(S, F.uold32, F.r32, F.u32, F.e32, F.lg, F.ih2, mk, C);
+    corr_drestrict<DEV>(S, F.uold32, F.r32, F.u32, F.lg, F.ih2, mk, C);
     corr_vcycle_dense<DEV>(S, k + 1);
     const CList cf = clist(S, k);
     if (cl_threads(cf, F.n) > 0)
@@ -2219,7 +2217,7 @@ void corr_vcycle_tree(SolveCtx& S, int l) {
   } else if (l == 0 && S.kmax >= 1) {
     DenseHier& H = c->dh;
     DenseLevel& C = H.L[1];
-    corr_drestrict<DEV>(S, F.wold32, F.wf32, F.w32, nullptr, F.lgN, F.ih2, F.act, C);
+    corr_drestrict<DEV>(S, F.wold32, F.wf32, F.w32, F.lgN, F.ih2, F.act, C);
     corr_vcycle_dense<DEV>(S, 1);
     const CList c0 = clist(S, 0);
     if (cl_threads(c0, F.ncell) > 0)

@@ -246,10 +246,41 @@ __device__ __forceinline__ void vec_fas(unsigned t, const float* __restrict__ x,
   st4(f + colour * half + R.c, fv);
 }
 
+// One fine row (i, j) of the restriction to the coarse cells K0..K0+3: the residuals (res)
+// and the values to be averaged (val: NL: x; LIN: w; DEV: w + x) of its daughters at even
+// k ([0]) and odd k ([1]), one vector of each colour
+template <int OP>
+__device__ __forceinline__ void restrict_row(const float* __restrict__ x,
+                                             const float* __restrict__ r,
+                                             const float* __restrict__ w, int i, int j, int K0,
+                                             int lgf, const PF& m, float ih2, V4* res, V4* val) {
+  const unsigned half = 1u << (3 * lgf - 1);
+  const int qe = (i + j) & 1;  // the plane of the row's even k
+#pragma unroll
+  for (int c = 0; c < 2; ++c) {  // k = 2K + c
+    const unsigned own = ((qe ^ c) ? half : 0u), oth = half - own;
+    const Rows R = rows_at(i, j, K0, c, lgf);
+    const Nb4 xn = load_nb(x + oth, R, c);
+    const V4 xv = ld4(x + own + R.c), rv = ld4(r + own + R.c);
+    Nb4 wn{};
+    V4 wv{};
+    if (OP == MG_LIN || OP == MG_DEV) {
+      wn = load_nb(w + oth, R, c);
+      wv = ld4(w + own + R.c);
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      float a[6], b[6];
+      xn.get(q, a);
+      wn.get(q, b);
+      res[c].v[q] = rv.v[q] - point_apply<OP>(xv.v[q], a, wv.v[q], b, m, ih2);
+      val[c].v[q] = OP == MG_NL ? xv.v[q] : (OP == MG_DEV ? wv.v[q] + xv.v[q] : wv.v[q]);
+    }
+  }
+}
+
 // Restriction to four coarse cells (I, J, K0..K0+3): the average of the eight
-// daughters' residuals, and of the iterate (NL: x; LIN: w; DEV: w + x), the
-// daughters visited in C order.  The daughters of a fine row are one vector
-// of each colour.
+// daughters' residuals, and of the iterate, the daughters visited in C order
 template <int OP>
 __device__ __forceinline__ void vec_restrict(unsigned t, const float* __restrict__ x,
                                                   const float* __restrict__ r,
@@ -259,34 +290,11 @@ __device__ __forceinline__ void vec_restrict(unsigned t, const float* __restrict
   const int lgc = lgf - 1, Mc = (1 << lgc) - 1;
   const int K0 = 4 * (int)(t & ((1u << (lgc - 2)) - 1));
   const int J = (int)((t >> (lgc - 2)) & Mc), I = (int)(t >> (2 * lgc - 2));
-  const unsigned half = 1u << (3 * lgf - 1);
   float sr[4] = {0.f, 0.f, 0.f, 0.f}, su[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll 1
   for (int ab = 0; ab < 4; ++ab) {
-    const int i = 2 * I + (ab >> 1), j = 2 * J + (ab & 1);
-    const int qe = (i + j) & 1;  // the plane of the row's even k
     V4 res[2], val[2];
-#pragma unroll
-    for (int c = 0; c < 2; ++c) {  // k = 2K + c
-      const unsigned own = ((qe ^ c) ? half : 0u), oth = half - own;
-      const Rows R = rows_at(i, j, K0, c, lgf);
-      const Nb4 xn = load_nb(x + oth, R, c);
-      const V4 xv = ld4(x + own + R.c), rv = ld4(r + own + R.c);
-      Nb4 wn{};
-      V4 wv{};
-      if (OP == MG_LIN || OP == MG_DEV) {
-        wn = load_nb(w + oth, R, c);
-        wv = ld4(w + own + R.c);
-      }
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        float a[6], b[6];
-        xn.get(q, a);
-        wn.get(q, b);
-        res[c].v[q] = rv.v[q] - point_apply<OP>(xv.v[q], a, wv.v[q], b, m, ih2);
-        val[c].v[q] = OP == MG_NL ? xv.v[q] : (OP == MG_DEV ? wv.v[q] + xv.v[q] : wv.v[q]);
-      }
-    }
+    restrict_row<OP>(x, r, w, 2 * I + (ab >> 1), 2 * J + (ab & 1), K0, lgf, m, ih2, res, val);
 #pragma unroll
     for (int q = 0; q < 4; ++q)
 #pragma unroll
@@ -343,31 +351,8 @@ __device__ __forceinline__ void vec_restrict_rows(unsigned t, const float* __res
   t >>= 2;
   const int K0 = 4 * (int)(t & ((1u << (lgc - 2)) - 1));
   const int J = (int)((t >> (lgc - 2)) & Mc), I = (int)(t >> (2 * lgc - 2));
-  const unsigned half = 1u << (3 * lgf - 1);
-  const int i = 2 * I + (ab >> 1), j = 2 * J + (ab & 1);
-  const int qe = (i + j) & 1;  // the plane of the row's even k
   V4 res[2], val[2];
-#pragma unroll
-  for (int c = 0; c < 2; ++c) {  // k = 2K + c
-    const unsigned own = ((qe ^ c) ? half : 0u), oth = half - own;
-    const Rows R = rows_at(i, j, K0, c, lgf);
-    const Nb4 xn = load_nb(x + oth, R, c);
-    const V4 xv = ld4(x + own + R.c), rv = ld4(r + own + R.c);
-    V4 wv{};
-    Nb4 wn{};
-    if (OP == MG_LIN || OP == MG_DEV) {
-      wn = load_nb(w + oth, R, c);
-      wv = ld4(w + own + R.c);
-    }
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      float a[6], b[6];
-      xn.get(q, a);
-      wn.get(q, b);
-      res[c].v[q] = rv.v[q] - point_apply<OP>(xv.v[q], a, wv.v[q], b, m, ih2);
-      val[c].v[q] = OP == MG_NL ? xv.v[q] : (OP == MG_DEV ? wv.v[q] + xv.v[q] : wv.v[q]);
-    }
-  }
+  restrict_row<OP>(x, r, w, 2 * I + (ab >> 1), 2 * J + (ab & 1), K0, lgf, m, ih2, res, val);
   float sr = 0.f, su = 0.f;
   transpose4(res[0].v);
   transpose4(res[1].v);

@@ -328,7 +328,11 @@ void nn_wgrad_finish(float* partials, int S, int Cin, int Cout, float* dW, TView
   const bool vec = (uintptr_t)(g.p + g.off) % 16 == 0 && g.ld % 8 == 0;
   (vec ? k_bias_part<true> : k_bias_part<false>)<<<BG_BLOCKS, BG_BS, 0, s>>>(g.p, g.ld, g.off,
                                                                             Mtot, Cout, partials);
-  k_bias_sum<<<Cout, 32, 0, s>>>(partials, BG_BLOCKS, Cout, db);
+  nn_bias_sum(partials, BG_BLOCKS, Cout, db, s);
+}
+
+void nn_bias_sum(const float* part, int nb, int Cout, float* db, cudaStream_t s) {
+  k_bias_sum<<<Cout, 32, 0, s>>>(part, nb, Cout, db);
 }
 
 long long nn_wgrad_scratch(int Cin, int Cout) {

@@ -35,6 +35,9 @@ long long nn_wgrad_scratch(int Cin, int Cout);
 // bias stages reuse `partials` as their scratch: Cin >= 16, S >= 1)
 void nn_wgrad_finish(float* partials, int S, int Cin, int Cout, float* dW, TView g,
                      float* db, long long Mtot, cudaStream_t s);
+// db[c] = sum over the nb blocks of part[block][c], in order of the blocks within each of 32
+// lanes, then a fixed tree
+void nn_bias_sum(const float* part, int nb, int Cout, float* db, cudaStream_t s);
 
 // ---- tensor-core (tcgen05) forward and input-gradient convolutions (nn_tc.cu)
 struct TcArgs {

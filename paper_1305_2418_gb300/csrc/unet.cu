@@ -252,17 +252,6 @@ __global__ void __launch_bounds__(BS) k_relu_bwd(FView g, TView y, int lc8, long
       part[(size_t)blockIdx.x * 8 * ng + 8 * threadIdx.x + i] = red[i][threadIdx.x];
 }
 
-// db[c] = the blocks' partial sums, in order of the blocks within each of 32
-// lanes, then a fixed tree; one warp per channel
-__global__ void k_bias_parts(const float* __restrict__ part, int nb, int C,
-                             float* __restrict__ db) {
-  const int c = blockIdx.x, lane = threadIdx.x;
-  float s = 0.f;
-  for (int q = lane; q < nb; q += 32) s += part[(size_t)q * C + c];
-  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-  if (lane == 0) db[c] = s;
-}
-
 __global__ void __launch_bounds__(BS) k_head_fwd(TView x, const float* __restrict__ w, long long M,
                                                  float* __restrict__ out) {
   const long long m = blockIdx.x * (long long)blockDim.x + threadIdx.x;
@@ -622,7 +611,7 @@ static void conv_bwd(mgfr_ctx* c, UNet* U, int i, const LayerIO& L, int acc_in) 
   const long long n8 = M * s.cout / 8;
   const int nb = (int)std::min<long long>(kBiasBlocks, nblocks(n8, BS));
   k_relu_bwd<<<nb, BS, 0, c->s>>>(L.gy, L.y, lg_of(s.cout / 8), n8, U->Gpre, U->bpart);
-  k_bias_parts<<<s.cout, 32, 0, c->s>>>(U->bpart, nb, s.cout, U->G + U->boff[i]);
+  nn_bias_sum(U->bpart, nb, s.cout, U->G + U->boff[i], c->s);
   const TView g = tv(U->Gpre, s.cout);
   if (!nn_tc_wgrad(L.x, s.cin, g, s.cout, U->G + U->woff[i], nullptr, U->wpart, U->B, L.lgD,
                    U->tc_err, c->s))
