@@ -29,7 +29,8 @@
  *  - Memory: every pointer named *_dev is device memory owned by the caller;
  *    it must stay valid until the call returns.  The library allocates its
  *    own workspaces inside the context (freed by mgfr_destroy): a dense grid
- *    takes 43 bytes per cell in the FP64 form and 55 in the mixed form, a
+ *    takes 43 bytes per cell in the FP64 form (29 where there is no room for
+ *    more: its cycles are then slower) and 55 in the mixed form, a
  *    particle-mesh potential 29 per cell of its grid and its force 32 more.  The
  *    arrays of refined levels (about 140 bytes per cell) are kept from one
  *    particle solve to the next while they are at most twice too large, and made

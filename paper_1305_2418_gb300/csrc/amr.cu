@@ -1138,9 +1138,14 @@ static bool give_back_levels(mgfr_ctx* c) {
   return any;
 }
 
+static bool give_back(mgfr_ctx* c) {
+  const bool levels = give_back_levels(c), conv = conv_scratch_trim(c->device);
+  return levels || conv;
+}
+
 cudaError_t dev_malloc_bytes(mgfr_ctx* c, void** p, size_t bytes) {
   const cudaError_t e = cudaMalloc(p, bytes);
-  if (e != cudaErrorMemoryAllocation || !give_back_levels(c)) return e;
+  if (e != cudaErrorMemoryAllocation || !give_back(c)) return e;
   (void)cudaGetLastError();
   return cudaMalloc(p, bytes);
 }
@@ -1504,26 +1509,30 @@ static mgfr_status solve_particles_once(mgfr_ctx* c, const double* pos, long lon
   return worst;
 }
 
-// Where the device's memory runs out, once more from the start with all refined levels
-// given back and made exactly as large as they have to be.
+// Where the device's memory runs out, again from the start with all refined levels given
+// back and made exactly as large as they have to be, and in the FP64 form, if that is not
+// enough, without the dense grids' FP32 arrays.
 static mgfr_status solve_particles(mgfr_ctx* c, const double* pos, long long Np, int N0, double box,
                                    double a, const double* u_init, double* fr_out,
                                    double* acc_out, double* acc_host, mgfr_stats* st) {
   if (!c) return MGFR_E_INVALID;
   TRY(check_particle_args(c, pos, Np, N0, box, a));
-  const mgfr_status rs =
-      solve_particles_once(c, pos, Np, N0, box, a, u_init, fr_out, acc_out, acc_host, st);
-  if (rs != MGFR_E_OOM || !c->amr) return rs;
-  AmrWork* A = W(c);
-  MG_CK(c, cudaStreamSynchronize(c->s));
-  amr_invalidate(c);
-  if (!give_back_levels(c)) return rs;
-  c->err.clear();
-  A->exact = true;
-  const mgfr_status again =
-      solve_particles_once(c, pos, Np, N0, box, a, u_init, fr_out, acc_out, acc_host, st);
-  A->exact = false;
-  return again;
+  auto once = [&]() {
+    return solve_particles_once(c, pos, Np, N0, box, a, u_init, fr_out, acc_out, acc_host, st);
+  };
+  mgfr_status rs = once();
+  for (int less = 1; rs == MGFR_E_OOM && c->amr && less <= 2; ++less) {
+    if (less == 2 && (c->cfg.precision == MGFR_PREC_MIXED || c->dh.mixed)) break;
+    MG_CK(c, cudaStreamSynchronize(c->s));
+    amr_invalidate(c);
+    if (!give_back(c) && less == 1) continue;
+    c->err.clear();
+    W(c)->exact = true;
+    c->no_fp32 = less == 2;
+    rs = once();
+    W(c)->exact = c->no_fp32 = false;
+  }
+  return rs;
 }
 
 mgfr_status mgfr_solve_particles(mgfr_ctx* c, const double* pos, long long Np, int N0, double box,

@@ -2472,7 +2472,7 @@ mgfr_status amr_solve_level(mgfr_ctx* c, AmrWork* A, int Lv, const Model& m, mgf
   // solve was in the FP64 oct sweeps alone), in FP64 throughout while the residual
   // is beyond kDevMax ||f|| and from the first FP32 cycle that gains nothing
   constexpr double kDevMax = 2.0;
-  bool dev_ok = !mixed, coarse64 = mixed;
+  bool dev_ok = !mixed && H.fp32, coarse64 = mixed;
   if (dev_ok && r > target) TRY(zero_corr());
   while (r > target && it < g.max_vcycles) {
     if (dev_ok && r <= kDevMax * ref) {

@@ -54,6 +54,7 @@ struct DenseLevel {
 struct DenseHier {
   int N = 0, nlev = 0;
   bool mixed = false;
+  bool fp32 = false;  // the FP32 arrays exist
   DenseLevel L[MGFR_MAX_DENSE];
   double* partials = nullptr;  // reduction scratch (2 doubles per block)
   double* scal = nullptr;      // device scalars: [0..1] last norm, [2..7] spare
@@ -127,6 +128,7 @@ struct mgfr_ctx {
   cudaEvent_t ev_chunk[8] = {}, ev_copy = nullptr;
   std::string err;
   DenseHier dh;
+  bool no_fp32 = false;         // a solve in the FP64 form without the dense FP32 arrays
   double* host_scal = nullptr;  // pinned: norms read back by the host
   // captured V-cycle graphs (FP64 all through / FP64 with FP32 corrections /
   // FP32 nonlinear / linear phase)
@@ -179,7 +181,8 @@ mgfr_status set_err(mgfr_ctx* c, mgfr_status st, const std::string& msg);
 // Range checks of a configuration (false and the reason in why if invalid).
 bool validate_cfg(const mgfr_config* c, std::string& why);
 // cudaMalloc for a context's workspaces: where memory runs out, once more after the
-// refined levels of the context have given back what they hold beyond need (amr.cu).
+// refined levels of the context have given back what they hold beyond need (amr.cu) and
+// the convolution primitive its scratch.
 // Not for the arrays of a hierarchy that is being built.
 cudaError_t dev_malloc_bytes(mgfr_ctx* c, void** p, size_t bytes);
 template <class T>
@@ -188,8 +191,9 @@ cudaError_t dev_malloc(mgfr_ctx* c, T** p, size_t bytes) {
 }
 void batch_free(mgfr_ctx* c);
 void unet_free(mgfr_ctx* c);
-// give back the convolution primitive's scratch on this device (unet.cu)
-void conv_scratch_trim(int dev);
+// give back the convolution primitive's scratch on this device (unet.cu); whether there was
+// any
+bool conv_scratch_trim(int dev);
 void pm_free(mgfr_ctx* c);
 #define MG_CK(ctx, call)                                                                  \
   do {                                                                                    \

@@ -286,22 +286,31 @@ struct PmWork {
   double* part = nullptr;     // block sums (device)
   double* part_h = nullptr;   // block sums (page-locked host)
   int nparts = 0;
+  bool solve_gone = false;    // only phi and the force's arrays are left
 };
 
+// what the solve needs beside phi; the next solve then starts from nothing
+void pm_free_solve(PmWork* P) {
+  auto drop = [](auto*& p) {
+    if (p) cudaFree(p);
+    p = nullptr;
+  };
+  drop(P->rhs), drop(P->rlo);
+  for (int l = 0; l < PM_MAXL; ++l) drop(P->e[l]), drop(P->r[l]);
+  P->solve_gone = true;
+}
+
 void pm_free_work(PmWork* P) {
-  void* ps[] = {P->phi, P->rhs, P->rlo, P->grad, P->part};
+  pm_free_solve(P);
+  void* ps[] = {P->phi, P->grad, P->part};
   for (void* p : ps)
     if (p) cudaFree(p);
-  for (int l = 0; l < PM_MAXL; ++l) {
-    if (P->e[l]) cudaFree(P->e[l]);
-    if (P->r[l]) cudaFree(P->r[l]);
-  }
   if (P->part_h) cudaFreeHost(P->part_h);
   *P = PmWork();
 }
 
 mgfr_status pm_alloc(mgfr_ctx* c, PmWork* P, int lg, double box) {
-  if (P->lg != lg) {
+  if (P->lg != lg || P->solve_gone) {
     pm_free_work(P);
     mgfr_status ps = mg32_prepare(c);
     if (ps != MGFR_OK) return ps;
@@ -487,7 +496,14 @@ extern "C" mgfr_status mgfr_pm_accel(mgfr_ctx* c, int lpm, int what, const doubl
   PmWork* P = nullptr;
   mgfr_status rs = pm_solve(c, lpm, what, nullptr, nullptr, st, &P);
   if (rs != MGFR_OK && rs != MGFR_E_NOCONVERGE) return rs;
-  if (!P->grad) MG_CK(c, dev_malloc(c, &P->grad, 2 * sizeof(float4) * (size_t)P->n));
+  const size_t gb = 2 * sizeof(float4) * (size_t)P->n;
+  if (!P->grad && dev_malloc(c, &P->grad, gb) != cudaSuccess) {
+    // the force needs phi alone: the solve's other arrays make room (21 of the 32 bytes per
+    // cell) and are made again by the next solve
+    (void)cudaGetLastError();
+    pm_free_solve(P);
+    MG_CK(c, dev_malloc(c, &P->grad, gb));
+  }
   k_pm_grad<<<nblocks(P->n, BS), BS, 0, c->s>>>(P->phi, P->lg, df_from_double(0.5 / P->h), P->grad);
   k_pm_cic<<<nblocks(Np, BS), BS, 0, c->s>>>(pos_dev, Np, P->lg, 1.0 / P->h, P->grad, acc_out_dev);
   c->launches += 2;

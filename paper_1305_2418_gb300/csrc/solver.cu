@@ -215,8 +215,47 @@ static void drop_graphs(mgfr_ctx* c) {
   for (int g = 0; g < 5; ++g) prof_clear(c, g);
 }
 
-// The arrays of the dense hierarchy N, N/2, ..., 4 (f and the double-float copy
-// of it for the mixed form only).
+// The FP32 arrays: the correction cycles of both forms, and for the mixed form f and its
+// double-float copy
+static mgfr_status alloc_dense32(mgfr_ctx* c, DenseHier& H, bool mixed) {
+  for (int l = 0; l < H.nlev; ++l) {
+    DenseLevel& L = H.L[l];
+    const size_t b4 = sizeof(float) * (size_t)L.n;
+    MG_CK(c, dev_malloc(c, &L.u32, b4));
+    MG_CK(c, dev_malloc(c, &L.e32, b4));
+    MG_CK(c, dev_malloc(c, &L.r32, b4));
+    if (l > 0) MG_CK(c, dev_malloc(c, &L.uold32, b4));
+    if (mixed) MG_CK(c, dev_malloc(c, &L.f32, b4));
+  }
+  if (mixed) MG_CK(c, dev_malloc(c, &H.fdf, sizeof(double) * (size_t)H.L[0].n));
+  H.fp32 = true;
+  return MGFR_OK;
+}
+
+static void free_dense32(DenseHier& H) {
+  auto drop = [](auto*& p) {
+    if (p) cudaFree(p);
+    p = nullptr;
+  };
+  for (int l = 0; l < H.nlev; ++l) {
+    DenseLevel& L = H.L[l];
+    drop(L.u32), drop(L.e32), drop(L.r32), drop(L.uold32), drop(L.f32);
+  }
+  drop(H.fdf);
+  H.fp32 = false;
+}
+
+// The FP32 arrays of the FP64 form: without the memory for them (12 of its 43 bytes per
+// cell) its cycles run in FP64 throughout
+static mgfr_status try_dense32(mgfr_ctx* c, DenseHier& H) {
+  const mgfr_status rs = alloc_dense32(c, H, false);
+  if (rs != MGFR_E_OOM) return rs;
+  free_dense32(H);
+  c->err.clear();
+  return MGFR_OK;
+}
+
+// The arrays of the dense hierarchy N, N/2, ..., 4
 static mgfr_status alloc_dense(mgfr_ctx* c, DenseHier& H, int N, bool mixed) {
   int lg = 0;
   while ((1 << lg) < N) ++lg;
@@ -226,21 +265,18 @@ static mgfr_status alloc_dense(mgfr_ctx* c, DenseHier& H, int N, bool mixed) {
     L.lg = lg - l;
     L.N = 1 << L.lg;
     L.n = 1LL << (3 * L.lg);
-    size_t b8 = sizeof(double) * (size_t)L.n, b4 = sizeof(float) * (size_t)L.n;
+    const size_t b8 = sizeof(double) * (size_t)L.n;
     MG_CK(c, dev_malloc(c, &L.u, b8));
     MG_CK(c, dev_malloc(c, &L.E, b8));
     MG_CK(c, dev_malloc(c, &L.f, b8));
     if (l > 0) MG_CK(c, dev_malloc(c, &L.uold, b8));
-    MG_CK(c, dev_malloc(c, &L.u32, b4));
-    MG_CK(c, dev_malloc(c, &L.e32, b4));
-    MG_CK(c, dev_malloc(c, &L.r32, b4));
-    if (l > 0) MG_CK(c, dev_malloc(c, &L.uold32, b4));
-    if (mixed) MG_CK(c, dev_malloc(c, &L.f32, b4));
   }
   H.nparts = 152 * 8;
-  if (mixed) MG_CK(c, dev_malloc(c, &H.fdf, sizeof(double) * (size_t)H.L[0].n));
   MG_CK(c, dev_malloc(c, &H.partials, sizeof(double) * 2 * H.nparts));
   MG_CK(c, dev_malloc(c, &H.scal, sizeof(double) * 16));
+  const mgfr_status rs =
+      mixed ? alloc_dense32(c, H, true) : (c->no_fp32 ? MGFR_OK : try_dense32(c, H));
+  if (rs != MGFR_OK) return rs;
   H.N = N;
   H.mixed = mixed;
   return MGFR_OK;
@@ -248,7 +284,14 @@ static mgfr_status alloc_dense(mgfr_ctx* c, DenseHier& H, int N, bool mixed) {
 
 static mgfr_status ensure_dense(mgfr_ctx* c, int N, bool mixed) {
   DenseHier& H = c->dh;
-  if (H.N == N && (H.mixed || !mixed)) return MGFR_OK;
+  if (H.N == N && (H.mixed || !mixed)) {
+    if (!c->no_fp32) return H.fp32 ? MGFR_OK : try_dense32(c, H);
+    if (!H.mixed && H.fp32) {
+      drop_graphs(c);  // the cycles captured on them
+      free_dense32(H);
+    }
+    return MGFR_OK;
+  }
   mgfr_status ps = mg32_prepare(c);
   if (ps != MGFR_OK) return ps;
   drop_graphs(c);
@@ -418,7 +461,10 @@ mgfr_status dense_solve64(mgfr_ctx* c, const Model& m, double box, mgfr_stats* s
   const mgfr_config& g = c->cfg;
   double* hs = c->host_scal;
   f64::norm(L0.f, L0.n, H.partials, H.nparts, H.scal + 2, c->s);
-  f64::resid_dev(L0, m, H.partials, H.nparts, H.scal, c->s);
+  if (H.fp32)
+    f64::resid_dev(L0, m, H.partials, H.nparts, H.scal, c->s);
+  else
+    f64::resid_norm(L0, m, H.partials, H.nparts, H.scal, c->s);
   c->launches += 4;
   MG_CK(c, cudaMemcpyAsync(hs, H.scal, 4 * sizeof(double), cudaMemcpyDeviceToHost, c->s));
   mgfr_status rs = sync_read(c);
@@ -443,7 +489,7 @@ mgfr_status dense_solve64(mgfr_ctx* c, const Model& m, double box, mgfr_stats* s
     updates_per = cycle32(c, MG_DEV, m, 0);
     if (!pairs) fp64_dev();
   };
-  if (!c->g_dev || std::strcmp(key, c->keydev) != 0) {
+  if (H.fp32 && (!c->g_dev || std::strcmp(key, c->keydev) != 0)) {
     if (c->g_dev) cudaGraphExecDestroy(c->g_dev);
     c->g_dev = nullptr;
     mgfr_status cs = capture(c, 4, &c->g_dev, bodydev);
@@ -454,7 +500,7 @@ mgfr_status dense_solve64(mgfr_ctx* c, const Model& m, double box, mgfr_stats* s
   // the V-cycle in FP64 throughout, for a start far from the solution, whose
   // residual (kDevMax ||f|| and more; ||f|| at the zero start) FP32 cannot
   // resolve against f, and from the first FP32 cycle that gains nothing (its
-  // correction is taken back)
+  // correction is taken back); without the FP32 arrays always
   constexpr double kDevMax = 2.0;
   auto body64 = [&]() {
     updates_per = 0;
@@ -463,7 +509,7 @@ mgfr_status dense_solve64(mgfr_ctx* c, const Model& m, double box, mgfr_stats* s
     cudaMemcpyAsync(hs, H.scal, 2 * sizeof(double), cudaMemcpyDeviceToHost, c->s);
   };
   const double ref = fn > 0.0 ? fn : r0;
-  bool dev_ok = true;
+  bool dev_ok = H.fp32;
   double r = r0, rho = 0.0;  // rho: reduction of the last cycle
   int it = 0;
   long long updates = 0;

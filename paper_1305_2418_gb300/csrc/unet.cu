@@ -1043,13 +1043,16 @@ mgfr_status scratch_finish(ConvScratch& b, cudaStream_t s) {
 }
 }  // namespace
 
-void conv_scratch_trim(int dev) {
+bool conv_scratch_trim(int dev) {
   std::lock_guard<std::mutex> lk(g_scratch_mu);
+  bool any = false;
   for (size_t i = g_scratch.size(); i-- > 0;)
     if (g_scratch[i].dev == dev) {
       scratch_drop(g_scratch[i]);
       g_scratch.erase(g_scratch.begin() + i);
+      any = true;
     }
+  return any;
 }
 
 extern "C" {

@@ -2,7 +2,8 @@
 context work, and what the library holds in reserve never makes a call fail.
 
 The device is filled by one torch allocation (nothing is written to it) up to some
-memory left."""
+memory left.  What the driver itself frees when memory runs out is of the order of 0.1 GB:
+the sizes leave or lack several times that."""
 import contextlib
 import gc
 
@@ -55,21 +56,45 @@ def field(dev, N, seed):
 
 @pytest.mark.parametrize("prec", [mgfr.PREC_FP64, mgfr.PREC_MIXED])
 def test_a_dense_solve_after_one_without_memory(dev, prec):
-    """256^3 takes 0.7 GB and more beside its 0.13 GB result: with 0.65 GB it fails twice, a
-    small solve after that works, and 256^3 works once there is room."""
+    """512^3 takes 3.7 GB and more beside its 1 GB result: with 2.5 GB it fails twice, a
+    small solve after that works, and 512^3 works once there is room."""
     box = 100.0
-    big, small = field(dev, 256, 1), field(dev, 32, 2)
+    big, small = field(dev, 512, 1), field(dev, 32, 2)
     with mgfr_solver(precision=prec) as s:
         want_small = s.solve_density(small, box)["fr"].clone()
         want_big = s.solve_density(big, box)["fr"].clone()
     torch.cuda.empty_cache()
     with mgfr_solver(precision=prec) as s:
-        with only(dev, 0.65 * GB):
+        with only(dev, 2.5 * GB):
             fails_for_memory(lambda: s.solve_density(big, box, want_acc=False))
             fails_for_memory(lambda: s.solve_density(big, box, want_acc=False))
             assert torch.equal(s.solve_density(small, box)["fr"], want_small)
         assert torch.equal(s.solve_density(big, box)["fr"], want_big)
         assert torch.equal(s.solve_density(small, box)["fr"], want_small)
+
+
+def test_an_fp64_solve_without_the_fp32_arrays(dev):
+    """512^3 in the FP64 form: its FP64 arrays take 3.6 GB, the FP32 ones of the correction
+    cycles 1.8 GB more.  Without room for those the cycles run in FP64: the same field
+    within the tolerance (1e-8 of the source, 1e2 for the operator's inverse); with room
+    again they are back."""
+    box, big = 100.0, field(dev, 512, 1)
+    with mgfr_solver() as s:
+        out = s.solve_density(big, box)
+        want, launches = out["fr"].cpu(), out["stats"]["gpu_launches"]
+        del out
+    with mgfr_solver() as s:
+        with only(dev, (1.0 + 3.6 + 0.7) * GB):
+            for _ in range(2):
+                out = s.solve_density(big, box, want_acc=False)
+                assert out["status"] == mgfr.MGFR_OK
+                got = out["fr"].cpu()
+                # a launch per half-sweep of every grid: more than the cycles in FP32
+                assert out["stats"]["gpu_launches"] > 1.5 * launches
+                del out
+                assert float((got / want - 1.0).abs().max()) <= 1e-6
+        out = s.solve_density(big, box)
+        assert torch.equal(out["fr"].cpu(), want) and out["stats"]["gpu_launches"] == launches
 
 
 def test_a_prediction_after_one_without_memory(dev):
@@ -163,3 +188,46 @@ def test_a_kept_level_does_not_take_a_later_solves_memory(dev):
         assert [s.level_info(l) for l in range(3)] == levels
         fr = s.level_field(2, mgfr.FIELD_FR)
         assert np.isfinite(fr).all() and (fr < 0.0).all()
+
+
+def test_an_fp64_particle_solve_without_the_fp32_arrays(dev):
+    """512^3 base, one level of some 60 M cells: room for exact level arrays, but for half of
+    the dense grids' FP32 arrays (1.8 GB) only.  Two solutions to 1e-9 of the source,
+    the force at the particles within 1e-5 (1e2 for the operator's inverse, 1e2 for its
+    gradient)."""
+    pos = particles(dev, 80_000_000, 0.05, 7)
+    cfg = dict(max_level=1, tol_rel=1e-9)
+    with mgfr_solver(**cfg) as s:
+        need = held(dev, lambda: s.solve_particles(pos, 512, BOX))
+        out = s.solve_particles(pos, 512, BOX)
+        want, n = out["acc"].cpu(), s.level_info(1)[0]
+        launches = out["stats"]["gpu_launches"]
+        del out
+    reserve = n // 16 * 8 * 139
+    own = pos.numel() * 8 + 512 ** 3 * 8
+    with mgfr_solver(**cfg) as s:
+        with only(dev, need - reserve - (900 << 20) + own):
+            out = s.solve_particles(pos, 512, BOX)
+            assert out["status"] == mgfr.MGFR_OK
+            got = out["acc"].cpu()
+            assert out["stats"]["gpu_launches"] > 1.2 * launches
+            del out
+        assert rel(got, want) <= 1e-5
+        assert rel(s.solve_particles(pos, 512, BOX)["acc"].cpu(), want) <= 1e-9
+
+
+def test_a_force_in_the_room_of_the_solve(dev):
+    """The particle-mesh force's arrays (32 bytes per cell of 512^3: 4.3 GB) in what phi and
+    the solve's 21 bytes per cell leave: the solve's arrays make room, and come back."""
+    pos = particles(dev, 300_000, 1.0, 9)
+    with mgfr_solver(precision=mgfr.PREC_MIXED, tol_rel=1e-5) as s:
+        s.solve_particles(pos, 64, BOX)
+        want = s.pm_accel(pos, 3)[0].clone()
+    with mgfr_solver(precision=mgfr.PREC_MIXED, tol_rel=1e-5) as s:
+        s.solve_particles(pos, 64, BOX)
+        with only(dev, (8 + 32 + 4) * 512 ** 3):
+            assert rel(s.pm_accel(pos, 3)[0], want) <= 1e-9
+            assert rel(s.pm_accel(pos, 3)[0], want) <= 1e-9
+        assert rel(s.pm_accel(pos, 3)[0], want) <= 1e-9
+        phi = s.pm_potential(64, 3)[0]
+        assert bool(torch.isfinite(phi).all())
