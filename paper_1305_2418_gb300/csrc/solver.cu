@@ -215,20 +215,14 @@ static void drop_graphs(mgfr_ctx* c) {
   for (int g = 0; g < 5; ++g) prof_clear(c, g);
 }
 
-// The FP32 arrays: the correction cycles of both forms, and for the mixed form f and its
-// double-float copy
-static mgfr_status alloc_dense32(mgfr_ctx* c, DenseHier& H, bool mixed) {
-  for (int l = 0; l < H.nlev; ++l) {
-    DenseLevel& L = H.L[l];
-    const size_t b4 = sizeof(float) * (size_t)L.n;
-    MG_CK(c, dev_malloc(c, &L.u32, b4));
-    MG_CK(c, dev_malloc(c, &L.e32, b4));
-    MG_CK(c, dev_malloc(c, &L.r32, b4));
-    if (l > 0) MG_CK(c, dev_malloc(c, &L.uold32, b4));
-    if (mixed) MG_CK(c, dev_malloc(c, &L.f32, b4));
-  }
-  if (mixed) MG_CK(c, dev_malloc(c, &H.fdf, sizeof(double) * (size_t)H.L[0].n));
-  H.fp32 = true;
+// The FP32 arrays of level l: the correction cycles of both forms, f for the mixed one
+static mgfr_status alloc_level32(mgfr_ctx* c, DenseLevel& L, int l, bool mixed) {
+  const size_t b4 = sizeof(float) * (size_t)L.n;
+  MG_CK(c, dev_malloc(c, &L.u32, b4));
+  MG_CK(c, dev_malloc(c, &L.e32, b4));
+  MG_CK(c, dev_malloc(c, &L.r32, b4));
+  if (l > 0) MG_CK(c, dev_malloc(c, &L.uold32, b4));
+  if (mixed) MG_CK(c, dev_malloc(c, &L.f32, b4));
   return MGFR_OK;
 }
 
@@ -241,22 +235,11 @@ static void free_dense32(DenseHier& H) {
     DenseLevel& L = H.L[l];
     drop(L.u32), drop(L.e32), drop(L.r32), drop(L.uold32), drop(L.f32);
   }
-  drop(H.fdf);
   H.fp32 = false;
 }
 
-// The FP32 arrays of the FP64 form: without the memory for them (12 of its 43 bytes per
-// cell) its cycles run in FP64 throughout
-static mgfr_status try_dense32(mgfr_ctx* c, DenseHier& H) {
-  const mgfr_status rs = alloc_dense32(c, H, false);
-  if (rs != MGFR_E_OOM) return rs;
-  free_dense32(H);
-  c->err.clear();
-  return MGFR_OK;
-}
-
-// The arrays of the dense hierarchy N, N/2, ..., 4
-static mgfr_status alloc_dense(mgfr_ctx* c, DenseHier& H, int N, bool mixed) {
+// The arrays of the dense hierarchy N, N/2, ..., 4, with (fp32) or without the FP32 ones
+static mgfr_status alloc_dense(mgfr_ctx* c, DenseHier& H, int N, bool mixed, bool fp32) {
   int lg = 0;
   while ((1 << lg) < N) ++lg;
   H.nlev = lg - 1;  // N ... 4
@@ -270,34 +253,50 @@ static mgfr_status alloc_dense(mgfr_ctx* c, DenseHier& H, int N, bool mixed) {
     MG_CK(c, dev_malloc(c, &L.E, b8));
     MG_CK(c, dev_malloc(c, &L.f, b8));
     if (l > 0) MG_CK(c, dev_malloc(c, &L.uold, b8));
+    const mgfr_status rs = fp32 ? alloc_level32(c, L, l, mixed) : MGFR_OK;
+    if (rs != MGFR_OK) return rs;
   }
   H.nparts = 152 * 8;
+  if (mixed) MG_CK(c, dev_malloc(c, &H.fdf, sizeof(double) * (size_t)H.L[0].n));
   MG_CK(c, dev_malloc(c, &H.partials, sizeof(double) * 2 * H.nparts));
   MG_CK(c, dev_malloc(c, &H.scal, sizeof(double) * 16));
-  const mgfr_status rs =
-      mixed ? alloc_dense32(c, H, true) : (c->no_fp32 ? MGFR_OK : try_dense32(c, H));
-  if (rs != MGFR_OK) return rs;
   H.N = N;
   H.mixed = mixed;
+  H.fp32 = fp32;
   return MGFR_OK;
 }
 
+// The dense hierarchy of an N^3 grid.  The FP64 form does without the FP32 arrays (12 of
+// its 43 bytes per cell) where there is no memory for them: its cycles then run in FP64
+// throughout.
 static mgfr_status ensure_dense(mgfr_ctx* c, int N, bool mixed) {
   DenseHier& H = c->dh;
   if (H.N == N && (H.mixed || !mixed)) {
-    if (!c->no_fp32) return H.fp32 ? MGFR_OK : try_dense32(c, H);
-    if (!H.mixed && H.fp32) {
-      drop_graphs(c);  // the cycles captured on them
+    if (H.mixed || H.fp32 == !c->no_fp32) return MGFR_OK;
+    drop_graphs(c);  // the cycles captured on the arrays
+    free_dense32(H);
+    mgfr_status rs = MGFR_OK;
+    for (int l = 0; l < H.nlev && !c->no_fp32 && rs == MGFR_OK; ++l)
+      rs = alloc_level32(c, H.L[l], l, false);
+    H.fp32 = !c->no_fp32 && rs == MGFR_OK;
+    if (rs == MGFR_E_OOM) {
       free_dense32(H);
+      c->err.clear();
+      return MGFR_OK;
     }
-    return MGFR_OK;
+    return rs;
   }
-  mgfr_status ps = mg32_prepare(c);
-  if (ps != MGFR_OK) return ps;
+  mgfr_status rs = mg32_prepare(c);
+  if (rs != MGFR_OK) return rs;
   drop_graphs(c);
   free_dense(H);
   c->u_prev_N = 0;
-  const mgfr_status rs = alloc_dense(c, H, N, mixed);
+  rs = alloc_dense(c, H, N, mixed, mixed || !c->no_fp32);
+  if (rs == MGFR_E_OOM && !mixed && !c->no_fp32) {
+    free_dense(H);
+    c->err.clear();
+    rs = alloc_dense(c, H, N, false, false);
+  }
   if (rs != MGFR_OK) free_dense(H);  // the next call must not take a part for the whole
   return rs;
 }
