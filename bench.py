@@ -682,7 +682,7 @@ def main():
         pm[name] = {"ms": g0.elapsed_time(g1), "vcycles": pst["vcycles"],
                     "res_rel": pst["res_l2_final"] / pst["f_l2"],
                     "gs_cell_updates_per_s": pst["linear_updates"] / (g0.elapsed_time(g1) / 1e3)}
-    pm["grid"] = f"{w['N']}^3 periodic PM grid (the base grid), FP64 linear multigrid to 1e-8"
+    pm["grid"] = f"{w['N']}^3 periodic PM grid (the base grid), linear multigrid (FP32 corrections, FP64 stopping test) to 1e-8"
     sm.close()
 
     # ---- the same steps with CUDA events around each profiled launch ----

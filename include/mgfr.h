@@ -190,6 +190,9 @@ mgfr_status mgfr_set_config(mgfr_ctx* ctx, const mgfr_config* cfg);
  *   acc_out_dev [3][N^3] FP64 a_MG / c^2, or NULL.
  *   u_out_dev   [N^3] FP64 solution u, or NULL.
  *   st          statistics, or NULL.
+ * Precision FP64: u, e^u, the residual and the stopping test in FP64, each
+ * V-cycle's correction in FP32 (in FP64 where FP32 cannot resolve it).  Mixed:
+ * FP32 V-cycles, then the residual and u in pairs of floats (48 bits).
  * Returns MGFR_E_NOCONVERGE (outputs filled from the last iterate) when the
  * stopping test fails within max_vcycles.
  */
@@ -300,15 +303,19 @@ mgfr_status mgfr_effective_mass_pm(mgfr_ctx* ctx, int lpm, double* out_dev);
  *          potential is -(c^2/2) f_R up to a constant and discretisation),
  *          MGFR_PM_MATTER: the matter contrast delta (Newtonian gravity),
  *          MGFR_PM_TOTAL: delta + delta_eff (Eq. (30)).
- * The 7-point periodic Poisson problem is solved in FP64 by linear multigrid
- * V-cycles (cfg.n_pre / n_post red-black Gauss-Seidel sweeps, down to 4^3) to
- * ||rhs - lap phi||_2 <= cfg.tol_rel ||rhs||_2 (at most cfg.max_vcycles).
+ * The 7-point periodic Poisson problem is solved by linear multigrid V-cycles
+ * (cfg.n_pre / n_post red-black Gauss-Seidel sweeps, down to 4^3) to
+ * ||rhs - lap phi||_2 <= cfg.tol_rel ||rhs||_2 (at most cfg.max_vcycles).  phi and
+ * the residual of the stopping test are FP64; a cycle forms its correction in
+ * FP32, and the residual is carried between the cycles in pairs of floats (48
+ * bits).
  *   phi_out_dev  [N_pm^3] device FP64, C order (required).
  *   dens_out_dev [N_pm^3] device FP64: delta_pm, or NULL.
  *   st           vcycles, res_l2_init / final (of the scaled right-hand side),
  *                linear_updates, t_solve_ms; or NULL.
- * Workspace (three FP64 arrays of the PM grid and its coarse levels) is held
- * by the context.  MGFR_E_INVALID without a particle solve, for a bad lpm or
+ * The workspace (phi and the right-hand side in FP64, the low part of the residual,
+ * and two FP32 arrays of the PM grid and its coarse levels) is held by the
+ * context.  MGFR_E_INVALID without a particle solve, for a bad lpm or
  * what; MGFR_E_NOCONVERGE (phi filled) if the tolerance is not reached.
  */
 typedef enum { MGFR_PM_EFFECTIVE = 0, MGFR_PM_MATTER = 1, MGFR_PM_TOTAL = 2 } mgfr_pm_what;
@@ -321,7 +328,8 @@ mgfr_status mgfr_pm_potential(mgfr_ctx* ctx, int lpm, int what, double* phi_out_
  * grid (periodic) is interpolated to each particle with cloud-in-cell weights
  * of the PM grid (the 8 cells around x N_pm / box - 1/2).  With what =
  * MGFR_PM_TOTAL this is the long-range force of Eq. (30) including the
- * effective mass (Sec. 2.4); MGFR_PM_MATTER gives the Newtonian one.
+ * effective mass (Sec. 2.4); MGFR_PM_MATTER gives the Newtonian one.  The gradient's
+ * scaling and the interpolation run in pairs of floats (48 bits).
  *   pos_dev     [Np][3] FP64 comoving positions (Mpc/h), any values (wrapped).
  *   acc_out_dev [Np][3] FP64 -grad_x phi in (km/s)^2 per Mpc/h (the comoving
  *               gradient; the peculiar acceleration is this divided by a).
@@ -357,9 +365,11 @@ typedef struct {
 /*
  * Solve `nsolves` independent periodic grids of mixed sizes in ONE persistent
  * cooperative kernel launch (replayed from a CUDA graph): every solve runs the
- * mixed-precision form of mgfr_solve_density (FP32 FAS V-cycles, then FP64
- * residual with FP32 linear V-cycles on the Jacobian system) to
- * ||f - L(u)||_2 <= tol_rel ||f||_2.  Solves of different sizes share each
+ * mixed-precision form of mgfr_solve_density (FP32 FAS V-cycles, then a
+ * residual in pairs of floats, 48 bits, or for tol_rel < 1e-10 in FP64, with
+ * FP32 linear V-cycles on the Jacobian system) to
+ * ||f - L(u)||_2 <= tol_rel ||f||_2; at cfg.max_vcycles the outputs are those of
+ * the last iterate.  Solves of different sizes share each
  * V-cycle phase (aligned on grid size); phases are separated by a software
  * grid barrier whose waits are bounded by cfg.max_spins (MGFR_E_TIMEOUT if
  * one gives up; the context stays usable).  per_solve (nullable) receives one

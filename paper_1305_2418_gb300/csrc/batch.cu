@@ -368,10 +368,10 @@ __device__ __forceinline__ void load_modes(const BArgs& A, unsigned char* smode)
 // DF: the iterate of the defect correction in double-float pairs on the FP32
 // pipes (its residual took 43 FP64 instructions per cell); FP64 for tolerances
 // that come near the pairs' 48 bits.  Bound by issue slots (55% busy at 32
-// warps per SM; 64 registers, a few spilled, against one block of 128: 45 and
+// warps per SM; 64 registers, a few spilled, against one block of 128 per SM: 45 and
 // 50 ms).  96 solves of 32^3..128^3: 157 ms with one cell per thread in C order
 // (half of every line unused per half-sweep), FP64 residuals and a warp
-// reduction per 32 cells; 45 ms now.
+// reduction per 32 cells; 42 ms now.
 template <bool DF>
 __global__ void __launch_bounds__(512, 2) k_batch(BArgs A) {
   __shared__ unsigned char smode[kMaxBatch];

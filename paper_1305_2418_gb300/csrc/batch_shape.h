@@ -3,7 +3,8 @@
 // cells each).  Plain C++.
 //
 // Beyond 2^20 items the device is full either way and 512 threads x 2 per SM are the
-// fastest (96 solves of 32^3..128^3, ms: 45.0; 256 x 2 54.5, 256 x 3 47.1, 128 x 8 50.3),
+// fastest (96 solves of 32^3..128^3, ms, all on one build: 45.0; 256 x 2 54.5, 256 x 3
+// 47.1, 128 x 8 50.3; 42 for 512 x 2 now),
 // below it smaller blocks spread the items better (one 64^3 1.68 for 1.82, one 128^3 3.46
 // for 3.64).  A batch of few items is little but barriers, whose time grows with the
 // blocks that arrive at them: no more blocks than there are items for (and one per solve,

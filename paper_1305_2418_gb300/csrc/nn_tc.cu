@@ -213,8 +213,6 @@ __device__ __forceinline__ unsigned tc_nbr(unsigned m, int lgD, int dx, int dy, 
   return (((((b << lgD) + ((i + dx) & M)) << lgD) + ((j + dy) & M)) << lgD) + ((k + dz) & M);
 }
 
-// KC: channels of an A row (the reduction per tap); NC: output columns.
-// DGRAD: the input-gradient form (mirrored tap, FP32 output, optional add).
 // threads of a convolution CTA: two warps per scheduler, because staging the
 // operands is a chain of address arithmetic and copies per 16-byte chunk (with
 // four warps the 96 -> 32 halo kernel spent 20 of 27 us per CTA there)
@@ -258,6 +256,8 @@ __device__ __forceinline__ void store16(const float* v, long long m, int n0,
   }
 }
 
+// KC: channels of an A row (the reduction per tap); NC: output columns.
+// DGRAD: the input-gradient form (mirrored tap, FP32 output, optional add).
 template <int KC, int NC, bool DGRAD>
 __global__ void __launch_bounds__(HT) k_conv_tc(
     const __nv_bfloat16* __restrict__ x, int ldx, int offx, const __nv_bfloat16* __restrict__ Wp,
@@ -776,9 +776,9 @@ void launch_halo(const TcArgs& a, cudaStream_t s) {
 
 // The same halo-tiled form for layers whose 27 weight slices do not fit beside
 // the input block: the block stays resident while the taps' weight slices
-// stream through NS shared-memory stages (one bulk copy each).  Thread 0 alone
-// loads the slices and issues the MMAs, so the loop over taps has no block-wide
-// synchronisation.  A tap's MMAs take about 0.3 us and a copy's latency is 1 us:
+// stream through NS shared-memory stages (one bulk copy each).  One warp, by its
+// elected lane, loads the slices and issues the MMAs, so the loop over taps has no
+// block-wide synchronisation.  A tap's MMAs take about 0.3 us and a copy's latency is 1 us:
 // as many slices are in flight as the shared memory holds, up to 8 (with two,
 // 96 -> 32 waited for every slice: 110 us on 4 x 32^3).
 constexpr int halo_s_fit(int kc, int nc, int tx, int bytes) {
