@@ -38,11 +38,15 @@ int main() {
           // no more blocks per SM than the launch fills
           least = least && (r.per_sm == 1 || (long long)nsm * (r.per_sm - 1) < g);
         }
+  // one 8^3 and one 16^3: more than one block, 32 items in each
+  const BatchShape f = batch_rule(64, 1, 152), g = batch_rule(512, 1, 152);
+  const bool tiny = f.threads == 128 && batch_grid(f, 64, 1, 152) == 4 && g.threads == 128 &&
+                    batch_grid(g, 512, 1, 152) == 16;
   const BatchShape a = batch_rule(4096, 1, 152), b = batch_rule(32768, 1, 152),
                    d = batch_rule(24 * 32768, 24, 152), e = batch_rule(1 << 21, 96, 152);
-  const bool known = a.threads == 128 && batch_grid(a, 4096, 1, 152) == 64 && b.threads == 256 &&
+  const bool known = a.threads == 128 && batch_grid(a, 4096, 1, 152) == 128 && b.threads == 256 &&
                      batch_grid(b, 32768, 1, 152) == 128 && d.threads == 256 && d.per_sm == 3 &&
                      e.threads == 512 && e.per_sm == 2;
-  std::printf("%d %d %d %d %d %d\n", first, reached, once, spread, least, known);
+  std::printf("%d %d %d %d %d %d\n", first, reached, once, spread, least, known && tiny);
   return 0;
 }
